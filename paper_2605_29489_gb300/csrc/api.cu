@@ -768,14 +768,18 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
     o_est = slot(KG * 4);
     o_rank = slot(KG * 8);
   }
-  // the sampling CTAs' spans: up to 64 blocks of one trim group each
+  // the sampling CTAs' spans: up to span_blocks blocks of one trim group each, 64 for large
+  // families and as few as 8 (one per warp) for small ones, so that about 300 CTAs (two per
+  // SM) share the sample of a small family too
   std::vector<uint32_t> h_spans;
+  uint64_t span_blocks = 64;
+  while (span_blocks > 8 && g.n_blocks < span_blocks * 304) span_blocks /= 2;
   size_t o_shist = 0, o_scnt = 0, o_spans = 0;
   if (windowed) {
     for (uint32_t q = 0; q < n_groups; ++q) {
       const uint64_t b0 = scope == 0 ? g.t_first_block[q] : 0;
       const uint64_t b1 = scope == 0 ? (q + 1 < g.n_tensors ? g.t_first_block[q + 1] : g.n_blocks) : g.n_blocks;
-      for (uint64_t b = b0; b < b1; b += 64) {
+      for (uint64_t b = b0; b < b1; b += span_blocks) {
         h_spans.push_back(q);
         h_spans.push_back((uint32_t)b);
       }
@@ -843,6 +847,7 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
     p.scnt = (unsigned long long*)(m + o_scnt);
     p.samp_span = (const uint2*)(m + o_spans);
     p.n_samp_spans = (uint32_t)(h_spans.size() / 2);
+    p.samp_blocks = (uint32_t)span_blocks;
     if ((e = launch_fill(m + o_wfine, 0, o_wend - o_wfine, cs)) != cudaSuccess) return bail(e, "fill");
     if ((e = upload(ix, m + o_spans, h_spans.data(), h_spans.size() * 4, cs)) != cudaSuccess)
       return bail(e, "span copy");

@@ -727,31 +727,72 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
   }
 }
 
+// The k-th largest of the keys counted in h[0 .. 32 N), by one warp: lane l sums the N bins
+// that rank l-th from the top, a warp scan finds the lane where the running count reaches k,
+// and that lane walks its own bins.  True (on every lane) when h holds at least k keys; then
+// bin is the bin of the k-th largest and before the number of keys above it.  One thread
+// walking the bins waits for a load per bin: 256 to 384 of them took 30-46 us whatever the
+// number of pairs, this takes two.
+template <int N>
+__device__ __forceinline__ bool warp_kth(const unsigned long long* h, unsigned long long k, uint32_t& bin,
+                                         unsigned long long& before) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t top = 32u * N - 1u - lane * N;  // this lane's highest bin
+  unsigned long long c[N], sum = 0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    c[j] = h[top - j];
+    sum += c[j];
+  }
+  unsigned long long cum = sum;
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, cum, s);
+    if (lane >= (uint32_t)s) cum += o;
+  }
+  const uint32_t hit = __ballot_sync(0xFFFFFFFFu, cum >= k);
+  if (hit == 0u) return false;
+  const int src = __ffs(hit) - 1;
+  unsigned long long run = cum - sum;
+  uint32_t e = top;
+  bool done = false;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    if (!done && run + c[j] >= k) {
+      e = top - j;
+      done = true;
+    }
+    if (!done) run += c[j];
+  }
+  bin = __shfl_sync(0xFFFFFFFFu, e, src);
+  before = __shfl_sync(0xFFFFFFFFu, run, src);
+  return true;
+}
+
+// the pair (expert, trim group) of this warp in the select kernels, one warp each
+constexpr int kSelThreads = 128;
+__device__ __forceinline__ uint64_t select_pair() {
+  return (uint64_t)blockIdx.x * (kSelThreads / 32) + (threadIdx.x >> 5);
+}
+inline unsigned select_grid(uint64_t pairs) { return (unsigned)((pairs + kSelThreads / 32 - 1) / (kSelThreads / 32)); }
+
 // coarse select: bin e* of the upper 8 key bits holding the k-th largest key, and the
 // rank of that key inside the bin
-__global__ void ties_coarse_select(const IndexLaunch p) {
-  uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kSelThreads) ties_coarse_select(const IndexLaunch p) {
+  const uint64_t x = select_pair();
   if (x >= (uint64_t)p.K * p.n_groups) return;
   if (p.gmiss && p.gmiss[x] == 0u) return;  // its window already gave the threshold
-  uint32_t grp = (uint32_t)(x % p.n_groups);
-  unsigned long long k = p.kth[grp];
-  if (k == 0) {
-    p.estar[x] = kNoBin;
-    p.rank[x] = 0;
-    return;
+  const unsigned long long k = p.kth[x % p.n_groups];
+  uint32_t e = kNoBin;
+  unsigned long long before = 0, r = 0;
+  if (k != 0) {
+    if (!warp_kth<8>(p.coarse + x * 256u, k, e, before)) e = 0u;  // unreachable for k <= numel
+    r = k - before;
   }
-  const unsigned long long* h = p.coarse + x * 256u;
-  unsigned long long cum = 0;
-  for (int e = 255; e >= 0; --e) {
-    if (cum + h[e] >= k) {
-      p.estar[x] = (uint32_t)e;
-      p.rank[x] = k - cum;
-      return;
-    }
-    cum += h[e];
+  if ((threadIdx.x & 31u) == 0) {
+    p.estar[x] = e;
+    p.rank[x] = r;
   }
-  p.estar[x] = 0u;  // unreachable for k <= numel
-  p.rank[x] = k - cum;
 }
 
 template <bool BF16, int KG>
@@ -820,26 +861,19 @@ __global__ void __launch_bounds__(256) ties_fine_kernel(const IndexLaunch p) {
   }
 }
 
-__global__ void ties_fine_select(const IndexLaunch p) {
-  uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kSelThreads) ties_fine_select(const IndexLaunch p) {
+  const uint64_t x = select_pair();
   if (x >= (uint64_t)p.K * p.n_groups) return;
   if (p.gmiss && p.gmiss[x] == 0u) return;  // its window already gave the threshold
-  uint32_t es = p.estar[x];
-  if (es == kNoBin) {
-    p.tau[x] = kTauNone;
-    return;
+  const uint32_t es = p.estar[x];
+  uint32_t tau = kTauNone, m;
+  unsigned long long before;
+  if (es != kNoBin) {
+    // only bin 0 can fall short: its uncounted members are exact zeros, key 0
+    tau = es << 7;
+    if (warp_kth<4>(p.fine + x * 128u, p.rank[x], m, before)) tau |= m;
   }
-  const unsigned long long* f = p.fine + x * 128u;
-  unsigned long long r = p.rank[x], cum = 0;
-  for (int m = 127; m >= 0; --m) {
-    cum += f[m];
-    if (cum >= r) {
-      p.tau[x] = (es << 7) | (uint32_t)m;
-      return;
-    }
-  }
-  // only bin 0 can fall short: its uncounted members are exact zeros, key 0
-  p.tau[x] = es << 7;
+  if ((threadIdx.x & 31u) == 0) p.tau[x] = tau;
 }
 
 // TIES after masking: the coarse bins of (expert i, group) summed over a window of blocks:
@@ -872,10 +906,10 @@ __global__ void __launch_bounds__(256) ties_masked_coarse(const IndexLaunch p, u
 // ---- TIES thresholds with a predicted window ----------------------------------------------
 //
 // The threshold of a trim group is the k-th largest key of its deltas.  A sample predicts
-// the coarse bin e (upper 8 key bits) that holds it: from every block of the group, 32
-// vectors at jittered, evenly spaced positions (every vector of a block of at most 4096
-// elements), binned like the coarse catalog — every block contributes because the scale of
-// the deltas changes from block to block; e is the bin of the k_s-th largest sampled key,
+// the coarse bin e (upper 8 key bits) that holds it: from every block of the group, vectors at
+// jittered, evenly spaced positions (sample_vectors), binned like the coarse catalog — every
+// block contributes because the scale of the deltas changes from block to block; e is the bin
+// of the k_s-th largest sampled key,
 // k_s = max(1, floor(rho * sampled elements)).  The catalog pass then counts the 384 keys
 // of the window starting at L = 128 clamp(e - 1, 0, 253) at full resolution, plus the keys
 // above it, and ties_window_finish takes the threshold from those counts.  A pair whose
@@ -883,14 +917,24 @@ __global__ void __launch_bounds__(256) ties_masked_coarse(const IndexLaunch p, u
 // the marked pairs' groups, coarse select, fine pass, fine select) runs for the marked
 // pairs only; it does nothing when none is marked.  The prediction affects only which of
 // the two exact paths gives a threshold, never its value.
-constexpr uint32_t kSampleSpan = 64;  // blocks of one group per sampling CTA
+
+// Vectors sampled from a block of nvec vectors in a group of n_b blocks.  The window holds the
+// predicted binade and one on each side, so a few hundred vectors per group are enough: 8 of
+// each block in groups of 64 blocks or more, 32 in groups of 16 or more, up to 128 (every one
+// of a small tensor) in smaller groups.  Reading every vector of each block up to 4096 elements,
+// and 32 of larger ones, cost 241 us on 371 blocks of 4096 elements with 3 experts.
+constexpr uint32_t kSampleWide = 8;
+__device__ __forceinline__ uint32_t sample_vectors(uint32_t n_b, uint32_t nvec) {
+  const uint32_t want = n_b >= 64u ? kSampleWide : (n_b >= 16u ? 32u : 128u);
+  return min(want, nvec);
+}
 
 template <bool BF16, int KG>
 __global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
   constexpr uint32_t V = BF16 ? 8u : 4u;
   __shared__ uint32_t hist[KG][256];
   __shared__ unsigned long long s_n;  // sampled elements
-  const uint2 span = p.samp_span[blockIdx.x];  // {group, first block}: up to kSampleSpan blocks
+  const uint2 span = p.samp_span[blockIdx.x];  // {group, first block}: up to p.samp_blocks blocks
   const uint32_t g = span.x, i0 = blockIdx.y * KG;
   const uint32_t kc = min((uint32_t)KG, p.K - i0);
   if (kChecked && (g >= p.n_groups || i0 >= p.K)) {  // uniform over the CTA
@@ -901,19 +945,23 @@ __global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
   for (uint32_t x = tid; x < (uint32_t)KG * 256u; x += blockDim.x) (&hist[0][0])[x] = 0u;
   if (tid == 0) s_n = 0;
   __syncthreads();
-  const uint64_t gb1 = p.n_groups == 1 ? p.n_blocks : p.grp_blk0[g + 1];
-  const uint64_t b1 = min((uint64_t)span.y + kSampleSpan, gb1);
+  const uint64_t gb0 = p.n_groups == 1 ? 0 : p.grp_blk0[g], gb1 = p.n_groups == 1 ? p.n_blocks : p.grp_blk0[g + 1];
+  const uint64_t b1 = min((uint64_t)span.y + p.samp_blocks, gb1);
+  const uint32_t n_b = (uint32_t)min(gb1 - gb0, (uint64_t)0xFFFFFFFFu);
+  // a warp takes one block with 32 lanes, or (8 vectors each) four blocks with 8 lanes each
+  const bool wide = n_b >= 64u;
+  const uint32_t per_warp = wide ? 32u / kSampleWide : 1u, step = wide ? kSampleWide : 32u;
+  const uint32_t sub = wide ? lane / kSampleWide : 0u, l = wide ? lane % kSampleWide : lane;
   unsigned long long my_n = 0;
-  for (uint64_t b = span.y + warp; b < b1; b += 8) {
-    if (!checked_item<false>(p, b, i0, kc, BF16 ? 2u : 4u)) continue;  // uniform over the warp
+  for (uint64_t b = span.y + warp * per_warp + sub; b < b1; b += 8u * per_warp) {
+    if (!checked_item<false>(p, b, i0, kc, BF16 ? 2u : 4u)) continue;
     const uint32_t len = p.blk_len[b];
     const uint64_t off = p.blk_off[b];
     const uint32_t nvec = (len + V - 1) / V;
-    const bool every = len <= 4096u;
-    const uint32_t per = every ? 1u : nvec / 32u;
-    for (uint32_t v0 = lane; v0 < (every ? nvec : 32u); v0 += 32u) {
+    const uint32_t n_v = sample_vectors(n_b, nvec), per = nvec / n_v;
+    for (uint32_t v0 = l; v0 < n_v; v0 += step) {
       uint32_t v = v0;
-      if (!every) {  // a position in stretch v0 from a hash of (block, stretch)
+      if (n_v < nvec) {  // a position in stretch v0 from a hash of (block, stretch)
         uint32_t h = (uint32_t)b * 0x9E3779B1u ^ (v0 + 1u) * 0x85EBCA77u;
         h ^= h >> 15;
         h *= 0x2C1B3C6Du;
@@ -954,57 +1002,43 @@ __global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
 }
 
 // the window of each (expert, group) from its sampled coarse bins
-__global__ void ties_window_select(const IndexLaunch p) {
-  const uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kSelThreads) ties_window_select(const IndexLaunch p) {
+  const uint64_t x = select_pair();
   if (x >= (uint64_t)p.K * p.n_groups) return;
-  const uint32_t g = (uint32_t)(x % p.n_groups);
-  unsigned long long ks = (unsigned long long)floor((double)p.density * (double)p.scnt[g]);
+  unsigned long long ks = (unsigned long long)floor((double)p.density * (double)p.scnt[x % p.n_groups]), before;
   if (ks == 0) ks = 1;
-  const unsigned long long* h = p.shist + x * 256u;
   uint32_t e = 0;
-  unsigned long long cum = 0;
-  for (int j = 255; j >= 0; --j) {
-    cum += h[j];
-    if (cum >= ks) {
-      e = (uint32_t)j;
-      break;
-    }
-  }
+  if (!warp_kth<8>(p.shist + x * 256u, ks, e, before)) e = 0;  // fewer nonzero samples than k_s
   const uint32_t lo = e == 0 ? 0u : min(e - 1u, 253u);
-  p.wlo[x] = lo << 7;
+  if ((threadIdx.x & 31u) == 0) p.wlo[x] = lo << 7;
 }
 
 // the threshold of each (expert, group) from its window counts, or a mark for the
 // two-level select when it lies outside the window
-__global__ void ties_window_finish(const IndexLaunch p) {
-  const uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kSelThreads) ties_window_finish(const IndexLaunch p) {
+  const uint64_t x = select_pair();
   if (x >= (uint64_t)p.K * p.n_groups) return;
-  const uint32_t g = (uint32_t)(x % p.n_groups);
-  const unsigned long long k = p.kth[g];
-  if (k == 0) {
-    p.tau[x] = kTauNone;
-    return;
-  }
+  const unsigned long long k = p.kth[x % p.n_groups];
   const unsigned long long above = p.wabove[x];
   const uint32_t L = p.wlo[x];
-  if (above < k) {
-    const unsigned long long r = k - above;
-    const unsigned long long* f = p.wfine + x * kWinKeys;
-    unsigned long long cum = 0;
-    for (int j = (int)kWinKeys - 1; j >= 0; --j) {
-      cum += f[j];
-      if (cum >= r) {
-        p.tau[x] = L + (uint32_t)j;
-        return;
-      }
-    }
-    if (L == 0) {  // every uncounted delta is an exact zero, key 0
-      p.tau[x] = 0;
-      return;
+  uint32_t tau = kTauNone, j;
+  unsigned long long before;
+  bool miss = false;
+  if (k != 0) {
+    miss = above >= k;
+    if (!miss) {
+      if (warp_kth<(int)kWinKeys / 32>(p.wfine + x * kWinKeys, k - above, j, before)) tau = L + j;
+      else if (L == 0) tau = 0;  // every uncounted delta is an exact zero, key 0
+      else miss = true;
     }
   }
-  p.gmiss[x] = 1u;
-  atomicOr(p.miss, 1u);
+  if ((threadIdx.x & 31u) != 0) return;
+  if (miss) {
+    p.gmiss[x] = 1u;
+    atomicOr(p.miss, 1u);
+  } else {
+    p.tau[x] = tau;
+  }
 }
 
 // the TIES threshold from the coarse bins of the whole family: select the bin, count
@@ -1014,7 +1048,7 @@ template <bool BF16, int KG>
 cudaError_t ties_finish_t(const IndexLaunch& p, cudaStream_t st) {
   const uint32_t G = (p.K + KG - 1) / KG;
   const uint64_t nsel = (uint64_t)p.K * p.n_groups;
-  const unsigned sgrid = (unsigned)((nsel + 127) / 128);
+  const unsigned sgrid = select_grid(nsel);
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1025,9 +1059,9 @@ cudaError_t ties_finish_t(const IndexLaunch& p, cudaStream_t st) {
   uint64_t fgrid = (uint64_t)sms * (per_sm > 0 ? per_sm : 1);
   if (fgrid > p.n_blocks * G) fgrid = p.n_blocks * G;
   if (fgrid == 0) fgrid = 1;
-  ties_coarse_select<<<sgrid, 128, 0, st>>>(p);
+  ties_coarse_select<<<sgrid, kSelThreads, 0, st>>>(p);
   ties_fine_kernel<BF16, KG><<<(unsigned)fgrid, 256, 0, st>>>(p);
-  ties_fine_select<<<sgrid, 128, 0, st>>>(p);
+  ties_fine_select<<<sgrid, kSelThreads, 0, st>>>(p);
   count_launches(3);
   return cudaGetLastError();
 }
@@ -1074,11 +1108,11 @@ cudaError_t launch_t(const IndexLaunch& p, cudaStream_t st) {
   // two-level select for the pairs whose threshold left its window (a no-op when none did)
   const uint64_t nsel = (uint64_t)p.K * p.n_groups;
   ties_sample_kernel<BF16, KG><<<dim3(p.n_samp_spans, G), 256, 0, st>>>(p);
-  ties_window_select<<<(unsigned)((nsel + 127) / 128), 128, 0, st>>>(p);
+  ties_window_select<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
   count_launches(2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_pass<BF16, KG, kBinWindow>(p, G, n_items, sms, st)) != cudaSuccess) return e;
-  ties_window_finish<<<(unsigned)((nsel + 127) / 128), 128, 0, st>>>(p);
+  ties_window_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
   count_launches(1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, st)) != cudaSuccess) return e;
@@ -1091,7 +1125,7 @@ cudaError_t window_begin_t(const IndexLaunch& p, cudaStream_t st) {
   const uint64_t nsel = (uint64_t)p.K * p.n_groups;
   if (p.n_samp_spans == 0 || nsel == 0) return cudaSuccess;
   ties_sample_kernel<BF16, KG><<<dim3(p.n_samp_spans, G), 256, 0, st>>>(p);
-  ties_window_select<<<(unsigned)((nsel + 127) / 128), 128, 0, st>>>(p);
+  ties_window_select<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
   count_launches(2);
   return cudaGetLastError();
 }
@@ -1146,7 +1180,7 @@ cudaError_t launch_ties_window_end(const IndexLaunch& p, cudaStream_t st) {
   if (!p.wlo || !p.coarse) return cudaErrorInvalidValue;
   const uint64_t nsel = (uint64_t)p.K * p.n_groups;
   if (nsel == 0) return cudaSuccess;
-  ties_window_finish<<<(unsigned)((nsel + 127) / 128), 128, 0, st>>>(p);
+  ties_window_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
   count_launches(1);
   return cudaGetLastError();
 }

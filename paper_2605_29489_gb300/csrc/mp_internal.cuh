@@ -217,6 +217,7 @@ struct IndexLaunch {
   const uint32_t* grp_blk0;       // [n_groups + 1] first block of each trim group, then n_blocks
   const uint2* samp_span;         // [n_samp_spans] {group, first block} of each sampling CTA
   uint32_t n_samp_spans;
+  uint32_t samp_blocks;           // blocks per span at most
   unsigned long long* shist;      // [K][n_groups][256] coarse bins of the sampled deltas
   unsigned long long* scnt;       // [n_groups] sampled elements
   uint32_t* wlo;                  // [K][n_groups] first key L of the window
