@@ -1050,8 +1050,8 @@ mp_status mp_plan(const mp_index* index, const mp_op* op, uint64_t budget_bytes,
   put_u32(hdr, op->score_mode);
   const std::vector<uint8_t> order_key = hdr;  // everything the traversal order depends on
   put_u64(hdr, budget_bytes);
-  memcpy(p.hdr_prefix, hdr.data(), hdr.size());
-  p.hdr_prefix_len = (uint32_t)hdr.size();
+  p.digest_state = plan_digest_state(hdr.data(), hdr.size());
+  p.host_summary = pl->h_summary;
 
   // the first operator planned on this index leaves its traversal order behind; later
   // plans with the same operator start from it (the order is written once, by a launch
@@ -1072,8 +1072,6 @@ mp_status mp_plan(const mp_index* index, const mp_op* op, uint64_t budget_bytes,
         ixw->d_order_q = reinterpret_cast<unsigned long long*>(static_cast<char*>(ixw->order_mem.ptr) + align_up(U * 4));
         p.cache_order_out = ixw->d_order_cache;
         p.cache_q_out = ixw->d_order_q;
-        // an invalid count until the filling plan completes its sort
-        if ((e = launch_fill(ixw->d_order_q, 0xFF, 8, cs)) != cudaSuccess) return bail(e, "fill");
         fill = true;
       }
     }
@@ -1088,8 +1086,6 @@ mp_status mp_plan(const mp_index* index, const mp_op* op, uint64_t budget_bytes,
   }
   if ((e = cudaFreeAsync(scratch.ptr, cs)) != cudaSuccess) return bail(e, "free scratch");
   scratch.ptr = nullptr;
-  if ((e = launch_copy(pl->h_summary, pl->d_summary, 64, cs)) != cudaSuccess)
-    return bail(e, "summary copy");
   if ((e = cudaEventCreateWithFlags(&pl->done, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "event");
   if ((e = cudaEventRecord(pl->done, cs)) != cudaSuccess) return bail(e, "event record");
   *out = pl;

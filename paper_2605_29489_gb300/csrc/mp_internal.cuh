@@ -286,10 +286,11 @@ struct PlanLaunch {
   uint32_t* mask;
   uint32_t* order;
   uint64_t* summary;
-  // digest header fields (host-built, hashed on the device after C_hat is known)
-  uint8_t hdr_prefix[256];
-  uint32_t hdr_prefix_len;
+  uint64_t* host_summary;  // pinned host copy of the summary, or null
+  uint64_t digest_state;   // FNV-1a state after the digest header (plan_digest_state)
 };
+// FNV-1a 64 over the digest header (op, theta, B): the part of the digest known to the host
+uint64_t plan_digest_state(const uint8_t* header, size_t n);
 // scratch bytes the planner needs for n_units units and n_pairs (expert, tensor) pairs
 // (n_pairs = 0 without the tensor-level fallback)
 size_t plan_scratch_bytes(uint64_t n_units, uint64_t n_pairs);

@@ -1,8 +1,8 @@
-// Alg. 1 PlanGen on the device, as one cooperative persistent kernel.
+// Alg. 1 PlanGen on the device, as one persistent kernel.
 //
-// The grid's CTAs all stay resident (cooperative launch) and move through the phases
-// below together, separated by grid barriers whose waits are bounded.  Every phase
-// gives CTA c a contiguous slice of the data, so order is preserved wherever it matters.
+// The grid's CTAs all stay resident and move through the phases below together, separated by
+// grid-wide barriers.  Every phase gives warp w of CTA c a contiguous slice of the data, so
+// order is preserved wherever it matters.
 //
 //  0  tensor-level fallback (only for catalogs with entries lacking statistics, nnz =
 //     kNnzMissing): flag every (expert, tensor) pair holding one; then one warp per flagged
@@ -11,55 +11,65 @@
 //     The pair's unit is b0(t)*K + i; the tensor's other units are not candidates.
 //  A  score: unit u = b*K + i is a candidate iff nnz > 0 (TIES: and key(maxabs) >= tau);
 //     score = |coef_i| * norm (fp32), divided by the block's bytes in the score-per-byte
-//     mode; sort key = ~bits(score), so ascending key order is
-//     decreasing score.  Each CTA counts the candidates of its unit slice.
-//  B  stable compaction of the candidates in unit order (so equal scores stay in
-//     ascending unit order).
-//  C  stable LSD radix sort of (key, unit) pairs, four 8-bit digits; a digit that is the
-//     same for every key is skipped.  Stability plus the unit-ordered input gives the
-//     total order (score desc, unit asc).
+//     mode; sort key = ~bits(score), so ascending key order is decreasing score.  Each warp
+//     counts the lowest digit of its slice's candidate keys.
+//  C  stable LSD radix sort of (key, unit) pairs, four 8-bit digits; the first pass scatters
+//     the candidates straight from the unit order, so equal scores stay in ascending unit
+//     order; a later digit that is the same for every key is skipped.  A pass is two barriers:
+//     every warp counts its slice's digits, and after the barrier every CTA adds up the
+//     counts before its own and scatters.
 //  D  costs in that order: every position before the first prefix sum > B is selected.
 //  E  after that first overflow only candidates with cost <= the remaining budget R0 can
-//     ever be taken (R only shrinks): they are compacted, then one warp of CTA 0 runs the
-//     greedy with skip over them in order, from shared memory.
-//  F  the mask, the set hash and the count are scattered from the selected positions
-//     (a taken fallback unit sets its expert's bit in a per-tensor word, which the
-//     touched-block pass ORs into every block of the tensor); the last CTA computes the
-//     digest.
+//     ever be taken (R only shrinks): every CTA compacts those of its slice while the
+//     positions before the overflow enter the mask, the set hash and the counts; then CTA 0
+//     runs the greedy with skip over the compacted tail, in order, from shared memory.
+//     (A taken fallback unit sets its expert's bit in a per-tensor word, which a last pass
+//     ORs into every block of the tensor.)
+//  F  CTA 0 computes the digest and writes the summary, also to the host's pinned copy.
+//
+// What bounds it is latency: a plan of 62 K units touches about 2 MB, in 11 phases.  Two
+// launches of the same code: up to kClusterUnits units one thread-block cluster of up to 16 CTAs
+// of 1024 threads, whose barrier is the hardware's (about 1 us with what the writes before it
+// take, where the cooperative grid's in global memory takes 3 us) and whose CTAs read each
+// other's digit counts from shared memory; above, a cooperative grid of one 256-thread CTA per
+// SM, because a pass is then bound by the SMs' scattered stores.  Measured, first plan of an
+// index / later plan, us: 2,048 units 45 / 15 in the cluster, 80 / 20 in the grid; 62 K 65 / 22
+// and 82 / 23; 384 K 184 / 40 and 114 / 32.  (Before, as 21 phases of the grid alone, with a
+// compaction, a scan phase in every pass and one atomic ballot per taken tail candidate:
+// 119 / 35 at 2,048 units, 116 / 43 at 62 K, 180 / 70 at 384 K, 1124 / 348 at 3.9 M where it now
+// takes 750 / 160.)
 #include "mp_internal.cuh"
 
 namespace mp {
 namespace {
 
-constexpr int kPT = 256;            // threads per CTA
-constexpr uint32_t kMaxGrid = 1024;  // upper bound of the cooperative grid (scratch sizing)
-constexpr uint32_t kTailChunk = 4096;
+constexpr uint32_t kMaxGrid = 256;       // upper bound of the cooperative grid (scratch sizing)
+constexpr uint32_t kClusterMax = 16;     // CTAs of the cluster launch (non-portable size)
+constexpr int kClusterThreads = 1024;    // threads per CTA of the cluster launch
+constexpr int kGridThreads = 256;        // threads per CTA of the cooperative launch
+constexpr uint64_t kClusterUnits = 1ull << 17;  // most units planned by one cluster
 constexpr uint32_t kBarrierLimit = 1u << 24;
 
 // summary words (plan handle)
 enum { S_CHAT = 0, S_NSEL = 1, S_NCAND = 2, S_SETHASH = 3, S_DIGEST = 4, S_TOUCHED = 5, S_ERR = 6 };
 // scratch scalars
-enum { X_BAR_COUNT = 0, X_BAR_GEN = 1, X_P = 2, X_PBP = 3, X_TAILSUM = 4, X_DONE = 5, X_TOTAL = 6, X_MISSING = 7,
-       X_TAILMIN = 8, X_BADORDER = 9, X_COUNT = 16 };
+enum { X_BAR_COUNT = 0, X_BAR_GEN = 1, X_P = 2, X_PBP = 3, X_MISSING = 4, X_TAILMIN = 5, X_COUNT = 16 };
 
 constexpr unsigned long long kNoP = ~0ull;
 
 struct Scratch {
-  uint32_t* keys_a;             // [U]
-  uint32_t* keys_b;             // [U]
-  uint32_t* vals_b;             // [U]
-  uint32_t* tail_pos;           // [U]
-  unsigned long long* tail_cost;  // [U] costs of the compacted tail, in order
-  uint8_t* tailsel;             // [U]
-  uint32_t* hist;               // [256][kMaxGrid]
-  uint32_t* tot;                // [256]
+  uint2* kv_a;                  // [U] (key, unit) pairs of the sort: one scattered store each
+  uint2* kv_b;                  // [U]
+  uint32_t* tail_pos;           // [U] positions of the tail's candidates, compacted per CTA slice
+  unsigned long long* tail_cost;  // [U] their costs
+  uint32_t* hist;               // [kMaxGrid][256]
   unsigned long long* cta_a;    // [kMaxGrid]
   unsigned long long* cta_b;    // [kMaxGrid]
   unsigned long long* x;        // [X_COUNT]
-  uint32_t* pair_flag;          // [K * n_tensors] (fallback only; cleared by the host)
+  uint32_t* pair_flag;          // [K * n_tensors] (fallback only)
   uint32_t* pair_key;           // [K * n_tensors]
   unsigned long long* pair_cost;  // [K * n_tensors]
-  uint32_t* sel_bits;           // [n_tensors] experts whose fallback unit of the tensor was taken (cleared by the host)
+  uint32_t* sel_bits;           // [n_tensors] experts whose fallback unit of the tensor was taken
 };
 
 inline size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -69,14 +79,11 @@ size_t carve(void* base, uint64_t U, uint64_t n_pairs, Scratch* s) {
   size_t o = 0;
   auto take = [&](size_t bytes) { char* r = p + o; o += align_up(bytes); return r; };
   Scratch t;
-  t.keys_a = (uint32_t*)take(U * 4);
-  t.keys_b = (uint32_t*)take(U * 4);
-  t.vals_b = (uint32_t*)take(U * 4);
+  t.kv_a = (uint2*)take(U * 8);
+  t.kv_b = (uint2*)take(U * 8);
   t.tail_pos = (uint32_t*)take(U * 4);
   t.tail_cost = (unsigned long long*)take(U * 8);
-  t.tailsel = (uint8_t*)take(U);
   t.hist = (uint32_t*)take((size_t)256 * kMaxGrid * 4);
-  t.tot = (uint32_t*)take(256 * 4);
   t.cta_a = (unsigned long long*)take(kMaxGrid * 8);
   t.cta_b = (unsigned long long*)take(kMaxGrid * 8);
   t.x = (unsigned long long*)take(X_COUNT * 8);
@@ -107,7 +114,7 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned long long* p) {
   return (unsigned)v;
 }
 
-// grid barrier: the last CTA to arrive bumps the generation; the others wait for it with
+// barrier of the cooperative grid: the last CTA to arrive bumps the generation; the others wait for it with
 // a bounded number of polls.  Returns false (uniformly inside the CTA) if the wait expired.
 __device__ __forceinline__ bool grid_sync(unsigned long long* x, unsigned& gen, uint64_t* summary) {
   __shared__ int s_ok;
@@ -139,10 +146,28 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* x, unsigned& gen, 
   return s_ok != 0;
 }
 
-// block-wide exclusive scan (256 threads) with total
-template <typename T>
+// barrier of the cluster: every thread arrives, and what any of them wrote before is visible
+// to all of them after
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// the barrier between phases; false (uniformly inside the CTA) when the wait expired
+template <bool CL>
+__device__ __forceinline__ bool phase_sync(unsigned long long* x, unsigned& gen, uint64_t* summary) {
+  if constexpr (CL) {
+    cluster_sync();
+    return true;
+  } else {
+    return grid_sync(x, gen, summary);
+  }
+}
+
+// block-wide exclusive scan (PT threads) with total
+template <int PT, typename T>
 __device__ __forceinline__ T block_scan(T v, T& total) {
-  __shared__ T s_w[kPT / 32];
+  __shared__ T s_w[PT / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   T x = v;
 #pragma unroll
@@ -153,48 +178,60 @@ __device__ __forceinline__ T block_scan(T v, T& total) {
   if (lane == 31) s_w[warp] = x;
   __syncthreads();
   if (warp == 0) {
-    T t = lane < kPT / 32 ? s_w[lane] : T(0);
+    T t = lane < PT / 32 ? s_w[lane] : T(0);
 #pragma unroll
-    for (int s = 1; s < kPT / 32; s <<= 1) {
+    for (int s = 1; s < PT / 32; s <<= 1) {
       T y = __shfl_up_sync(0xFFFFFFFFu, t, s);
       if (lane >= s) t += y;
     }
-    if (lane < kPT / 32) s_w[lane] = t;
+    if (lane < PT / 32) s_w[lane] = t;
   }
   __syncthreads();
   const T before = warp > 0 ? s_w[warp - 1] : T(0);
-  total = s_w[kPT / 32 - 1];
+  total = s_w[PT / 32 - 1];
   __syncthreads();
   return before + x - v;
 }
 
-template <typename T>
+template <int PT, typename T>
 __device__ __forceinline__ T block_sum(T v) {
   T t;
-  block_scan<T>(v, t);
+  block_scan<PT, T>(v, t);
   return t;
 }
 
-// sum of a[0..n) (n <= kMaxGrid), computed by the whole CTA
-__device__ __forceinline__ unsigned long long block_sum_prefix(const unsigned long long* a, uint32_t n) {
-  unsigned long long s = 0;
-  for (uint32_t k = threadIdx.x; k < n; k += kPT) s += a[k];
-  return block_sum<unsigned long long>(s);
+// sums of a[0..c) and a[0..n), by every warp for itself
+__device__ __forceinline__ unsigned long long warp_prefix(const unsigned long long* a, uint32_t c, uint32_t n,
+                                                          unsigned long long& total) {
+  unsigned long long t = 0, v = 0;
+  for (uint32_t k = threadIdx.x & 31u; k < n; k += 32) {
+    const unsigned long long x = a[k];
+    t += x;
+    v += k < c ? x : 0ull;
+  }
+#pragma unroll
+  for (int sh = 16; sh > 0; sh >>= 1) {
+    t += __shfl_xor_sync(0xFFFFFFFFu, t, sh);
+    v += __shfl_xor_sync(0xFFFFFFFFu, v, sh);
+  }
+  total = t;
+  return v;
 }
 
 struct Unit {
   bool cand;
   uint32_t key;
+  bool missing;  // no statistics and no fallback
 };
 
-__device__ __forceinline__ Unit score_unit(const PlanLaunch& p, const Scratch& s, uint64_t u) {
-  const uint64_t b = u / p.K;
-  const uint32_t i = (uint32_t)(u % p.K);
+__device__ __forceinline__ Unit score_unit(const PlanLaunch& p, const Scratch& s, uint32_t u) {
+  const uint32_t b = u / p.K;
+  const uint32_t i = u - b * p.K;
   const uint64_t st = (uint64_t)i * p.n_blocks + b;
   if (p.fallback) {
     const uint32_t t = p.blk_tensor[b];
     const uint32_t pr = i * p.n_tensors + t;
-    if (s.pair_flag[pr]) return Unit{b == p.t_blk0[t], s.pair_key[pr]};
+    if (s.pair_flag[pr]) return Unit{b == p.t_blk0[t], s.pair_key[pr], false};
   }
   const uint32_t nz = p.nnz[st];
   bool cand = nz != 0u && nz != kNnzMissing;
@@ -203,7 +240,7 @@ __device__ __forceinline__ Unit score_unit(const PlanLaunch& p, const Scratch& s
   float score = __fmul_rn(p.coef[i], p.norm[st]);
   // score per byte: one IEEE division by the block's byte cost (exact in fp32, <= 2^20)
   if (p.score_mode) score = __fdiv_rn(score, (float)(p.blk_len[b] * p.elem_size));
-  return Unit{cand, ~__float_as_uint(score)};
+  return Unit{cand, ~__float_as_uint(score), !p.fallback && nz == kNnzMissing};
 }
 
 __device__ __forceinline__ unsigned long long unit_cost(const PlanLaunch& p, const Scratch& s, uint32_t u) {
@@ -263,361 +300,495 @@ __device__ __forceinline__ void fallback_pair(const PlanLaunch& p, const Scratch
   }
 }
 
-__device__ __forceinline__ void slice(uint64_t n, uint64_t& a, uint64_t& b) {
-  a = n * blockIdx.x / gridDim.x;
-  b = n * (blockIdx.x + 1) / gridDim.x;
+// elements of n that each warp of the grid takes: whole tiles of 32, so that few lanes idle
+template <int PT>
+__device__ __forceinline__ uint32_t slice_len(uint32_t n) {
+  const uint32_t parts = gridDim.x * (PT / 32);
+  const uint32_t tiles = n / 32u + (n % 32u ? 1u : 0u);
+  return (tiles / parts + (tiles % parts ? 1u : 0u)) * 32u;
 }
 
-__global__ void __launch_bounds__(kPT) plan_kernel(const PlanLaunch p, Scratch s) {
-  __shared__ uint32_t s_run[256];
-  __shared__ uint32_t s_wcnt[kPT / 32][256];
-  __shared__ unsigned long long s_cost[kTailChunk];
-  __shared__ unsigned long long s_bcast[1];
+// the first element of slice k of n elements cut into slices of len
+__device__ __forceinline__ uint32_t slice_begin(uint32_t n, uint32_t len, uint32_t k) {
+  return (uint32_t)min((uint64_t)len * k, (uint64_t)n);
+}
+
+// what a thread has put into the mask: added up over the CTA by add_selected
+struct Selected {
+  unsigned long long hash = 0, n = 0, touched = 0;
+};
+
+__device__ __forceinline__ void select_unit(const PlanLaunch& p, const Scratch& s, uint32_t u, Selected& sel) {
+  if (kChecked && (uint64_t)u >= p.n_blocks * p.K) {  // checked build: a unit id past U
+    atomicOr((unsigned long long*)&p.summary[S_ERR], (unsigned long long)kErrBounds);
+    return;
+  }
+  const uint32_t b = u / p.K, i = u - b * p.K;
+  const uint32_t t = p.fallback ? p.blk_tensor[b] : 0u;
+  if (p.fallback && s.pair_flag[i * p.n_tensors + t]) {
+    atomicOr(&s.sel_bits[t], 1u << i);  // every block of t gets bit i in the last pass
+  } else {
+    sel.touched += atomicOr(&p.mask[b], 1u << i) == 0u ? 1ull : 0ull;
+  }
+  sel.hash += splitmix64(u);
+  ++sel.n;
+}
+
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
+#pragma unroll
+  for (int sh = 16; sh > 0; sh >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, sh);
+  return v;
+}
+
+// adds a CTA's selections to the summary (the last pass counts the touched blocks when
+// fallback units put whole tensors into the mask)
+template <int PT>
+__device__ __forceinline__ void add_selected(const PlanLaunch& p, const Selected& sel) {
+  __shared__ unsigned long long s_sel[3][PT / 32];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const unsigned long long v[3] = {warp_sum(sel.hash), warp_sum(sel.n), warp_sum(sel.touched)};
+  if (lane < 3) s_sel[lane][warp] = lane == 0 ? v[0] : (lane == 1 ? v[1] : v[2]);
+  __syncthreads();
+  if (warp >= 3) return;  // warp k adds up value k
+  const unsigned long long t = warp_sum(lane < PT / 32 ? s_sel[warp][lane] : 0ull);
+  if (lane != 0 || t == 0) return;
+  if (warp == 0) atomicAdd((unsigned long long*)&p.summary[S_SETHASH], t);
+  else if (warp == 1) atomicAdd((unsigned long long*)&p.summary[S_NSEL], t);
+  else if (!p.fallback) atomicAdd((unsigned long long*)&p.summary[S_TOUCHED], t);
+}
+
+// inclusive scan over the warp
+__device__ __forceinline__ unsigned long long warp_scan(unsigned long long v, uint32_t lane) {
+#pragma unroll
+  for (int sh = 1; sh < 32; sh <<= 1) {
+    const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, v, sh);
+    if ((int)lane >= sh) v += o;
+  }
+  return v;
+}
+
+// lanes of `who` whose digit d (8 bits) equals this lane's
+__device__ __forceinline__ uint32_t same_digit(uint32_t d, uint32_t who) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const bool bit = (d >> k) & 1u;
+    const uint32_t v = __ballot_sync(0xFFFFFFFFu, bit);
+    who &= bit ? v : ~v;
+  }
+  return who;
+}
+
+// the digit counts of CTA g of the cluster, in its shared memory
+__device__ __forceinline__ uint32_t peer_count(const uint32_t* own, uint32_t g) {
+  uint32_t a, v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(own)), "r"(g));
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+
+template <int PT, bool CL>
+__global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch s) {
+  constexpr int W = PT / 32;
+  constexpr uint32_t kTailChunk = W * 128;  // tail costs held at once, in the digit counters' memory
+  constexpr int kHold = 4;                  // tiles of a warp's slice whose keys stay in registers
+  __shared__ __align__(16) uint32_t s_cnt[W][256];
+  __shared__ uint32_t s_hist[256];
+  __shared__ unsigned long long s_wsum[W];
+  __shared__ uint32_t s_take[kTailChunk / 32];
+  __shared__ uint32_t s_pre[kMaxGrid + 1];
+  __shared__ unsigned long long s_bcast;
+  unsigned long long* s_cost = reinterpret_cast<unsigned long long*>(&s_cnt[0][0]);
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t G = gridDim.x, c = blockIdx.x;
-  const uint64_t U = (uint64_t)p.K * p.n_blocks;
+  const uint32_t gt = c * PT + tid, gn = G * PT;  // this thread of the grid's threads
+  const uint32_t gw = c * W + warp;               // this warp of the grid's warps
+  const uint32_t U = (uint32_t)((uint64_t)p.K * p.n_blocks);  // below 2^32 (launch_plan)
+  const uint32_t lt = (1u << lane) - 1u;
   unsigned gen = 0;
 
-  // ---- zero the outputs; A: count the candidates of this CTA's unit slice ----
-  for (uint64_t k = (uint64_t)c * kPT + tid; k < p.n_blocks; k += (uint64_t)G * kPT) p.mask[k] = 0u;
-  for (uint64_t k = (uint64_t)c * kPT + tid; k < U; k += (uint64_t)G * kPT) s.tailsel[k] = 0;
+  // ---- zero the outputs and the scalars (first used after a barrier) ----
+  for (uint64_t k = gt; k < p.n_blocks; k += gn) p.mask[k] = 0u;
   if (c == 0 && tid < 8) p.summary[tid] = 0;
   if (c == 0 && tid == 0) {
     s.x[X_P] = kNoP;
     s.x[X_TAILMIN] = ~0ull;
+    s.x[X_MISSING] = 0;
+    if (p.cache_q_out) *p.cache_q_out = ~0ull;  // an invalid count until the sort is complete
   }
-  uint64_t Q = 0, q0 = 0, q1 = 0;
+  bool bad_order = false, miss = false;
+  uint32_t Q = 0, len = 0, a = 0, b = 0;  // candidates; this warp's slice [a, b) of them
+  auto own_slice = [&](uint32_t q) {
+    Q = q;
+    len = slice_len<PT>(q);
+    a = slice_begin(q, len, gw);
+    b = slice_begin(q, len, gw + 1);
+  };
   if (p.cache_q_in) {
     // the candidates in traversal order from an earlier plan of this index and operator:
     // phases 0 to C depend on the operator and the catalog, not on the budget
-    Q = *p.cache_q_in;
-    if (Q > U) {  // the plan that was to leave the order did not finish: report, plan nothing
-      if (c == 0 && tid == 0) s.x[X_BADORDER] = 1ull;
-      Q = 0;
-    }
-    slice(Q, q0, q1);
-    for (uint64_t j = q0 + tid; j < q1; j += kPT) p.order[j] = p.cache_order_in[j];
-    if (!grid_sync(s.x, gen, p.summary)) return;
+    const unsigned long long q = *p.cache_q_in;
+    bad_order = q > U;  // the plan that was to leave the order did not finish: report, plan nothing
+    own_slice(bad_order ? 0u : (uint32_t)q);
+    for (uint64_t j = a + lane; j < b; j += 32) p.order[j] = p.cache_order_in[j];
+    __syncwarp();  // the warp reads its own slice of the order below
   } else {
-    uint64_t u0, u1;
-    slice(U, u0, u1);
+    const uint32_t ul = slice_len<PT>(U), ua = slice_begin(U, ul, gw), ub = slice_begin(U, ul, gw + 1);
     if (p.fallback) {
+      const uint32_t n_pairs = p.K * p.n_tensors;
+      for (uint32_t k = gt; k < n_pairs; k += gn) s.pair_flag[k] = 0u;
+      for (uint32_t k = gt; k < p.n_tensors; k += gn) s.sel_bits[k] = 0u;
+      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
       // 0a: flag the pairs holding an entry without statistics (one atomic per pair and warp)
-      for (uint64_t t0 = u0; t0 < u1; t0 += kPT) {
-        const uint64_t u = t0 + tid;
+      for (uint64_t t0 = ua; t0 < ub; t0 += 32) {
+        const uint64_t u = t0 + lane;
         uint32_t pr = 0xFFFFFFFFu;
-        if (u < u1) {
-          const uint64_t b = u / p.K;
-          const uint32_t i = (uint32_t)(u % p.K);
-          if (p.nnz[(uint64_t)i * p.n_blocks + b] == kNnzMissing) pr = i * p.n_tensors + p.blk_tensor[b];
+        if (u < ub) {
+          const uint32_t bb = (uint32_t)u / p.K, i = (uint32_t)u - bb * p.K;
+          if (p.nnz[(uint64_t)i * p.n_blocks + bb] == kNnzMissing) pr = i * p.n_tensors + p.blk_tensor[bb];
         }
         const uint32_t peers = __match_any_sync(0xFFFFFFFFu, pr);
         if (pr != 0xFFFFFFFFu && lane == (uint32_t)(__ffs(peers) - 1)) atomicOr(&s.pair_flag[pr], 1u);
       }
-      if (!grid_sync(s.x, gen, p.summary)) return;
+      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
       // 0b: the flagged pairs' units, one warp each
-      const uint32_t n_pairs = p.K * p.n_tensors, nw = G * (kPT / 32);
-      for (uint32_t pr = c * (kPT / 32) + warp; pr < n_pairs; pr += nw)
+      for (uint32_t pr = gw; pr < n_pairs; pr += G * W)
         if (s.pair_flag[pr]) fallback_pair(p, s, pr, lane);
-      if (!grid_sync(s.x, gen, p.summary)) return;
+      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
     }
-    {
-      // without the fallback an entry lacking statistics cannot be planned: it is reported
-      unsigned long long cnt = 0;
-      bool miss = false;
-      for (uint64_t u = u0 + tid; u < u1; u += kPT) {
-        cnt += score_unit(p, s, u).cand ? 1ull : 0ull;
-        miss |= !p.fallback && p.nnz[(u % p.K) * p.n_blocks + u / p.K] == kNnzMissing;
-      }
-      if (__syncthreads_or(miss) && tid == 0) s.x[X_MISSING] = 1ull;
-      cnt = block_sum<unsigned long long>(cnt);
-      if (tid == 0) s.cta_a[c] = cnt;
-    }
-    if (!grid_sync(s.x, gen, p.summary)) return;
 
-    // ---- B: stable compaction into (keys_a, order) ----
-    {
-      const unsigned long long before = block_sum_prefix(s.cta_a, c);
-      Q = block_sum_prefix(s.cta_a, G);
-      unsigned long long run = before;
-      for (uint64_t t0 = u0; t0 < u1; t0 += kPT) {
-        const uint64_t u = t0 + tid;
-        Unit x = u < u1 ? score_unit(p, s, u) : Unit{false, 0u};
-        uint32_t tot;
-        const uint32_t pos = block_scan<uint32_t>(x.cand ? 1u : 0u, tot);
-        if (x.cand) {
-          if (kChecked && run + pos >= p.n_blocks * p.K) {  // checked build: a compaction slot past U
-            atomicOr((unsigned long long*)&p.summary[S_ERR], (unsigned long long)kErrBounds);
-          } else {
-            s.keys_a[run + pos] = x.key;
-            p.order[run + pos] = (uint32_t)u;
-          }
-        }
-        run += tot;
-      }
-    }
-    if (!grid_sync(s.x, gen, p.summary)) return;
-
-    // ---- C: stable LSD radix sort, 8-bit digits ----
-    uint32_t *kin = s.keys_a, *vin = p.order, *kout = s.keys_b, *vout = s.vals_b;
-    slice(Q, q0, q1);
+    // ---- A and C: candidates, then a stable LSD radix sort by 8-bit digits ----
+    // Pass 0 takes the candidates of this warp's slice of the units, later passes its slice of
+    // the pass before; the first kHold tiles' keys stay in registers from count to scatter.
+    const uint2* in = nullptr;
+    uint2* out = s.kv_a;
+    bool ordered = false;  // the last pass has put the units into p.order
     for (uint32_t pass = 0; pass < 4; ++pass) {
       const uint32_t shift = 8u * pass;
-      // C1: digit histogram of this CTA's slice
-      s_run[tid] = 0;
-      __syncthreads();
-      for (uint64_t j = q0 + tid; j < q1; j += kPT) atomicAdd(&s_run[(kin[j] >> shift) & 255u], 1u);
-      __syncthreads();
-      s.hist[(uint64_t)tid * G + c] = s_run[tid];
-      if (!grid_sync(s.x, gen, p.summary)) return;
-      // C2: per digit, exclusive prefix over the CTAs (one warp per digit) and the total
-      for (uint32_t d = c + warp * G; d < 256u; d += (kPT / 32) * G) {
-        uint32_t* h = s.hist + (uint64_t)d * G;
-        uint32_t carry = 0;
-        for (uint32_t k0 = 0; k0 < G; k0 += 32) {
-          const uint32_t v = k0 + lane < G ? h[k0 + lane] : 0u;
-          uint32_t x = v;
-  #pragma unroll
-          for (int sh = 1; sh < 32; sh <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, sh);
-            if ((int)lane >= sh) x += y;
-          }
-          if (k0 + lane < G) h[k0 + lane] = carry + x - v;
-          carry += __shfl_sync(0xFFFFFFFFu, x, 31);
+      const uint64_t r0 = pass == 0 ? ua : a, r1 = pass == 0 ? ub : b;
+      auto load = [&](uint64_t j, uint32_t& key, uint32_t& val) -> bool {  // false: no candidate
+        if (j >= r1) return false;
+        if (pass > 0) {
+          const uint2 kv = in[j];
+          key = kv.x;
+          val = kv.y;
+          return true;
         }
-        if (lane == 0) s.tot[d] = carry;
+        const Unit x = score_unit(p, s, (uint32_t)j);
+        // without the fallback an entry lacking statistics cannot be planned: it is reported
+        miss |= x.missing;
+        key = x.key;
+        val = (uint32_t)j;
+        return x.cand;
+      };
+      for (uint32_t k = lane; k < 256u; k += 32) s_cnt[warp][k] = 0u;
+      __syncwarp();
+      uint32_t hk[kHold], hv[kHold];
+      uint32_t hvalid = 0u;
+#pragma unroll
+      for (int t = 0; t < kHold; ++t)
+        if (load(r0 + 32u * t + lane, hk[t], hv[t])) hvalid |= 1u << t;
+#pragma unroll
+      for (int t = 0; t < kHold; ++t)
+        if ((hvalid >> t) & 1u) atomicAdd(&s_cnt[warp][(hk[t] >> shift) & 255u], 1u);
+#pragma unroll 4
+      for (uint64_t j = r0 + 32u * kHold + lane; j < r1; j += 32) {
+        uint32_t key, val;
+        if (load(j, key, val)) atomicAdd(&s_cnt[warp][(key >> shift) & 255u], 1u);
       }
-      if (!grid_sync(s.x, gen, p.summary)) return;
-      // C3: digit starts; skip the pass if one digit holds every key; stable scatter
+      __syncthreads();
+      if (tid < 256u) {
+        uint32_t n = 0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) n += s_cnt[w][tid];
+        if constexpr (CL) s_hist[tid] = n;
+        else s.hist[(uint64_t)c * 256u + tid] = n;
+      }
+      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+      // digit starts, the counts of the CTAs before this one, then each warp's start
+      uint32_t before = 0, tot = 0;
+      if (tid < 256u) {
+#pragma unroll 8
+        for (uint32_t g = 0; g < G; ++g) {
+          const uint32_t v = CL ? peer_count(&s_hist[tid], g) : s.hist[(uint64_t)g * 256u + tid];
+          before += g < c ? v : 0u;
+          tot += v;
+        }
+      }
       uint32_t total;
-      const uint32_t t_d = s.tot[tid];
-      const uint32_t start = block_scan<uint32_t>(t_d, total);
-      const bool skip = __syncthreads_or(t_d == (uint32_t)Q && Q > 0) != 0 || Q == 0;
-      if (skip) continue;  // uniform over the grid: every CTA reads the same totals
-      s_run[tid] = start + s.hist[(uint64_t)tid * G + c];
-      const uint32_t lt = (1u << lane) - 1u;
-      for (uint64_t t0 = q0; t0 < q1; t0 += kPT) {
-        for (int w = 0; w < kPT / 32; ++w) s_wcnt[w][tid] = 0;
-        __syncthreads();
-        const uint64_t j = t0 + tid;
-        const bool valid = j < q1;
-        const uint32_t key = valid ? kin[j] : 0u;
-        const uint32_t val = valid ? vin[j] : 0u;
-        const uint32_t d = valid ? ((key >> shift) & 255u) : 256u;
-        const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
-        const uint32_t rank = __popc(peers & lt);
-        if (valid && rank == 0) s_wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        {
-          uint32_t acc = s_run[tid];
-          for (int w = 0; w < kPT / 32; ++w) {
-            const uint32_t cw = s_wcnt[w][tid];
-            s_wcnt[w][tid] = acc;
-            acc += cw;
-          }
-          s_run[tid] = acc;
-        }
-        __syncthreads();
-        if (valid) {
-          const uint32_t pos = s_wcnt[warp][d] + rank;
-          kout[pos] = key;
-          vout[pos] = val;
-        }
-        __syncthreads();  // every warp has read its offsets before the next tile clears them
+      const uint32_t start = block_scan<PT, uint32_t>(tot, total);
+      if (pass == 0) {
+        if (miss) s.x[X_MISSING] = 1ull;  // cleared before the barrier
+        own_slice(total);
       }
-      if (!grid_sync(s.x, gen, p.summary)) return;
-      uint32_t* t;
-      t = kin, kin = kout, kout = t;
-      t = vin, vin = vout, vout = t;
+      // one digit holds every key: nothing moves (uniform over the grid: the same totals)
+      if (pass > 0 && (__syncthreads_or(tid < 256u && tot == Q) != 0 || Q == 0)) {
+        if (!phase_sync<CL>(s.x, gen, p.summary)) return;  // every CTA has read the counts
+        continue;
+      }
+      if (tid < 256u) {
+        uint32_t acc = start + before;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          const uint32_t n = s_cnt[w][tid];
+          s_cnt[w][tid] = acc;
+          acc += n;
+        }
+      }
+      __syncthreads();
+      auto scatter = [&](bool valid, uint32_t key, uint32_t val) {
+        const uint32_t d = (key >> shift) & 255u;
+        const uint32_t peers = same_digit(d, __ballot_sync(0xFFFFFFFFu, valid));
+        const uint32_t rank = __popc(peers & lt);
+        const uint32_t pos = valid ? s_cnt[warp][d] + rank : 0u;
+        __syncwarp();
+        if (valid && rank == 0) s_cnt[warp][d] = pos + __popc(peers);
+        __syncwarp();
+        if (!valid) return;
+        if (kChecked && pos >= U) {  // checked build: a slot past U
+          atomicOr((unsigned long long*)&p.summary[S_ERR], (unsigned long long)kErrBounds);
+          return;
+        }
+        if (pass < 3) out[pos] = make_uint2(key, val);
+        else p.order[pos] = val;  // nobody reads the keys after the last pass
+      };
+#pragma unroll
+      for (int t = 0; t < kHold; ++t)
+        if (r0 + 32u * t < r1) scatter((hvalid >> t) & 1u, hk[t], hv[t]);  // uniform over the warp
+      for (uint64_t t0 = r0 + 32u * kHold; t0 < r1; t0 += 32) {
+        uint32_t key = 0u, val = 0u;
+        const bool valid = load(t0 + lane, key, val);
+        scatter(valid, key, val);
+      }
+      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+      ordered = pass == 3;
+      in = out;
+      out = in == s.kv_a ? s.kv_b : s.kv_a;
     }
-    // the sorted units end in p.order, or in vals_b if an odd number of passes ran (a
-    // uniform fact: every CTA made the same skip decisions)
-    if (vin != p.order) {
-      for (uint64_t j = q0 + tid; j < q1; j += kPT) p.order[j] = vin[j];
-      if (!grid_sync(s.x, gen, p.summary)) return;
-    }
+    // the sorted units are in p.order unless the last pass was skipped (a uniform fact: every
+    // CTA made the same skip decisions)
+    if (!ordered)
+      for (uint64_t j = a + lane; j < b; j += 32) p.order[j] = in[j].y;
     if (p.cache_order_out) {  // keep the order for later plans with the same operator
-      for (uint64_t j = q0 + tid; j < q1; j += kPT) p.cache_order_out[j] = p.order[j];
-      if (c == 0 && tid == 0) *p.cache_q_out = Q;
+      for (uint64_t j = a + lane; j < b; j += 32) p.cache_order_out[j] = ordered ? p.order[j] : in[j].y;
+      if (gt == 0) *p.cache_q_out = Q;
     }
+    __syncwarp();  // the warp reads its own slice of the order below
   }
   const uint32_t* order = p.order;
 
   // ---- D: cost prefix in sorted order; the first position where it exceeds B ----
   {
     unsigned long long sum = 0;
-    for (uint64_t j = q0 + tid; j < q1; j += kPT) sum += unit_cost(p, s, order[j]);
-    sum = block_sum<unsigned long long>(sum);
-    if (tid == 0) s.cta_b[c] = sum;
+#pragma unroll 4
+    for (uint64_t j = a + lane; j < b; j += 32) sum += unit_cost(p, s, order[j]);
+    sum = warp_sum(sum);
+    if (lane == 0) s_wsum[warp] = sum;
+    __syncthreads();
+    if (warp == 0) {
+      const unsigned long long t = warp_sum(lane < W ? s_wsum[lane] : 0ull);
+      if (lane == 0) s.cta_b[c] = t;
+    }
   }
-  if (!grid_sync(s.x, gen, p.summary)) return;
+  if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+  unsigned long long total_cost;
   {
-    unsigned long long run = block_sum_prefix(s.cta_b, c);
-    const unsigned long long total_cost = block_sum_prefix(s.cta_b, G);
-    if (c == 0 && tid == 0) s.x[X_TOTAL] = total_cost;
-    for (uint64_t t0 = q0; t0 < q1; t0 += kPT) {
-      const uint64_t j = t0 + tid;
-      const unsigned long long cj = j < q1 ? unit_cost(p, s, order[j]) : 0ull;
-      unsigned long long tot;
-      const unsigned long long before = run + block_scan<unsigned long long>(cj, tot);
-      if (j < q1 && before + cj > p.budget && before <= p.budget) {  // unique: prefixes only grow
-        s.x[X_P] = j;
-        s.x[X_PBP] = before;
-      }
-      run += tot;
-    }
-  }
-  if (!grid_sync(s.x, gen, p.summary)) return;
-  const unsigned long long P = s.x[X_P];
-  const unsigned long long R0 = P == kNoP ? 0ull : p.budget - s.x[X_PBP];
-
-  // ---- E: the tail after the first overflow ----
-  if (P != kNoP) {
-    {
-      unsigned long long cnt = 0;
-      for (uint64_t j = q0 + tid; j < q1; j += kPT) cnt += (j > P && unit_cost(p, s, order[j]) <= R0) ? 1ull : 0ull;
-      cnt = block_sum<unsigned long long>(cnt);
-      if (tid == 0) s.cta_a[c] = cnt;
-    }
-    if (!grid_sync(s.x, gen, p.summary)) return;
-    const unsigned long long L = block_sum_prefix(s.cta_a, G);
-    {
-      unsigned long long run = block_sum_prefix(s.cta_a, c);
-      unsigned long long cmin = ~0ull;
-      for (uint64_t t0 = q0; t0 < q1; t0 += kPT) {
-        const uint64_t j = t0 + tid;
-        const unsigned long long cj = j < q1 ? unit_cost(p, s, order[j]) : ~0ull;
-        const bool f = j < q1 && j > P && cj <= R0;
-        uint32_t tot;
-        const uint32_t pos = block_scan<uint32_t>(f ? 1u : 0u, tot);
-        if (f) {
-          s.tail_pos[run + pos] = (uint32_t)j;
-          s.tail_cost[run + pos] = cj;
-          cmin = cj < cmin ? cj : cmin;
-        }
-        run += tot;
-      }
-#pragma unroll
-      for (int sh = 16; sh > 0; sh >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, cmin, sh);
-        cmin = o < cmin ? o : cmin;
-      }
-      if (lane == 0 && cmin != ~0ull) atomicMin(&s.x[X_TAILMIN], cmin);
-    }
-    if (!grid_sync(s.x, gen, p.summary)) return;
-    if (c == 0) {
-      // greedy with skip over the compacted tail, in order, from shared memory; once R is
-      // below the smallest tail cost nothing more can be taken
-      const unsigned long long cmin = __ldcg(&s.x[X_TAILMIN]);
-      unsigned long long R = R0;
-      for (unsigned long long k0 = 0; k0 < L && R >= cmin; k0 += kTailChunk) {
-        const uint32_t n = (uint32_t)min((unsigned long long)kTailChunk, L - k0);
-        for (uint32_t k = tid; k < n; k += kPT) s_cost[k] = __ldcg(s.tail_cost + k0 + k);
-        __syncthreads();
-        if (warp == 0) {
-          for (uint32_t b0 = 0; b0 < n && R >= cmin; b0 += 32) {
-            const uint32_t k = b0 + lane;
-            const unsigned long long ck = k < n ? s_cost[k] : ~0ull;
-            uint32_t done = 0u;
-            for (;;) {
-              const uint32_t m = __ballot_sync(0xFFFFFFFFu, ck <= R) & ~done;
-              if (m == 0u) break;
-              const int f = __ffs(m) - 1;
-              if ((int)lane == f) s.tailsel[s.tail_pos[k0 + k]] = 1;
-              R -= __shfl_sync(0xFFFFFFFFu, ck, f);
-              done = f == 31 ? 0xFFFFFFFFu : ((2u << f) - 1u);
-            }
+    unsigned long long own;
+    unsigned long long run = warp_prefix(s.cta_b, c, G, total_cost) + warp_prefix(s_wsum, warp, W, own);
+    // only the warp whose slice holds the crossing walks it (prefixes only grow: it is unique)
+    if (run <= p.budget && run + s_wsum[warp] > p.budget) {
+      for (uint64_t t0 = a; t0 < b; t0 += 32) {
+        const uint64_t j = t0 + lane;
+        const unsigned long long cj = j < b ? unit_cost(p, s, order[j]) : 0ull;
+        const unsigned long long cum = run + warp_scan(cj, lane);
+        const uint32_t over = __ballot_sync(0xFFFFFFFFu, cum > p.budget);
+        if (over) {
+          if ((int)lane == __ffs(over) - 1) {
+            s.x[X_P] = j;
+            s.x[X_PBP] = cum - cj;
           }
-          if (lane == 0) s_bcast[0] = R;
+          break;
         }
-        __syncthreads();
-        R = s_bcast[0];
+        run = __shfl_sync(0xFFFFFFFFu, cum, 31);
       }
-      if (tid == 0) s.x[X_TAILSUM] = R0 - R;
     }
-    if (!grid_sync(s.x, gen, p.summary)) return;
   }
+  if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+  const unsigned long long P = s.x[X_P];
+  const unsigned long long pbp = P == kNoP ? 0ull : s.x[X_PBP];
+  const unsigned long long R0 = P == kNoP ? 0ull : p.budget - pbp;
 
-  // ---- F: mask, set hash, count; then touched blocks and the digest (last CTA) ----
+  // ---- E: the positions before the overflow are selected; the tail after it is compacted ----
   {
-    unsigned long long h = 0, n = 0;
-    for (uint64_t j = q0 + tid; j < q1; j += kPT) {
-      if ((P == kNoP || j < P) || s.tailsel[j]) {
-        const uint32_t u = order[j];
-        if (kChecked && (uint64_t)u >= p.n_blocks * p.K) {  // checked build: a unit id past U
-          atomicOr((unsigned long long*)&p.summary[S_ERR], (unsigned long long)kErrBounds);
-          continue;
+    Selected sel;
+    uint32_t cnt = 0;
+    const uint32_t n_sel = P == kNoP ? Q : (uint32_t)P;
+#pragma unroll 4
+    for (uint64_t j = gt; j < n_sel; j += gn) select_unit(p, s, order[j], sel);  // over the whole grid
+    add_selected<PT>(p, sel);
+    if (P != kNoP) {
+      if (b > P)
+        for (uint64_t j = a + lane; j < b; j += 32) cnt += (j > P && unit_cost(p, s, order[j]) <= R0) ? 1u : 0u;
+#pragma unroll
+      for (int sh = 16; sh > 0; sh >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, sh);
+      uint32_t n_cta;
+      const uint32_t w0 = block_scan<PT, uint32_t>(lane == 0 ? cnt : 0u, n_cta);
+      uint32_t o = slice_begin(Q, len, c * W) + __shfl_sync(0xFFFFFFFFu, w0, 0);
+      unsigned long long cmin = ~0ull;
+      if (cnt) {
+        for (uint64_t t0 = a; t0 < b; t0 += 32) {
+          const uint64_t j = t0 + lane;
+          const unsigned long long cj = j < b && j > P ? unit_cost(p, s, order[j]) : ~0ull;
+          const bool f = cj <= R0;
+          const uint32_t m = __ballot_sync(0xFFFFFFFFu, f);
+          if (f) {
+            s.tail_pos[o + __popc(m & lt)] = (uint32_t)j;
+            s.tail_cost[o + __popc(m & lt)] = cj;
+            cmin = cj < cmin ? cj : cmin;
+          }
+          o += __popc(m);
         }
-        const uint32_t b = u / p.K, i = u % p.K;
-        const uint32_t t = p.fallback ? p.blk_tensor[b] : 0u;
-        if (p.fallback && s.pair_flag[i * p.n_tensors + t]) {
-          atomicOr(&s.sel_bits[t], 1u << i);  // every block of t gets bit i in the next pass
-        } else {
-          atomicOr(&p.mask[b], 1u << i);
+#pragma unroll
+        for (int sh = 16; sh > 0; sh >>= 1) {
+          const unsigned long long v = __shfl_xor_sync(0xFFFFFFFFu, cmin, sh);
+          cmin = v < cmin ? v : cmin;
         }
-        h += splitmix64(u);
-        ++n;
+        if (lane == 0) atomicMin(&s.x[X_TAILMIN], cmin);
       }
-    }
-    h = block_sum<unsigned long long>(h);
-    n = block_sum<unsigned long long>(n);
-    if (tid == 0 && n) {
-      atomicAdd((unsigned long long*)&p.summary[S_SETHASH], h);
-      atomicAdd((unsigned long long*)&p.summary[S_NSEL], n);
+      if (tid == 0) s.cta_a[c] = n_cta;
     }
   }
-  if (!grid_sync(s.x, gen, p.summary)) return;
-  {
-    uint64_t b0, b1;
-    slice(p.n_blocks, b0, b1);
-    unsigned long long t = 0;
-    for (uint64_t b = b0 + tid; b < b1; b += kPT) {
-      uint32_t m = p.mask[b];
-      if (p.fallback) {
-        const uint32_t sb = __ldcg(s.sel_bits + p.blk_tensor[b]);
-        if (sb) {
-          m |= sb;
-          p.mask[b] = m;  // one thread per block in this pass
+  if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+  unsigned long long tail_sum = 0;
+  if (c == 0 && P != kNoP) {
+    // greedy with skip over the compacted tail, in order, from shared memory; once R is
+    // below the smallest tail cost nothing more can be taken
+    Selected sel;
+    uint32_t L;
+    {
+      const uint32_t v = tid < G ? (uint32_t)s.cta_a[tid] : 0u;
+      const uint32_t e = block_scan<PT, uint32_t>(v, L);
+      if (tid < G) s_pre[tid] = e;
+      if (tid == 0) s_pre[G] = L;
+      __syncthreads();
+    }
+    // slot of the k-th tail candidate: in the slice of the last CTA with s_pre <= k
+    auto slot = [&](uint32_t k) -> uint32_t {
+      uint32_t lo = 0, hi = G;  // s_pre[lo] <= k < s_pre[hi]
+      while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (s_pre[mid] <= k) lo = mid;
+        else hi = mid;
+      }
+      return slice_begin(Q, len, lo * W) + (k - s_pre[lo]);
+    };
+    const unsigned long long cmin = __ldcg(&s.x[X_TAILMIN]);
+    unsigned long long R = R0;
+    for (uint32_t k0 = 0; k0 < L && R >= cmin; k0 += kTailChunk) {
+      const uint32_t n = min(kTailChunk, L - k0);
+      unsigned long long sum = 0;
+      for (uint32_t k = tid; k < n; k += PT) {
+        const unsigned long long ck = __ldcg(s.tail_cost + slot(k0 + k));
+        s_cost[k] = ck;
+        sum += ck <= R ? ck : 0ull;
+      }
+      sum = block_sum<PT, unsigned long long>(sum);
+      if (sum <= R) {  // everything that fits now fits together
+        for (uint32_t k = tid; k < n; k += PT)
+          if (s_cost[k] <= R) select_unit(p, s, order[__ldcg(s.tail_pos + slot(k0 + k))], sel);
+        R -= sum;
+        __syncthreads();  // the next chunk overwrites s_cost
+        continue;
+      }
+      if (warp == 0) {
+        for (uint32_t b0 = 0; b0 < n; b0 += 32) {
+          const uint32_t k = b0 + lane;
+          const unsigned long long ck = k < n ? s_cost[k] : ~0ull;
+          uint32_t taken = 0u, rem = 0xFFFFFFFFu;
+          // R only shrinks, so what does not fit now never will; of what fits now, everything
+          // up to the first whose prefix exceeds R is taken, that one is skipped, and the
+          // lanes after it are looked at again
+          while (rem) {
+            const bool e = ((rem >> lane) & 1u) && ck <= R;
+            const uint32_t fit = __ballot_sync(0xFFFFFFFFu, e);
+            if (fit == 0u) break;
+            const unsigned long long v = e ? ck : 0ull, cum = warp_scan(v, lane);
+            const uint32_t over = __ballot_sync(0xFFFFFFFFu, e && cum > R);
+            if (over == 0u) {
+              taken |= fit;
+              R -= __shfl_sync(0xFFFFFFFFu, cum, 31);
+              break;
+            }
+            const int f = __ffs(over) - 1;
+            taken |= fit & ((1u << f) - 1u);
+            R -= __shfl_sync(0xFFFFFFFFu, cum - v, f);
+            rem &= f == 31 ? 0u : ~((2u << f) - 1u);
+          }
+          if (lane == 0) s_take[b0 / 32] = taken;
         }
+        if (lane == 0) s_bcast = R;
+      }
+      __syncthreads();
+      R = s_bcast;
+      for (uint32_t k = tid; k < n; k += PT)
+        if ((s_take[k / 32] >> (k & 31u)) & 1u) select_unit(p, s, order[__ldcg(s.tail_pos + slot(k0 + k))], sel);
+      __syncthreads();  // the next chunk overwrites s_cost and s_take
+    }
+    tail_sum = R0 - R;
+    add_selected<PT>(p, sel);
+    __syncthreads();  // three warps have added to the summary that thread 0 reads
+  }
+  if (p.fallback) {
+    // a taken fallback unit's expert bit goes into every block of its tensor
+    if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+    unsigned long long t = 0;
+    for (uint64_t k = gt; k < p.n_blocks; k += gn) {
+      uint32_t m = p.mask[k];
+      const uint32_t sb = s.sel_bits[p.blk_tensor[k]];
+      if (sb) {
+        m |= sb;
+        p.mask[k] = m;  // one thread per block in this pass
       }
       t += m != 0u ? 1ull : 0ull;
     }
-    t = block_sum<unsigned long long>(t);
-    __shared__ bool last;
-    if (tid == 0) {
-      if (t) atomicAdd((unsigned long long*)&p.summary[S_TOUCHED], t);
-      __threadfence();
-      last = atomicAdd(&s.x[X_DONE], 1ull) == (unsigned long long)(G - 1);
-    }
-    __syncthreads();
-    if (!last || tid != 0) return;
+    t = block_sum<PT, unsigned long long>(t);
+    if (tid == 0 && t) atomicAdd((unsigned long long*)&p.summary[S_TOUCHED], t);
+    if (!phase_sync<CL>(s.x, gen, p.summary)) return;
   }
-  // the digest: FNV-1a 64 over the host-built prefix and C_hat, n_sel, set_hash
+  if (gt != 0) return;
+  // ---- F: the digest: FNV-1a 64 over the header (hashed by the host) and C_hat, n_sel, set_hash ----
   __threadfence();
   volatile unsigned long long* sum = (volatile unsigned long long*)p.summary;
-  const unsigned long long chat = P == kNoP ? s.x[X_TOTAL] : s.x[X_PBP] + s.x[X_TAILSUM];
+  const unsigned long long chat = P == kNoP ? total_cost : pbp + tail_sum;
   const unsigned long long nsel = sum[S_NSEL], sh = sum[S_SETHASH];
-  uint64_t h = 14695981039346656037ull;
-  for (uint32_t k = 0; k < p.hdr_prefix_len; ++k) {
-    h ^= p.hdr_prefix[k];
-    h *= 1099511628211ull;
-  }
+  uint64_t h = p.digest_state;
   const unsigned long long tail[3] = {chat, nsel, sh};
   for (int w = 0; w < 3; ++w)
     for (int k = 0; k < 8; ++k) {
       h ^= (tail[w] >> (8 * k)) & 0xFFu;
       h *= 1099511628211ull;
     }
-  sum[S_CHAT] = chat;
-  sum[S_NCAND] = Q;
-  sum[S_DIGEST] = h;
-  sum[S_ERR] = sum[S_ERR] | (unsigned long long)*p.index_err | (s.x[X_MISSING] ? (unsigned long long)kErrMissing : 0ull) |
-               (s.x[X_BADORDER] ? (unsigned long long)kErrInternal : 0ull);
+  const unsigned long long err = sum[S_ERR] | (unsigned long long)*p.index_err |
+                                 (s.x[X_MISSING] ? (unsigned long long)kErrMissing : 0ull) |
+                                 (bad_order ? (unsigned long long)kErrInternal : 0ull);
+  const unsigned long long words[8] = {chat, nsel, Q, sh, h, sum[S_TOUCHED], err, 0ull};
+  for (int k = 0; k < 8; ++k) {
+    sum[k] = words[k];
+    if (p.host_summary) p.host_summary[k] = words[k];
+  }
 }
 
 }  // namespace
 
 size_t plan_scratch_bytes(uint64_t n_units, uint64_t n_pairs) { return carve(nullptr, n_units, n_pairs, nullptr); }
+
+uint64_t plan_digest_state(const uint8_t* header, size_t n) {
+  uint64_t h = 14695981039346656037ull;
+  for (size_t k = 0; k < n; ++k) {
+    h ^= header[k];
+    h *= 1099511628211ull;
+  }
+  return h;
+}
 
 cudaError_t launch_plan(const PlanLaunch& p, void* scratch, cudaStream_t st) {
   const uint64_t U = (uint64_t)p.K * p.n_blocks;
@@ -626,24 +797,43 @@ cudaError_t launch_plan(const PlanLaunch& p, void* scratch, cudaStream_t st) {
   if (p.fallback && (!p.blk_tensor || !p.t_blk0 || n_pairs == 0)) return cudaErrorInvalidValue;
   Scratch s;
   carve(scratch, U, n_pairs, &s);
-  int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e;
+  if (U <= kClusterUnits) {
+    // half a unit per thread, then more, in one cluster
+    uint32_t grid = 1;
+    while (grid < kClusterMax && grid * 512ull < U) grid *= 2;
+    auto k = plan_kernel<kClusterThreads, true>;
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = grid;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if ((e = cudaLaunchKernelEx(&cfg, k, p, s)) != cudaSuccess) return e;
+    count_launches(1);
+    return cudaGetLastError();
+  }
+  int dev = 0, sms = 0, per_sm = 0;
+  auto kern = plan_kernel<kGridThreads, false>;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan_kernel, kPT, 0)) != cudaSuccess) return e;
-  // about 512 units per CTA (two tiles), at most one CTA per SM, all co-resident
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGridThreads, 0)) != cudaSuccess) return e;
+  // at most one CTA per SM, all co-resident
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  uint64_t grid = (U + 511) / 512;
-  const uint64_t cap = (uint64_t)sms;
-  if (grid > cap) grid = cap;
+  uint64_t grid = (uint64_t)sms;
   if (grid > kMaxGrid) grid = kMaxGrid;
-  if (grid < 1) grid = 1;
+  static_assert(kMaxGrid <= (uint32_t)kGridThreads && kClusterMax <= (uint32_t)kClusterThreads,
+                "one thread per CTA where the CTAs' counts are added up");
   if ((e = launch_fill(s.x, 0, X_COUNT * sizeof(unsigned long long), st)) != cudaSuccess) return e;
-  if (n_pairs && (e = launch_fill(s.pair_flag, 0, n_pairs * 4, st)) != cudaSuccess) return e;
-  if (n_pairs && (e = launch_fill(s.sel_bits, 0, (size_t)p.n_tensors * 4, st)) != cudaSuccess) return e;
   PlanLaunch pc = p;
   void* args[] = {&pc, &s};
-  if ((e = cudaLaunchCooperativeKernel((const void*)plan_kernel, dim3((unsigned)grid), dim3(kPT), args, 0, st)) !=
+  if ((e = cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(kGridThreads), args, 0, st)) !=
       cudaSuccess)
     return e;
   count_launches(1);

@@ -143,20 +143,21 @@ extern "C" mp_status mp_plan_noalloc(uint32_t K, uint64_t n_blocks, uint32_t n_g
   p.mask = mask;
   p.order = order;
   p.summary = summary;
+  uint8_t hdr[256];  // 4 * 32 coefficients and 52 bytes of other fields at most
   uint32_t o = 0;
-  put_u32(p.hdr_prefix, o, (uint32_t)op->kind);
-  put_u32(p.hdr_prefix, o, K);
-  for (uint32_t i = 0; i < K; ++i) put_u32(p.hdr_prefix, o, op->alpha ? fbits(op->alpha[i]) : 0u);
-  put_u32(p.hdr_prefix, o, fbits(op->lambda));
-  put_u32(p.hdr_prefix, o, fbits(op->density));
-  put_u32(p.hdr_prefix, o, op->trim_scope);
+  put_u32(hdr, o, (uint32_t)op->kind);
+  put_u32(hdr, o, K);
+  for (uint32_t i = 0; i < K; ++i) put_u32(hdr, o, op->alpha ? fbits(op->alpha[i]) : 0u);
+  put_u32(hdr, o, fbits(op->lambda));
+  put_u32(hdr, o, fbits(op->density));
+  put_u32(hdr, o, op->trim_scope);
   uint64_t pb;
   memcpy(&pb, &op->drop_p, 8);
-  put_u64(p.hdr_prefix, o, pb);
-  put_u64(p.hdr_prefix, o, op->seed);
-  put_u32(p.hdr_prefix, o, op->score_mode);
-  put_u64(p.hdr_prefix, o, budget_bytes);
-  p.hdr_prefix_len = o;
+  put_u64(hdr, o, pb);
+  put_u64(hdr, o, op->seed);
+  put_u32(hdr, o, op->score_mode);
+  put_u64(hdr, o, budget_bytes);
+  p.digest_state = mp::plan_digest_state(hdr, o);
 
   cudaError_t e = mp::launch_plan(p, scratch, reinterpret_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) {
