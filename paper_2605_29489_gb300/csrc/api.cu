@@ -138,16 +138,17 @@ void pin_put(void* p, size_t bytes) {
 
 size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Host data into the index's device memory by kernel: staged in a pinned slot that the handle
-// keeps until mp_free, read by launch_copy over the host mapping.  Data larger than the
-// largest slot goes by cudaMemcpyAsync.
-cudaError_t upload(mp_index_s* ix, void* dst, const void* src, size_t bytes, cudaStream_t cs) {
+// Host data into the index's device memory: staged in a pinned slot that the handle keeps until
+// mp_free, and copied by the init kernel over the host mapping.  Data larger than the largest
+// slot goes by cudaMemcpyAsync.
+cudaError_t upload(mp_index_s* ix, InitList& init, void* dst, const void* src, size_t bytes, cudaStream_t cs) {
   if (bytes == 0) return cudaSuccess;
   void* h = pin_get(bytes);
   if (!h) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, cs);
   memcpy(h, src, bytes);
   ix->pinned.push_back({h, bytes});
-  return launch_copy(dst, h, bytes, cs);
+  init.add(dst, h, bytes);
+  return cudaSuccess;
 }
 
 void release_pinned(mp_index_s* ix) {
@@ -352,7 +353,7 @@ mp_status cuda_fail(cudaError_t e, const char* what) {
 }
 
 mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, size_t work_bytes, cudaStream_t cs,
-                    mp_index_s** out, char** work);
+                    InitList& init, mp_index_s** out, char** work);
 cudaError_t finish_index(mp_index_s* ix, cudaStream_t cs);
 void discard_index(mp_index_s* ix, cudaStream_t cs);
 mp_status alloc_hashes(mp_index_s* ix, cudaStream_t cs);
@@ -520,6 +521,7 @@ cudaError_t walk_segments(const IndexLaunch& p, const mp_index_s* ix, cudaStream
     ps.expert_origin = g.e0;
     ps.ext.x_span = span;
     ps.defer_ties_select = 1;
+    ps.work = p.work + s;
     for (uint32_t i = 0; i < p.K; ++i) ps.experts.p[i] = hp.buf(b, i);
     const int tk = trace_begin(MP_TRACE_SEGMENT, (uint32_t)s, 0, cs);
     e = stage(ps);
@@ -543,7 +545,9 @@ cudaError_t index_host_pool(IndexLaunch p, const mp_index_s* ix, cudaStream_t cs
         cudaSuccess)
       return e;
     if ((e = launch_ties_window_end(p, cs)) != cudaSuccess) return e;
-    if ((e = walk_segments(p, ix, cs, p.miss, [&](const IndexLaunch& ps) { return launch_index_pass(ps, false, cs); })) !=
+    IndexLaunch q = p;
+    q.work = p.work + 2 * (size_t)(ix->g.n_params / kSegmentElems) + 2;  // the second walk's counters
+    if ((e = walk_segments(q, ix, cs, p.miss, [&](const IndexLaunch& ps) { return launch_index_pass(ps, false, cs); })) !=
         cudaSuccess)
       return e;
   } else {
@@ -601,6 +605,8 @@ cudaError_t merge_host_pool(MergeLaunch p, const mp_index_s* ix, cudaStream_t cs
     ps.expert_origin = g.e0;
     ps.ext.x_span = span;
     ps.experts = gl.dst;
+    ps.work = p.work + s;
+    if (s + 1 < segs.size()) ps.back_host = nullptr;  // the last segment's launch sends the manifest back
     const int tk = trace_begin(MP_TRACE_SEGMENT, (uint32_t)s, 0, cs);
     e = launch_merge(ps, cs);
     trace_end(tk, cs);
@@ -613,10 +619,11 @@ cudaError_t merge_host_pool(MergeLaunch p, const mp_index_s* ix, cudaStream_t cs
 
 // A new index handle for geometry g: one device allocation holding the block table
 // (offset, length, TIES trim group and tensor of each block, first block of each tensor),
-// the statistics, the error word and work_bytes of scratch for the caller (*work).  The
-// table is uploaded and the error word and tau cleared on cs.
+// the statistics, the error word and work_bytes of scratch for the caller (*work).  What
+// uploads the table and clears the error word and tau is left in init, which the caller
+// launches on cs with what it adds of its own.
 mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, size_t work_bytes, cudaStream_t cs,
-                    mp_index_s** out, char** work) {
+                    InitList& init, mp_index_s** out, char** work) {
   const bool ties = op && (op->kind == MP_OP_TIES || op->kind == MP_OP_TIES_MASKED);
   const bool masked = op && op->kind == MP_OP_TIES_MASKED;
   const uint32_t scope = ties ? op->trim_scope : 0u;
@@ -684,7 +691,6 @@ mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, size_t w
   ix->d_err = (uint32_t*)(m + o_err);
   ix->d_unit_hist = masked ? (uint32_t*)(m + o_uh) : nullptr;
   cudaError_t e = cudaSuccess;
-  const char* what = "block table copy";
   {
     // the five table arrays are consecutive in the allocation: one staged upload
     const size_t t_end = o_tb0 + ((size_t)g.n_tensors + 1) * 4;
@@ -694,15 +700,14 @@ mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, size_t w
     memcpy(tab.data() + o_grp, h_grp.data(), nb * 4);
     memcpy(tab.data() + o_tens, h_tens.data(), nb * 4);
     memcpy(tab.data() + o_tb0, h_tb0.data(), ((size_t)g.n_tensors + 1) * 4);
-    e = upload(ix, m, tab.data(), t_end, cs);
+    e = upload(ix, init, m, tab.data(), t_end, cs);
   }
-  if (e == cudaSuccess) what = "fill", e = launch_fill(ix->d_err, 0, 16, cs);
-  if (e == cudaSuccess) e = launch_fill(ix->d_tau, 0, KG * 4, cs);
   if (e != cudaSuccess) {
-    mp_status r = cuda_fail(e, what);
+    mp_status r = cuda_fail(e, "block table copy");
     discard_index(ix, cs);
     return r;
   }
+  init.add(ix->d_tau, nullptr, o_err + 16 - o_tau);  // tau, then the error word
   if (host_pool) {
     ix->h_blk_off = std::move(h_off);
     ix->h_blk_len = std::move(h_len);
@@ -803,7 +808,11 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   // the index kernels' work space after the handle's own arrays
   size_t o = 0;
   auto slot = [&](size_t bytes) { size_t r = o; o += align_up(bytes); return r; };
-  const size_t o_work = slot(16);  // the index kernel's work counter
+  // the index kernels' work counters: for device-resident experts the two passes' and the two
+  // counts of finished CTAs; for a host pool one per segment of both walks (any two consecutive
+  // segments together exceed kSegmentElems)
+  const size_t n_work = family->experts_location == 0 ? 4 : 2 * (2 * (size_t)(g.n_params / kSegmentElems) + 2);
+  const size_t o_work = slot(n_work * 8);
   size_t o_coarse = 0, o_fine = 0, o_kth = 0, o_est = 0, o_rank = 0;
   size_t o_wfine = 0, o_wabove = 0, o_wlo = 0, o_gmiss = 0, o_miss = 0, o_wend = 0;
   // device-resident TIES (not after masking) takes its thresholds from predicted windows
@@ -844,7 +853,8 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   }
   mp_index_s* ix = nullptr;
   char* m = nullptr;
-  if ((st = new_index(g, op, family->experts_location != 0, o, cs, &ix, &m)) != MP_OK) return st;
+  InitList init;
+  if ((st = new_index(g, op, family->experts_location != 0, o, cs, init, &ix, &m)) != MP_OK) return st;
 
   cudaError_t e;
   auto bail = [&](cudaError_t err, const char* what) {
@@ -878,9 +888,8 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
     p.rank = (unsigned long long*)(m + o_rank);
     p.tau = ix->d_tau;
     p.unit_hist = ix->d_unit_hist;
-    if ((e = launch_fill(p.coarse, 0, KG * 256 * 8, cs)) != cudaSuccess) return bail(e, "fill");
-    if ((e = launch_fill(p.fine, 0, KG * 128 * 8, cs)) != cudaSuccess) return bail(e, "fill");
-    if ((e = upload(ix, (void*)p.kth, h_kth.data(), n_groups * 8, cs)) != cudaSuccess) return bail(e, "k copy");
+    init.add(p.coarse, nullptr, o_kth - o_coarse);  // coarse and fine bins
+    if ((e = upload(ix, init, (void*)p.kth, h_kth.data(), n_groups * 8, cs)) != cudaSuccess) return bail(e, "k copy");
   }
   if (windowed) {
     p.density = op->density;
@@ -895,10 +904,12 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
     p.samp_span = (const uint2*)(m + o_spans);
     p.n_samp_spans = (uint32_t)(h_spans.size() / 2);
     p.samp_blocks = (uint32_t)span_blocks;
-    if ((e = launch_fill(m + o_wfine, 0, o_wend - o_wfine, cs)) != cudaSuccess) return bail(e, "fill");
-    if ((e = upload(ix, m + o_spans, h_spans.data(), h_spans.size() * 4, cs)) != cudaSuccess)
+    init.add(m + o_wfine, nullptr, o_wend - o_wfine);
+    if ((e = upload(ix, init, m + o_spans, h_spans.data(), h_spans.size() * 4, cs)) != cudaSuccess)
       return bail(e, "span copy");
   }
+  init.add(m + o_work, nullptr, n_work * 8);
+  if ((e = launch_init(init, cs)) != cudaSuccess) return bail(e, "index start");
   p.b_begin = 0;
   p.b_end = g.n_blocks;
   p.expert_origin = 0;
@@ -957,7 +968,8 @@ mp_status mp_index_import(const mp_family* family, const mp_op* op, const float*
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
   mp_index_s* ix = nullptr;
   char* m = nullptr;
-  if ((st = new_index(g, op, family->experts_location != 0, 0, cs, &ix, &m)) != MP_OK) return st;
+  InitList init;
+  if ((st = new_index(g, op, family->experts_location != 0, 0, cs, init, &ix, &m)) != MP_OK) return st;
   ix->has_missing = missing;
   cudaError_t e;
   auto bail = [&](cudaError_t err, const char* what) {
@@ -965,6 +977,7 @@ mp_status mp_index_import(const mp_family* family, const mp_op* op, const float*
     discard_index(ix, cs);
     return r;
   };
+  if ((e = launch_init(init, cs)) != cudaSuccess) return bail(e, "index start");
   if ((e = cudaMemcpyAsync(ix->d_norm, norm, U * 4, cudaMemcpyHostToDevice, cs)) != cudaSuccess)
     return bail(e, "catalog copy");
   if ((e = cudaMemcpyAsync(ix->d_maxabs, maxabs, U * 4, cudaMemcpyHostToDevice, cs)) != cudaSuccess)
@@ -1197,7 +1210,7 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   const size_t counters_bytes = (size_t)kCounterSlots * g.K * 8;
   // the counters (64 slots x K), the plan summary, the error word and the TIES_MASKED
   // threshold reads come back in one copy
-  const size_t back_bytes = counters_bytes + 64 + 16 + 16;
+  const size_t back_bytes = counters_bytes + 64 + kBackTail * 8;
   mf->h_realized = static_cast<unsigned long long*>(pin_get(back_bytes));
   if (!mf->h_realized) {
     delete mf;
@@ -1211,14 +1224,16 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   auto mslot = [&](size_t bytes) { size_t r = mo; mo += align_up(bytes); return r; };
   const size_t m_coarse = mslot(KG * 256 * 8), m_fine = mslot(KG * 128 * 8), m_kth = mslot(plan->n_groups * 8);
   const size_t m_est = mslot(KG * 4), m_rank = mslot(KG * 8), m_tau = mslot(KG * 4);
-  const size_t scratch_off = align_up(back_bytes + 16);
+  // the merge kernel's work counter (one per segment of a host pool) and its count of finished CTAs
+  const size_t n_work = family->experts_location == 0 ? 1 : 2 * (size_t)(g.n_params / kSegmentElems) + 2;
+  const size_t zero_bytes = back_bytes + (n_work + 1) * 8;
+  const size_t scratch_off = align_up(zero_bytes);
   if ((st = dev_alloc(mf->mem, scratch_off + (masked ? mo : 0), cs)) != MP_OK) {
     release_pinned();
     delete mf;
     return st;
   }
   mf->d_realized = static_cast<unsigned long long*>(mf->mem.ptr);
-  uint64_t* d_sum_copy = reinterpret_cast<uint64_t*>(static_cast<char*>(mf->mem.ptr) + counters_bytes);
   mf->d_err = reinterpret_cast<uint32_t*>(static_cast<char*>(mf->mem.ptr) + counters_bytes + 64);
   auto bail = [&](cudaError_t err, const char* what) {
     mp_status r = cuda_fail(err, what);
@@ -1232,7 +1247,7 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   cudaError_t e;
   if ((e = stream_wait(cs, index->done, index->captured, mf->captured)) != cudaSuccess) return bail(e, "stream wait");
   if ((e = stream_wait(cs, plan->done, plan->captured, mf->captured)) != cudaSuccess) return bail(e, "stream wait");
-  if ((e = launch_fill(mf->mem.ptr, 0, back_bytes, cs)) != cudaSuccess) return bail(e, "fill");
+  if ((e = launch_fill(mf->mem.ptr, 0, zero_bytes, cs)) != cudaSuccess) return bail(e, "fill");
   uint32_t* masked_tau = nullptr;
   if (masked) {
     // TIES after masking: the threshold of the zero-completed masked deltas of this plan
@@ -1312,6 +1327,9 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   }
   p.realized = mf->d_realized;
   p.work = reinterpret_cast<unsigned long long*>(static_cast<char*>(mf->mem.ptr) + back_bytes);
+  p.done = p.work + n_work;
+  p.back_host = mf->h_realized;
+  p.back_summary = plan->d_summary;
   p.err = mf->d_err;
   p.b_begin = 0;
   p.b_end = g.n_blocks;
@@ -1327,10 +1345,6 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
       return bail(cudaErrorInvalidValue, "an index of a host-resident pool is needed for a host-pool merge");
     if ((e = merge_host_pool(p, index, cs)) != cudaSuccess) return bail(e, "merge (host pool)");
   }
-  if ((e = launch_copy(d_sum_copy, plan->d_summary, 64, cs)) != cudaSuccess)
-    return bail(e, "summary copy");
-  if ((e = launch_copy(mf->h_realized, mf->mem.ptr, back_bytes, cs)) != cudaSuccess)
-    return bail(e, "manifest copy");
   if ((e = cudaEventCreateWithFlags(&mf->done, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "event");
   if ((e = cudaEventRecord(mf->done, cs)) != cudaSuccess) return bail(e, "event record");
   *man_out = mf;

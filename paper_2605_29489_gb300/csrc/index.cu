@@ -128,7 +128,7 @@ struct __align__(128) IxSmem {
   float red_mx[KG][8];
   uint32_t red_nz[KG][8];
   uint64_t cbar;  // consumer-only barrier (one arrival per consumer warp)
-  int abort;
+  int abort, last;
 };
 
 // raw 16-byte vector at element k0 of a fill: from the slot when inside the bulk-copied
@@ -306,6 +306,102 @@ __device__ __forceinline__ bool checked_item(const IndexLaunch& p, uint64_t b, u
   return false;
 }
 
+// The k-th largest of the keys counted in h[0 .. 32 N), by one warp: lane l sums the N bins
+// that rank l-th from the top, a warp scan finds the lane where the running count reaches k,
+// and that lane walks its own bins.  True (on every lane) when h holds at least k keys; then
+// bin is the bin of the k-th largest and before the number of keys above it.  One thread
+// walking the bins waits for a load per bin: 256 to 384 of them took 30-46 us whatever the
+// number of pairs, this takes two.
+template <int N>
+__device__ __forceinline__ bool warp_kth(const unsigned long long* h, unsigned long long k, uint32_t& bin,
+                                         unsigned long long& before) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t top = 32u * N - 1u - lane * N;  // this lane's highest bin
+  unsigned long long c[N], sum = 0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    c[j] = h[top - j];
+    sum += c[j];
+  }
+  unsigned long long cum = sum;
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, cum, s);
+    if (lane >= (uint32_t)s) cum += o;
+  }
+  const uint32_t hit = __ballot_sync(0xFFFFFFFFu, cum >= k);
+  if (hit == 0u) return false;
+  const int src = __ffs(hit) - 1;
+  unsigned long long run = cum - sum;
+  uint32_t e = top;
+  bool done = false;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    if (!done && run + c[j] >= k) {
+      e = top - j;
+      done = true;
+    }
+    if (!done) run += c[j];
+  }
+  bin = __shfl_sync(0xFFFFFFFFu, e, src);
+  before = __shfl_sync(0xFFFFFFFFu, run, src);
+  return true;
+}
+
+// coarse select of pair x = (expert, trim group), by one warp: bin e* of the upper 8 key bits
+// holding the k-th largest key, and the rank of that key inside the bin
+__device__ __forceinline__ void coarse_select_pair(const IndexLaunch& p, uint64_t x) {
+  if (p.gmiss && p.gmiss[x] == 0u) return;  // its window already gave the threshold
+  const unsigned long long k = p.kth[x % p.n_groups];
+  uint32_t e = kNoBin;
+  unsigned long long before = 0, r = 0;
+  if (k != 0) {
+    if (!warp_kth<8>(p.coarse + x * 256u, k, e, before)) e = 0u;  // unreachable for k <= numel
+    r = k - before;
+  }
+  if ((threadIdx.x & 31u) == 0) {
+    p.estar[x] = e;
+    p.rank[x] = r;
+  }
+}
+
+// fine select of pair x, by one warp: the threshold from the fine bins of its coarse bin
+__device__ __forceinline__ void fine_select_pair(const IndexLaunch& p, uint64_t x) {
+  if (p.gmiss && p.gmiss[x] == 0u) return;  // its window already gave the threshold
+  const uint32_t es = p.estar[x];
+  uint32_t tau = kTauNone, m;
+  unsigned long long before;
+  if (es != kNoBin) {
+    // only bin 0 can fall short: its uncounted members are exact zeros, key 0
+    tau = es << 7;
+    if (warp_kth<4>(p.fine + x * 128u, p.rank[x], m, before)) tau |= m;
+  }
+  if ((threadIdx.x & 31u) == 0) p.tau[x] = tau;
+}
+
+// true on every thread of the launch's last CTA to get here (barrier id 1, THREADS threads,
+// which may come from different places); what the others wrote before is then visible
+template <int THREADS>
+__device__ __forceinline__ bool last_cta(unsigned long long* done, volatile int* s_last) {
+  __syncwarp();
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+  if (threadIdx.x == 0) {
+    __threadfence();
+    *s_last = atomicAdd(done, 1ull) == (unsigned long long)(gridDim.x - 1) ? 1 : 0;
+  }
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+  if (!*s_last) return false;
+  __threadfence();
+  return true;
+}
+
+// the end of a fallback coarse pass: its last CTA makes the coarse select of the marked pairs
+// (few or none as a rule), which saves a launch that would return at once
+__device__ __forceinline__ void coarse_pass_end(const IndexLaunch& p, volatile int* s_last) {
+  if (!p.select_in_pass || !last_cta<kIxThreads>(p.work + 2, s_last)) return;
+  for (uint64_t x = threadIdx.x >> 5; x < (uint64_t)p.K * p.n_groups; x += kIxThreads / 32) coarse_select_pair(p, x);
+}
+
 template <bool BF16, int KG, int BM>
 __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPerSm)
     index_tma_kernel(const IndexLaunch p, uint32_t G, uint64_t n_items, unsigned long long* work) {
@@ -476,6 +572,10 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
         if (lastf == 0 && p.stall) continue;  // never armed: nothing in flight
         mbar_wait_drain(&S.full[s], (lastf / kIxSlots) & 1u);
       }
+    }
+    if constexpr (BM == kBinCoarse) {
+      __syncwarp();
+      coarse_pass_end(p, &S.last);
     }
     return;
   }
@@ -725,48 +825,7 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
       break;
     }
   }
-}
-
-// The k-th largest of the keys counted in h[0 .. 32 N), by one warp: lane l sums the N bins
-// that rank l-th from the top, a warp scan finds the lane where the running count reaches k,
-// and that lane walks its own bins.  True (on every lane) when h holds at least k keys; then
-// bin is the bin of the k-th largest and before the number of keys above it.  One thread
-// walking the bins waits for a load per bin: 256 to 384 of them took 30-46 us whatever the
-// number of pairs, this takes two.
-template <int N>
-__device__ __forceinline__ bool warp_kth(const unsigned long long* h, unsigned long long k, uint32_t& bin,
-                                         unsigned long long& before) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t top = 32u * N - 1u - lane * N;  // this lane's highest bin
-  unsigned long long c[N], sum = 0;
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    c[j] = h[top - j];
-    sum += c[j];
-  }
-  unsigned long long cum = sum;
-#pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, cum, s);
-    if (lane >= (uint32_t)s) cum += o;
-  }
-  const uint32_t hit = __ballot_sync(0xFFFFFFFFu, cum >= k);
-  if (hit == 0u) return false;
-  const int src = __ffs(hit) - 1;
-  unsigned long long run = cum - sum;
-  uint32_t e = top;
-  bool done = false;
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    if (!done && run + c[j] >= k) {
-      e = top - j;
-      done = true;
-    }
-    if (!done) run += c[j];
-  }
-  bin = __shfl_sync(0xFFFFFFFFu, e, src);
-  before = __shfl_sync(0xFFFFFFFFu, run, src);
-  return true;
+  if constexpr (BM == kBinCoarse) coarse_pass_end(p, &S.last);
 }
 
 // the pair (expert, trim group) of this warp in the select kernels, one warp each
@@ -776,29 +835,16 @@ __device__ __forceinline__ uint64_t select_pair() {
 }
 inline unsigned select_grid(uint64_t pairs) { return (unsigned)((pairs + kSelThreads / 32 - 1) / (kSelThreads / 32)); }
 
-// coarse select: bin e* of the upper 8 key bits holding the k-th largest key, and the
-// rank of that key inside the bin
 __global__ void __launch_bounds__(kSelThreads) ties_coarse_select(const IndexLaunch p) {
   const uint64_t x = select_pair();
-  if (x >= (uint64_t)p.K * p.n_groups) return;
-  if (p.gmiss && p.gmiss[x] == 0u) return;  // its window already gave the threshold
-  const unsigned long long k = p.kth[x % p.n_groups];
-  uint32_t e = kNoBin;
-  unsigned long long before = 0, r = 0;
-  if (k != 0) {
-    if (!warp_kth<8>(p.coarse + x * 256u, k, e, before)) e = 0u;  // unreachable for k <= numel
-    r = k - before;
-  }
-  if ((threadIdx.x & 31u) == 0) {
-    p.estar[x] = e;
-    p.rank[x] = r;
-  }
+  if (x < (uint64_t)p.K * p.n_groups) coarse_select_pair(p, x);
 }
 
 template <bool BF16, int KG>
 __global__ void __launch_bounds__(256) ties_fine_kernel(const IndexLaunch p) {
   constexpr int V = BF16 ? 8 : 4;
   __shared__ uint32_t s_fine[KG][128];
+  __shared__ int s_last;
   if (p.miss && *p.miss == 0u) return;  // windowed thresholds: no pair needs this pass
   const uint32_t G = (p.K + KG - 1) / KG;
   const uint64_t n_items = p.n_blocks * G;
@@ -859,21 +905,14 @@ __global__ void __launch_bounds__(256) ties_fine_kernel(const IndexLaunch p) {
     }
     __syncthreads();  // the next item clears s_fine
   }
+  // the windowed catalog's fallback: the last CTA makes the fine select of the marked pairs
+  if (!p.select_in_pass || !last_cta<256>(p.work + 3, &s_last)) return;
+  for (uint64_t x = tid >> 5; x < (uint64_t)p.K * p.n_groups; x += 8) fine_select_pair(p, x);
 }
 
 __global__ void __launch_bounds__(kSelThreads) ties_fine_select(const IndexLaunch p) {
   const uint64_t x = select_pair();
-  if (x >= (uint64_t)p.K * p.n_groups) return;
-  if (p.gmiss && p.gmiss[x] == 0u) return;  // its window already gave the threshold
-  const uint32_t es = p.estar[x];
-  uint32_t tau = kTauNone, m;
-  unsigned long long before;
-  if (es != kNoBin) {
-    // only bin 0 can fall short: its uncounted members are exact zeros, key 0
-    tau = es << 7;
-    if (warp_kth<4>(p.fine + x * 128u, p.rank[x], m, before)) tau |= m;
-  }
-  if ((threadIdx.x & 31u) == 0) p.tau[x] = tau;
+  if (x < (uint64_t)p.K * p.n_groups) fine_select_pair(p, x);
 }
 
 // TIES after masking: the coarse bins of (expert i, group) summed over a window of blocks:
@@ -1059,16 +1098,17 @@ cudaError_t ties_finish_t(const IndexLaunch& p, cudaStream_t st) {
   uint64_t fgrid = (uint64_t)sms * (per_sm > 0 ? per_sm : 1);
   if (fgrid > p.n_blocks * G) fgrid = p.n_blocks * G;
   if (fgrid == 0) fgrid = 1;
-  ties_coarse_select<<<sgrid, kSelThreads, 0, st>>>(p);
+  if (!p.select_in_pass) ties_coarse_select<<<sgrid, kSelThreads, 0, st>>>(p);
   ties_fine_kernel<BF16, KG><<<(unsigned)fgrid, 256, 0, st>>>(p);
-  ties_fine_select<<<sgrid, kSelThreads, 0, st>>>(p);
-  count_launches(3);
+  if (!p.select_in_pass) ties_fine_select<<<sgrid, kSelThreads, 0, st>>>(p);
+  count_launches(p.select_in_pass ? 1 : 3);
   return cudaGetLastError();
 }
 
 // one persistent launch of the catalog kernel with binning mode BM
 template <bool BF16, int KG, int BM>
-cudaError_t launch_pass(const IndexLaunch& p, uint32_t G, uint64_t n_items, int sms, cudaStream_t st) {
+cudaError_t launch_pass(const IndexLaunch& p, uint32_t G, uint64_t n_items, int sms, unsigned long long* work,
+                        cudaStream_t st) {
   constexpr bool ties = BM != kBinNone;
   constexpr uint32_t NB = BM == kBinNone ? 1u : (BM == kBinWindow ? kWinBins : 256u);
   const size_t smem = sizeof(IxSmem<KG, IxGeo<ties, KG>::kSlots, IxGeo<ties, KG>::kSlotBytes, NB>);
@@ -1079,10 +1119,9 @@ cudaError_t launch_pass(const IndexLaunch& p, uint32_t G, uint64_t n_items, int 
   uint64_t grid = (uint64_t)sms * IxGeo<ties, KG>::kCtasPerSm;
   if (grid > n_items) grid = n_items;
   cudaError_t e;
-  if ((e = launch_fill(p.work, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
   auto k = index_tma_kernel<BF16, KG, BM>;
   if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  k<<<(unsigned)grid, kIxThreads, smem, st>>>(p, G, n_items, p.work);
+  k<<<(unsigned)grid, kIxThreads, smem, st>>>(p, G, n_items, work);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1098,9 +1137,9 @@ cudaError_t launch_t(const IndexLaunch& p, cudaStream_t st) {
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if (!ties) return launch_pass<BF16, KG, kBinNone>(p, G, n_items, sms, st);
+  if (!ties) return launch_pass<BF16, KG, kBinNone>(p, G, n_items, sms, p.work, st);
   if (!p.wlo) {  // the two-level select for every pair
-    if ((e = launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, st)) != cudaSuccess) return e;
+    if ((e = launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
     if (p.defer_ties_select) return cudaSuccess;
     return ties_finish_t<BF16, KG>(p, st);
   }
@@ -1111,12 +1150,14 @@ cudaError_t launch_t(const IndexLaunch& p, cudaStream_t st) {
   ties_window_select<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
   count_launches(2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_pass<BF16, KG, kBinWindow>(p, G, n_items, sms, st)) != cudaSuccess) return e;
+  if ((e = launch_pass<BF16, KG, kBinWindow>(p, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
   ties_window_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
   count_launches(1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, st)) != cudaSuccess) return e;
-  return ties_finish_t<BF16, KG>(p, st);
+  IndexLaunch q = p;  // the selects of the fallback ride in its passes
+  q.select_in_pass = 1;
+  if ((e = launch_pass<BF16, KG, kBinCoarse>(q, G, n_items, sms, p.work + 1, st)) != cudaSuccess) return e;
+  return ties_finish_t<BF16, KG>(q, st);
 }
 
 template <bool BF16, int KG>
@@ -1140,8 +1181,8 @@ cudaError_t pass_t(const IndexLaunch& p, bool window, cudaStream_t st) {
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  return window ? launch_pass<BF16, KG, kBinWindow>(p, G, n_items, sms, st)
-                : launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, st);
+  return window ? launch_pass<BF16, KG, kBinWindow>(p, G, n_items, sms, p.work, st)
+                : launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, p.work, st);
 }
 
 template <bool BF16>

@@ -100,7 +100,7 @@ struct __align__(128) Smem {
   uint64_t empty[NS];
   unsigned long long realized[kMaxK];
   float2 ctab[kMaxK + 1];  // TIES: {c, RN(1/c)} for the counts c = 0..kMaxK (entry 0: {1, 1})
-  int abort;
+  int abort, last;
 };
 
 // packed fp32x2 arithmetic (two independent IEEE round-to-nearest operations per
@@ -334,6 +334,27 @@ __device__ __forceinline__ void dare_keep_words(const MergeLaunch& p, uint32_t i
   }
 }
 
+// The end of a merge kernel, reached by every warp of the CTA (a named barrier: the producer
+// warp and the consumers come from different places): when all of them are done, so are the
+// CTA's realized counts and error bits, and the last CTA of the launch writes the manifest to
+// the host's pinned copy.  It replaces two copy kernels after every merge.
+template <int THREADS>
+__device__ __forceinline__ void merge_end(const MergeLaunch& p, volatile int* s_last) {
+  if (!p.back_host) return;
+  __syncwarp();
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+  if (threadIdx.x == 0) {
+    __threadfence();
+    *s_last = atomicAdd(p.done, 1ull) == (unsigned long long)(gridDim.x - 1) ? 1 : 0;
+  }
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+  if (!*s_last) return;
+  __threadfence();
+  const uint32_t n = (uint32_t)kCounterSlots * p.K;
+  for (uint32_t k = threadIdx.x; k < n + 8u + (uint32_t)kBackTail; k += THREADS)
+    p.back_host[k] = k >= n && k < n + 8u ? (unsigned long long)p.back_summary[k - n] : __ldcg(p.realized + k);
+}
+
 template <bool BF16, int OPC>
 __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
     merge_tma_kernel(const MergeLaunch p, uint32_t cpb, uint64_t n_chunks, unsigned long long* work) {
@@ -475,6 +496,7 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
         if (S.realized[i])
           atomicAdd(p.realized + (uint64_t)(blockIdx.x % kCounterSlots) * p.K + i, S.realized[i]);
     }
+    merge_end<kConsumers + 32>(p, &S.last);
     return;
   }
 
@@ -647,6 +669,7 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
       }
     }
   }
+  merge_end<kConsumers + 32>(p, &S.last);
 }
 
 // ---------------- TIES (at most 8 experts) and DARE (at most 16): whole-chunk consumers ----------------
@@ -702,7 +725,7 @@ struct __align__(128) TcSmem {
   unsigned long long realized[KC];
   float2 ntab[kTcMaxK + 1];  // {-c, RN(1/c)} for the counts c = 0..16 (entry 0: {-1, 1})
   uint32_t nf[NS];           // producer only: fills held by the chunk of each entry
-  int abort;
+  int abort, last;
 };
 
 template <bool BF16, int OPC, int KC>
@@ -864,6 +887,7 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
         if (S.realized[i])
           atomicAdd(p.realized + (uint64_t)(blockIdx.x % kCounterSlots) * p.K + i, S.realized[i]);
     }
+    merge_end<kConsumers + 32>(p, &S.last);
     return;
   }
   // ---------------- consumers: thread t owns vector t of every chunk ----------------
@@ -1086,6 +1110,7 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
     }
     if (k0 < n) store_vec<BF16>(p.out, off + k0, n - k0, y);
   }
+  merge_end<kConsumers + 32>(p, &S.last);
 }
 
 template <bool BF16, int OPC, int KC>
@@ -1109,7 +1134,6 @@ cudaError_t launch_chunk(const MergeLaunch& p, cudaStream_t st) {
     return e;
   uint64_t grid = (uint64_t)sms * TcGeo<OPC, KC>::kCtasPerSm;
   if (grid > n_chunks) grid = n_chunks;
-  if ((e = launch_fill(p.work, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
   kern<<<(unsigned)grid, TcGeo<OPC, KC>::kThreads, smem, st>>>(p, cpb, n_chunks, p.work);
   count_launches(1);
   return cudaGetLastError();
@@ -1132,7 +1156,6 @@ cudaError_t launch_op(const MergeLaunch& p, cudaStream_t st) {
     return e;
   uint64_t grid = (uint64_t)sms * Geo<OPC>::kCtasPerSm;
   if (grid > n_chunks) grid = n_chunks;
-  if ((e = launch_fill(p.work, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
   merge_tma_kernel<BF16, OPC><<<(unsigned)grid, Geo<OPC>::kThreads, smem, st>>>(p, cpb, n_chunks, p.work);
   count_launches(1);
   return cudaGetLastError();

@@ -23,6 +23,7 @@ constexpr uint32_t kTauNone = 0x8000u;  // TIES threshold meaning "keep nothing"
 constexpr int kLanes = 256;             // lanes of the canonical norm order (one CTA)
 constexpr int kMaxK = 32;
 constexpr int kCounterSlots = 64;  // realized-byte counters are spread over slots
+constexpr int kBackTail = 4;       // words after the summary: the error word (16 bytes), the threshold reads (16)
 
 // device error word bits
 // (kErrBounds: a range failed a check of the checked build and was skipped)
@@ -227,7 +228,11 @@ struct IndexLaunch {
   uint32_t* miss;                 // [1] nonzero when some pair does
   const uint32_t* mask;        // the access mask for the fine pass, or null (every block)
   unsigned long long* thr_reads;  // expert bytes read by the fine pass, or null
-  unsigned long long* work;    // item counter of the dynamic scheduler (zeroed per launch)
+  // item counters of the dynamic scheduler, zeroed with the handle: work[0] of the catalog
+  // pass, work[1] of the fallback pass; work[2] and work[3] count the CTAs of the fallback pass
+  // and of the fine pass that are done (the last one selects, when select_in_pass is set)
+  unsigned long long* work;
+  uint32_t select_in_pass;
   // the launch covers blocks [b_begin, b_end); expert pointers address element
   // expert_origin of the flat layout (0 for resident experts, a segment start when they
   // point into a staging buffer)
@@ -322,8 +327,14 @@ struct MergeLaunch {
   uint32_t dare_rk[10][2];  // DARE: Philox round keys of the seed (precomputed on the host)
   uint64_t seed;
   unsigned long long* realized;  // [kCounterSlots][K]
-  unsigned long long* work;      // chunk counter of the dynamic scheduler (zeroed per launch)
+  unsigned long long* work;      // chunk counter of the dynamic scheduler (zeroed with the manifest)
   uint32_t* err;
+  // the manifest's way back, by the last CTA of the launch that has it set: the realized
+  // counters and kBackTail words after the summary's place, with the plan's summary between
+  // them, into the host's pinned copy; done counts the CTAs (zeroed with the manifest)
+  unsigned long long* back_host;  // or null
+  const uint64_t* back_summary;
+  unsigned long long* done;
   uint64_t b_begin, b_end, expert_origin;  // as in IndexLaunch
   Extents ext;                             // as in IndexLaunch
   uint32_t touched_only;  // 1: blocks with an empty mask are neither read nor written
@@ -351,9 +362,24 @@ struct GatherLaunch {
   uint32_t* err;                 // the call's error word (checked build)
 };
 cudaError_t launch_gather(const GatherLaunch& g, cudaStream_t st);
-// copies and fills by kernel on st (no copy engine); host buffers must be pinned memory
-cudaError_t launch_copy(void* dst, const void* src, size_t bytes, cudaStream_t st);
+// fills by kernel on st (no copy engine)
 cudaError_t launch_fill(void* dst, uint32_t byte_value, size_t bytes, cudaStream_t st);
+// what a handle's memory starts from, in one launch: copies from pinned host memory (src) and
+// zeroed ranges (src null); every address is 16-byte aligned
+struct InitSeg {
+  void* dst;
+  const void* src;
+  size_t bytes;
+};
+struct InitList {
+  static constexpr uint32_t kMax = 8;
+  InitSeg seg[kMax];
+  uint32_t n = 0;
+  void add(void* dst, const void* src, size_t bytes) {
+    if (bytes) seg[n++] = InitSeg{dst, src, bytes};
+  }
+};
+cudaError_t launch_init(const InitList& l, cudaStream_t st);
 
 // ---- block content hashes (hash.cu) --------------------------------------------------------
 // catalog mode (validate = 0): hash every block of the base and of each expert into
