@@ -246,16 +246,36 @@ __device__ __forceinline__ uint4 read_raw(const uint8_t* slot, const void* gsrc,
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// elements 2k and 2k + 1 of a raw vector as fp32 (k is a compile-time index)
+// the deltas of elements 2k and 2k + 1 of a raw vector against the base elements a and b (k is a
+// compile-time index), each one IEEE fp32 subtraction.  bf16 elements are converted by the
+// mixed-precision subtract itself (128 lanes per clock and SM): two instructions per pair where
+// moving both up to fp32 and a packed subtract take three, two of them at half rate (DARE with 4
+// experts 1.436 -> 1.385 ms, TIES with 8 experts 0.851 -> 0.819 ms).
 template <bool BF16, int k>
-__device__ __forceinline__ void pair_of(const uint4 r, float& a, float& b) {
+__device__ __forceinline__ void delta_pair(const uint4 r, float a, float b, float& d0, float& d1) {
   if constexpr (BF16) {
     const uint32_t w = k == 0 ? r.x : (k == 1 ? r.y : (k == 2 ? r.z : r.w));
-    a = __uint_as_float(w * 65536u);
-    b = __uint_as_float(w & 0xFFFF0000u);
+    asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n sub.rn.f32.bf16 %0, l, %3;\n sub.rn.f32.bf16 %1, h, %4;\n}"
+        : "=f"(d0), "=f"(d1)
+        : "r"(w), "f"(a), "f"(b));
   } else {
-    a = __uint_as_float(k == 0 ? r.x : r.z);
-    b = __uint_as_float(k == 0 ? r.y : r.w);
+    f2_sub(__uint_as_float(k == 0 ? r.x : r.z), __uint_as_float(k == 0 ? r.y : r.w), a, b, d0, d1);
+  }
+}
+
+// fold(v, d0, d1) for the deltas of elements v and v + 1 of a raw vector, v = 0, 2, ...
+template <bool BF16, typename Fold>
+__device__ __forceinline__ void delta_pairs(const uint4 r, const float* x0, Fold fold) {
+  float d0, d1;
+  delta_pair<BF16, 0>(r, x0[0], x0[1], d0, d1);
+  fold(0, d0, d1);
+  delta_pair<BF16, 1>(r, x0[2], x0[3], d0, d1);
+  fold(2, d0, d1);
+  if constexpr (BF16) {
+    delta_pair<BF16, 2>(r, x0[4], x0[5], d0, d1);
+    fold(4, d0, d1);
+    delta_pair<BF16, 3>(r, x0[6], x0[7], d0, d1);
+    fold(6, d0, d1);
   }
 }
 
@@ -314,23 +334,45 @@ __device__ __forceinline__ bool checked_chunk(const MergeLaunch& p, uint64_t b, 
   return false;
 }
 
-// DARE keep words of the vector at flat element j0 for expert i: element j keeps its delta
-// iff 16-bit word j mod 8 of the Philox4x32-10 output for counter j / 8 is >= T.  A bf16
-// vector is exactly the 8 words of one call (chunk and tensor offsets are multiples of 8
-// elements); an fp32 vector is half of one.  Word j mod 8 of element j is returned in the
-// upper half of a 32-bit register: the upper word as it stands, the lower one moved up by a
-// multiply (FMA pipe; the ALU pipe is the busy one); it is kept iff that register >= T << 16.
+// DARE keep words: element j of expert i keeps its delta iff 16-bit word j mod 8 of the
+// Philox4x32-10 output for counter (j / 8, i, tag) is >= T.  A bf16 vector is exactly the 8 words
+// of one call (chunk and tensor offsets are multiples of 8 elements); an fp32 vector is half of
+// one.  The whole-chunk kernel keeps the experts' share of the first two rounds in shared memory,
+// for the kDareHi lowest values of a group number's upper word (a test for larger ones in its
+// loop cost 10 instructions per vector and expert, 5 % of the DARE merge); families past
+// kDareSpan elements take the streaming kernel, which makes that share for each fill.
+constexpr uint32_t kDareHi = 4;
+constexpr uint64_t kDareSpan = (uint64_t)kDareHi << 35;
+constexpr uint32_t kDareTag = 0x44415245u;
+
+struct DareVec {
+  PhiloxGroup grp;
+  uint32_t g_hi;  // upper word of the group number
+  bool upper;     // fp32: the vector is the upper half of its group
+};
+
+__device__ __forceinline__ DareVec dare_vec(const MergeLaunch& p, uint64_t j0) {
+  const uint64_t g = j0 >> 3;
+  return DareVec{philox_group((uint32_t)g, kDareTag, p.dare_rk), (uint32_t)(g >> 32), (j0 & 4u) != 0u};
+}
+
+__device__ __forceinline__ uint4 dare_expert(const MergeLaunch& p, uint32_t g_hi, uint32_t i) {
+  const PhiloxExpert e = philox_expert(g_hi, i, p.dare_rk);
+  return make_uint4(e.x0, e.x2, e.x3, __float_as_uint(p.alpha[i]));
+}
+
+// word j mod 8 of element j in the upper half of a 32-bit register: the upper word as it
+// stands, the lower one moved up by a multiply (FMA pipe; the ALU pipe is the busy one); it is
+// kept iff that register >= T << 16
 template <bool BF16>
-__device__ __forceinline__ void dare_keep_words(const MergeLaunch& p, uint32_t i, uint64_t j0,
+__device__ __forceinline__ void dare_keep_words(const MergeLaunch& p, const DareVec& v, const uint4 pe,
                                                 uint32_t (&kw)[BF16 ? 8 : 4]) {
   constexpr int V = BF16 ? 8 : 4;
-  const uint64_t g = j0 >> 3;
-  const Philox4 r = philox4x32_10_rk((uint32_t)g, (uint32_t)(g >> 32), i, 0x44415245u, p.dare_rk);
-  const uint32_t e0 = (uint32_t)(j0 & 7u);  // 0 for bf16; 0 or 4 for fp32
+  const Philox4 r = philox_finish(v.grp, PhiloxExpert{pe.x, pe.y, pe.z}, p.dare_rk);
 #pragma unroll
-  for (int e = 0; e < V; ++e) {
-    const uint32_t wd = BF16 ? r.w[e >> 1] : (e0 ? r.w[2 + (e >> 1)] : r.w[e >> 1]);
-    kw[e] = (e & 1) ? wd : wd * 65536u;
+  for (int k = 0; k < V; ++k) {
+    const uint32_t wd = BF16 ? r.w[k >> 1] : (v.upper ? r.w[2 + (k >> 1)] : r.w[k >> 1]);
+    kw[k] = (k & 1) ? wd : wd * 65536u;
   }
 }
 
@@ -382,6 +424,7 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
     mbar_fence_init();
   }
   if (tid < (uint32_t)kMaxK) S.realized[tid] = 0;
+  constexpr bool kDare = OPC == OP_DARE || OPC == OP_DTIES;
   if (tid <= (uint32_t)kMaxK) {
     const float c = tid == 0 ? 1.0f : (float)tid;
     S.ctab[tid] = make_float2(c, __fdiv_rn(1.0f, c));
@@ -508,10 +551,11 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
   uint32_t m_chunk = 0, m_rest = 0;  // the chunk's access mask; its experts still to come
   float s_sel = 0.0f;  // renormalised AVG: sum of the counted experts' alpha (ascending)
   // DARE keep decisions of the vector's elements (dare_keep_words)
-  auto dare_words = [&](uint32_t i, uint64_t j0, uint32_t (&kw)[V]) { dare_keep_words<BF16>(p, i, j0, kw); };
-  auto dare_kept = [&](uint32_t i, uint64_t j0, bool (&kept)[V]) {
+  DareVec dv[VPT];
+  auto dare_words = [&](uint32_t i, int u, uint32_t (&kw)[V]) { dare_keep_words<BF16>(p, dv[u], dare_expert(p, dv[u].g_hi, i), kw); };
+  auto dare_kept = [&](uint32_t i, int u, bool (&kept)[V]) {
     uint32_t kw[V];
-    dare_words(i, j0, kw);
+    dare_words(i, u, kw);
 #pragma unroll
     for (int e = 0; e < V; ++e) kept[e] = kw[e] >= p.dare_T16;
   };
@@ -542,6 +586,7 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
         const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
         read_vec<BF16>(slot, p.base, off, k0, n, n_tma, x0[u]);
         if (remaining) {
+          if constexpr (kDare) dv[u] = dare_vec(p, off + k0);
 #pragma unroll
           for (int e = 0; e < V; ++e) {
             acc[u][e] = 0.0f;
@@ -567,7 +612,7 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
           float xe[V];
           read_vec<BF16>(slot, src, off - p.expert_origin, k0, n, n_tma, xe);
           uint32_t kw[V];
-          if constexpr (OPC == OP_DTIES) dare_words(i, off + k0, kw);
+          if constexpr (OPC == OP_DTIES) dare_words(i, u, kw);
 #pragma unroll
           for (int e = 0; e < V; e += 2) {
             // the deltas of an element pair in one packed fp32x2 subtract
@@ -593,7 +638,7 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
           float xe[V];
           read_vec<BF16>(slot, src, off - p.expert_origin, k0, n, n_tma, xe);
           bool kept[V];
-          if constexpr (OPC == OP_DARE) dare_kept(i, off + k0, kept);
+          if constexpr (OPC == OP_DARE) dare_kept(i, u, kept);
 #pragma unroll
           for (int e = 0; e < V; e += 2) {
             float d0, d1;
@@ -684,23 +729,30 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
 // streaming kernel disappear.  The ring must hold every fill of one chunk (1 + K slots), so
 // this kernel serves TIES with K <= 8 and DARE with K <= 16; the streaming kernel above
 // serves the other operators and larger expert counts.
-constexpr uint32_t kTcSlotBytes = 4096u;
 constexpr uint32_t kTcMaxK = 16;
 
 // ring slots and CTAs per SM by expert count: K <= 4 holds two chunks of 5 fills in 11
 // slots at four CTAs per SM (three for DARE-TIES, whose state needs more registers); K <= 8
 // two chunks of 9 fills in 18 slots at three; K <= 16 one chunk of 17 fills, or several of
-// the usual few selected experts, in 17 slots at three
+// the usual few selected experts, in 17 slots at three.  A fill is 4 KiB: 256 consumer threads
+// take one vector each, but for TIES with K <= 4 128 threads take two (a chunk's wait, release
+// and metadata reads are then shared by two vectors, and 96 registers a thread hold both: 1.015
+// -> 0.980 ms on four Llama layers at the full budget).  Measured and not taken, on DARE and
+// DARE-TIES with 16 experts (1.41 and 2.17 ms here): two vectors per thread 1.47 and 2.47 ms,
+// 2 KiB fills at six CTAs per SM 1.55 and 2.37, 3 KiB fills at four 1.46 and 2.42; TIES with 8
+// experts (0.82 ms): two vectors 0.83, 3 KiB fills 0.99.
 template <int OPC, int KC>
 struct TcGeo {
   static constexpr int kSlots = KC <= 4 ? 11 : (KC <= 8 ? 18 : 17);
   static constexpr int kCtasPerSm = KC <= 4 && OPC != OP_DTIES ? 4 : 3;
-  static constexpr int kConsumers = 256;
+  static constexpr int kVpt = KC <= 4 && OPC == OP_TIES ? 2 : 1;  // vectors per consumer thread and fill
+  static constexpr int kConsumers = 256 / kVpt;
   static constexpr int kThreads = kConsumers + 32;
+  static constexpr uint32_t kSlotBytes = kConsumers * kVpt * 16u;
   static constexpr uint32_t kGrab = 8;
 };
 
-template <int KC>
+template <int KC, int NT>
 struct TcEntry {
   uint64_t off;          // element offset of the chunk
   uint32_t q;            // chunk id, or kEnd
@@ -709,22 +761,24 @@ struct TcEntry {
   uint32_t s0;           // ring slot of the base fill; expert fill j sits in slot s0 + 1 + j (mod NS)
   uint32_t nsel;         // selected experts
   uint32_t fast;         // 1: every selected threshold is >= 2^-100 (no numerator needs the IEEE division)
-  float thr[KC];         // TIES: trim thresholds (as floats) in fill order
+  float thr[NT];         // TIES: trim thresholds (as floats) in fill order
   uint8_t ex[KC];        // the selected experts in fill order
 };
 
 // sized by the expert count KC so that three CTAs of 18 slots fit one SM's 228 KB
-template <int NS, uint32_t G, int KC>
+template <int NS, uint32_t SB, uint32_t G, int KC, bool TIES>
 struct __align__(128) TcSmem {
-  uint8_t slot[NS][kTcSlotBytes];
-  TcEntry<KC> ce[NS];
+  static constexpr int NT = TIES ? KC : 1, NE = TIES ? 1 : KC;
+  uint8_t slot[NS][SB];
+  TcEntry<KC, NT> ce[NS];
   ChunkMeta chunk[G];
-  uint32_t thr[G][KC];  // bits threshold of (chunk of the grab, expert)
+  uint32_t thr[G][NT];  // TIES: bits threshold of (chunk of the grab, expert)
   uint64_t full[NS];
   uint64_t empty[NS];
   unsigned long long realized[KC];
   float2 ntab[kTcMaxK + 1];  // {-c, RN(1/c)} for the counts c = 0..16 (entry 0: {-1, 1})
   uint32_t nf[NS];           // producer only: fills held by the chunk of each entry
+  uint4 pe[TIES ? 1 : kDareHi][NE];  // DARE, DARE-TIES: dare_expert of every expert, by the group's upper word
   int abort, last;
 };
 
@@ -738,12 +792,16 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
   constexpr int kConsumers = TcGeo<OPC, KC>::kConsumers;
   constexpr uint32_t G = TcGeo<OPC, KC>::kGrab;
   constexpr uint32_t ES = BF16 ? 2u : 4u;
-  constexpr uint32_t CH = kTcSlotBytes / ES;  // elements per chunk
+  constexpr uint32_t SB = TcGeo<OPC, KC>::kSlotBytes;
+  constexpr uint32_t CH = SB / ES;  // elements per chunk
   constexpr int V = BF16 ? 8 : 4;
-  static_assert(CH == (uint32_t)(kConsumers * V), "one vector per consumer thread and chunk");
+  constexpr int VPT = TcGeo<OPC, KC>::kVpt;
+  constexpr int kThreads = kConsumers + 32;
+  static_assert(CH == (uint32_t)(kConsumers * VPT * V), "whole vectors per consumer thread and chunk");
   static_assert(NS >= KC + 1, "the ring holds every fill of a chunk");
   extern __shared__ __align__(128) uint8_t smem_raw[];
-  TcSmem<NS, G, KC>& S = *reinterpret_cast<TcSmem<NS, G, KC>*>(smem_raw);
+  using Sm = TcSmem<NS, SB, G, KC, OPC == OP_TIES>;
+  Sm& S = *reinterpret_cast<Sm*>(smem_raw);
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
   volatile int* abort_flag = &S.abort;
   const uint32_t wl = wait_limit_of(p.wait_limit);
@@ -757,6 +815,9 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
     mbar_fence_init();
   }
   if (tid < (uint32_t)KC) S.realized[tid] = 0;
+  if (OPC != OP_TIES)
+    for (uint32_t k = tid; k < kDareHi * KC; k += kThreads)
+      if (k % KC < p.K) S.pe[k / KC][k % KC] = dare_expert(p, k / KC, k % KC);
   if (tid <= kTcMaxK) {
     const float c = tid == 0 ? 1.0f : (float)tid;
     S.ntab[tid] = make_float2(-c, __fdiv_rn(1.0f, c));
@@ -824,7 +885,7 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
           if (fill >= (uint32_t)NS) fence_proxy_async_smem();  // slots the consumers have read are refilled
           const uint32_t e = seq % NS;
           const uint32_t bytes = (cm.n * ES) & ~15u;
-          TcEntry<KC>& ce = S.ce[e];
+          auto& ce = S.ce[e];
           ce.off = cm.off;
           ce.q = (uint32_t)(q0 + c);
           ce.n = cm.n;
@@ -890,8 +951,7 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
     merge_end<kConsumers + 32>(p, &S.last);
     return;
   }
-  // ---------------- consumers: thread t owns vector t of every chunk ----------------
-  const uint32_t k0 = tid * (uint32_t)V;
+  // ---------------- consumers: thread t owns vectors t, t + kConsumers, ... of every chunk ----------------
   for (uint32_t c = 0;; ++c) {
     const uint32_t e = c % NS;
     if (!warp_wait<true>(&S.full[e], (c / NS) & 1u, abort_flag, wl)) {
@@ -899,140 +959,147 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
       S.abort = 1;
       break;
     }
-    const TcEntry<KC>& ce = S.ce[e];
+    const auto& ce = S.ce[e];
     if (ce.q == kEnd) break;
     uint32_t s = ce.s0;
     const uint32_t nsel = ce.nsel;
-    float x0[V];
-    bool in_slot;  // the thread's vector lies inside the bulk-copied bytes
+    float x0[VPT][V];
+    bool in_slot = true;  // the thread's vectors lie inside the bulk-copied bytes
     {
       const uint32_t n = ce.n, n_tma = ((n * ES) & ~15u) / ES;
-      in_slot = k0 + V <= n_tma;
-      read_vec<BF16>(S.slot[s], p.base, ce.off, k0, n, n_tma, x0);
+#pragma unroll
+      for (int u = 0; u < VPT; ++u) {
+        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
+        in_slot = in_slot && k0 + V <= n_tma;
+        read_vec<BF16>(S.slot[s], p.base, ce.off, k0, n, n_tma, x0[u]);
+      }
     }
-    float y[V];
+    float y[VPT][V];
+    auto store = [&](uint64_t off, uint32_t n) {
+#pragma unroll
+      for (int u = 0; u < VPT; ++u) {
+        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
+        if (k0 < n) store_vec<BF16>(p.out, off + k0, n - k0, y[u]);
+      }
+    };
     if (nsel == 0) {  // uniform over the CTA
       // no expert selected: the output is M_0 plus the zero the operator adds (lambda * +0
       // for TIES, +0 for DARE)
       const float z = kTiesLike<OPC> ? __fmul_rn(p.lambda, 0.0f) : 0.0f;
 #pragma unroll
-      for (int v = 0; v < V; ++v) y[v] = __fadd_rn(x0[v], z);
+      for (int u = 0; u < VPT; ++u)
+#pragma unroll
+        for (int v = 0; v < V; ++v) y[u][v] = __fadd_rn(x0[u][v], z);
       const uint64_t off = ce.off;
       const uint32_t n = ce.n;
       mbar_arrive(&S.empty[e]);
-      if (k0 < n) store_vec<BF16>(p.out, off + k0, n - k0, y);
+      store(off, n);
       continue;
     }
+    DareVec dv[VPT];
+    if constexpr (OPC != OP_TIES) {
+#pragma unroll
+      for (int u = 0; u < VPT; ++u) dv[u] = dare_vec(p, ce.off + (tid + (uint32_t)u * kConsumers) * V);
+    }
+    // the raw vector u of the fill in slot sl, expert j of the chunk's selected ones
+    auto raw = [&](uint32_t sl, uint32_t j, int u) -> uint4 {
+      const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
+      if (in_slot) return *reinterpret_cast<const uint4*>(S.slot[sl] + k0 * ES);
+      // the ragged tail of a tensor, from global memory
+      const uint32_t n = ce.n;
+      return read_raw<BF16>(S.slot[sl], p.experts.p[ce.ex[j]], ce.off - p.expert_origin, k0, n, ((n * ES) & ~15u) / ES);
+    };
     if constexpr (OPC == OP_DARE) {
       // acc = fma(alpha_i, v_i, acc) over the selected experts whose keep word passes, in
       // ascending order, with v_i = delta_i * sigma (a dropped entry is omitted)
-      float acc[V];
+      float acc[VPT][V];
 #pragma unroll
-      for (int v = 0; v < V; ++v) acc[v] = 0.0f;
+      for (int u = 0; u < VPT; ++u)
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[u][v] = 0.0f;
 #pragma unroll 1
       for (uint32_t j = 0; j < nsel; ++j) {
         s = s + 1 == (uint32_t)NS ? 0u : s + 1;
         const uint32_t i = ce.ex[j];
-        const float a = p.alpha[i];
-        uint4 r;
-        if (in_slot) {
-          r = *reinterpret_cast<const uint4*>(S.slot[s] + k0 * ES);
-        } else {  // the ragged tail of a tensor, from global memory
-          const uint32_t n = ce.n;
-          r = read_raw<BF16>(S.slot[s], p.experts.p[i], ce.off - p.expert_origin, k0, n, ((n * ES) & ~15u) / ES);
-        }
-        uint32_t kw[V];
-        dare_keep_words<BF16>(p, i, ce.off + k0, kw);
-        auto fold_pair = [&](int v, float e0, float e1) {
-          float d0, d1, s0, s1;
-          f2_sub(e0, e1, x0[v], x0[v + 1], d0, d1);
-          f2_mul(d0, d1, p.sigma, p.sigma, s0, s1);
-          // a dropped entry is omitted from the sum, as an unselected one is
-          if (kw[v] >= p.dare_T16) acc[v] = __fmaf_rn(a, s0, acc[v]);
-          if (kw[v + 1] >= p.dare_T16) acc[v + 1] = __fmaf_rn(a, s1, acc[v + 1]);
-        };
-        float e0, e1;
-        pair_of<BF16, 0>(r, e0, e1);
-        fold_pair(0, e0, e1);
-        pair_of<BF16, 1>(r, e0, e1);
-        fold_pair(2, e0, e1);
-        if constexpr (BF16) {
-          pair_of<BF16, 2>(r, e0, e1);
-          fold_pair(4, e0, e1);
-          pair_of<BF16, 3>(r, e0, e1);
-          fold_pair(6, e0, e1);
+#pragma unroll
+        for (int u = 0; u < VPT; ++u) {
+          const uint4 pe = S.pe[dv[u].g_hi][i];
+          const float a = __uint_as_float(pe.w);
+          const uint4 r = raw(s, j, u);
+          uint32_t kw[V];
+          dare_keep_words<BF16>(p, dv[u], pe, kw);
+          auto fold_pair = [&](int v, float d0, float d1) {
+            float s0, s1;
+            f2_mul(d0, d1, p.sigma, p.sigma, s0, s1);
+            // a dropped entry is omitted from the sum, as an unselected one is
+            if (kw[v] >= p.dare_T16) acc[u][v] = __fmaf_rn(a, s0, acc[u][v]);
+            if (kw[v + 1] >= p.dare_T16) acc[u][v + 1] = __fmaf_rn(a, s1, acc[u][v + 1]);
+          };
+          delta_pairs<BF16>(r, x0[u], fold_pair);
         }
       }
       const uint64_t off = ce.off;
       const uint32_t n = ce.n;
       mbar_arrive(&S.empty[e]);  // every read of the chunk's slots and entry is done
 #pragma unroll
-      for (int v = 0; v < V; v += 2) f2_add(x0[v], x0[v + 1], acc[v], acc[v + 1], y[v], y[v + 1]);
-      if (k0 < n) store_vec<BF16>(p.out, off + k0, n - k0, y);
+      for (int u = 0; u < VPT; ++u)
+#pragma unroll
+        for (int v = 0; v < V; v += 2)
+          f2_add(x0[u][v], x0[u][v + 1], acc[u][v], acc[u][v + 1], y[u][v], y[u][v + 1]);
+      store(off, n);
       continue;
     }
     // Per element: P and N, the sums of the kept positive and negative deltas, and both
     // counts in one float C = 2^23 + c+ + 2^CB c- (exact: every value is an integer below
     // 2^24, so the low bits of C hold c+ and c-).  DARE-TIES keeps, instead, every nonzero
-    // rescaled delta s = d sigma whose keep word passes (no magnitude trim).  A delta d is kept positive when d >= thr and kept
-    // negative when d <= -thr (thr > 0: |d| >= thr and the sign in one compare each); the
-    // keep factors k+ and k- are 1 or 0, and P = fma(k+, d, P), N = fma(k-, d, N): a factor 1
-    // adds d with the one rounding of P + d, a factor 0 adds a zero, which leaves P and N
-    // unchanged (they start at +0 and are never -0).  Two elements per packed instruction.
-    float Pp[V], Nn[V], Cc[V];
+    // rescaled delta s = d sigma whose keep word passes (no magnitude trim).  A delta d is
+    // kept positive when d >= thr and kept negative when d <= -thr (thr > 0: |d| >= thr and
+    // the sign in one compare each); the keep factors k+ and k- are 1 or 0, and
+    // P = fma(k+, d, P), N = fma(k-, d, N): a factor 1 adds d with the one rounding of P + d,
+    // a factor 0 adds a zero, which leaves P and N unchanged (they start at +0 and are never
+    // -0).  Two elements per packed instruction.
+    float Pp[VPT][V], Nn[VPT][V], Cc[VPT][V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      Pp[v] = 0.0f;
-      Nn[v] = 0.0f;
-      Cc[v] = 8388608.0f;  // 2^23
-    }
+    for (int u = 0; u < VPT; ++u)
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        Pp[u][v] = 0.0f;
+        Nn[u][v] = 0.0f;
+        Cc[u][v] = 8388608.0f;  // 2^23
+      }
     // the selected experts in ascending order: fill j of the chunk sits in slot s0 + 1 + j
 #pragma unroll 1
     for (uint32_t j = 0; j < nsel; ++j) {
       s = s + 1 == (uint32_t)NS ? 0u : s + 1;
       const float thr = OPC == OP_TIES ? ce.thr[j] : 0.0f;
-      uint32_t kw[V];
-      if constexpr (OPC == OP_DTIES) dare_keep_words<BF16>(p, ce.ex[j], ce.off + k0, kw);
-      uint4 r;
-      if (in_slot) {
-        r = *reinterpret_cast<const uint4*>(S.slot[s] + k0 * ES);
-      } else {  // the ragged tail of a tensor, from global memory (expert = j-th selected)
-        const uint32_t i = __fns(ce.m, 0, (int)j + 1), n = ce.n;
-        r = read_raw<BF16>(S.slot[s], p.experts.p[i], ce.off - p.expert_origin, k0, n, ((n * ES) & ~15u) / ES);
-      }
-      // one element pair at a time, so that only the raw vector stays live
-      auto tally_pair = [&](int v, float e0, float e1) {
-        float d0, d1, t0, t1, kp0, kp1, kn0, kn1;
-        f2_sub(e0, e1, x0[v], x0[v + 1], d0, d1);
-        if constexpr (OPC == OP_DTIES) {
-          f2_mul(d0, d1, p.sigma, p.sigma, d0, d1);
-          // keep factors as 1.0 / 0.0 straight from compares joined with the keep test
-          asm("{\n .reg .pred q;\n setp.ge.u32 q, %4, %5;\n set.gt.and.f32.f32 %0, %6, 0f00000000, q;\n"
-              " set.lt.and.f32.f32 %1, %6, 0f00000000, q;\n setp.ge.u32 q, %7, %5;\n"
-              " set.gt.and.f32.f32 %2, %8, 0f00000000, q;\n set.lt.and.f32.f32 %3, %8, 0f00000000, q;\n}"
-              : "=f"(kp0), "=f"(kn0), "=f"(kp1), "=f"(kn1)
-              : "r"(kw[v]), "r"(p.dare_T16), "f"(d0), "r"(kw[v + 1]), "f"(d1));
-        } else {
-          kp0 = d0 >= thr ? 1.0f : 0.0f;
-          kp1 = d1 >= thr ? 1.0f : 0.0f;
-          kn0 = d0 <= -thr ? 1.0f : 0.0f;
-          kn1 = d1 <= -thr ? 1.0f : 0.0f;
-        }
-        f2_fma(kp0, kp1, d0, d1, Pp[v], Pp[v + 1], Pp[v], Pp[v + 1]);
-        f2_fma(kn0, kn1, d0, d1, Nn[v], Nn[v + 1], Nn[v], Nn[v + 1]);
-        f2_fma(kn0, kn1, (float)(1u << CB), (float)(1u << CB), kp0, kp1, t0, t1);
-        f2_add(Cc[v], Cc[v + 1], t0, t1, Cc[v], Cc[v + 1]);
-      };
-      float e0, e1;
-      pair_of<BF16, 0>(r, e0, e1);
-      tally_pair(0, e0, e1);
-      pair_of<BF16, 1>(r, e0, e1);
-      tally_pair(2, e0, e1);
-      if constexpr (BF16) {
-        pair_of<BF16, 2>(r, e0, e1);
-        tally_pair(4, e0, e1);
-        pair_of<BF16, 3>(r, e0, e1);
-        tally_pair(6, e0, e1);
+#pragma unroll
+      for (int u = 0; u < VPT; ++u) {
+        uint32_t kw[V];
+        if constexpr (OPC == OP_DTIES) dare_keep_words<BF16>(p, dv[u], S.pe[dv[u].g_hi][ce.ex[j]], kw);
+        const uint4 r = raw(s, j, u);
+        // one element pair at a time, so that only the raw vector stays live
+        auto tally_pair = [&](int v, float d0, float d1) {
+          float t0, t1, kp0, kp1, kn0, kn1;
+          if constexpr (OPC == OP_DTIES) {
+            f2_mul(d0, d1, p.sigma, p.sigma, d0, d1);
+            // keep factors as 1.0 / 0.0 straight from compares joined with the keep test
+            asm("{\n .reg .pred q;\n setp.ge.u32 q, %4, %5;\n set.gt.and.f32.f32 %0, %6, 0f00000000, q;\n"
+                " set.lt.and.f32.f32 %1, %6, 0f00000000, q;\n setp.ge.u32 q, %7, %5;\n"
+                " set.gt.and.f32.f32 %2, %8, 0f00000000, q;\n set.lt.and.f32.f32 %3, %8, 0f00000000, q;\n}"
+                : "=f"(kp0), "=f"(kn0), "=f"(kp1), "=f"(kn1)
+                : "r"(kw[v]), "r"(p.dare_T16), "f"(d0), "r"(kw[v + 1]), "f"(d1));
+          } else {
+            kp0 = d0 >= thr ? 1.0f : 0.0f;
+            kp1 = d1 >= thr ? 1.0f : 0.0f;
+            kn0 = d0 <= -thr ? 1.0f : 0.0f;
+            kn1 = d1 <= -thr ? 1.0f : 0.0f;
+          }
+          f2_fma(kp0, kp1, d0, d1, Pp[u][v], Pp[u][v + 1], Pp[u][v], Pp[u][v + 1]);
+          f2_fma(kn0, kn1, d0, d1, Nn[u][v], Nn[u][v + 1], Nn[u][v], Nn[u][v + 1]);
+          f2_fma(kn0, kn1, (float)(1u << CB), (float)(1u << CB), kp0, kp1, t0, t1);
+          f2_add(Cc[u][v], Cc[u][v + 1], t0, t1, Cc[u][v], Cc[u][v + 1]);
+        };
+        delta_pairs<BF16>(r, x0[u], tally_pair);
       }
     }
     const uint64_t off = ce.off;
@@ -1041,10 +1108,10 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
     // the elected side's sum and count: the sign of P + N taken exactly as P > -N or P < -N
     // (then that side holds at least one entry, so c >= 1); otherwise the numerator +0, whose
     // quotient is +0 whatever count (<= 16, a valid table entry) is paired with it
-    auto num_c = [&](int v, float& num, uint32_t& cv) {
-      const bool pos = Pp[v] > -Nn[v], any = Pp[v] != -Nn[v];
-      num = any ? (pos ? Pp[v] : Nn[v]) : 0.0f;
-      const uint32_t cb = __float_as_uint(Cc[v]);
+    auto num_c = [&](int u, int v, float& num, uint32_t& cv) {
+      const bool pos = Pp[u][v] > -Nn[u][v], any = Pp[u][v] != -Nn[u][v];
+      num = any ? (pos ? Pp[u][v] : Nn[u][v]) : 0.0f;
+      const uint32_t cb = __float_as_uint(Cc[u][v]);
       cv = (pos ? cb : cb >> CB) & ((1u << CB) - 1u);
     };
     // q = RN(num * y), then Markstein's correction q + RN(num - q c) * y, and the output
@@ -1055,28 +1122,32 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
       // 2 * bits(2^-100) - 2 exactly when some numerator has 0 < |num| < 2^-100
       uint32_t lowest = 0xFFFFFFFFu;
 #pragma unroll
-      for (int v = 0; v < V; v += 2) {
+      for (int u = 0; u < VPT; ++u)
+#pragma unroll
+        for (int v = 0; v < V; v += 2) {
         float a0, a1, q0, q1, r0, r1;
         uint32_t c0, c1;
-        num_c(v, a0, c0);
-        num_c(v + 1, a1, c1);
+        num_c(u, v, a0, c0);
+        num_c(u, v + 1, a1, c1);
         if constexpr (decltype(checked)::value)
           lowest = min(lowest, min(__float_as_uint(a0) * 2u - 2u, __float_as_uint(a1) * 2u - 2u));
         const float2 t0 = S.ntab[c0], t1 = S.ntab[c1];
         f2_mul(a0, a1, t0.y, t1.y, q0, q1);
         f2_fma(q0, q1, t0.x, t1.x, a0, a1, r0, r1);
         f2_fma(r0, r1, t0.y, t1.y, q0, q1, q0, q1);
-        f2_fma(p.lambda, p.lambda, q0, q1, x0[v], x0[v + 1], y[v], y[v + 1]);
+        f2_fma(p.lambda, p.lambda, q0, q1, x0[u][v], x0[u][v + 1], y[u][v], y[u][v + 1]);
       }
       static_assert(0x0D800000u * 2u - 2u == 0x1AFFFFFEu, "bits of 2^-100");
       const bool exact = decltype(checked)::value && lowest < 0x1AFFFFFEu;
       if (decltype(checked)::value && __any_sync(0xFFFFFFFFu, exact)) {
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
+        for (int u = 0; u < VPT; ++u)
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
           float a;
           uint32_t cv;
-          num_c(v, a, cv);
-          if (div_small_needs_ieee(a)) y[v] = __fmaf_rn(p.lambda, __fdiv_rn(a, -S.ntab[cv].x), x0[v]);
+          num_c(u, v, a, cv);
+          if (div_small_needs_ieee(a)) y[u][v] = __fmaf_rn(p.lambda, __fdiv_rn(a, -S.ntab[cv].x), x0[u][v]);
         }
       }
     };
@@ -1088,34 +1159,41 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
       // TIES chunks with a threshold below 2^-100 (rare): one element at a time
       bool exact = false;
 #pragma unroll
-      for (int v = 0; v < V; ++v) {
+      for (int u = 0; u < VPT; ++u)
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
         float a;
         uint32_t cv;
-        num_c(v, a, cv);
+        num_c(u, v, a, cv);
         const float2 t = S.ntab[cv];
-        y[v] = div_small_fast(a, -t.x, t.y);
+        y[u][v] = div_small_fast(a, -t.x, t.y);
         exact = exact || div_small_needs_ieee(a);
       }
       if (__any_sync(0xFFFFFFFFu, exact)) {
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
+        for (int u = 0; u < VPT; ++u)
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
           float a;
           uint32_t cv;
-          num_c(v, a, cv);
-          if (div_small_needs_ieee(a)) y[v] = __fdiv_rn(a, -S.ntab[cv].x);
+          num_c(u, v, a, cv);
+          if (div_small_needs_ieee(a)) y[u][v] = __fdiv_rn(a, -S.ntab[cv].x);
         }
       }
 #pragma unroll
-      for (int v = 0; v < V; ++v) y[v] = __fmaf_rn(p.lambda, y[v], x0[v]);
+      for (int u = 0; u < VPT; ++u)
+#pragma unroll
+        for (int v = 0; v < V; ++v) y[u][v] = __fmaf_rn(p.lambda, y[u][v], x0[u][v]);
     }
-    if (k0 < n) store_vec<BF16>(p.out, off + k0, n - k0, y);
+    store(off, n);
   }
   merge_end<kConsumers + 32>(p, &S.last);
 }
 
 template <bool BF16, int OPC, int KC>
 cudaError_t launch_chunk(const MergeLaunch& p, cudaStream_t st) {
-  constexpr uint32_t chunk = kTcSlotBytes / (BF16 ? 2u : 4u);
+  using Geo = TcGeo<OPC, KC>;
+  constexpr uint32_t chunk = Geo::kSlotBytes / (BF16 ? 2u : 4u);
   const uint32_t cpb = (p.block_elems + chunk - 1) / chunk;
   const uint64_t n_chunks = (p.b_end - p.b_begin) * cpb;
   if (n_chunks == 0) return cudaSuccess;
@@ -1124,17 +1202,17 @@ cudaError_t launch_chunk(const MergeLaunch& p, cudaStream_t st) {
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  using Smem = TcSmem<TcGeo<OPC, KC>::kSlots, TcGeo<OPC, KC>::kGrab, KC>;
+  using Smem = TcSmem<Geo::kSlots, Geo::kSlotBytes, Geo::kGrab, KC, OPC == OP_TIES>;
   // every CTA also holds 1 KB of the SM's 228 KB for the system
-  static_assert(TcGeo<OPC, KC>::kCtasPerSm * (sizeof(Smem) + 1024) <= 228u * 1024u,
+  static_assert(Geo::kCtasPerSm * (sizeof(Smem) + 1024) <= 228u * 1024u,
                 "the CTAs per SM that the grid assumes fit one SM's shared memory");
   const size_t smem = sizeof(Smem);
   auto kern = merge_chunk_kernel<BF16, OPC, KC>;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return e;
-  uint64_t grid = (uint64_t)sms * TcGeo<OPC, KC>::kCtasPerSm;
+  uint64_t grid = (uint64_t)sms * Geo::kCtasPerSm;
   if (grid > n_chunks) grid = n_chunks;
-  kern<<<(unsigned)grid, TcGeo<OPC, KC>::kThreads, smem, st>>>(p, cpb, n_chunks, p.work);
+  kern<<<(unsigned)grid, Geo::kThreads, smem, st>>>(p, cpb, n_chunks, p.work);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1171,12 +1249,14 @@ cudaError_t launch_dtype(const MergeLaunch& p, cudaStream_t st) {
       if (p.K <= 8) return launch_chunk<BF16, OP_TIES, 8>(p, st);
       return launch_op<BF16, OP_TIES>(p, st);
     case MP_OP_DARE:
+      if (p.ext.span > kDareSpan) return launch_op<BF16, OP_DARE>(p, st);
       if (p.K <= 4) return launch_chunk<BF16, OP_DARE, 4>(p, st);
       if (p.K <= 8) return launch_chunk<BF16, OP_DARE, 8>(p, st);
       if (p.K <= 16) return launch_chunk<BF16, OP_DARE, 16>(p, st);
       return launch_op<BF16, OP_DARE>(p, st);
     case MP_OP_AVG_RENORM: return launch_op<BF16, OP_RENORM>(p, st);
     case MP_OP_DARE_TIES:
+      if (p.ext.span > kDareSpan) return launch_op<BF16, OP_DTIES>(p, st);
       if (p.K <= 4) return launch_chunk<BF16, OP_DTIES, 4>(p, st);
       if (p.K <= 8) return launch_chunk<BF16, OP_DTIES, 8>(p, st);
       if (p.K <= 16) return launch_chunk<BF16, OP_DTIES, 16>(p, st);
