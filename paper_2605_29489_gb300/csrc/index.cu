@@ -85,16 +85,25 @@ constexpr int kIxThreads = kIxConsumers + 32;
 static_assert(kIxConsumers == 256, "one consumer thread per coarse TIES bin at the end of a block");
 constexpr uint32_t kIxEnd = 0xFFFFFFFFu;
 
-// ring geometry.  The plain catalog is bound by HBM: two CTAs per SM with twelve 8 KiB
-// slots.  The TIES catalog also bins every delta, which makes it bound by instruction
-// latency: four CTAs per SM (more warps to hide it; the state fits 56 registers) with twelve
-// 4 KiB slots (one vector per consumer thread and fill).  With eight experts per item the
+// ring geometry.  The plain catalog is bound by HBM: three CTAs per SM with 72 KiB rings (two
+// with 96 KiB held fewer warps: 1.52 -> 1.42 ms on Qwen2.5-0.5B with 8 experts, 0.80 -> 0.73 with
+// 4, with the mixed-precision subtract on both sides of the second).  With 8 experts per item a
+// chunk is nine fills, each of which a consumer waited for and released: 4 KiB slots published a
+// chunk at a time took that to 1.30 ms (16 experts on 8 layers of Qwen2.5-1.5B: 3.59 -> 3.00 ms
+// in all).  With up to 4 experts 8 KiB slots stay, released fill by fill:
+// a chunk published at once leaves too little of the ring for the next (0.77 ms with 4 KiB slots,
+// 0.85 with 8 KiB ones).  The TIES catalog also bins every delta, which makes it bound by
+// instruction latency: four CTAs per SM (more warps to hide it; the state fits 56 registers) with
+// twelve 4 KiB slots (one vector per consumer thread and fill).  With eight experts per item the
 // histograms make a CTA too large for four per SM: three run, with the registers of three.
 template <bool TIES, int KG = 1>
 struct IxGeo {
-  static constexpr int kCtasPerSm = TIES ? (KG > 4 ? 3 : 4) : 2;
-  static constexpr uint32_t kSlotBytes = TIES ? 4096u : 8192u;
-  static constexpr int kSlots = 12;
+  static constexpr int kCtasPerSm = TIES && KG <= 4 ? 4 : 3;
+  static constexpr uint32_t kSlotBytes = TIES || KG > 4 ? 4096u : 8192u;
+  static constexpr int kSlots = TIES ? 12 : (KG > 4 ? 18 : 9);
+  // whole chunks: the base fill and the item's expert fills of one chunk sit in consecutive
+  // ring slots under one "full" and one "empty" mbarrier
+  static constexpr bool kWhole = TIES ? KG <= 4 : KG > 4;
 };
 
 struct IxMeta {
@@ -186,6 +195,24 @@ __device__ __forceinline__ void f2_sub(float a0, float a1, float b0, float b1, f
       " mov.b64 {%0, %1}, rd;\n}"
       : "=f"(d0), "=f"(d1)
       : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+
+// the deltas of a raw vector against the base elements x0, each one IEEE fp32 subtraction; bf16
+// elements are converted by the mixed-precision subtract itself (8 instructions per vector where
+// unpacking and a packed subtract take 12: 1.519 -> 1.442 ms on Qwen2.5-0.5B with 8 experts)
+template <bool BF16>
+__device__ __forceinline__ void deltas(const uint4 r, const float* x0, float* d) {
+  if constexpr (BF16) {
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n sub.rn.f32.bf16 %0, l, %3;\n sub.rn.f32.bf16 %1, h, %4;\n}"
+          : "=f"(d[2 * k]), "=f"(d[2 * k + 1])
+          : "r"(w[k]), "f"(x0[2 * k]), "f"(x0[2 * k + 1]));
+  } else {
+    f2_sub(__uint_as_float(r.x), __uint_as_float(r.y), x0[0], x0[1], d[0], d[1]);
+    f2_sub(__uint_as_float(r.z), __uint_as_float(r.w), x0[2], x0[3], d[2], d[3]);
+  }
 }
 
 // TIES window bins of two deltas: a nonzero delta with key k adds 1 to bin
@@ -407,11 +434,10 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
     index_tma_kernel(const IndexLaunch p, uint32_t G, uint64_t n_items, unsigned long long* work) {
   constexpr bool TIES = BM != kBinNone;
   constexpr uint32_t NB = BM == kBinNone ? 1u : (BM == kBinWindow ? kWinBins : 256u);  // key bins per expert
-  // The TIES catalog with up to 4 experts per item publishes whole chunks: the base fill and
-  // the item's expert fills of one chunk sit in consecutive ring slots under one "full"
-  // mbarrier (counting all their bytes) and one "empty" mbarrier, so that a consumer waits
-  // and releases once per chunk instead of once per fill.
-  constexpr bool CW = TIES && KG <= 4;
+  // Whole chunks (IxGeo): one "full" mbarrier counts all the bytes of a chunk's fills and one
+  // "empty" mbarrier its releases, so that a consumer waits and releases once per chunk instead
+  // of once per fill.
+  constexpr bool CW = IxGeo<TIES, KG>::kWhole;
   // window bins of bf16 deltas: the nonzero count comes from the keys (ties_win2k,
   // nz_halves) and the zeros share the below-window bin
   constexpr bool KNZ = BM == kBinWindow && BF16;
@@ -662,11 +688,8 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
         }
 #pragma unroll
         for (int u = 0; u < VPT; ++u) {
-          float xe[V];
-          unpack<BF16>(re[u], xe);
           float d[V];
-#pragma unroll
-          for (int e = 0; e < V; e += 2) f2_sub(xe[e], xe[e + 1], xb[u][e], xb[u][e + 1], d[e], d[e + 1]);
+          deltas<BF16>(re[u], xb[u], d);
           // the sum of squares is one fma chain in element order (the canonical order);
           // max |d| and the counts are exact in any order, so they take a tree
 #pragma unroll
