@@ -535,7 +535,7 @@ cudaError_t walk_segments(const IndexLaunch& p, const mp_index_s* ix, cudaStream
 
 cudaError_t index_host_pool(IndexLaunch p, const mp_index_s* ix, cudaStream_t cs) {
   cudaError_t e;
-  if (p.wlo) {
+  if (p.win) {
     // the windowed TIES catalog: the sample reads the host experts in place (32 vectors per
     // block), one walk counts every pair's window, the finish marks the pairs whose threshold
     // left it; a second walk, whose gathers and kernels do nothing unless some pair was
@@ -814,7 +814,7 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   const size_t n_work = family->experts_location == 0 ? 4 : 2 * (2 * (size_t)(g.n_params / kSegmentElems) + 2);
   const size_t o_work = slot(n_work * 8);
   size_t o_coarse = 0, o_fine = 0, o_kth = 0, o_est = 0, o_rank = 0;
-  size_t o_wfine = 0, o_wabove = 0, o_wlo = 0, o_gmiss = 0, o_miss = 0, o_wend = 0;
+  size_t o_wfine = 0, o_wabove = 0, o_win = 0, o_gmiss = 0, o_miss = 0, o_wend = 0;
   // device-resident TIES (not after masking) takes its thresholds from predicted windows
   const bool windowed = ties && op->kind == MP_OP_TIES;
   if (ties) {
@@ -845,10 +845,10 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
     o_wabove = slot(KG * 8);
     o_gmiss = slot(KG * 4);
     o_miss = slot(16);
-    o_shist = slot(KG * 256 * 8);
+    o_shist = slot(KG * 1024 * 4);
     o_scnt = slot(n_groups * 8);
     o_wend = o;
-    o_wlo = slot(KG * 4);
+    o_win = slot(KG * 4);
     o_spans = slot(h_spans.size() * 4);
   }
   mp_index_s* ix = nullptr;
@@ -898,12 +898,13 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
     p.wabove = (unsigned long long*)(m + o_wabove);
     p.gmiss = (uint32_t*)(m + o_gmiss);
     p.miss = (uint32_t*)(m + o_miss);
-    p.wlo = (uint32_t*)(m + o_wlo);
-    p.shist = (unsigned long long*)(m + o_shist);
+    p.win = (uint32_t*)(m + o_win);
+    p.shist = (uint32_t*)(m + o_shist);
     p.scnt = (unsigned long long*)(m + o_scnt);
     p.samp_span = (const uint2*)(m + o_spans);
     p.n_samp_spans = (uint32_t)(h_spans.size() / 2);
     p.samp_blocks = (uint32_t)span_blocks;
+    p.max_blk_len = g.max_blk_len;
     init.add(m + o_wfine, nullptr, o_wend - o_wfine);
     if ((e = upload(ix, init, m + o_spans, h_spans.data(), h_spans.size() * 4, cs)) != cudaSuccess)
       return bail(e, "span copy");

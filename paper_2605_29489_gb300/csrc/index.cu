@@ -15,6 +15,8 @@
 // finishes the threshold.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "mp_internal.cuh"
 #include "tma.cuh"
 
@@ -94,16 +96,16 @@ constexpr uint32_t kIxEnd = 0xFFFFFFFFu;
 // a chunk published at once leaves too little of the ring for the next (0.77 ms with 4 KiB slots,
 // 0.85 with 8 KiB ones).  The TIES catalog also bins every delta, which makes it bound by
 // instruction latency: four CTAs per SM (more warps to hide it; the state fits 56 registers) with
-// twelve 4 KiB slots (one vector per consumer thread and fill).  With eight experts per item the
-// histograms make a CTA too large for four per SM: three run, with the registers of three.
+// twelve 4 KiB slots (one vector per consumer thread and fill), and at most 4 experts per item.
 template <bool TIES, int KG = 1>
 struct IxGeo {
-  static constexpr int kCtasPerSm = TIES && KG <= 4 ? 4 : 3;
+  static_assert(!TIES || KG <= 4, "the TIES catalog takes at most 4 experts per item");
+  static constexpr int kCtasPerSm = TIES ? 4 : 3;
   static constexpr uint32_t kSlotBytes = TIES || KG > 4 ? 4096u : 8192u;
   static constexpr int kSlots = TIES ? 12 : (KG > 4 ? 18 : 9);
   // whole chunks: the base fill and the item's expert fills of one chunk sit in consecutive
   // ring slots under one "full" and one "empty" mbarrier
-  static constexpr bool kWhole = TIES ? KG <= 4 : KG > 4;
+  static constexpr bool kWhole = TIES || KG > 4;
 };
 
 struct IxMeta {
@@ -112,18 +114,36 @@ struct IxMeta {
   uint32_t n;      // elements in the chunk
   uint32_t last;   // 1 on the block's last chunk
   uint32_t s0;     // whole-chunk publication: ring slot of the base fill (experts follow)
-  int32_t wlo[4];  // whole-chunk publication, window bins: L - 1 of the item's experts' windows
+  // whole-chunk publication, window bins: the windows of the item's experts (win_words)
+  uint32_t wneg[4], wtop[4];
 };
 
 // How the TIES catalog bins the keys of the deltas:
 //  * kBinCoarse: 256 bins of the upper 8 key bits (the two-level select: a second pass then
 //    counts the lower 7 bits inside the chosen bin);
-//  * kBinWindow: the 384 keys [L, L + 384) of a window predicted from a sample (three
-//    coarse bins at full resolution), one bin below and one above it, so that the
-//    threshold is found without a second pass whenever it lies inside the window.
+//  * kBinWindow: the W keys [L, L + W) of a window predicted from a sample, one bin each, and
+//    one bin below and one above it, so that the threshold is found without a second pass
+//    whenever it lies inside the window.
 enum { kBinNone = 0, kBinCoarse = 1, kBinWindow = 2 };
-constexpr uint32_t kWinKeys = 384;           // keys of the window
+constexpr uint32_t kWinKeys = 384;           // most keys of a window (three binades)
 constexpr uint32_t kWinBins = kWinKeys + 2;  // + below + above
+
+// The window of one (expert, trim group), as ties_window_select leaves it: L | W << 16.
+// Groups of kWinNarrowBlocks blocks or more get a window of kWinNarrow keys (64 keys, a factor of
+// 1.4 or more, either side of the predicted bin of 32), smaller ones, whose sample is small, three
+// whole binades.  The increments are what bounds the pass: with three binades for every group
+// they took 5.5 wavefronts each and the LSU data pipe was 88 % busy (every block active); in a
+// narrow window most lanes share the bins below and above it (1.5 wavefronts).  Index of four
+// Llama layers with 4 experts 1.82 -> 1.61 ms, of two with every block active 1.26 -> 0.94, of
+// Qwen2.5-0.5B with 8 experts (items of 4 instead of 8 besides) 2.65 -> 1.88.  128 keys gave 1.59,
+// 0.92 and, with missed windows, 2.49 ms (items of 8), 192 keys 1.59, 0.93 and 2.44.
+constexpr uint32_t kWinNarrow = 160, kWinNarrowBlocks = 16;
+
+// the window in 16-bit lanes: 1 - L (added to the keys) and W + 1 (the clamp, the bin above)
+__device__ __forceinline__ void win_words(uint32_t win, uint32_t& neg, uint32_t& top) {
+  neg = ((1u - (win & 0xFFFFu)) & 0xFFFFu) * 0x00010001u;
+  top = ((win >> 16) + 1u) * 0x00010001u;
+}
 
 template <int KG, int NS, uint32_t SB, uint32_t NB>
 struct __align__(128) IxSmem {
@@ -215,54 +235,22 @@ __device__ __forceinline__ void deltas(const uint4 r, const float* x0, float* d)
   }
 }
 
-// TIES window bins of two deltas: a nonzero delta with key k adds 1 to bin
-// clamp(k - lo, 0, 385) of the shared histogram at hist0, with lo = L - 1: bin 0 below the
-// window, bins 1..384 for the keys L..L + 383, bin 385 above it.  Both keys at once in
-// 16-bit lanes: one add and one clamp at zero and 385 (k - lo lies in [-32383, 32768]; it
-// wraps only for the NaN key 0x7FFF at lo = -1, whose bin the clamp still keeps in range and
-// whose NaN the statistics report).  Predicated, no branch.
-__device__ __forceinline__ void ties_win2(float d0, float d1, int32_t lo, uint32_t hist0) {
-  const __nv_bfloat162 h2 = __floats2bfloat162_rn(d0, d1);
-  const uint32_t w = *reinterpret_cast<const uint32_t*>(&h2) & 0x7FFF7FFFu;
-  static_assert(kWinKeys + 1u == 0x181u, "the clamp bound is the above-window bin");
-  const uint32_t nlo2 = ((uint32_t)(-lo) & 0xFFFFu) * 0x00010001u;
-  uint32_t kk;
-  asm("{\n .reg .b32 t;\n add.s16x2 t, %1, %2;\n min.s16x2.relu %0, t, %3;\n}"
-      : "=r"(kk)
-      : "r"(w), "r"(nlo2), "r"(0x01810181u));
-  // byte addresses by multiply-add (FMA pipe; the ALU pipe carries the rest)
-  uint32_t a0, a1;
-  asm("mad.lo.u32 %0, %1, 4, %2;" : "=r"(a0) : "r"(kk & 0xFFFFu), "r"(hist0));
-  asm("mad.lo.u32 %0, %1, 4, %2;" : "=r"(a1) : "r"(kk >> 16), "r"(hist0));
-  asm volatile(
-      "{\n"
-      " .reg .pred p0, p1;\n"
-      " setp.ne.f32 p0, %2, 0f00000000;\n"
-      " setp.ne.f32 p1, %3, 0f00000000;\n"
-      " @p0 red.shared.add.u32 [%0], 1;\n"
-      " @p1 red.shared.add.u32 [%1], 1;\n"
-      "}\n" ::"r"(a0),
-      "r"(a1), "f"(d0), "f"(d1)
-      : "memory");
-}
-
-// The same bins for deltas of two bf16 checkpoints, where key 0 holds exactly the zero
-// deltas (the difference of two distinct bf16 values is at least the smallest bf16
-// subnormal, whose key is 1).  Every delta adds 1 to its bin, zeros included: a zero has
-// key 0 and lands below the window, in bin 0, which no threshold reads (with the window at
-// the bottom, L = 0 and lo = -1, it lands in key 0's bin, where it can only decide a
-// threshold of key 0, the one that an uncounted zero gives too).  The nonzero deltas are
-// counted from the returned key word instead (nz_halves).  Both byte addresses come from one
-// multiply-add in 16-bit lanes: h2 = the histogram's byte address in both lanes, which the
-// caller keeps below 2^16 - 4 * 385.  No predicate and no branch.
-__device__ __forceinline__ uint32_t ties_win2k(float d0, float d1, int32_t lo, uint32_t h2) {
+// TIES window bins of two deltas: key k adds 1 to bin clamp(k - L + 1, 0, W + 1) of the shared
+// histogram at h, also to bin 0 (below the window), which nothing reads: lanes that increment
+// one address share a wavefront, and a predicate on the increment cost more than it saved (it
+// becomes a branch: 537 instead of 425 million warp instructions on a Llama layer).  Both keys
+// at once in 16-bit lanes:
+// one add and one clamp at zero and W + 1 (k - L + 1 lies in [-32383, 32768]; it wraps only for
+// the NaN key 0x7FFF at L = 0, whose bin the clamp still keeps in range and whose NaN the
+// statistics report), and one multiply-add for both byte addresses (h2 = h in both lanes, which
+// the caller keeps below 2^16 - 4 * 385).  An exact zero has key 0: below the window, or, with
+// L = 0, in key 0's bin, where it can only decide a threshold of key 0, the one that an
+// uncounted zero gives too.  Returns the two keys.
+__device__ __forceinline__ uint32_t ties_win2(float d0, float d1, uint32_t neg, uint32_t top, uint32_t h2) {
   const __nv_bfloat162 hb = __floats2bfloat162_rn(d0, d1);
   const uint32_t w = *reinterpret_cast<const uint32_t*>(&hb) & 0x7FFF7FFFu;
-  const uint32_t nlo2 = ((uint32_t)(-lo) & 0xFFFFu) * 0x00010001u;
   uint32_t kk;
-  asm("{\n .reg .b32 t;\n add.s16x2 t, %1, %2;\n min.s16x2.relu %0, t, %3;\n}"
-      : "=r"(kk)
-      : "r"(w), "r"(nlo2), "r"(0x01810181u));
+  asm("{\n .reg .b32 t;\n add.s16x2 t, %1, %2;\n min.s16x2.relu %0, t, %3;\n}" : "=r"(kk) : "r"(w), "r"(neg), "r"(top));
   const uint32_t a2 = kk * 4u + h2;  // lanes: h + 4 b0 and h + 4 b1 (no carry between them)
   asm volatile(
       "{\n"
@@ -438,9 +426,11 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
   // "empty" mbarrier its releases, so that a consumer waits and releases once per chunk instead
   // of once per fill.
   constexpr bool CW = IxGeo<TIES, KG>::kWhole;
-  // window bins of bf16 deltas: the nonzero count comes from the keys (ties_win2k,
-  // nz_halves) and the zeros share the below-window bin
-  constexpr bool KNZ = BM == kBinWindow && BF16;
+  // window bins: the nonzero deltas are counted apart (the bins leave out those below the
+  // window); for bf16 from the keys (nz_halves), where key 0 holds exactly the zero deltas (the
+  // difference of two distinct bf16 values is at least the smallest bf16 subnormal, whose key
+  // is 1)
+  constexpr bool KNZ = BM == kBinWindow;
   constexpr int kIxSlots = IxGeo<TIES, KG>::kSlots;
   static_assert(!CW || kIxSlots >= 2 * (KG + 1), "two whole chunks fit the ring");
   constexpr uint32_t kIxSlotBytes = IxGeo<TIES, KG>::kSlotBytes;
@@ -494,7 +484,7 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
         return true;
       };
       // publishes one chunk: the base fill and kc expert fills in consecutive slots
-      int32_t item_wlo[4] = {0, 0, 0, 0};  // window bins: L - 1 of the current item's experts
+      uint32_t item_neg[4] = {0, 0, 0, 0}, item_top[4] = {0, 0, 0, 0};  // the current item's windows
       auto publish = [&](uint32_t item, uint64_t off, uint32_t n, uint32_t last, uint32_t i0,
                          uint32_t kc) -> bool {
         const uint32_t nfill = item == kIxEnd ? 0u : 1u + kc;
@@ -509,7 +499,10 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
         S.meta[e].s0 = fill % kIxSlots;
         if constexpr (BM == kBinWindow) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) S.meta[e].wlo[k] = item_wlo[k];
+          for (int k = 0; k < 4; ++k) {
+            S.meta[e].wneg[k] = item_neg[k];
+            S.meta[e].wtop[k] = item_top[k];
+          }
         }
         S.nf[e] = nfill;
         const bool arm = !(seq == 0 && p.stall);  // test hook: the first chunk is never armed
@@ -568,7 +561,7 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
           const uint32_t grp = p.blk_group[b];
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            item_wlo[k] = (uint32_t)k < kc ? (int32_t)p.wlo[(uint64_t)(i0 + k) * p.n_groups + grp] - 1 : 0;
+            if ((uint32_t)k < kc) win_words(p.win[(uint64_t)(i0 + k) * p.n_groups + grp], item_neg[k], item_top[k]);
         }
         for (uint32_t c = 0; c < nch && ok; ++c) {
           const uint32_t n = min(CH, len - c * CH);
@@ -680,11 +673,11 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
       // a warp whose vectors all match skips them (warp-uniform, so the summation order is
       // untouched)
       if (!__all_sync(0xFFFFFFFFu, same)) {
-        // kBinWindow: L - 1 of this expert's window in the block's trim group
-        int32_t wlo_k = 0;
+        // kBinWindow: this expert's window in the block's trim group
+        uint32_t wneg = 0, wtop = 0;
         if constexpr (BM == kBinWindow) {
-          if constexpr (CW) wlo_k = mt.wlo[k < 4 ? k : 0];
-          else wlo_k = (int32_t)__ldg(p.wlo + (uint64_t)(i0 + k) * p.n_groups + __ldg(p.blk_group + b)) - 1;
+          wneg = mt.wneg[k < 4 ? k : 0];
+          wtop = mt.wtop[k < 4 ? k : 0];
         }
 #pragma unroll
         for (int u = 0; u < VPT; ++u) {
@@ -702,23 +695,20 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
 #pragma unroll
             for (int e = 0; e < w; ++e) m[e] = fmaxf(m[e], m[e + w]);
           mx[k] = fmaxf(mx[k], m[0]);
-          if constexpr (KNZ) {
+          if constexpr (BM == kBinWindow) {
             const uint32_t h2 = su32(&S.hist[k][0]) * 0x00010001u;
             uint32_t wk[V / 2];
 #pragma unroll
-            for (int e = 0; e < V; e += 2) wk[e / 2] = ties_win2k(d[e], d[e + 1], wlo_k, h2);
-            nz[k] += nz_halves(wk[0], wk[1], wk[2], wk[3]);
-          } else {
+            for (int e = 0; e < V; e += 2) wk[e / 2] = ties_win2(d[e], d[e + 1], wneg, wtop, h2);
+            if constexpr (BF16) nz[k] += nz_halves(wk[0], wk[1], wk[2], wk[3]);
+          }
 #pragma unroll
-            for (int e = 0; e < V; e += 2) {
-              if constexpr (BM == kBinWindow) {
-                ties_win2(d[e], d[e + 1], wlo_k, su32(&S.hist[k][0]));
-              } else if constexpr (BM == kBinCoarse) {
-                ties_bin2(d[e], d[e + 1], su32(&S.hist[k][0]));
-              } else {
-                nz[k] += d[e] != 0.0f ? 1u : 0u;
-                nz[k] += d[e + 1] != 0.0f ? 1u : 0u;
-              }
+          for (int e = 0; e < V; e += 2) {
+            if constexpr (BM == kBinCoarse) {
+              ties_bin2(d[e], d[e + 1], su32(&S.hist[k][0]));
+            } else if constexpr (BM == kBinNone || !BF16) {
+              nz[k] += d[e] != 0.0f ? 1u : 0u;
+              nz[k] += d[e + 1] != 0.0f ? 1u : 0u;
             }
           }
         }
@@ -737,7 +727,7 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
     // end of the block: the canonical combine, then the statistics (and TIES bins)
 #pragma unroll
     for (int k = 0; k < KG; ++k) {
-      if constexpr (KNZ) nz[k] = (nz[k] & 0xFFFFu) + (nz[k] >> 16);  // the two 16-bit lanes
+      if constexpr (KNZ && BF16) nz[k] = (nz[k] & 0xFFFFu) + (nz[k] >> 16);  // the two 16-bit lanes
 #pragma unroll
       for (int s = 16; s >= 1; s >>= 1) {
         ss[k] = __fadd_rn(ss[k], __shfl_xor_sync(0xFFFFFFFFu, ss[k], s));
@@ -783,8 +773,7 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
       if (lane == 0 && bad) atomicOr(p.err, kErrNonfinite);
     }
     if constexpr (TIES) {
-      // every nonzero delta added 1 to exactly one bin: the histogram's total is nnz (not
-      // for KNZ, whose nonzero deltas were counted by key and whose bin 0 holds the zeros too)
+      // coarse bins: every nonzero delta added 1 to exactly one bin, the histogram's total is nnz
       if (!consumer_barrier(&S.cbar, cphase, abort_flag, wl)) {
         atomicOr(p.err, kErrTimeout);
         S.abort = 1;
@@ -833,12 +822,13 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
           if (p.unit_hist) p.unit_hist[(((uint64_t)(i0 + k) * p.n_blocks + b) << 8) + tid] = (uint32_t)c;
           if (c) atomicAdd(&p.coarse[x * 256u + tid], c);
         } else {
-          // bin 0 (below the window) only counts toward nnz; bins 1..384 are the window's
-          // keys; bin 385 is above it
-          if (tid > 0 && hc[k]) atomicAdd(&p.wfine[x * kWinKeys + tid - 1u], (unsigned long long)hc[k]);
-          const uint32_t j = tid + 256u;
-          if (j <= kWinKeys && hd[k]) atomicAdd(&p.wfine[x * kWinKeys + j - 1u], (unsigned long long)hd[k]);
-          if (j == kWinKeys + 1u && hd[k]) atomicAdd(&p.wabove[x], (unsigned long long)hd[k]);
+          // bins 1..W are the window's keys, bin W + 1 is above it (bin 0, below it, is dropped)
+          const uint32_t W = p.win[x] >> 16;
+          auto flush = [&](uint32_t j, uint32_t n) {
+            if (n) atomicAdd(j <= W ? &p.wfine[x * kWinKeys + j - 1u] : &p.wabove[x], (unsigned long long)n);
+          };
+          if (tid > 0) flush(tid, hc[k]);
+          flush(tid + 256u, hd[k]);
         }
       }
     }
@@ -968,33 +958,41 @@ __global__ void __launch_bounds__(256) ties_masked_coarse(const IndexLaunch p, u
 // ---- TIES thresholds with a predicted window ----------------------------------------------
 //
 // The threshold of a trim group is the k-th largest key of its deltas.  A sample predicts
-// the coarse bin e (upper 8 key bits) that holds it: from every block of the group, vectors at
-// jittered, evenly spaced positions (sample_vectors), binned like the coarse catalog — every
-// block contributes because the scale of the deltas changes from block to block; e is the bin
-// of the k_s-th largest sampled key,
-// k_s = max(1, floor(rho * sampled elements)).  The catalog pass then counts the 384 keys
-// of the window starting at L = 128 clamp(e - 1, 0, 253) at full resolution, plus the keys
-// above it, and ties_window_finish takes the threshold from those counts.  A pair whose
+// the bin e of 32 keys that holds it: from every block of the group, vectors at jittered, evenly
+// spaced positions (sample_vectors) — every block contributes because the scale of the deltas
+// changes from block to block; e is the bin of the k_s-th largest sampled key,
+// k_s = max(1, floor(rho * sampled elements)).  The catalog pass then counts the keys of a window
+// around it at full resolution (ties_window_select), plus the keys above it, and
+// ties_window_finish takes the threshold from those counts.  A pair whose
 // threshold lies outside its window is marked, and the two-level select (coarse pass over
 // the marked pairs' groups, coarse select, fine pass, fine select) runs for the marked
 // pairs only; it does nothing when none is marked.  The prediction affects only which of
 // the two exact paths gives a threshold, never its value.
 
-// Vectors sampled from a block of nvec vectors in a group of n_b blocks.  The window holds the
-// predicted binade and one on each side, so a few hundred vectors per group are enough: 8 of
-// each block in groups of 64 blocks or more, 32 in groups of 16 or more, up to 128 (every one
-// of a small tensor) in smaller groups.  Reading every vector of each block up to 4096 elements,
-// and 32 of larger ones, cost 241 us on 371 blocks of 4096 elements with 3 experts.
-constexpr uint32_t kSampleWide = 8;
-__device__ __forceinline__ uint32_t sample_vectors(uint32_t n_b, uint32_t nvec) {
-  const uint32_t want = n_b >= 64u ? kSampleWide : (n_b >= 16u ? 32u : 128u);
-  return min(want, nvec);
+// Vectors sampled from a block of nvec vectors in a group of n_b blocks whose whole blocks have
+// nvec0: 8 of each whole block in groups of 256 blocks or more, 32 in groups of 64 or more, up to
+// 128 (every one of a small tensor) in smaller groups, so that every group that gets a narrow
+// window has 2,000 vectors or more (with 500, one pair in some hundred missed it); a partial
+// block in proportion, so that it weighs in the sample what it weighs in the group.  Reading
+// every vector of each block up to 4096 elements, and 32 of larger ones, cost 241 us on 371 blocks
+// of 4096 elements with 3 experts.
+constexpr uint32_t kSampleWide = 8, kSampleWideBlocks = 256;
+__device__ __forceinline__ uint32_t sample_vectors(uint32_t n_b, uint32_t nvec, uint32_t nvec0) {
+  const uint32_t want = n_b >= kSampleWideBlocks ? kSampleWide : (n_b >= 64u ? 32u : 128u);
+  const uint32_t share = (uint32_t)(((uint64_t)want * nvec + nvec0 / 2u) / nvec0);
+  return min(max(share, 1u), nvec);
 }
+
+// The sample counts 1024 bins of 32 keys.  The deltas of bf16 checkpoints are multiples of the
+// elements' last place, so their keys sit on a few values of each binade and a whole binade's
+// count does not say where in it the threshold lies (a narrow window placed by interpolation
+// missed it, and with the second pass the index of four Llama layers took 2.45 instead of 1.82 ms).
+constexpr uint32_t kSampleBins = 1024;
 
 template <bool BF16, int KG>
 __global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
   constexpr uint32_t V = BF16 ? 8u : 4u;
-  __shared__ uint32_t hist[KG][256];
+  __shared__ uint32_t hist[KG][kSampleBins];
   __shared__ unsigned long long s_n;  // sampled elements
   const uint2 span = p.samp_span[blockIdx.x];  // {group, first block}: up to p.samp_blocks blocks
   const uint32_t g = span.x, i0 = blockIdx.y * KG;
@@ -1004,14 +1002,15 @@ __global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
     return;
   }
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
-  for (uint32_t x = tid; x < (uint32_t)KG * 256u; x += blockDim.x) (&hist[0][0])[x] = 0u;
+  for (uint32_t x = tid; x < (uint32_t)KG * kSampleBins; x += blockDim.x) (&hist[0][0])[x] = 0u;
   if (tid == 0) s_n = 0;
   __syncthreads();
   const uint64_t gb0 = p.n_groups == 1 ? 0 : p.grp_blk0[g], gb1 = p.n_groups == 1 ? p.n_blocks : p.grp_blk0[g + 1];
   const uint64_t b1 = min((uint64_t)span.y + p.samp_blocks, gb1);
   const uint32_t n_b = (uint32_t)min(gb1 - gb0, (uint64_t)0xFFFFFFFFu);
+  const uint32_t nvec0 = ((p.n_groups == 1 ? p.max_blk_len : p.blk_len[gb0]) + V - 1) / V;  // of a whole block
   // a warp takes one block with 32 lanes, or (8 vectors each) four blocks with 8 lanes each
-  const bool wide = n_b >= 64u;
+  const bool wide = n_b >= kSampleWideBlocks;
   const uint32_t per_warp = wide ? 32u / kSampleWide : 1u, step = wide ? kSampleWide : 32u;
   const uint32_t sub = wide ? lane / kSampleWide : 0u, l = wide ? lane % kSampleWide : lane;
   unsigned long long my_n = 0;
@@ -1020,7 +1019,7 @@ __global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
     const uint32_t len = p.blk_len[b];
     const uint64_t off = p.blk_off[b];
     const uint32_t nvec = (len + V - 1) / V;
-    const uint32_t n_v = sample_vectors(n_b, nvec), per = nvec / n_v;
+    const uint32_t n_v = sample_vectors(n_b, nvec, nvec0), per = nvec / n_v;
     for (uint32_t v0 = l; v0 < n_v; v0 += step) {
       uint32_t v = v0;
       if (n_v < nvec) {  // a position in stretch v0 from a hash of (block, stretch)
@@ -1047,7 +1046,7 @@ __global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
 #pragma unroll
         for (uint32_t e = 0; e < V; ++e) {
           const float d = __fsub_rn(xe[e], xb[e]);
-          if (d != 0.0f) atomicAdd(&hist[k][ties_key(d) >> 7], 1u);
+          if (d != 0.0f) atomicAdd(&hist[k][ties_key(d) >> 5], 1u);
         }
       }
     }
@@ -1056,23 +1055,58 @@ __global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
   for (int s = 16; s >= 1; s >>= 1) my_n += __shfl_xor_sync(0xFFFFFFFFu, my_n, s);
   if (lane == 0) atomicAdd(&s_n, my_n);
   __syncthreads();
-  for (uint32_t x = tid; x < kc * 256u; x += blockDim.x) {
-    const uint32_t k = x >> 8, e = x & 255u;
-    if (hist[k][e]) atomicAdd(&p.shist[((uint64_t)(i0 + k) * p.n_groups + g) * 256u + e], (unsigned long long)hist[k][e]);
+  for (uint32_t x = tid; x < kc * kSampleBins; x += blockDim.x) {
+    const uint32_t k = x / kSampleBins, e = x % kSampleBins;
+    if (hist[k][e]) atomicAdd(&p.shist[((uint64_t)(i0 + k) * p.n_groups + g) * kSampleBins + e], hist[k][e]);
   }
   if (tid == 0 && blockIdx.y == 0) atomicAdd(&p.scnt[g], s_n);
 }
 
-// the window of each (expert, group) from its sampled coarse bins
+// the window of each (expert, group) from its sample, by one warp: around the bin e of the k_s-th
+// largest sampled key, or the three binades around that bin's binade
 __global__ void __launch_bounds__(kSelThreads) ties_window_select(const IndexLaunch p) {
   const uint64_t x = select_pair();
   if (x >= (uint64_t)p.K * p.n_groups) return;
-  unsigned long long ks = (unsigned long long)floor((double)p.density * (double)p.scnt[x % p.n_groups]), before;
+  const uint32_t lane = threadIdx.x & 31u, g = (uint32_t)(x % p.n_groups);
+  const uint64_t n_b = p.n_groups == 1 ? p.n_blocks : p.grp_blk0[g + 1] - p.grp_blk0[g];
+  unsigned long long ks = (unsigned long long)floor((double)p.density * (double)p.scnt[g]);
   if (ks == 0) ks = 1;
-  uint32_t e = 0;
-  if (!warp_kth<8>(p.shist + x * 256u, ks, e, before)) e = 0;  // fewer nonzero samples than k_s
-  const uint32_t lo = e == 0 ? 0u : min(e - 1u, 253u);
-  if ((threadIdx.x & 31u) == 0) p.wlo[x] = lo << 7;
+  // lane l sums the 32 bins that rank l-th from the top; the first lane whose running count
+  // reaches k_s holds e, and its bins go one to a lane for the same again
+  static_assert(kSampleBins == 32 * 32, "one run of 32 bins per lane");
+  const uint32_t* h = p.shist + x * kSampleBins;
+  auto suffix = [&](unsigned long long v) {
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const unsigned long long o = __shfl_up_sync(0xFFFFFFFFu, v, s);
+      if (lane >= (uint32_t)s) v += o;
+    }
+    return v;
+  };
+  unsigned long long sum = 0;
+  const uint4* h4 = reinterpret_cast<const uint4*>(h + (31u - lane) * 32u);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint4 c = h4[j];
+    sum += (unsigned long long)c.x + c.y + c.z + c.w;
+  }
+  unsigned long long cum = suffix(sum);
+  uint32_t hit = __ballot_sync(0xFFFFFFFFu, cum >= ks), e = 0;
+  const bool found = hit != 0u;  // or: fewer nonzero samples than k_s
+  if (found) {
+    const uint32_t run = 31u - (uint32_t)(__ffs(hit) - 1);
+    const unsigned long long before = __shfl_sync(0xFFFFFFFFu, cum - sum, 31 - (int)run);
+    cum = before + suffix(h[run * 32u + 31u - lane]);
+    hit = __ballot_sync(0xFFFFFFFFu, cum >= ks);
+    e = run * 32u + 31u - (uint32_t)(__ffs(hit) - 1);
+  }
+  if (lane != 0) return;
+  uint32_t L = e >= 4u ? min(e / 4u - 1u, 253u) << 7 : 0u, W = kWinKeys;
+  if (found && n_b >= kWinNarrowBlocks) {
+    L = (uint32_t)min(max((int32_t)(e * 32u + 16u) - (int32_t)kWinNarrow / 2, 0), 32768 - (int32_t)kWinNarrow);
+    W = kWinNarrow;
+  }
+  p.win[x] = L | W << 16;
 }
 
 // the threshold of each (expert, group) from its window counts, or a mark for the
@@ -1082,7 +1116,7 @@ __global__ void __launch_bounds__(kSelThreads) ties_window_finish(const IndexLau
   if (x >= (uint64_t)p.K * p.n_groups) return;
   const unsigned long long k = p.kth[x % p.n_groups];
   const unsigned long long above = p.wabove[x];
-  const uint32_t L = p.wlo[x];
+  const uint32_t L = p.win[x] & 0xFFFFu;
   uint32_t tau = kTauNone, j;
   unsigned long long before;
   bool miss = false;
@@ -1150,18 +1184,29 @@ cudaError_t launch_pass(const IndexLaunch& p, uint32_t G, uint64_t n_items, int 
 }
 
 template <bool BF16, int KG>
-cudaError_t launch_t(const IndexLaunch& p, cudaStream_t st) {
+cudaError_t launch_plain_t(const IndexLaunch& p, cudaStream_t st) {
   const uint32_t G = (p.K + KG - 1) / KG;
   const uint64_t n_items = (p.b_end - p.b_begin) * G;
   if (n_items == 0) return cudaSuccess;
   if (n_items > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-  const bool ties = p.coarse != nullptr;
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if (!ties) return launch_pass<BF16, KG, kBinNone>(p, G, n_items, sms, p.work, st);
-  if (!p.wlo) {  // the two-level select for every pair
+  return launch_pass<BF16, KG, kBinNone>(p, G, n_items, sms, p.work, st);
+}
+
+template <bool BF16, int KG>
+cudaError_t launch_ties_t(const IndexLaunch& p, cudaStream_t st) {
+  const uint32_t G = (p.K + KG - 1) / KG;
+  const uint64_t n_items = (p.b_end - p.b_begin) * G;
+  if (n_items == 0) return cudaSuccess;
+  if (n_items > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+  int dev = 0, sms = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if (!p.win) {  // the two-level select for every pair
     if ((e = launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
     if (p.defer_ties_select) return cudaSuccess;
     return ties_finish_t<BF16, KG>(p, st);
@@ -1208,12 +1253,26 @@ cudaError_t pass_t(const IndexLaunch& p, bool window, cudaStream_t st) {
                 : launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, p.work, st);
 }
 
+// f(KG) with the experts per item of the TIES kernels as a constant.  More than 4 experts take
+// several items of 4, which read the base again (from L2: neighbouring items run together):
+// with 8 per item the histograms leave three CTAs per SM and a chunk's nine fills are waited for
+// one by one, 2.45 instead of 1.95 ms on Qwen2.5-0.5B with 8 experts, 4.45 instead of 3.63 with 16.
+template <int KG>
+using Kg = std::integral_constant<int, KG>;
+template <typename F>
+cudaError_t by_ties_items(uint32_t K, F f) {
+  if (K <= 1) return f(Kg<1>());
+  if (K <= 2) return f(Kg<2>());
+  return f(Kg<4>());
+}
+
 template <bool BF16>
 cudaError_t launch_dtype(const IndexLaunch& p, cudaStream_t st) {
-  if (p.K <= 1) return launch_t<BF16, 1>(p, st);
-  if (p.K <= 2) return launch_t<BF16, 2>(p, st);
-  if (p.K <= 4) return launch_t<BF16, 4>(p, st);
-  return launch_t<BF16, 8>(p, st);
+  if (p.coarse) return by_ties_items(p.K, [&](auto kg) { return launch_ties_t<BF16, decltype(kg)::value>(p, st); });
+  if (p.K <= 1) return launch_plain_t<BF16, 1>(p, st);
+  if (p.K <= 2) return launch_plain_t<BF16, 2>(p, st);
+  if (p.K <= 4) return launch_plain_t<BF16, 4>(p, st);
+  return launch_plain_t<BF16, 8>(p, st);
 }
 
 }  // namespace
@@ -1223,25 +1282,23 @@ cudaError_t launch_index(const IndexLaunch& p, cudaStream_t st) {
 }
 
 cudaError_t launch_ties_window_begin(const IndexLaunch& p, cudaStream_t st) {
-  if (!p.wlo || !p.coarse) return cudaErrorInvalidValue;
-  const bool bf = p.dtype == MP_BF16;
-  if (p.K <= 1) return bf ? window_begin_t<true, 1>(p, st) : window_begin_t<false, 1>(p, st);
-  if (p.K <= 2) return bf ? window_begin_t<true, 2>(p, st) : window_begin_t<false, 2>(p, st);
-  if (p.K <= 4) return bf ? window_begin_t<true, 4>(p, st) : window_begin_t<false, 4>(p, st);
-  return bf ? window_begin_t<true, 8>(p, st) : window_begin_t<false, 8>(p, st);
+  if (!p.win || !p.coarse) return cudaErrorInvalidValue;
+  return by_ties_items(p.K, [&](auto kg) {
+    constexpr int KG = decltype(kg)::value;
+    return p.dtype == MP_BF16 ? window_begin_t<true, KG>(p, st) : window_begin_t<false, KG>(p, st);
+  });
 }
 
 cudaError_t launch_index_pass(const IndexLaunch& p, bool window, cudaStream_t st) {
-  if (!p.wlo || !p.coarse) return cudaErrorInvalidValue;
-  const bool bf = p.dtype == MP_BF16;
-  if (p.K <= 1) return bf ? pass_t<true, 1>(p, window, st) : pass_t<false, 1>(p, window, st);
-  if (p.K <= 2) return bf ? pass_t<true, 2>(p, window, st) : pass_t<false, 2>(p, window, st);
-  if (p.K <= 4) return bf ? pass_t<true, 4>(p, window, st) : pass_t<false, 4>(p, window, st);
-  return bf ? pass_t<true, 8>(p, window, st) : pass_t<false, 8>(p, window, st);
+  if (!p.win || !p.coarse) return cudaErrorInvalidValue;
+  return by_ties_items(p.K, [&](auto kg) {
+    constexpr int KG = decltype(kg)::value;
+    return p.dtype == MP_BF16 ? pass_t<true, KG>(p, window, st) : pass_t<false, KG>(p, window, st);
+  });
 }
 
 cudaError_t launch_ties_window_end(const IndexLaunch& p, cudaStream_t st) {
-  if (!p.wlo || !p.coarse) return cudaErrorInvalidValue;
+  if (!p.win || !p.coarse) return cudaErrorInvalidValue;
   const uint64_t nsel = (uint64_t)p.K * p.n_groups;
   if (nsel == 0) return cudaSuccess;
   ties_window_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
@@ -1260,11 +1317,10 @@ cudaError_t launch_ties_masked(const IndexLaunch& p, cudaStream_t st) {
 }
 
 cudaError_t launch_ties_finish(const IndexLaunch& p, cudaStream_t st) {
-  const bool bf = p.dtype == MP_BF16;
-  if (p.K <= 1) return bf ? ties_finish_t<true, 1>(p, st) : ties_finish_t<false, 1>(p, st);
-  if (p.K <= 2) return bf ? ties_finish_t<true, 2>(p, st) : ties_finish_t<false, 2>(p, st);
-  if (p.K <= 4) return bf ? ties_finish_t<true, 4>(p, st) : ties_finish_t<false, 4>(p, st);
-  return bf ? ties_finish_t<true, 8>(p, st) : ties_finish_t<false, 8>(p, st);
+  return by_ties_items(p.K, [&](auto kg) {
+    constexpr int KG = decltype(kg)::value;
+    return p.dtype == MP_BF16 ? ties_finish_t<true, KG>(p, st) : ties_finish_t<false, KG>(p, st);
+  });
 }
 
 }  // namespace mp
