@@ -1,22 +1,21 @@
 // Alg. 2 ExecuteMerge on the device: M_A[t,b] = M_0[t,b] + Psi_op(A_{.,t,b}, Delta_{.,t,b})
 // (Eq. 4) for every block, reading only the experts the access mask selects.
 //
-// Pipeline (persistent CTAs, 2 or 3 per SM, 256 consumer threads + 1 producer warp):
+// Pipeline (persistent CTAs, 2 to 4 per SM, 128 or 256 consumer threads + 1 producer warp):
 //  * work unit = one chunk of a block (8 KiB for AVG/TA, 4 KiB for TIES/DARE); chunks are
 //    handed out dynamically through a global counter, GRAB at a time;
 //  * the producer warp takes a grab: its lanes load the chunks' block metadata (and, for
-//    TIES, every expert's trim threshold) in parallel into shared memory, and the counter
-//    value of the next grab is requested before this one is issued, so that no fill waits
-//    on a global-memory round trip;
-//  * lane 0 then walks each chunk's fills — the base chunk, then every selected expert's
+//    TIES, every expert's trim threshold) in parallel, and the counter value of the next grab is
+//    requested before this one is issued, so that no fill waits on a global-memory round trip;
+//  * it then walks each chunk's fills — the base chunk, then every selected expert's
 //    chunk in ascending expert order — and streams each fill into the next slot of a ring
 //    of NS shared-memory slots with one cp.async.bulk (TMA 1-D bulk copy), completing on
-//    the slot's "full" mbarrier; it writes the slot's metadata (chunk, offset, length,
-//    mask, TIES threshold) before arming the barrier;
-//  * consumers take the slots in the same order: the base fill loads M_0 into registers,
+//    a "full" mbarrier (AVG/TA one per slot, the others one per group of slots); it writes the
+//    metadata (chunk, offset, length, mask, TIES threshold) before arming the barrier;
+//  * consumers take the fills in the same order: the base fill loads M_0 into registers,
 //    each expert fill folds Delta_i into fp32 accumulators, the last fill of a chunk
 //    writes the output with 16-byte streaming stores; every consumer thread arrives on the
-//    slot's "empty" mbarrier as soon as it has read it;
+//    "empty" mbarrier as soon as it has read the slot or the group;
 //  * the bytes in flight are the ring (NS slots per CTA), independent of registers and of
 //    how many experts a block selects.
 // Per element, in the fixed ascending expert order:
@@ -49,27 +48,18 @@ constexpr uint32_t kEnd = 0xFFFFFFFFu;
 enum { OP_ADD = 0, OP_TIES = 1, OP_DARE = 2, OP_RENORM = 3, OP_DTIES = 4 };
 
 // TIES and DARE-TIES share the sign election and disjoint mean (DARE and DARE-TIES share
-// the random keep mask); AVG/TA and the renormalised AVG share the additive geometry
+// the random keep mask)
 template <int OPC>
 constexpr bool kTiesLike = OPC == OP_TIES || OPC == OP_DTIES;
-template <int OPC>
-constexpr bool kAddGeo = OPC == OP_ADD || OPC == OP_RENORM;
 
-// slot geometry per operator.  The additive merges are bound by HBM: two CTAs per SM with a
-// 96 KiB ring each (two 16-byte vectors per consumer thread and fill).  TIES, DARE and
-// DARE-TIES spend more arithmetic per byte, so they run more warps per SM to hide latency
-// (measured better than fewer consumer threads with more work each), with 4 KiB slots (one
-// vector per consumer thread and fill, so that their state fits the register budget): TIES
-// and DARE four CTAs per SM with a 44 KiB ring (their state fits 56 registers), DARE-TIES
-// three with a 64 KiB ring (it would spill at 56).
-template <int OPC>
+// slot geometry of the streaming kernel (AVG/TA and the renormalised AVG), which is bound by
+// HBM: two CTAs per SM with a 96 KiB ring each (two 16-byte vectors per consumer thread and fill)
 struct Geo {
   static constexpr int kConsumers = 256;
   static constexpr int kThreads = kConsumers + 32;  // + one producer warp
-  static constexpr int kCtasPerSm = kAddGeo<OPC> ? 2 : (OPC == OP_DTIES ? 3 : 4);
-  static constexpr uint32_t kRingBytes = kAddGeo<OPC> ? 98304u : (OPC == OP_DTIES ? 65536u : 45056u);
-  static constexpr uint32_t kSlotBytes = kAddGeo<OPC> ? 8192u : 4096u;  // one chunk of one checkpoint
-  static constexpr int kSlots = (int)(kRingBytes / kSlotBytes);
+  static constexpr int kCtasPerSm = 2;
+  static constexpr uint32_t kSlotBytes = 8192u;  // one chunk of one checkpoint
+  static constexpr int kSlots = 12;
   static constexpr uint32_t kGrab = 8;  // chunks taken per counter increment (<= 32)
 };
 
@@ -78,8 +68,8 @@ struct SlotMeta {
   uint32_t q;     // chunk id, or kEnd
   uint32_t n;     // elements in the chunk
   uint32_t m;     // the block's access mask
-  uint32_t aux;   // TIES: bits threshold of this (expert, trim group); renormalised AVG: the
-                  // experts counted in the normaliser (selected or with a zero delta block)
+  uint32_t aux;   // renormalised AVG: the experts counted in the normaliser (selected or with a
+                  // zero delta block)
 };
 
 // block metadata of one chunk of a grab, staged by the producer warp
@@ -94,12 +84,10 @@ struct __align__(128) Smem {
   uint8_t slot[NS][SB];
   SlotMeta meta[NS];
   ChunkMeta chunk[G];
-  uint32_t thr[G][kMaxK];  // TIES: bits threshold of (chunk, expert)
   uint32_t zmask[G];       // renormalised AVG: experts whose delta block is exactly zero
   uint64_t full[NS];
   uint64_t empty[NS];
   unsigned long long realized[kMaxK];
-  float2 ctab[kMaxK + 1];  // TIES: {c, RN(1/c)} for the counts c = 0..kMaxK (entry 0: {1, 1})
   int abort, last;
 };
 
@@ -142,49 +130,6 @@ __device__ __forceinline__ void f2_fma(float a0, float a1, float b0, float b1, f
 // float compare against it is never true.
 __host__ __device__ __forceinline__ uint32_t ties_bits_threshold(uint32_t tau) {
   return tau == 0u ? 0u : (tau << 16) - 0x8000u + (tau & 1u);
-}
-
-// One expert's contribution to an element's TIES tally, with predicated adds: the delta d
-// is kept when |d| >= thr; a kept d goes into P (with count +1) when positive or into N
-// (count + 0x10000) otherwise.  thr is at least the smallest subnormal, so a kept d is
-// never zero and "not positive" means negative; one compare with two destination
-// predicates splits the kept entries by sign.  A skipped add is the same as adding the +0
-// of a trimmed entry: P and N are never -0, so +0 leaves them unchanged.  The elected
-// sign is that of P + N (compared exactly at the end).
-__device__ __forceinline__ void ties_tally(float d, float thr, float& P, float& N, uint32_t& cnt) {
-  asm("{\n"
-      " .reg .pred pk, pp, pn;\n"
-      " .reg .f32 ad;\n"
-      " abs.f32 ad, %3;\n"
-      " setp.ge.f32 pk, ad, %4;\n"
-      " setp.gt.and.f32 pp|pn, %3, 0f00000000, pk;\n"
-      " @pp add.rn.f32 %0, %0, %3;\n"
-      " @pn add.rn.f32 %1, %1, %3;\n"
-      " @pp add.u32 %2, %2, 1;\n"
-      " @pn add.u32 %2, %2, 65536;\n"
-      "}\n"
-      : "+f"(P), "+f"(N), "+r"(cnt)
-      : "f"(d), "f"(thr));
-}
-
-// One expert's contribution to an element's DARE-TIES tally: the rescaled delta s enters
-// when its keep word kw (the 16-bit word in the upper half of a 32-bit register) reaches
-// T16 and s is nonzero, into P (count +1) when positive or N (count + 0x10000) when
-// negative; no magnitude trim.  A dropped or zero entry adds nothing (the +0 of Eq. 4's
-// dropped delta leaves P and N unchanged).
-__device__ __forceinline__ void dties_tally(float s, uint32_t kw, uint32_t T16, float& P, float& N, uint32_t& cnt) {
-  asm("{\n"
-      " .reg .pred pk, pp, pn;\n"
-      " setp.ge.u32 pk, %4, %5;\n"
-      " setp.gt.and.f32 pp, %3, 0f00000000, pk;\n"
-      " setp.lt.and.f32 pn, %3, 0f00000000, pk;\n"
-      " @pp add.rn.f32 %0, %0, %3;\n"
-      " @pn add.rn.f32 %1, %1, %3;\n"
-      " @pp add.u32 %2, %2, 1;\n"
-      " @pn add.u32 %2, %2, 65536;\n"
-      "}\n"
-      : "+f"(P), "+f"(N), "+r"(cnt)
-      : "f"(s), "r"(kw), "r"(T16));
 }
 
 // bf16 -> fp32: the upper element by a mask, the lower one moved up by a multiply (which runs
@@ -279,34 +224,33 @@ __device__ __forceinline__ void delta_pairs(const uint4 r, const float* x0, Fold
   }
 }
 
-// the tail loops are unrolled over the vector with a predicate, so that h and y stay in
-// registers (a loop bounded by navail would index them at run time, through local memory)
+// elements e and e + 1 of an output vector into its words: bf16 two per conversion, each rounded
+// to nearest-even, element e in the low half
 template <bool BF16>
-__device__ __forceinline__ void store_vec(void* ptr, uint64_t elem, uint32_t navail, const float* y) {
-  constexpr uint32_t V = BF16 ? 8u : 4u;
+__device__ __forceinline__ void put_pair(uint32_t (&w)[4], int e, float y0, float y1) {
   if constexpr (BF16) {
-    // two elements per conversion, each rounded to nearest-even: element 2k in the low half
-    uint32_t w[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const __nv_bfloat162 h2 = __floats2bfloat162_rn(y[2 * k], y[2 * k + 1]);
-      w[k] = *reinterpret_cast<const uint32_t*>(&h2);
-    }
-    if (navail >= V) {
-      __stcs(reinterpret_cast<uint4*>(static_cast<char*>(ptr) + elem * 2u), make_uint4(w[0], w[1], w[2], w[3]));
-    } else {
-#pragma unroll
-      for (uint32_t e = 0; e < V; ++e)
-        if (e < navail) static_cast<uint16_t*>(ptr)[elem + e] = (uint16_t)(w[e >> 1] >> (16u * (e & 1u)));
-    }
+    const __nv_bfloat162 h2 = __floats2bfloat162_rn(y0, y1);
+    w[e >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
   } else {
-    if (navail >= V) {
-      __stcs(reinterpret_cast<float4*>(static_cast<char*>(ptr) + elem * 4u), make_float4(y[0], y[1], y[2], y[3]));
-    } else {
+    w[e] = __float_as_uint(y0);
+    w[e + 1] = __float_as_uint(y1);
+  }
+}
+
+// the tail is unrolled over the vector with a predicate, so that w stays in registers (a loop
+// bounded by navail would index it at run time, through local memory)
+template <bool BF16>
+__device__ __forceinline__ void store_words(void* ptr, uint64_t elem, uint32_t navail, const uint32_t (&w)[4]) {
+  constexpr uint32_t V = BF16 ? 8u : 4u, ES = BF16 ? 2u : 4u;
+  if (navail >= V) {
+    __stcs(reinterpret_cast<uint4*>(static_cast<char*>(ptr) + elem * ES), make_uint4(w[0], w[1], w[2], w[3]));
+    return;
+  }
 #pragma unroll
-      for (uint32_t e = 0; e < V; ++e)
-        if (e < navail) static_cast<float*>(ptr)[elem + e] = y[e];
-    }
+  for (uint32_t e = 0; e < V; ++e) {
+    if (e >= navail) break;
+    if constexpr (BF16) static_cast<uint16_t*>(ptr)[elem + e] = (uint16_t)(w[e >> 1] >> (16u * (e & 1u)));
+    else static_cast<uint32_t*>(ptr)[elem + e] = w[e];
   }
 }
 
@@ -337,23 +281,18 @@ __device__ __forceinline__ bool checked_chunk(const MergeLaunch& p, uint64_t b, 
 // DARE keep words: element j of expert i keeps its delta iff 16-bit word j mod 8 of the
 // Philox4x32-10 output for counter (j / 8, i, tag) is >= T.  A bf16 vector is exactly the 8 words
 // of one call (chunk and tensor offsets are multiples of 8 elements); an fp32 vector is half of
-// one.  The whole-chunk kernel keeps the experts' share of the first two rounds in shared memory,
-// for the kDareHi lowest values of a group number's upper word (a test for larger ones in its
-// loop cost 10 instructions per vector and expert, 5 % of the DARE merge); families past
-// kDareSpan elements take the streaming kernel, which makes that share for each fill.
-constexpr uint32_t kDareHi = 4;
-constexpr uint64_t kDareSpan = (uint64_t)kDareHi << 35;
+// one.  The experts' share of the first two rounds comes with each group of fills (dare_expert,
+// made by the producer; consumers that made it themselves for groups past 2^32 tested for them in
+// every call: 10 instructions per vector and expert, 5 % of the DARE merge).
 constexpr uint32_t kDareTag = 0x44415245u;
 
 struct DareVec {
   PhiloxGroup grp;
-  uint32_t g_hi;  // upper word of the group number
-  bool upper;     // fp32: the vector is the upper half of its group
+  bool upper;  // fp32: the vector is the upper half of its group
 };
 
-__device__ __forceinline__ DareVec dare_vec(const MergeLaunch& p, uint64_t j0) {
-  const uint64_t g = j0 >> 3;
-  return DareVec{philox_group((uint32_t)g, kDareTag, p.dare_rk), (uint32_t)(g >> 32), (j0 & 4u) != 0u};
+__device__ __forceinline__ DareVec dare_vec(uint64_t j0, const MergeLaunch& p) {
+  return DareVec{philox_group((uint32_t)(j0 >> 3), kDareTag, p.dare_rk), (j0 & 4u) != 0u};
 }
 
 __device__ __forceinline__ uint4 dare_expert(const MergeLaunch& p, uint32_t g_hi, uint32_t i) {
@@ -398,13 +337,14 @@ __device__ __forceinline__ void merge_end(const MergeLaunch& p, volatile int* s_
 }
 
 template <bool BF16, int OPC>
-__global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
+__global__ void __launch_bounds__(Geo::kThreads, Geo::kCtasPerSm)
     merge_tma_kernel(const MergeLaunch p, uint32_t cpb, uint64_t n_chunks, unsigned long long* work) {
-  constexpr int kConsumers = Geo<OPC>::kConsumers;
+  static_assert(OPC == OP_ADD || OPC == OP_RENORM, "streaming consumers: AVG/TA and the renormalised AVG");
+  constexpr int kConsumers = Geo::kConsumers;
   constexpr uint32_t ES = BF16 ? 2u : 4u;
-  constexpr uint32_t SB = Geo<OPC>::kSlotBytes;
-  constexpr int kSlots = Geo<OPC>::kSlots;
-  constexpr uint32_t G = Geo<OPC>::kGrab;
+  constexpr uint32_t SB = Geo::kSlotBytes;
+  constexpr int kSlots = Geo::kSlots;
+  constexpr uint32_t G = Geo::kGrab;
   constexpr uint32_t CH = SB / ES;  // elements per chunk
   constexpr int V = BF16 ? 8 : 4;
   constexpr int VPT = (int)(CH / (kConsumers * V));  // vectors per consumer thread per chunk
@@ -424,11 +364,6 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
     mbar_fence_init();
   }
   if (tid < (uint32_t)kMaxK) S.realized[tid] = 0;
-  constexpr bool kDare = OPC == OP_DARE || OPC == OP_DTIES;
-  if (tid <= (uint32_t)kMaxK) {
-    const float c = tid == 0 ? 1.0f : (float)tid;
-    S.ctab[tid] = make_float2(c, __fdiv_rn(1.0f, c));
-  }
   __syncthreads();
 
   if (warp == kConsumers / 32) {
@@ -462,7 +397,6 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
       if (q0 >= n_chunks || !ok) break;
       if (lane == 0) q_next = atomicAdd(work, (unsigned long long)G);  // used by the next grab
       // lanes c < G: metadata of chunk q0 + c
-      uint32_t grp = 0;
       uint64_t bq = 0;  // block of chunk q0 + lane
       if (lane < G) {
         const unsigned long long q = q0 + lane;
@@ -476,19 +410,9 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
           cm.m = p.mask[b];
           cm.n = start < len ? min(CH, len - start) : 0u;
           if (p.touched_only && cm.m == 0u) cm.n = 0u;  // left as it is: a reference to M_0
-          if constexpr (OPC == OP_TIES) grp = p.blk_group[b];
-          if (!checked_chunk<OPC == OP_TIES>(p, b, cm, grp, ES)) cm.n = 0u, grp = 0u;
+          if (!checked_chunk<false>(p, b, cm, 0u, ES)) cm.n = 0u;
         }
         S.chunk[lane] = cm;
-      }
-      if constexpr (OPC == OP_TIES) {
-        // lane i < K: the trim thresholds of expert i for every chunk of the grab, at least
-        // the smallest subnormal (a zero delta is never kept: it would add nothing)
-#pragma unroll
-        for (uint32_t c = 0; c < G; ++c) {
-          const uint32_t g = __shfl_sync(0xFFFFFFFFu, grp, c);
-          if (lane < p.K) S.thr[c][lane] = max(ties_bits_threshold(p.tau[(uint64_t)lane * p.n_groups + g]), 1u);
-        }
       }
       if constexpr (OPC == OP_RENORM) {
         // lane i < K: is expert i's delta block exactly zero (catalog nnz = 0)?  Such an
@@ -513,8 +437,7 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
           ok = produce(q, cm.off, cm.n, cm.m, aux0, static_cast<const char*>(p.base) + cm.off * ES, bytes);
           for (uint32_t mm = cm.m; ok && mm; mm &= mm - 1) {
             const uint32_t i = __ffs(mm) - 1;
-            // DARE-TIES keeps every nonzero rescaled delta: threshold = the smallest subnormal
-            ok = produce(q, cm.off, cm.n, cm.m, OPC == OP_TIES ? S.thr[c][i] : 1u,
+            ok = produce(q, cm.off, cm.n, cm.m, 0u,
                          static_cast<const char*>(p.experts.p[i]) + (cm.off - p.expert_origin) * ES, bytes);
             S.realized[i] += (unsigned long long)cm.n * ES;
           }
@@ -544,21 +467,11 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
   }
 
   // ---------------- consumers ----------------
-  float x0[VPT][V], acc[VPT][V], Pp[VPT][V], Nn[VPT][V];
-  uint32_t cnt[VPT][V];  // TIES: positive count | negative count << 16
+  float x0[VPT][V], acc[VPT][V];
   uint64_t off = 0;
   uint32_t n = 0, n_tma = 0, remaining = 0;
   uint32_t m_chunk = 0, m_rest = 0;  // the chunk's access mask; its experts still to come
   float s_sel = 0.0f;  // renormalised AVG: sum of the counted experts' alpha (ascending)
-  // DARE keep decisions of the vector's elements (dare_keep_words)
-  DareVec dv[VPT];
-  auto dare_words = [&](uint32_t i, int u, uint32_t (&kw)[V]) { dare_keep_words<BF16>(p, dv[u], dare_expert(p, dv[u].g_hi, i), kw); };
-  auto dare_kept = [&](uint32_t i, int u, bool (&kept)[V]) {
-    uint32_t kw[V];
-    dare_words(i, u, kw);
-#pragma unroll
-    for (int e = 0; e < V; ++e) kept[e] = kw[e] >= p.dare_T16;
-  };
   for (uint32_t fill = 0;; ++fill) {
     const uint32_t s = fill % kSlots, r = fill / kSlots;
     if (!warp_wait<true>(&S.full[s], r & 1u, abort_flag, wl)) {
@@ -586,73 +499,23 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
         const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
         read_vec<BF16>(slot, p.base, off, k0, n, n_tma, x0[u]);
         if (remaining) {
-          if constexpr (kDare) dv[u] = dare_vec(p, off + k0);
 #pragma unroll
-          for (int e = 0; e < V; ++e) {
-            acc[u][e] = 0.0f;
-            Pp[u][e] = 0.0f;
-            Nn[u][e] = 0.0f;
-            cnt[u][e] = 0u;
-          }
+          for (int e = 0; e < V; ++e) acc[u][e] = 0.0f;
         }
       }
     } else {
       const uint32_t i = __ffs(m_rest) - 1;
       m_rest &= m_rest - 1;
       const void* src = p.experts.p[i];
-      if constexpr (kTiesLike<OPC>) {
-        // TIES: trim test on the magnitude's bits: key(|d|) >= tau exactly when bits(|d|) >=
-        // the producer's threshold (a NaN pattern, never true, when nothing is kept).
-        // DARE-TIES: the delta is rescaled, and it enters when its keep word passes and the
-        // result is nonzero (no magnitude trim).
-        const float thr = __uint_as_float(OPC == OP_TIES ? S.meta[s].aux : 1u);
+      // renormalised AVG: beta_i = alpha_i / (sum of the selected alpha), one IEEE division
+      const float a = OPC == OP_RENORM ? __fdiv_rn(p.alpha[i], s_sel) : p.alpha[i];
 #pragma unroll
-        for (int u = 0; u < VPT; ++u) {
-          const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
-          float xe[V];
-          read_vec<BF16>(slot, src, off - p.expert_origin, k0, n, n_tma, xe);
-          uint32_t kw[V];
-          if constexpr (OPC == OP_DTIES) dare_words(i, u, kw);
-#pragma unroll
-          for (int e = 0; e < V; e += 2) {
-            // the deltas of an element pair in one packed fp32x2 subtract
-            float d0, d1;
-            f2_sub(xe[e], xe[e + 1], x0[u][e], x0[u][e + 1], d0, d1);
-            if constexpr (OPC == OP_DTIES) {
-              float s0, s1;
-              f2_mul(d0, d1, p.sigma, p.sigma, s0, s1);
-              dties_tally(s0, kw[e], p.dare_T16, Pp[u][e], Nn[u][e], cnt[u][e]);
-              dties_tally(s1, kw[e + 1], p.dare_T16, Pp[u][e + 1], Nn[u][e + 1], cnt[u][e + 1]);
-            } else {
-              ties_tally(d0, thr, Pp[u][e], Nn[u][e], cnt[u][e]);
-              ties_tally(d1, thr, Pp[u][e + 1], Nn[u][e + 1], cnt[u][e + 1]);
-            }
-          }
-        }
-      } else {
-        // renormalised AVG: beta_i = alpha_i / (sum of the selected alpha), one IEEE division
-        const float a = OPC == OP_RENORM ? __fdiv_rn(p.alpha[i], s_sel) : p.alpha[i];
-#pragma unroll
-        for (int u = 0; u < VPT; ++u) {
-          const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
-          float xe[V];
-          read_vec<BF16>(slot, src, off - p.expert_origin, k0, n, n_tma, xe);
-          bool kept[V];
-          if constexpr (OPC == OP_DARE) dare_kept(i, u, kept);
-#pragma unroll
-          for (int e = 0; e < V; e += 2) {
-            float d0, d1;
-            f2_sub(xe[e], xe[e + 1], x0[u][e], x0[u][e + 1], d0, d1);
-            if constexpr (OPC == OP_DARE) {  // a dropped entry is omitted from the sum
-              float s0, s1;
-              f2_mul(d0, d1, p.sigma, p.sigma, s0, s1);
-              if (kept[e]) acc[u][e] = __fmaf_rn(a, s0, acc[u][e]);
-              if (kept[e + 1]) acc[u][e + 1] = __fmaf_rn(a, s1, acc[u][e + 1]);
-            } else {
-              f2_fma(a, a, d0, d1, acc[u][e], acc[u][e + 1], acc[u][e], acc[u][e + 1]);
-            }
-          }
-        }
+      for (int u = 0; u < VPT; ++u) {
+        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
+        const uint4 re = read_raw<BF16>(slot, src, off - p.expert_origin, k0, n, n_tma);
+        delta_pairs<BF16>(re, x0[u], [&](int e, float d0, float d1) {
+          f2_fma(a, a, d0, d1, acc[u][e], acc[u][e + 1], acc[u][e], acc[u][e + 1]);
+        });
       }
       --remaining;
     }
@@ -660,134 +523,98 @@ __global__ void __launch_bounds__(Geo<OPC>::kThreads, Geo<OPC>::kCtasPerSm)
     if (remaining == 0) {
 #pragma unroll
       for (int u = 0; u < VPT; ++u) {
-        // every lane of the warp runs the finalisation (a lane past the chunk's end holds
-        // zeros) so that the warp vote below is reached by all of them; only the store is
-        // limited to the chunk
         const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
-        const bool live = k0 < n;
-        float y[V];
-        if (m_chunk == 0) {  // uniform over the warp
-          // no expert selected: every accumulator is +0, so the output is M_0 plus the
-          // zero the operator adds (lambda * +0 for TIES, +0 otherwise)
-          const float z = kTiesLike<OPC> ? __fmul_rn(p.lambda, 0.0f) : 0.0f;
+        if (k0 >= n) continue;
+        // no expert selected: every accumulator would be +0, the output is M_0 plus that
+        uint32_t w[4];
 #pragma unroll
-          for (int e = 0; e < V; ++e) y[e] = __fadd_rn(x0[u][e], z);
-          if (live) store_vec<BF16>(p.out, off + k0, n - k0, y);
-          continue;
-        }
-        if constexpr (kTiesLike<OPC>) {
-          // one division per element: the mean of the entries whose sign was elected, the
-          // sign of P + N taken exactly as P > -N or P < -N (then that side holds at least
-          // one entry, so c >= 1; otherwise +0 / 1 = +0).  The rare numerators that need the
-          // IEEE division take it under one warp vote.
-          auto num_c = [&](int e, float& num, uint32_t& c) {
-            const bool pos = Pp[u][e] > -Nn[u][e], any = Pp[u][e] != -Nn[u][e];
-            num = any ? (pos ? Pp[u][e] : Nn[u][e]) : 0.0f;
-            c = any ? (pos ? (cnt[u][e] & 0xFFFFu) : (cnt[u][e] >> 16)) : 0u;
-          };
-          bool exact = false;
-#pragma unroll
-          for (int e = 0; e < V; ++e) {
-            float num;
-            uint32_t c;
-            num_c(e, num, c);
-            const float2 cy = S.ctab[c];
-            y[e] = div_small_fast(num, cy.x, cy.y);
-            exact = exact || div_small_needs_ieee(num);
-          }
-          if (__any_sync(0xFFFFFFFFu, exact)) {
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-              float num;
-              uint32_t c;
-              num_c(e, num, c);
-              if (div_small_needs_ieee(num)) y[e] = __fdiv_rn(num, S.ctab[c].x);
-            }
-          }
-#pragma unroll
-          for (int e = 0; e < V; ++e) y[e] = __fmaf_rn(p.lambda, y[e], x0[u][e]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < V; ++e) y[e] = __fadd_rn(x0[u][e], acc[u][e]);
-        }
-        if (live) store_vec<BF16>(p.out, off + k0, n - k0, y);
+        for (int e = 0; e < V; e += 2)
+          put_pair<BF16>(w, e, __fadd_rn(x0[u][e], m_chunk == 0 ? 0.0f : acc[u][e]),
+                         __fadd_rn(x0[u][e + 1], m_chunk == 0 ? 0.0f : acc[u][e + 1]));
+        store_words<BF16>(p.out, off + k0, n - k0, w);
       }
     }
   }
   merge_end<kConsumers + 32>(p, &S.last);
 }
 
-// ---------------- TIES (at most 8 experts) and DARE (at most 16): whole-chunk consumers ----------------
+// ---------------- TIES, DARE and DARE-TIES: groups of fills ----------------
 //
-// The same TMA ring, but a chunk (its base fill and its selected experts' fills, which sit in
-// consecutive ring slots) is published as one unit: one "full" mbarrier per chunk counts the
-// bytes of all its fills, one "empty" mbarrier per chunk counts the consumers' releases.
-// A consumer thread waits once per chunk, folds every selected expert of its vector in the
-// fixed ascending order while all of them are in shared memory, releases the chunk and only
-// then finalises: the per-element state (M_0 and P, N, counts for TIES, the accumulator for
-// DARE) lives for one chunk and the per-fill waits, arrivals and metadata reads of the
-// streaming kernel disappear.  The ring must hold every fill of one chunk (1 + K slots), so
-// this kernel serves TIES with K <= 8 and DARE with K <= 16; the streaming kernel above
-// serves the other operators and larger expert counts.
-constexpr uint32_t kTcMaxK = 16;
+// The same TMA ring, but fills are published in groups: a chunk's base fill and its first GF
+// selected experts' fills, then GF more at a time, each group in consecutive ring slots with
+// one "full" mbarrier that counts the bytes of its fills and one "empty" mbarrier that counts
+// the consumers' releases.  A consumer thread waits once per group, folds the group's experts
+// into its vector in the fixed ascending order, and releases the group; after a chunk's last
+// group it finalises.  The per-fill waits, arrivals and metadata reads of the streaming kernel
+// above disappear, and whatever a chunk selects the ring holds two groups or more, so that one
+// is brought in while another is folded.
+constexpr uint32_t kTcMaxK = 32;
 
-// ring slots and CTAs per SM by expert count: K <= 4 holds two chunks of 5 fills in 11
-// slots at four CTAs per SM (three for DARE-TIES, whose state needs more registers); K <= 8
-// two chunks of 9 fills in 18 slots at three; K <= 16 one chunk of 17 fills, or several of
-// the usual few selected experts, in 17 slots at three.  A fill is 4 KiB: 256 consumer threads
-// take one vector each, but for TIES with K <= 4 128 threads take two (a chunk's wait, release
-// and metadata reads are then shared by two vectors, and 96 registers a thread hold both: 1.015
-// -> 0.980 ms on four Llama layers at the full budget).  Measured and not taken, on DARE and
-// DARE-TIES with 16 experts (1.41 and 2.17 ms here): two vectors per thread 1.47 and 2.47 ms,
-// 2 KiB fills at six CTAs per SM 1.55 and 2.37, 3 KiB fills at four 1.46 and 2.42; TIES with 8
-// experts (0.82 ms): two vectors 0.83, 3 KiB fills 0.99.
+// Ring slots, experts per group and CTAs per SM by expert count: K <= 4 takes a chunk of up to 5
+// fills as one group, two of them in 11 slots, at four CTAs per SM (three for DARE-TIES, whose
+// state needs more registers); K <= 8 one group of up to 9 fills, two in 18 slots (17 where the
+// mask words fill the entries), at three; larger K groups of up to 8 experts in 17 slots at
+// three, whose consumers keep a chunk's state from group to group.  A fill is 4 KiB: 256 consumer
+// threads take one vector each, but for TIES and DARE with K <= 4 128 threads take two (a group's
+// wait, release and metadata reads are then shared by two vectors, and 96 registers a thread hold
+// both: TIES 1.006 -> 0.969 ms on four Llama layers at the full budget, DARE 1.304 -> 1.248).
+//
+// Merge times, ms, of the streaming kernel (K > 8 TIES, K > 16), of whole chunks in the ring, and
+// here: Qwen2.5-0.5B TIES K = 16 at f = 0.25 1.313 / 1.235 / 0.945, at f = 1 1.614 / 1.480 / 1.099;
+// K = 32 (8 layers) TIES 1.258 / - / 0.835, DARE 1.526 / - / 1.108, DARE-TIES 1.843 / - / 1.596;
+// Qwen2.5-1.5B (8 layers) K = 16 DARE - / 1.414 / 1.315; TIES K = 8 - / 0.819 / 0.712; four Llama
+// layers TIES K = 4 - / 0.978 / 0.926 at f = 1, - / 0.654 / 0.621 at f = 0.1.  Groups of 5 gave
+// 1.141 ms for TIES K = 16 at f = 1 (1.109 with 8 then), 7 1.119, 16 (one chunk) 1.240.  Measured
+// and not taken, on DARE with 16 experts: two vectors per thread 1.430 ms, four CTAs per SM with
+// groups of 6 in 13 slots 1.344, both 1.328; earlier, 2 KiB fills at six CTAs per SM 1.55 against
+// 1.41, 3 KiB fills at four 1.46.
 template <int OPC, int KC>
 struct TcGeo {
-  static constexpr int kSlots = KC <= 4 ? 11 : (KC <= 8 ? 18 : 17);
+  static constexpr int kSlots = KC <= 4 ? 11 : (KC <= 8 && OPC == OP_TIES ? 18 : 17);
+  static constexpr int kGroup = KC <= 4 ? 4 : 8;  // expert fills per group
   static constexpr int kCtasPerSm = KC <= 4 && OPC != OP_DTIES ? 4 : 3;
-  static constexpr int kVpt = KC <= 4 && OPC == OP_TIES ? 2 : 1;  // vectors per consumer thread and fill
+  static constexpr int kVpt = KC <= 4 && OPC != OP_DTIES ? 2 : 1;  // vectors per consumer thread and fill
   static constexpr int kConsumers = 256 / kVpt;
   static constexpr int kThreads = kConsumers + 32;
   static constexpr uint32_t kSlotBytes = kConsumers * kVpt * 16u;
   static constexpr uint32_t kGrab = 8;
 };
 
-template <int KC, int NT>
+enum : uint32_t { kFirst = 1u, kLast = 2u, kFast = 4u, kNone = 8u, kEndGroup = 16u };
+
+template <int GF, bool TIES>
 struct TcEntry {
-  uint64_t off;          // element offset of the chunk
-  uint32_t q;            // chunk id, or kEnd
-  uint32_t n;            // elements in the chunk
-  uint32_t m;            // the block's access mask
-  uint32_t s0;           // ring slot of the base fill; expert fill j sits in slot s0 + 1 + j (mod NS)
-  uint32_t nsel;         // selected experts
-  uint32_t fast;         // 1: every selected threshold is >= 2^-100 (no numerator needs the IEEE division)
-  float thr[NT];         // TIES: trim thresholds (as floats) in fill order
-  uint8_t ex[KC];        // the selected experts in fill order
+  uint64_t off;    // element offset of the chunk
+  uint32_t n;      // elements in the chunk
+  uint32_t flags;  // kFirst: the group begins with the base fill; kLast: it ends its chunk; kFast:
+                   // every selected threshold is >= 2^-100 (no numerator needs the IEEE division);
+                   // kNone: the chunk selects no expert
+  uint32_t s0;     // ring slot of the group's first fill; fill j sits in slot s0 + j (mod NS)
+  uint32_t nexp;   // expert fills
+  uint8_t ex[GF < 8 ? 8 : GF];    // their experts in fill order
+  float thr[TIES ? GF : 1];       // TIES: their trim thresholds
+  alignas(16) uint4 pe[TIES ? 1 : GF];  // DARE, DARE-TIES: dare_expert of each
 };
 
-// sized by the expert count KC so that three CTAs of 18 slots fit one SM's 228 KB
-template <int NS, uint32_t SB, uint32_t G, int KC, bool TIES>
+template <int NS, uint32_t SB, uint32_t G, int KC, int GF, bool TIES>
 struct __align__(128) TcSmem {
-  static constexpr int NT = TIES ? KC : 1, NE = TIES ? 1 : KC;
   uint8_t slot[NS][SB];
-  TcEntry<KC, NT> ce[NS];
-  ChunkMeta chunk[G];
-  uint32_t thr[G][NT];  // TIES: bits threshold of (chunk of the grab, expert)
+  TcEntry<GF, TIES> ce[NS];
+  uint32_t thr[TIES ? G : 1][KC];  // producer only, TIES: bits threshold of (chunk of the grab, expert)
   uint64_t full[NS];
   uint64_t empty[NS];
-  unsigned long long realized[KC];
-  float2 ntab[kTcMaxK + 1];  // {-c, RN(1/c)} for the counts c = 0..16 (entry 0: {-1, 1})
-  uint32_t nf[NS];           // producer only: fills held by the chunk of each entry
-  uint4 pe[TIES ? 1 : kDareHi][NE];  // DARE, DARE-TIES: dare_expert of every expert, by the group's upper word
+  float2 ntab[kTcMaxK + 1];  // {-c, RN(1/c)} for the counts c = 0..32 (entry 0: {-1, 1})
+  uint32_t nf[NS];           // producer only: fills held by the group of each entry
   int abort, last;
 };
 
 template <bool BF16, int OPC, int KC>
 __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCtasPerSm)
     merge_chunk_kernel(const MergeLaunch p, uint32_t cpb, uint64_t n_chunks, unsigned long long* work) {
-  static_assert(OPC == OP_TIES || OPC == OP_DARE || OPC == OP_DTIES, "whole-chunk consumers: TIES, DARE, DARE-TIES");
-  // the packed counts C = 2^23 + c+ + 2^CB c-: CB = 4 bits for up to 8 experts, 5 for 16
-  constexpr uint32_t CB = KC <= 8 ? 4u : 5u;
+  static_assert(OPC == OP_TIES || OPC == OP_DARE || OPC == OP_DTIES, "groups of fills: TIES, DARE, DARE-TIES");
+  // the packed counts C = 2^23 + c+ + 2^CB c-: CB = 4 bits for up to 8 experts, 6 for 32
+  constexpr uint32_t CB = KC <= 8 ? 4u : 6u;
+  constexpr int GF = TcGeo<OPC, KC>::kGroup;
   constexpr int NS = TcGeo<OPC, KC>::kSlots;
   constexpr int kConsumers = TcGeo<OPC, KC>::kConsumers;
   constexpr uint32_t G = TcGeo<OPC, KC>::kGrab;
@@ -796,11 +623,10 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
   constexpr uint32_t CH = SB / ES;  // elements per chunk
   constexpr int V = BF16 ? 8 : 4;
   constexpr int VPT = TcGeo<OPC, KC>::kVpt;
-  constexpr int kThreads = kConsumers + 32;
   static_assert(CH == (uint32_t)(kConsumers * VPT * V), "whole vectors per consumer thread and chunk");
-  static_assert(NS >= KC + 1, "the ring holds every fill of a chunk");
+  static_assert(NS >= 2 * GF + 1, "a group is brought in while another is folded");
   extern __shared__ __align__(128) uint8_t smem_raw[];
-  using Sm = TcSmem<NS, SB, G, KC, OPC == OP_TIES>;
+  using Sm = TcSmem<NS, SB, G, KC, GF, OPC == OP_TIES>;
   Sm& S = *reinterpret_cast<Sm*>(smem_raw);
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
   volatile int* abort_flag = &S.abort;
@@ -809,15 +635,11 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&S.full[s], 1);
-      mbar_init(&S.empty[s], kConsumers);  // every consumer thread arrives once per chunk
+      mbar_init(&S.empty[s], kConsumers);  // every consumer thread arrives once per group
     }
     S.abort = 0;
     mbar_fence_init();
   }
-  if (tid < (uint32_t)KC) S.realized[tid] = 0;
-  if (OPC != OP_TIES)
-    for (uint32_t k = tid; k < kDareHi * KC; k += kThreads)
-      if (k % KC < p.K) S.pe[k / KC][k % KC] = dare_expert(p, k / KC, k % KC);
   if (tid <= kTcMaxK) {
     const float c = tid == 0 ? 1.0f : (float)tid;
     S.ntab[tid] = make_float2(-c, __fdiv_rn(1.0f, c));
@@ -825,263 +647,269 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
   __syncthreads();
 
   if (warp == kConsumers / 32) {
-    // ---------------- producer ----------------
+    // ---------------- producer: lane i serves expert i ----------------
+    // The whole warp walks the chunks together.  A single lane that wrote each fill's metadata and
+    // issued its copy in a loop was what bounded these merges: TIES with 16 experts took 1.27 ms
+    // with it and 1.00 without, with 32 experts 1.14 and 0.88, DARE with 16 1.43 and 1.33 (groups
+    // of 7 on both sides).  Lane i keeps expert i's
+    // trim thresholds, mask words and realized bytes in registers; every lane waits for the ring
+    // itself, so that each has acquired the slots its copies refill.
     uint32_t fill = 0;  // ring slots used so far (monotonic)
-    uint32_t seq = 0;   // chunks published
-    uint32_t head = 0;  // oldest published chunk not yet seen released
-    uint32_t used = 0;  // slots held by chunks head .. seq - 1
+    uint32_t seq = 0;   // groups published
+    uint32_t head = 0;  // oldest published group not yet seen released
+    uint32_t used = 0;  // slots held by groups head .. seq - 1
     bool ok = true;
-    // lane 0: wait until entry seq % NS is free and nfill slots are free; chunks are
-    // released in order, so the oldest one is the next to free its slots
+    // wait until entry seq % NS is free and nfill slots are free; groups are released in order,
+    // so the oldest one is the next to free its slots
     auto reserve = [&](uint32_t nfill) -> bool {
       while (seq - head >= (uint32_t)NS || used + nfill > (uint32_t)NS) {
         const uint32_t he = head % NS;
-        if (!mbar_wait<true>(&S.empty[he], (head / NS) & 1u, abort_flag, wl)) return false;
+        if (!warp_wait(&S.empty[he], (head / NS) & 1u, abort_flag, wl)) return false;
         used -= S.nf[he];
         ++head;
       }
       return true;
     };
+    const bool mine = lane < p.K;  // this lane serves an expert
+    const char* src = mine ? static_cast<const char*>(p.experts.p[lane]) : nullptr;
+    unsigned long long realized = 0;
+    uint4 pe = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t pe_hi = 0xFFFFFFFFu;  // the upper word of the group number that pe is for
     unsigned long long q_next = 0;
     if (lane == 0) q_next = atomicAdd(work, (unsigned long long)G);
     for (;;) {
       const unsigned long long q0 = __shfl_sync(0xFFFFFFFFu, q_next, 0);
       if (q0 >= n_chunks || !ok) break;
       if (lane == 0) q_next = atomicAdd(work, (unsigned long long)G);  // used by the next grab
+      // lane c < G: metadata of chunk q0 + c
       uint32_t grp = 0;
+      ChunkMeta cl{0, 0, 0};
       if (lane < G) {
         const unsigned long long q = q0 + lane;
-        ChunkMeta cm{0, 0, 0};
         if (q < n_chunks && checked_block(p, p.b_begin + q / cpb)) {
           const uint64_t b = p.b_begin + q / cpb;
           const uint32_t start = (uint32_t)(q % cpb) * CH;
           const uint32_t len = p.blk_len[b];
-          cm.off = p.blk_off[b] + start;
-          cm.m = p.mask[b];
-          cm.n = start < len ? min(CH, len - start) : 0u;
-          if (p.touched_only && cm.m == 0u) cm.n = 0u;  // left as it is: a reference to M_0
+          cl.off = p.blk_off[b] + start;
+          cl.m = p.mask[b];
+          cl.n = start < len ? min(CH, len - start) : 0u;
+          if (p.touched_only && cl.m == 0u) cl.n = 0u;  // left as it is: a reference to M_0
           if (OPC == OP_TIES) grp = p.blk_group[b];
-          if (!checked_chunk<OPC == OP_TIES>(p, b, cm, grp, ES)) cm.n = 0u, grp = 0u;
+          if (!checked_chunk<OPC == OP_TIES>(p, b, cl, grp, ES)) cl.n = 0u, grp = 0u;
         }
-        S.chunk[lane] = cm;
       }
+      // TIES: this lane's expert's trim threshold for every chunk of the grab, at least the smallest
+      // subnormal (a zero delta is never kept: it would add nothing); each lane reads its own back
       if constexpr (OPC == OP_TIES) {
-        // lane i < K: the trim thresholds of expert i for every chunk of the grab, at least the
-        // smallest subnormal (a zero delta is never kept: it would add nothing)
 #pragma unroll
         for (uint32_t c = 0; c < G; ++c) {
           const uint32_t g = __shfl_sync(0xFFFFFFFFu, grp, c);
-          if (lane < p.K) S.thr[c][lane] = max(ties_bits_threshold(p.tau[(uint64_t)lane * p.n_groups + g]), 1u);
+          if (mine) S.thr[c][lane] = max(ties_bits_threshold(p.tau[(uint64_t)lane * p.n_groups + g]), 1u);
         }
       }
-      __syncwarp();
-      if (lane == 0) {
-        const uint32_t nq = (uint32_t)min((unsigned long long)G, n_chunks - q0);
-        for (uint32_t c = 0; c < nq && ok; ++c) {
-          const ChunkMeta cm = S.chunk[c];
-          if (cm.n == 0) continue;
-          const uint32_t nsel = __popc(cm.m);
-          if (!(ok = reserve(1u + nsel))) break;
-          if (fill >= (uint32_t)NS) fence_proxy_async_smem();  // slots the consumers have read are refilled
-          const uint32_t e = seq % NS;
-          const uint32_t bytes = (cm.n * ES) & ~15u;
-          auto& ce = S.ce[e];
-          ce.off = cm.off;
-          ce.q = (uint32_t)(q0 + c);
-          ce.n = cm.n;
-          ce.m = cm.m;
-          ce.s0 = fill % NS;
-          ce.nsel = nsel;
-          uint32_t fast = 1u, j = 0;
-          for (uint32_t mm = cm.m; mm; mm &= mm - 1, ++j) {
-            const uint32_t i = __ffs(mm) - 1;
-            ce.ex[j] = (uint8_t)i;
-            if constexpr (OPC == OP_TIES) {
-              const uint32_t t = S.thr[c][i];
-              ce.thr[j] = __uint_as_float(t);
-              fast &= t >= 0x0D800000u ? 1u : 0u;  // bits of 2^-100
+      // not unrolled, and without the loops that a class cannot take: the producer's code competes
+      // with the consumers' for the instruction cache (0.701 -> 0.623 ms at f = 0.1, with empty
+      // chunks apart in the consumers)
+#pragma unroll 1
+      for (uint32_t c = 0; c < G; ++c) {
+        uint64_t off = __shfl_sync(0xFFFFFFFFu, cl.off, c);
+        uint32_t left = __shfl_sync(0xFFFFFFFFu, cl.n, c);  // elements of the chunk still to be published
+        const uint32_t m = __shfl_sync(0xFFFFFFFFu, cl.m, c);
+        if (left == 0u || !ok) continue;
+        const bool sel = (m >> lane) & 1u;
+        const uint32_t rank = __popc(m & ((1u << lane) - 1u)), nsel = __popc(m);
+        uint32_t fast = 0u, thr = 0u;  // DARE-TIES: rescaled deltas may be tiny
+        if constexpr (OPC == OP_TIES) {
+          if (sel) thr = S.thr[c][lane];
+          fast = __any_sync(0xFFFFFFFFu, sel && thr < 0x0D800000u) ? 0u : kFast;  // bits of 2^-100
+        }
+        do {
+          uint32_t n = left;
+          if constexpr (OPC != OP_TIES) {
+            // an entry's share of the mask generator holds one upper word of the group number: a
+            // chunk that crosses a multiple of 2^35 elements goes as two
+            const uint32_t g_hi = (uint32_t)(off >> 35);
+            n = (uint32_t)min((uint64_t)left, ((uint64_t)g_hi + 1u << 35) - off);
+            if (g_hi != pe_hi && mine) pe = dare_expert(p, g_hi, lane);
+            pe_hi = g_hi;
+          }
+          left -= n;
+          const uint32_t bytes = (n * ES) & ~15u;
+          uint32_t done = 0u, first = 1u;
+          do {
+            const uint32_t nexp = min(nsel - done, (uint32_t)GF), nfill = nexp + first;
+            if (!(ok = reserve(nfill))) break;
+            if (fill >= (uint32_t)NS) fence_proxy_async_smem();  // slots the consumers have read are refilled
+            const uint32_t e = seq % NS;
+            const bool here = sel && rank >= done && rank < done + nexp;  // this lane's fill is in the group
+            auto& ce = S.ce[e];
+            if (here) {
+              ce.ex[rank - done] = (uint8_t)lane;
+              if constexpr (OPC == OP_TIES) ce.thr[rank - done] = __uint_as_float(thr);
+              else ce.pe[rank - done] = pe;
             }
-          }
-          ce.fast = OPC == OP_TIES ? fast : 0u;  // DARE-TIES: rescaled deltas may be tiny
-          S.nf[e] = 1u + nsel;
-          // test hook: the first chunk is never armed, so the consumers' wait for it runs out
-          const bool arm = !(seq == 0 && p.stall);
-          if (arm) mbar_arrive_expect_tx(&S.full[e], (1u + nsel) * bytes);
-          if (bytes && arm)
-            tma_load_1d(S.slot[fill % NS], static_cast<const char*>(p.base) + cm.off * ES, bytes, &S.full[e]);
-          ++fill;
-          for (uint32_t mm = cm.m; mm; mm &= mm - 1) {
-            const uint32_t i = __ffs(mm) - 1;
-            if (bytes && arm)
-              tma_load_1d(S.slot[fill % NS],
-                          static_cast<const char*>(p.experts.p[i]) + (cm.off - p.expert_origin) * ES, bytes,
-                          &S.full[e]);
-            ++fill;
-            S.realized[i] += (unsigned long long)cm.n * ES;
-          }
-          used += 1u + nsel;
-          ++seq;
-        }
+            if (lane == 0) {
+              ce.off = off;
+              ce.n = n;
+              ce.flags = (first ? kFirst : 0u) | (done + nexp == nsel ? kLast : 0u) | (nsel ? 0u : kNone) | fast;
+              ce.s0 = fill % NS;
+              ce.nexp = nexp;
+              S.nf[e] = nfill;
+            }
+            __syncwarp();  // the entry is written before it is published
+            // test hook: the first group is never armed, so the consumers' wait for it runs out
+            const bool arm = !(seq == 0 && p.stall);
+            if (lane == 0 && arm) {
+              mbar_arrive_expect_tx(&S.full[e], nfill * bytes);
+              if (first && bytes)
+                tma_load_1d(S.slot[fill % NS], static_cast<const char*>(p.base) + off * ES, bytes, &S.full[e]);
+            }
+            __syncwarp();  // armed before any lane's copy can complete
+            if (here) {
+              if (bytes && arm)
+                tma_load_1d(S.slot[(fill + first + rank - done) % NS], src + (off - p.expert_origin) * ES, bytes, &S.full[e]);
+              realized += (unsigned long long)n * ES;
+            }
+            fill += nfill;
+            used += nfill;
+            ++seq;
+            done += nexp;
+            first = 0u;
+          } while (GF < KC && done < nsel);
+          off += n;
+        } while (OPC != OP_TIES && left && ok);
       }
-      ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
-      __syncwarp();
     }
-    if (lane == 0) {
-      if (ok && (ok = reserve(0u))) {
-        const uint32_t e = seq % NS;
-        S.ce[e].q = kEnd;
+    if (ok && (ok = reserve(0u))) {
+      const uint32_t e = seq % NS;
+      if (lane == 0) {
+        S.ce[e].flags = kEndGroup;
         S.nf[e] = 0u;
         if (!(seq == 0 && p.stall)) mbar_arrive_expect_tx(&S.full[e], 0u);
-        ++seq;
       }
-      if (!ok) {
-        atomicOr(p.err, kErrTimeout);
-        S.abort = 1;
-      }
-      // drain: the last chunk of every entry must have landed before the CTA may exit
-      for (uint32_t e = 0; e < (uint32_t)NS && e < seq; ++e) {
-        const uint32_t last = seq - 1 - ((seq - 1 + NS - e) % NS);
-        if (last == 0 && p.stall) continue;  // never armed: nothing in flight
-        mbar_wait_drain(&S.full[e], (last / NS) & 1u);
-      }
-      for (uint32_t i = 0; i < p.K; ++i)
-        if (S.realized[i])
-          atomicAdd(p.realized + (uint64_t)(blockIdx.x % kCounterSlots) * p.K + i, S.realized[i]);
+      ++seq;
     }
+    if (!ok && lane == 0) {
+      atomicOr(p.err, kErrTimeout);
+      S.abort = 1;
+    }
+    // drain: the last group of every entry must have landed before the CTA may exit
+    for (uint32_t e = 0; e < (uint32_t)NS && e < seq; ++e) {
+      const uint32_t last = seq - 1 - ((seq - 1 + NS - e) % NS);
+      if (last == 0 && p.stall) continue;  // never armed: nothing in flight
+      mbar_wait_drain(&S.full[e], (last / NS) & 1u);
+    }
+    if (realized) atomicAdd(p.realized + (uint64_t)(blockIdx.x % kCounterSlots) * p.K + lane, realized);
     merge_end<kConsumers + 32>(p, &S.last);
     return;
   }
   // ---------------- consumers: thread t owns vectors t, t + kConsumers, ... of every chunk ----------------
+  float x0[VPT][V];
+  // DARE: acc = fma(alpha_i, v_i, acc) over the selected experts whose keep word passes, in
+  // ascending order, with v_i = delta_i * sigma (a dropped entry is omitted).
+  // TIES: P and N, the sums of the kept positive and negative deltas, and both counts in one
+  // float C = 2^23 + c+ + 2^CB c- (exact: every value is an integer below 2^24, so the low bits
+  // of C hold c+ and c-).  DARE-TIES keeps, instead, every nonzero rescaled delta s = d sigma
+  // whose keep word passes (no magnitude trim).  A delta d is kept positive when d >= thr and kept
+  // negative when d <= -thr (thr > 0: |d| >= thr and the sign in one compare each); the keep
+  // factors k+ and k- are 1 or 0, and P = fma(k+, d, P), N = fma(k-, d, N): a factor 1 adds d with
+  // the one rounding of P + d, a factor 0 adds a zero, which leaves P and N unchanged (they start
+  // at +0 and are never -0).  Two elements per packed instruction.
+  float Pp[VPT][V], Nn[VPT][V], Cc[VPT][V];
+  float (&acc)[VPT][V] = Pp;
+  // a class whose largest chunk is one group keeps its state for one group only
+  constexpr bool kWhole = GF >= KC;
   for (uint32_t c = 0;; ++c) {
     const uint32_t e = c % NS;
-    if (!warp_wait<true>(&S.full[e], (c / NS) & 1u, abort_flag, wl)) {
+    if (!warp_wait(&S.full[e], (c / NS) & 1u, abort_flag, wl)) {
       atomicOr(p.err, kErrTimeout);
       S.abort = 1;
       break;
     }
     const auto& ce = S.ce[e];
-    if (ce.q == kEnd) break;
+    const uint32_t begin = ce.flags;
+    if (begin & kEndGroup) break;
     uint32_t s = ce.s0;
-    const uint32_t nsel = ce.nsel;
-    float x0[VPT][V];
-    bool in_slot = true;  // the thread's vectors lie inside the bulk-copied bytes
-    {
-      const uint32_t n = ce.n, n_tma = ((n * ES) & ~15u) / ES;
-#pragma unroll
-      for (int u = 0; u < VPT; ++u) {
-        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
-        in_slot = in_slot && k0 + V <= n_tma;
-        read_vec<BF16>(S.slot[s], p.base, ce.off, k0, n, n_tma, x0[u]);
-      }
-    }
-    float y[VPT][V];
-    auto store = [&](uint64_t off, uint32_t n) {
-#pragma unroll
-      for (int u = 0; u < VPT; ++u) {
-        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
-        if (k0 < n) store_vec<BF16>(p.out, off + k0, n - k0, y[u]);
-      }
-    };
-    if (nsel == 0) {  // uniform over the CTA
+    const uint32_t nexp = ce.nexp;
+    // whether the thread's vectors lie inside the bulk-copied bytes
+    const bool in_slot = (tid + (uint32_t)(VPT - 1) * kConsumers + 1u) * V <= ((ce.n * ES) & ~15u) / ES;
+    if (begin & kNone) {  // uniform over the CTA
       // no expert selected: the output is M_0 plus the zero the operator adds (lambda * +0
       // for TIES, +0 for DARE)
-      const float z = kTiesLike<OPC> ? __fmul_rn(p.lambda, 0.0f) : 0.0f;
+      const uint32_t n = ce.n;
+      const uint64_t off = ce.off;
+      float xb[VPT][V];
 #pragma unroll
       for (int u = 0; u < VPT; ++u)
-#pragma unroll
-        for (int v = 0; v < V; ++v) y[u][v] = __fadd_rn(x0[u][v], z);
-      const uint64_t off = ce.off;
-      const uint32_t n = ce.n;
+        read_vec<BF16>(S.slot[s], p.base, off, (tid + (uint32_t)u * kConsumers) * V, n, ((n * ES) & ~15u) / ES, xb[u]);
       mbar_arrive(&S.empty[e]);
-      store(off, n);
+      const float z = kTiesLike<OPC> ? __fmul_rn(p.lambda, 0.0f) : 0.0f;
+#pragma unroll
+      for (int u = 0; u < VPT; ++u) {
+        uint32_t w[4];
+#pragma unroll
+        for (int v = 0; v < V; v += 2) {
+          float y0, y1;
+          f2_add(xb[u][v], xb[u][v + 1], z, z, y0, y1);
+          put_pair<BF16>(w, v, y0, y1);
+        }
+        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
+        if (k0 < n) store_words<BF16>(p.out, off + k0, n - k0, w);
+      }
       continue;
+    }
+    if (kWhole || (begin & kFirst)) {
+#pragma unroll
+      for (int u = 0; u < VPT; ++u) {
+        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V, n = ce.n;
+        read_vec<BF16>(S.slot[s], p.base, ce.off, k0, n, ((n * ES) & ~15u) / ES, x0[u]);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          Pp[u][v] = 0.0f;
+          if (OPC != OP_DARE) {
+            Nn[u][v] = 0.0f;
+            Cc[u][v] = 8388608.0f;  // 2^23
+          }
+        }
+      }
+      s = s + 1 == (uint32_t)NS ? 0u : s + 1;
     }
     DareVec dv[VPT];
     if constexpr (OPC != OP_TIES) {
 #pragma unroll
-      for (int u = 0; u < VPT; ++u) dv[u] = dare_vec(p, ce.off + (tid + (uint32_t)u * kConsumers) * V);
+      for (int u = 0; u < VPT; ++u) dv[u] = dare_vec(ce.off + (tid + (uint32_t)u * kConsumers) * V, p);
     }
-    // the raw vector u of the fill in slot sl, expert j of the chunk's selected ones
-    auto raw = [&](uint32_t sl, uint32_t j, int u) -> uint4 {
-      const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
-      if (in_slot) return *reinterpret_cast<const uint4*>(S.slot[sl] + k0 * ES);
-      // the ragged tail of a tensor, from global memory
-      const uint32_t n = ce.n;
-      return read_raw<BF16>(S.slot[sl], p.experts.p[ce.ex[j]], ce.off - p.expert_origin, k0, n, ((n * ES) & ~15u) / ES);
-    };
-    if constexpr (OPC == OP_DARE) {
-      // acc = fma(alpha_i, v_i, acc) over the selected experts whose keep word passes, in
-      // ascending order, with v_i = delta_i * sigma (a dropped entry is omitted)
-      float acc[VPT][V];
-#pragma unroll
-      for (int u = 0; u < VPT; ++u)
-#pragma unroll
-        for (int v = 0; v < V; ++v) acc[u][v] = 0.0f;
 #pragma unroll 1
-      for (uint32_t j = 0; j < nsel; ++j) {
-        s = s + 1 == (uint32_t)NS ? 0u : s + 1;
-        const uint32_t i = ce.ex[j];
-#pragma unroll
-        for (int u = 0; u < VPT; ++u) {
-          const uint4 pe = S.pe[dv[u].g_hi][i];
-          const float a = __uint_as_float(pe.w);
-          const uint4 r = raw(s, j, u);
-          uint32_t kw[V];
-          dare_keep_words<BF16>(p, dv[u], pe, kw);
-          auto fold_pair = [&](int v, float d0, float d1) {
-            float s0, s1;
-            f2_mul(d0, d1, p.sigma, p.sigma, s0, s1);
-            // a dropped entry is omitted from the sum, as an unselected one is
-            if (kw[v] >= p.dare_T16) acc[u][v] = __fmaf_rn(a, s0, acc[u][v]);
-            if (kw[v + 1] >= p.dare_T16) acc[u][v + 1] = __fmaf_rn(a, s1, acc[u][v + 1]);
-          };
-          delta_pairs<BF16>(r, x0[u], fold_pair);
-        }
-      }
-      const uint64_t off = ce.off;
-      const uint32_t n = ce.n;
-      mbar_arrive(&S.empty[e]);  // every read of the chunk's slots and entry is done
-#pragma unroll
-      for (int u = 0; u < VPT; ++u)
-#pragma unroll
-        for (int v = 0; v < V; v += 2)
-          f2_add(x0[u][v], x0[u][v + 1], acc[u][v], acc[u][v + 1], y[u][v], y[u][v + 1]);
-      store(off, n);
-      continue;
-    }
-    // Per element: P and N, the sums of the kept positive and negative deltas, and both
-    // counts in one float C = 2^23 + c+ + 2^CB c- (exact: every value is an integer below
-    // 2^24, so the low bits of C hold c+ and c-).  DARE-TIES keeps, instead, every nonzero
-    // rescaled delta s = d sigma whose keep word passes (no magnitude trim).  A delta d is
-    // kept positive when d >= thr and kept negative when d <= -thr (thr > 0: |d| >= thr and
-    // the sign in one compare each); the keep factors k+ and k- are 1 or 0, and
-    // P = fma(k+, d, P), N = fma(k-, d, N): a factor 1 adds d with the one rounding of P + d,
-    // a factor 0 adds a zero, which leaves P and N unchanged (they start at +0 and are never
-    // -0).  Two elements per packed instruction.
-    float Pp[VPT][V], Nn[VPT][V], Cc[VPT][V];
-#pragma unroll
-    for (int u = 0; u < VPT; ++u)
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        Pp[u][v] = 0.0f;
-        Nn[u][v] = 0.0f;
-        Cc[u][v] = 8388608.0f;  // 2^23
-      }
-    // the selected experts in ascending order: fill j of the chunk sits in slot s0 + 1 + j
-#pragma unroll 1
-    for (uint32_t j = 0; j < nsel; ++j) {
-      s = s + 1 == (uint32_t)NS ? 0u : s + 1;
+    for (uint32_t j = 0; j < nexp; ++j) {
       const float thr = OPC == OP_TIES ? ce.thr[j] : 0.0f;
 #pragma unroll
       for (int u = 0; u < VPT; ++u) {
+        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
+        uint4 r;
+        if (in_slot) {
+          r = *reinterpret_cast<const uint4*>(S.slot[s] + k0 * ES);
+        } else {  // the ragged tail of a tensor, from global memory
+          const uint32_t n = ce.n;
+          r = read_raw<BF16>(S.slot[s], p.experts.p[ce.ex[j]], ce.off - p.expert_origin, k0, n, ((n * ES) & ~15u) / ES);
+        }
         uint32_t kw[V];
-        if constexpr (OPC == OP_DTIES) dare_keep_words<BF16>(p, dv[u], S.pe[dv[u].g_hi][ce.ex[j]], kw);
-        const uint4 r = raw(s, j, u);
+        float a = 0.0f;
+        if constexpr (OPC != OP_TIES) {
+          const uint4 pe = ce.pe[j];
+          a = __uint_as_float(pe.w);
+          dare_keep_words<BF16>(p, dv[u], pe, kw);
+        }
         // one element pair at a time, so that only the raw vector stays live
-        auto tally_pair = [&](int v, float d0, float d1) {
+        auto fold_pair = [&](int v, float d0, float d1) {
+          if constexpr (OPC != OP_TIES) f2_mul(d0, d1, p.sigma, p.sigma, d0, d1);
+          if constexpr (OPC == OP_DARE) {
+            // a dropped entry is omitted from the sum, as an unselected one is
+            if (kw[v] >= p.dare_T16) acc[u][v] = __fmaf_rn(a, d0, acc[u][v]);
+            if (kw[v + 1] >= p.dare_T16) acc[u][v + 1] = __fmaf_rn(a, d1, acc[u][v + 1]);
+            return;
+          }
           float t0, t1, kp0, kp1, kn0, kn1;
           if constexpr (OPC == OP_DTIES) {
-            f2_mul(d0, d1, p.sigma, p.sigma, d0, d1);
             // keep factors as 1.0 / 0.0 straight from compares joined with the keep test
             asm("{\n .reg .pred q;\n setp.ge.u32 q, %4, %5;\n set.gt.and.f32.f32 %0, %6, 0f00000000, q;\n"
                 " set.lt.and.f32.f32 %1, %6, 0f00000000, q;\n setp.ge.u32 q, %7, %5;\n"
@@ -1099,15 +927,43 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
           f2_fma(kn0, kn1, (float)(1u << CB), (float)(1u << CB), kp0, kp1, t0, t1);
           f2_add(Cc[u][v], Cc[u][v + 1], t0, t1, Cc[u][v], Cc[u][v + 1]);
         };
-        delta_pairs<BF16>(r, x0[u], tally_pair);
+        delta_pairs<BF16>(r, x0[u], fold_pair);
       }
+      s = s + 1 == (uint32_t)NS ? 0u : s + 1;
     }
+    const uint32_t n = ce.n, flags = begin;
     const uint64_t off = ce.off;
-    const uint32_t n = ce.n, fast = ce.fast;
-    mbar_arrive(&S.empty[e]);  // every read of the chunk's slots and entry is done
+    mbar_arrive(&S.empty[e]);  // every read of the group's slots and entry is done
+    if (!kWhole && !(flags & kLast)) continue;
+    // the chunk's output from f(u, v, y0, y1), elements v and v + 1 of vector u
+    uint32_t w[VPT][4];
+    auto fill_words = [&](auto f) {
+#pragma unroll
+      for (int u = 0; u < VPT; ++u)
+#pragma unroll
+        for (int v = 0; v < V; v += 2) {
+          float y0, y1;
+          f(u, v, y0, y1);
+          put_pair<BF16>(w[u], v, y0, y1);
+        }
+    };
+    auto store = [&]() {
+#pragma unroll
+      for (int u = 0; u < VPT; ++u) {
+        const uint32_t k0 = (tid + (uint32_t)u * kConsumers) * V;
+        if (k0 < n) store_words<BF16>(p.out, off + k0, n - k0, w[u]);
+      }
+    };
+    if constexpr (OPC == OP_DARE) {
+      fill_words([&](int u, int v, float& y0, float& y1) {
+        f2_add(x0[u][v], x0[u][v + 1], acc[u][v], acc[u][v + 1], y0, y1);
+      });
+      store();
+      continue;
+    }
     // the elected side's sum and count: the sign of P + N taken exactly as P > -N or P < -N
     // (then that side holds at least one entry, so c >= 1); otherwise the numerator +0, whose
-    // quotient is +0 whatever count (<= 16, a valid table entry) is paired with it
+    // quotient is +0 whatever count (<= 32, a valid table entry) is paired with it
     auto num_c = [&](int u, int v, float& num, uint32_t& cv) {
       const bool pos = Pp[u][v] > -Nn[u][v], any = Pp[u][v] != -Nn[u][v];
       num = any ? (pos ? Pp[u][v] : Nn[u][v]) : 0.0f;
@@ -1115,77 +971,60 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
       cv = (pos ? cb : cb >> CB) & ((1u << CB) - 1u);
     };
     // q = RN(num * y), then Markstein's correction q + RN(num - q c) * y, and the output
-    // fma(lambda, q, M_0), two elements per instruction; `checked` also notes the numerators
-    // 0 < |num| < 2^-100, which then take the IEEE division under one warp vote
+    // fma(lambda, q, M_0), two elements per instruction.  Numerators 0 < |num| < 2^-100 need the
+    // IEEE division: where one may occur (`checked`: DARE-TIES, whose rescaled deltas may be tiny,
+    // and TIES chunks with a threshold below 2^-100) the warp looks for them, and then takes its
+    // elements one by one.
+    auto one = [&](int u, int v) {
+      float a;
+      uint32_t cv;
+      num_c(u, v, a, cv);
+      const float2 t = S.ntab[cv];
+      return __fmaf_rn(p.lambda, div_small(a, -t.x, t.y), x0[u][v]);
+    };
     auto finalise = [&](auto checked) {
       // 2 |bits| - 2 wraps the zeros to the top: its minimum over the vector is below
       // 2 * bits(2^-100) - 2 exactly when some numerator has 0 < |num| < 2^-100
+      static_assert(0x0D800000u * 2u - 2u == 0x1AFFFFFEu, "bits of 2^-100");
       uint32_t lowest = 0xFFFFFFFFu;
-#pragma unroll
-      for (int u = 0; u < VPT; ++u)
-#pragma unroll
-        for (int v = 0; v < V; v += 2) {
+      auto look = [&](float a0, float a1) {
+        lowest = min(lowest, min(__float_as_uint(a0) * 2u - 2u, __float_as_uint(a1) * 2u - 2u));
+      };
+      auto by_element = [&]() -> bool {
+        if (!__any_sync(0xFFFFFFFFu, lowest < 0x1AFFFFFEu)) return false;
+        fill_words([&](int u, int v, float& y0, float& y1) {
+          y0 = one(u, v);
+          y1 = one(u, v + 1);
+        });
+        return true;
+      };
+      auto fast = [&](int u, int v, float& y0, float& y1) {
         float a0, a1, q0, q1, r0, r1;
         uint32_t c0, c1;
         num_c(u, v, a0, c0);
         num_c(u, v + 1, a1, c1);
-        if constexpr (decltype(checked)::value)
-          lowest = min(lowest, min(__float_as_uint(a0) * 2u - 2u, __float_as_uint(a1) * 2u - 2u));
+        if constexpr (decltype(checked)::value && kWhole) look(a0, a1);
         const float2 t0 = S.ntab[c0], t1 = S.ntab[c1];
         f2_mul(a0, a1, t0.y, t1.y, q0, q1);
         f2_fma(q0, q1, t0.x, t1.x, a0, a1, r0, r1);
         f2_fma(r0, r1, t0.y, t1.y, q0, q1, q0, q1);
-        f2_fma(p.lambda, p.lambda, q0, q1, x0[u][v], x0[u][v + 1], y[u][v], y[u][v + 1]);
-      }
-      static_assert(0x0D800000u * 2u - 2u == 0x1AFFFFFEu, "bits of 2^-100");
-      const bool exact = decltype(checked)::value && lowest < 0x1AFFFFFEu;
-      if (decltype(checked)::value && __any_sync(0xFFFFFFFFu, exact)) {
+        f2_fma(p.lambda, p.lambda, q0, q1, x0[u][v], x0[u][v + 1], y0, y1);
+      };
+      // a class that keeps its state over groups has no registers for the words beside it: it
+      // looks first, at both sums (one of them is the numerator)
+      if constexpr (decltype(checked)::value && !kWhole) {
 #pragma unroll
         for (int u = 0; u < VPT; ++u)
 #pragma unroll
-          for (int v = 0; v < V; ++v) {
-          float a;
-          uint32_t cv;
-          num_c(u, v, a, cv);
-          if (div_small_needs_ieee(a)) y[u][v] = __fmaf_rn(p.lambda, __fdiv_rn(a, -S.ntab[cv].x), x0[u][v]);
-        }
+          for (int v = 0; v < V; ++v) look(Pp[u][v], Nn[u][v]);
+        if (by_element()) return;
       }
+      fill_words(fast);
+      if constexpr (decltype(checked)::value && kWhole) by_element();
     };
-    if constexpr (OPC == OP_DTIES) {
-      finalise(std::true_type{});  // rescaled deltas may be tiny: always checked
-    } else if (fast) {             // uniform over the CTA: every nonzero numerator >= 2^-100
-      finalise(std::false_type{});
-    } else {
-      // TIES chunks with a threshold below 2^-100 (rare): one element at a time
-      bool exact = false;
-#pragma unroll
-      for (int u = 0; u < VPT; ++u)
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-        float a;
-        uint32_t cv;
-        num_c(u, v, a, cv);
-        const float2 t = S.ntab[cv];
-        y[u][v] = div_small_fast(a, -t.x, t.y);
-        exact = exact || div_small_needs_ieee(a);
-      }
-      if (__any_sync(0xFFFFFFFFu, exact)) {
-#pragma unroll
-        for (int u = 0; u < VPT; ++u)
-#pragma unroll
-          for (int v = 0; v < V; ++v) {
-          float a;
-          uint32_t cv;
-          num_c(u, v, a, cv);
-          if (div_small_needs_ieee(a)) y[u][v] = __fdiv_rn(a, -S.ntab[cv].x);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < VPT; ++u)
-#pragma unroll
-        for (int v = 0; v < V; ++v) y[u][v] = __fmaf_rn(p.lambda, y[u][v], x0[u][v]);
-    }
-    store(off, n);
+    if (OPC == OP_TIES && (flags & kFast)) finalise(std::false_type{});  // uniform over the CTA
+    else finalise(std::true_type{});
+    store();
   }
   merge_end<kConsumers + 32>(p, &S.last);
 }
@@ -1202,7 +1041,7 @@ cudaError_t launch_chunk(const MergeLaunch& p, cudaStream_t st) {
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  using Smem = TcSmem<Geo::kSlots, Geo::kSlotBytes, Geo::kGrab, KC, OPC == OP_TIES>;
+  using Smem = TcSmem<Geo::kSlots, Geo::kSlotBytes, Geo::kGrab, KC, Geo::kGroup, OPC == OP_TIES>;
   // every CTA also holds 1 KB of the SM's 228 KB for the system
   static_assert(Geo::kCtasPerSm * (sizeof(Smem) + 1024) <= 228u * 1024u,
                 "the CTAs per SM that the grid assumes fit one SM's shared memory");
@@ -1218,8 +1057,15 @@ cudaError_t launch_chunk(const MergeLaunch& p, cudaStream_t st) {
 }
 
 template <bool BF16, int OPC>
+cudaError_t launch_groups(const MergeLaunch& p, cudaStream_t st) {
+  if (p.K <= 4) return launch_chunk<BF16, OPC, 4>(p, st);
+  if (p.K <= 8) return launch_chunk<BF16, OPC, 8>(p, st);
+  return launch_chunk<BF16, OPC, kMaxK>(p, st);
+}
+
+template <bool BF16, int OPC>
 cudaError_t launch_op(const MergeLaunch& p, cudaStream_t st) {
-  const uint32_t chunk = Geo<OPC>::kSlotBytes / (BF16 ? 2u : 4u);
+  const uint32_t chunk = Geo::kSlotBytes / (BF16 ? 2u : 4u);
   const uint32_t cpb = (p.block_elems + chunk - 1) / chunk;
   const uint64_t n_chunks = (p.b_end - p.b_begin) * cpb;
   if (n_chunks == 0) return cudaSuccess;
@@ -1228,13 +1074,13 @@ cudaError_t launch_op(const MergeLaunch& p, cudaStream_t st) {
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const size_t smem = sizeof(Smem<Geo<OPC>::kSlots, Geo<OPC>::kSlotBytes, Geo<OPC>::kGrab>);
+  const size_t smem = sizeof(Smem<Geo::kSlots, Geo::kSlotBytes, Geo::kGrab>);
   if ((e = cudaFuncSetAttribute(merge_tma_kernel<BF16, OPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
       cudaSuccess)
     return e;
-  uint64_t grid = (uint64_t)sms * Geo<OPC>::kCtasPerSm;
+  uint64_t grid = (uint64_t)sms * Geo::kCtasPerSm;
   if (grid > n_chunks) grid = n_chunks;
-  merge_tma_kernel<BF16, OPC><<<(unsigned)grid, Geo<OPC>::kThreads, smem, st>>>(p, cpb, n_chunks, p.work);
+  merge_tma_kernel<BF16, OPC><<<(unsigned)grid, Geo::kThreads, smem, st>>>(p, cpb, n_chunks, p.work);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1244,23 +1090,10 @@ cudaError_t launch_dtype(const MergeLaunch& p, cudaStream_t st) {
   switch (p.op_kind) {
     case MP_OP_AVG:
     case MP_OP_TA: return launch_op<BF16, OP_ADD>(p, st);
-    case MP_OP_TIES:
-      if (p.K <= 4) return launch_chunk<BF16, OP_TIES, 4>(p, st);
-      if (p.K <= 8) return launch_chunk<BF16, OP_TIES, 8>(p, st);
-      return launch_op<BF16, OP_TIES>(p, st);
-    case MP_OP_DARE:
-      if (p.ext.span > kDareSpan) return launch_op<BF16, OP_DARE>(p, st);
-      if (p.K <= 4) return launch_chunk<BF16, OP_DARE, 4>(p, st);
-      if (p.K <= 8) return launch_chunk<BF16, OP_DARE, 8>(p, st);
-      if (p.K <= 16) return launch_chunk<BF16, OP_DARE, 16>(p, st);
-      return launch_op<BF16, OP_DARE>(p, st);
+    case MP_OP_TIES: return launch_groups<BF16, OP_TIES>(p, st);
+    case MP_OP_DARE: return launch_groups<BF16, OP_DARE>(p, st);
     case MP_OP_AVG_RENORM: return launch_op<BF16, OP_RENORM>(p, st);
-    case MP_OP_DARE_TIES:
-      if (p.ext.span > kDareSpan) return launch_op<BF16, OP_DTIES>(p, st);
-      if (p.K <= 4) return launch_chunk<BF16, OP_DTIES, 4>(p, st);
-      if (p.K <= 8) return launch_chunk<BF16, OP_DTIES, 8>(p, st);
-      if (p.K <= 16) return launch_chunk<BF16, OP_DTIES, 16>(p, st);
-      return launch_op<BF16, OP_DTIES>(p, st);
+    case MP_OP_DARE_TIES: return launch_groups<BF16, OP_DTIES>(p, st);
     default: return cudaErrorInvalidValue;
   }
 }

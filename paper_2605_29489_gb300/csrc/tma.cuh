@@ -10,8 +10,8 @@ namespace mp {
 // A sleeping wait suspends the thread for up to kSuspendHintNs per try_wait round (it resumes
 // as soon as the phase completes), so waiting warps do not spin on the issue slots that working
 // warps need; a polling wait returns after each round.  Which one a kernel uses is a measured
-// choice (the merge kernel sleeps, the catalog kernel polls).  kWaitLimit rounds bound every
-// wait to a few seconds.
+// choice (the AVG/TA merge sleeps; the catalog and the other merges poll).  kWaitLimit rounds
+// bound every wait to a few seconds.
 constexpr uint32_t kSuspendHintNs = 2000;
 constexpr uint32_t kWaitLimit = 1u << 21;  // try_wait rounds before a wait gives up
 
