@@ -622,10 +622,9 @@ cudaError_t merge_host_pool(MergeLaunch p, const mp_index_s* ix, cudaStream_t cs
 // the statistics, the error word and work_bytes of scratch for the caller (*work).  What
 // uploads the table and clears the error word and tau is left in init, which the caller
 // launches on cs with what it adds of its own.
-mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, size_t work_bytes, cudaStream_t cs,
-                    InitList& init, mp_index_s** out, char** work) {
+mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, uint32_t unit_bins, size_t work_bytes,
+                    cudaStream_t cs, InitList& init, mp_index_s** out, char** work) {
   const bool ties = op && (op->kind == MP_OP_TIES || op->kind == MP_OP_TIES_MASKED);
-  const bool masked = op && op->kind == MP_OP_TIES_MASKED;
   const uint32_t scope = ties ? op->trim_scope : 0u;
   const uint32_t n_groups = scope == 0 ? g.n_tensors : 1u;
   const uint64_t nb = g.n_blocks, U = nb * g.K, KG = (uint64_t)g.K * n_groups;
@@ -650,7 +649,7 @@ mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, size_t w
   const size_t o_tb0 = slot(((size_t)g.n_tensors + 1) * 4);
   const size_t o_norm = slot(U * 4), o_max = slot(U * 4), o_nnz = slot(U * 4), o_tau = slot(KG * 4);
   const size_t o_err = slot(16);
-  const size_t o_uh = slot(masked ? U * 256 * 4 : 0);
+  const size_t o_uh = slot(U * unit_bins * 4);
   const size_t o_work = slot(work_bytes);
   mp_index_s* ix = new (std::nothrow) mp_index_s();
   if (!ix) return fail(MP_ERR_OOM, "host allocation failed");
@@ -689,7 +688,9 @@ mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, size_t w
   ix->d_nnz = (uint32_t*)(m + o_nnz);
   ix->d_tau = (uint32_t*)(m + o_tau);
   ix->d_err = (uint32_t*)(m + o_err);
-  ix->d_unit_hist = masked ? (uint32_t*)(m + o_uh) : nullptr;
+  ix->d_unit_hist = unit_bins ? (uint32_t*)(m + o_uh) : nullptr;
+  ix->d_win = nullptr;
+  ix->d_kth = nullptr;
   cudaError_t e = cudaSuccess;
   {
     // the five table arrays are consecutive in the allocation: one staged upload
@@ -815,11 +816,16 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   const size_t o_work = slot(n_work * 8);
   size_t o_coarse = 0, o_fine = 0, o_kth = 0, o_est = 0, o_rank = 0;
   size_t o_wfine = 0, o_wabove = 0, o_win = 0, o_gmiss = 0, o_miss = 0, o_wend = 0;
-  // device-resident TIES (not after masking) takes its thresholds from predicted windows
+  // TIES takes its thresholds from predicted windows, TIES after masking where the units' larger
+  // histograms (2.5 KiB) are small against what they count
   const bool windowed = ties && op->kind == MP_OP_TIES;
+  const bool masked = ties && !windowed;
+  const bool units = masked && family->experts_location == 0 && g.n_params >= g.n_blocks * kUnitHistElems;
+  size_t o_usum = 0;
   if (ties) {
-    o_coarse = slot(KG * 256 * 8);
+    o_coarse = slot(units ? 0 : KG * 256 * 8);
     o_fine = slot(KG * 128 * 8);
+    o_usum = slot(units ? KG * kUnitHistBins * 8 : 0);
     o_kth = slot(n_groups * 8);
     o_est = slot(KG * 4);
     o_rank = slot(KG * 8);
@@ -831,7 +837,7 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   uint64_t span_blocks = 64;
   while (span_blocks > 8 && g.n_blocks < span_blocks * 304) span_blocks /= 2;
   size_t o_shist = 0, o_scnt = 0, o_spans = 0;
-  if (windowed) {
+  if (windowed || units) {
     for (uint32_t q = 0; q < n_groups; ++q) {
       const uint64_t b0 = scope == 0 ? g.t_first_block[q] : 0;
       const uint64_t b1 = scope == 0 ? (q + 1 < g.n_tensors ? g.t_first_block[q + 1] : g.n_blocks) : g.n_blocks;
@@ -841,8 +847,8 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
       }
     }
     // zeroed together: window counts, keys above, marks, the flag, sampled bins and counts
-    o_wfine = slot(KG * 384 * 8);
-    o_wabove = slot(KG * 8);
+    o_wfine = slot(units ? 0 : KG * 384 * 8);
+    o_wabove = slot(units ? 0 : KG * 8);
     o_gmiss = slot(KG * 4);
     o_miss = slot(16);
     o_shist = slot(KG * 1024 * 4);
@@ -854,7 +860,9 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   mp_index_s* ix = nullptr;
   char* m = nullptr;
   InitList init;
-  if ((st = new_index(g, op, family->experts_location != 0, o, cs, init, &ix, &m)) != MP_OK) return st;
+  if ((st = new_index(g, op, family->experts_location != 0, units ? kUnitHistBins : (masked ? 256u : 0u), o, cs, init,
+                      &ix, &m)) != MP_OK)
+    return st;
 
   cudaError_t e;
   auto bail = [&](cudaError_t err, const char* what) {
@@ -881,17 +889,18 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   p.wait_limit = g_stall_rounds.load(std::memory_order_relaxed);
   p.stall = p.wait_limit ? 1u : 0u;
   if (ties) {
-    p.coarse = (unsigned long long*)(m + o_coarse);
+    if (!units) p.coarse = (unsigned long long*)(m + o_coarse);
+    else p.usum = (unsigned long long*)(m + o_usum);
     p.fine = (unsigned long long*)(m + o_fine);
-    p.kth = (const unsigned long long*)(m + o_kth);
+    p.kth = ix->d_kth = (const unsigned long long*)(m + o_kth);
     p.estar = (uint32_t*)(m + o_est);
     p.rank = (unsigned long long*)(m + o_rank);
     p.tau = ix->d_tau;
     p.unit_hist = ix->d_unit_hist;
-    init.add(p.coarse, nullptr, o_kth - o_coarse);  // coarse and fine bins
+    init.add(m + o_coarse, nullptr, o_kth - o_coarse);  // coarse and fine bins, sums of the units' bins
     if ((e = upload(ix, init, (void*)p.kth, h_kth.data(), n_groups * 8, cs)) != cudaSuccess) return bail(e, "k copy");
   }
-  if (windowed) {
+  if (windowed || units) {
     p.density = op->density;
     p.grp_blk0 = ix->d_t_blk0;
     p.wfine = (unsigned long long*)(m + o_wfine);
@@ -899,6 +908,7 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
     p.gmiss = (uint32_t*)(m + o_gmiss);
     p.miss = (uint32_t*)(m + o_miss);
     p.win = (uint32_t*)(m + o_win);
+    if (units) ix->d_win = p.win;
     p.shist = (uint32_t*)(m + o_shist);
     p.scnt = (unsigned long long*)(m + o_scnt);
     p.samp_span = (const uint2*)(m + o_spans);
@@ -970,7 +980,7 @@ mp_status mp_index_import(const mp_family* family, const mp_op* op, const float*
   mp_index_s* ix = nullptr;
   char* m = nullptr;
   InitList init;
-  if ((st = new_index(g, op, family->experts_location != 0, 0, cs, init, &ix, &m)) != MP_OK) return st;
+  if ((st = new_index(g, op, family->experts_location != 0, 0, 0, cs, init, &ix, &m)) != MP_OK) return st;
   ix->has_missing = missing;
   cudaError_t e;
   auto bail = [&](cudaError_t err, const char* what) {
@@ -1223,12 +1233,14 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   const uint64_t KG = (uint64_t)g.K * plan->n_groups;
   size_t mo = 0;
   auto mslot = [&](size_t bytes) { size_t r = mo; mo += align_up(bytes); return r; };
-  const size_t m_coarse = mslot(KG * 256 * 8), m_fine = mslot(KG * 128 * 8), m_kth = mslot(plan->n_groups * 8);
+  const bool units = masked && index->d_win;  // the threshold from the sums of the units' windows
+  const size_t m_hist = mslot(KG * (units ? kUnitHistBins : 256) * 8), m_fine = mslot(KG * 128 * 8);
+  const size_t m_gmiss = mslot(KG * 4), m_miss = mslot(16), m_work = mslot(4 * 8), m_zero = mo;
   const size_t m_est = mslot(KG * 4), m_rank = mslot(KG * 8), m_tau = mslot(KG * 4);
   // the merge kernel's work counter (one per segment of a host pool) and its count of finished CTAs
   const size_t n_work = family->experts_location == 0 ? 1 : 2 * (size_t)(g.n_params / kSegmentElems) + 2;
-  const size_t zero_bytes = back_bytes + (n_work + 1) * 8;
-  const size_t scratch_off = align_up(zero_bytes);
+  const size_t scratch_off = align_up(back_bytes + (n_work + 1) * 8);
+  const size_t zero_bytes = masked ? scratch_off + m_zero : back_bytes + (n_work + 1) * 8;
   if ((st = dev_alloc(mf->mem, scratch_off + (masked ? mo : 0), cs)) != MP_OK) {
     release_pinned();
     delete mf;
@@ -1253,16 +1265,6 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   if (masked) {
     // TIES after masking: the threshold of the zero-completed masked deltas of this plan
     char* sm = static_cast<char*>(mf->mem.ptr) + scratch_off;
-    std::vector<unsigned long long> kth(plan->n_groups, 0);
-    {
-      std::vector<uint64_t> gnumel(plan->n_groups, 0);
-      for (uint32_t t = 0; t < g.n_tensors; ++t) gnumel[plan->trim_scope == 0 ? t : 0] += g.t_numel[t];
-      for (uint32_t q = 0; q < plan->n_groups; ++q)
-        kth[q] = (unsigned long long)floor((double)plan->density * (double)gnumel[q]);
-    }
-    if ((e = cudaMemsetAsync(sm, 0, m_kth, cs)) != cudaSuccess) return bail(e, "memset");  // coarse + fine
-    if ((e = cudaMemcpyAsync(sm + m_kth, kth.data(), plan->n_groups * 8, cudaMemcpyHostToDevice, cs)) != cudaSuccess)
-      return bail(e, "k copy");
     IndexLaunch q;
     memset(&q, 0, sizeof(q));
     q.dtype = g.dtype;
@@ -1278,9 +1280,17 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
     q.maxabs = index->d_maxabs;
     q.nnz = index->d_nnz;
     q.err = mf->d_err;
-    q.coarse = (unsigned long long*)(sm + m_coarse);
+    if (units) {
+      q.usum = (unsigned long long*)(sm + m_hist);
+      q.win = index->d_win;
+      q.gmiss = (uint32_t*)(sm + m_gmiss);
+      q.miss = (uint32_t*)(sm + m_miss);
+    } else {
+      q.coarse = (unsigned long long*)(sm + m_hist);
+    }
+    q.work = (unsigned long long*)(sm + m_work);
     q.fine = (unsigned long long*)(sm + m_fine);
-    q.kth = (const unsigned long long*)(sm + m_kth);
+    q.kth = index->d_kth;  // a plan has its index's density and trim scope
     q.estar = (uint32_t*)(sm + m_est);
     q.rank = (unsigned long long*)(sm + m_rank);
     q.tau = masked_tau = (uint32_t*)(sm + m_tau);

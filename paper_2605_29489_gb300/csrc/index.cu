@@ -97,12 +97,12 @@ constexpr uint32_t kIxEnd = 0xFFFFFFFFu;
 // 0.85 with 8 KiB ones).  The TIES catalog also bins every delta, which makes it bound by
 // instruction latency: four CTAs per SM (more warps to hide it; the state fits 56 registers) with
 // twelve 4 KiB slots (one vector per consumer thread and fill), and at most 4 experts per item.
-template <bool TIES, int KG = 1>
+template <bool TIES, int KG = 1, bool UNITS = false>
 struct IxGeo {
   static_assert(!TIES || KG <= 4, "the TIES catalog takes at most 4 experts per item");
   static constexpr int kCtasPerSm = TIES ? 4 : 3;
   static constexpr uint32_t kSlotBytes = TIES || KG > 4 ? 4096u : 8192u;
-  static constexpr int kSlots = TIES ? 12 : (KG > 4 ? 18 : 9);
+  static constexpr int kSlots = TIES ? (UNITS ? 11 : 12) : (KG > 4 ? 18 : 9);  // UNITS: kBinUnits' larger histograms
   // whole chunks: the base fill and the item's expert fills of one chunk sit in consecutive
   // ring slots under one "full" and one "empty" mbarrier
   static constexpr bool kWhole = TIES || KG > 4;
@@ -123,8 +123,11 @@ struct IxMeta {
 //    counts the lower 7 bits inside the chosen bin);
 //  * kBinWindow: the W keys [L, L + W) of a window predicted from a sample, one bin each, and
 //    one bin below and one above it, so that the threshold is found without a second pass
-//    whenever it lies inside the window.
-enum { kBinNone = 0, kBinCoarse = 1, kBinWindow = 2 };
+//    whenever it lies inside the window;
+//  * kBinUnits (TIES after masking): both at once, and kept for each (expert, block), because a
+//    plan's threshold is that of the blocks it selects: the keys of a window one bin each, the
+//    others by their upper 8 bits.
+enum { kBinNone = 0, kBinCoarse = 1, kBinWindow = 2, kBinUnits = 3 };
 constexpr uint32_t kWinKeys = 384;           // most keys of a window (three binades)
 constexpr uint32_t kWinBins = kWinKeys + 2;  // + below + above
 
@@ -143,6 +146,21 @@ constexpr uint32_t kWinNarrow = 160, kWinNarrowBlocks = 16;
 __device__ __forceinline__ void win_words(uint32_t win, uint32_t& neg, uint32_t& top) {
   neg = ((1u - (win & 0xFFFFu)) & 0xFFFFu) * 0x00010001u;
   top = ((win >> 16) + 1u) * 0x00010001u;
+}
+
+// The bins of kBinUnits: key k adds to bin clamp(k - L, 0, W) + (k >> 7), which is one bin per key
+// inside [L, L + W) (W = 384, L a multiple of 128) and one per binade outside, in the order of the
+// keys.  Bin 0 of what is stored is the count of nonzero deltas: the zeros of a trim group are
+// what its other bins leave, also for the elements that a plan omits.  Three instructions more per
+// pair of keys than the window alone; without it the catalog read the experts twice (coarse, then
+// fine bins) and each plan's threshold read the selected ones a third time: two Llama layers with
+// 4 experts, catalog 1.71 -> 0.81 ms, merge with its thresholds 1.54 -> 0.59 ms (floors 0.65, 0.52).
+constexpr uint32_t kUnitBins = kUnitHistBins;
+static_assert(kUnitBins == 256 + kWinKeys, "bins of kBinUnits");
+
+template <int BM>
+constexpr uint32_t key_bins() {
+  return BM == kBinNone ? 1u : (BM == kBinWindow ? kWinBins : (BM == kBinUnits ? kUnitBins : 256u));
 }
 
 template <int KG, int NS, uint32_t SB, uint32_t NB>
@@ -264,6 +282,27 @@ __device__ __forceinline__ uint32_t ties_win2(float d0, float d1, uint32_t neg, 
   return w;
 }
 
+// kBinUnits bins of two deltas, both keys in 16-bit lanes as in ties_win2; neg = -L in both lanes
+__device__ __forceinline__ uint32_t ties_units2(float d0, float d1, uint32_t neg, uint32_t h2) {
+  const __nv_bfloat162 hb = __floats2bfloat162_rn(d0, d1);
+  const uint32_t w = *reinterpret_cast<const uint32_t*>(&hb) & 0x7FFF7FFFu;
+  uint32_t t;
+  asm("{\n .reg .b32 t;\n add.s16x2 t, %1, %2;\n min.s16x2.relu %0, t, %3;\n}"
+      : "=r"(t)
+      : "r"(w), "r"(neg), "r"(kWinKeys * 0x00010001u));
+  const uint32_t a2 = t * 4u + (((w >> 5) & 0x03FC03FCu) + h2);
+  asm volatile(
+      "{\n"
+      " .reg .b32 a0, a1;\n"
+      " and.b32 a0, %0, 65535;\n"
+      " shr.u32 a1, %0, 16;\n"
+      " red.shared.add.u32 [a0], 1;\n"
+      " red.shared.add.u32 [a1], 1;\n"
+      "}\n" ::"r"(a2)
+      : "memory");
+  return w;
+}
+
 // number of nonzero keys among the four key words of a vector, in two 16-bit lanes
 __device__ __forceinline__ uint32_t nz_halves(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
   uint32_t m0, m1, m2, m3;
@@ -321,13 +360,14 @@ __device__ __forceinline__ bool checked_item(const IndexLaunch& p, uint64_t b, u
   return false;
 }
 
-// The k-th largest of the keys counted in h[0 .. 32 N), by one warp: lane l sums the N bins
+// The k-th largest of the keys counted in h[0 .. 32 N) (SKIP0: h[0] apart), by one warp: lane l sums the N bins
 // that rank l-th from the top, a warp scan finds the lane where the running count reaches k,
 // and that lane walks its own bins.  True (on every lane) when h holds at least k keys; then
-// bin is the bin of the k-th largest and before the number of keys above it.  One thread
+// bin is the bin of the k-th largest and before the number of keys above it; false: before is
+// the number of keys.  One thread
 // walking the bins waits for a load per bin: 256 to 384 of them took 30-46 us whatever the
 // number of pairs, this takes two.
-template <int N>
+template <int N, bool SKIP0 = false>
 __device__ __forceinline__ bool warp_kth(const unsigned long long* h, unsigned long long k, uint32_t& bin,
                                          unsigned long long& before) {
   const uint32_t lane = threadIdx.x & 31u;
@@ -335,7 +375,7 @@ __device__ __forceinline__ bool warp_kth(const unsigned long long* h, unsigned l
   unsigned long long c[N], sum = 0;
 #pragma unroll
   for (int j = 0; j < N; ++j) {
-    c[j] = h[top - j];
+    c[j] = SKIP0 && top == (uint32_t)j ? 0ull : h[top - j];
     sum += c[j];
   }
   unsigned long long cum = sum;
@@ -345,7 +385,10 @@ __device__ __forceinline__ bool warp_kth(const unsigned long long* h, unsigned l
     if (lane >= (uint32_t)s) cum += o;
   }
   const uint32_t hit = __ballot_sync(0xFFFFFFFFu, cum >= k);
-  if (hit == 0u) return false;
+  if (hit == 0u) {
+    before = __shfl_sync(0xFFFFFFFFu, cum, 31);
+    return false;
+  }
   const int src = __ffs(hit) - 1;
   unsigned long long run = cum - sum;
   uint32_t e = top;
@@ -418,22 +461,23 @@ __device__ __forceinline__ void coarse_pass_end(const IndexLaunch& p, volatile i
 }
 
 template <bool BF16, int KG, int BM>
-__global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPerSm)
+__global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG, BM == kBinUnits>::kCtasPerSm)
     index_tma_kernel(const IndexLaunch p, uint32_t G, uint64_t n_items, unsigned long long* work) {
   constexpr bool TIES = BM != kBinNone;
-  constexpr uint32_t NB = BM == kBinNone ? 1u : (BM == kBinWindow ? kWinBins : 256u);  // key bins per expert
+  constexpr uint32_t NB = key_bins<BM>();  // key bins per expert
+  using Geo = IxGeo<TIES, KG, BM == kBinUnits>;
   // Whole chunks (IxGeo): one "full" mbarrier counts all the bytes of a chunk's fills and one
   // "empty" mbarrier its releases, so that a consumer waits and releases once per chunk instead
   // of once per fill.
-  constexpr bool CW = IxGeo<TIES, KG>::kWhole;
+  constexpr bool CW = Geo::kWhole;
   // window bins: the nonzero deltas are counted apart (the bins leave out those below the
   // window); for bf16 from the keys (nz_halves), where key 0 holds exactly the zero deltas (the
   // difference of two distinct bf16 values is at least the smallest bf16 subnormal, whose key
   // is 1)
-  constexpr bool KNZ = BM == kBinWindow;
-  constexpr int kIxSlots = IxGeo<TIES, KG>::kSlots;
+  constexpr bool KNZ = BM == kBinWindow || BM == kBinUnits;
+  constexpr int kIxSlots = Geo::kSlots;
   static_assert(!CW || kIxSlots >= 2 * (KG + 1), "two whole chunks fit the ring");
-  constexpr uint32_t kIxSlotBytes = IxGeo<TIES, KG>::kSlotBytes;
+  constexpr uint32_t kIxSlotBytes = Geo::kSlotBytes;
   constexpr uint32_t ES = BF16 ? 2u : 4u;
   constexpr uint32_t CH = kIxSlotBytes / ES;
   constexpr int V = BF16 ? 8 : 4;
@@ -445,8 +489,8 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
   // the fallback pass of the windowed catalog runs only when some threshold left its window
   if (BM == kBinCoarse && p.miss && *p.miss == 0u) return;
-  if constexpr (KNZ) {  // the packed bin addresses need the histogram below 2^16 - 4 * 385
-    if (su32(&S.hist[KG - 1][NB - 1]) >= 65536u - 4u * (kWinKeys + 1u)) {
+  if constexpr (KNZ) {  // the packed bin addresses need the histograms below 2^16 - 4 NB
+    if (su32(&S.hist[KG - 1][NB - 1]) >= 65536u - 4u * NB) {
       if (threadIdx.x == 0) atomicOr(p.err, kErrInternal);
       return;
     }
@@ -497,7 +541,7 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
         S.meta[e].n = n;
         S.meta[e].last = last;
         S.meta[e].s0 = fill % kIxSlots;
-        if constexpr (BM == kBinWindow) {
+        if constexpr (KNZ) {
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             S.meta[e].wneg[k] = item_neg[k];
@@ -557,11 +601,14 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
         const uint32_t len = p.blk_len[b];
         const uint64_t off0 = p.blk_off[b];
         const uint32_t nch = (len + CH - 1) / CH;
-        if constexpr (CW && BM == kBinWindow) {
+        if constexpr (CW && KNZ) {
           const uint32_t grp = p.blk_group[b];
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            if ((uint32_t)k < kc) win_words(p.win[(uint64_t)(i0 + k) * p.n_groups + grp], item_neg[k], item_top[k]);
+            if ((uint32_t)k < kc) {
+              win_words(p.win[(uint64_t)(i0 + k) * p.n_groups + grp], item_neg[k], item_top[k]);
+              if constexpr (BM == kBinUnits) item_neg[k] -= 0x00010001u;  // -L: no bin apart below the window
+            }
         }
         for (uint32_t c = 0; c < nch && ok; ++c) {
           const uint32_t n = min(CH, len - c * CH);
@@ -673,9 +720,9 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
       // a warp whose vectors all match skips them (warp-uniform, so the summation order is
       // untouched)
       if (!__all_sync(0xFFFFFFFFu, same)) {
-        // kBinWindow: this expert's window in the block's trim group
+        // kBinWindow, kBinUnits: this expert's window in the block's trim group
         uint32_t wneg = 0, wtop = 0;
-        if constexpr (BM == kBinWindow) {
+        if constexpr (KNZ) {
           wneg = mt.wneg[k < 4 ? k : 0];
           wtop = mt.wtop[k < 4 ? k : 0];
         }
@@ -695,11 +742,13 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
 #pragma unroll
             for (int e = 0; e < w; ++e) m[e] = fmaxf(m[e], m[e + w]);
           mx[k] = fmaxf(mx[k], m[0]);
-          if constexpr (BM == kBinWindow) {
+          if constexpr (KNZ) {
             const uint32_t h2 = su32(&S.hist[k][0]) * 0x00010001u;
             uint32_t wk[V / 2];
 #pragma unroll
-            for (int e = 0; e < V; e += 2) wk[e / 2] = ties_win2(d[e], d[e + 1], wneg, wtop, h2);
+            for (int e = 0; e < V; e += 2)
+              wk[e / 2] = BM == kBinUnits ? ties_units2(d[e], d[e + 1], wneg, h2)
+                                          : ties_win2(d[e], d[e + 1], wneg, wtop, h2);
             if constexpr (BF16) nz[k] += nz_halves(wk[0], wk[1], wk[2], wk[3]);
           }
 #pragma unroll
@@ -779,16 +828,20 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
         S.abort = 1;
         break;
       }
-      // thread t holds bin t (and, for the window bins, bin t + 256)
-      uint32_t hc[KG], hd[KG];
+      // thread t holds bin t (and bins t + 256 and t + 512 where there are as many)
+      uint32_t hc[KG], hd[KG], he[KG];
 #pragma unroll
       for (int k = 0; k < KG; ++k) {
         hc[k] = S.hist[k][tid];
         S.hist[k][tid] = 0u;
-        hd[k] = 0u;
-        if (BM == kBinWindow && tid + 256u < NB) {
+        hd[k] = he[k] = 0u;
+        if (KNZ && tid + 256u < NB) {
           hd[k] = S.hist[k][tid + 256u];
           S.hist[k][tid + 256u] = 0u;
+        }
+        if (KNZ && NB > 512u && tid + 512u < NB) {
+          he[k] = S.hist[k][tid + 512u];
+          S.hist[k][tid + 512u] = 0u;
         }
         if constexpr (!KNZ) {
           uint32_t w = hc[k] + hd[k];
@@ -821,6 +874,21 @@ __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG>::kCtasPe
           if (tid == 0) c += len - nzk;  // zero deltas have key 0
           if (p.unit_hist) p.unit_hist[(((uint64_t)(i0 + k) * p.n_blocks + b) << 8) + tid] = (uint32_t)c;
           if (c) atomicAdd(&p.coarse[x * 256u + tid], c);
+        } else if constexpr (BM == kBinUnits) {
+          if (tid == 0) {
+            hc[k] = 0u;
+#pragma unroll
+            for (int w = 0; w < kIxConsumers / 32; ++w) hc[k] += S.red_nz[k][w];
+          }
+          uint32_t* uh = p.unit_hist + ((uint64_t)(i0 + k) * p.n_blocks + b) * kUnitBins;
+          unsigned long long* us = p.usum + x * kUnitBins;
+          auto flush = [&](uint32_t j, uint32_t n) {
+            uh[j] = n;
+            if (n) atomicAdd(&us[j], (unsigned long long)n);
+          };
+          flush(tid, hc[k]);
+          flush(tid + 256u, hd[k]);
+          if (NB > 512u && tid + 512u < NB) flush(tid + 512u, he[k]);
         } else {
           // bins 1..W are the window's keys, bin W + 1 is above it (bin 0, below it, is dropped)
           const uint32_t W = p.win[x] >> 16;
@@ -990,7 +1058,7 @@ __device__ __forceinline__ uint32_t sample_vectors(uint32_t n_b, uint32_t nvec, 
 constexpr uint32_t kSampleBins = 1024;
 
 template <bool BF16, int KG>
-__global__ void __launch_bounds__(256) ties_sample_kernel(const IndexLaunch p) {
+__global__ void __launch_bounds__(256, 4) ties_sample_kernel(const IndexLaunch p) {
   constexpr uint32_t V = BF16 ? 8u : 4u;
   __shared__ uint32_t hist[KG][kSampleBins];
   __shared__ unsigned long long s_n;  // sampled elements
@@ -1102,7 +1170,12 @@ __global__ void __launch_bounds__(kSelThreads) ties_window_select(const IndexLau
   }
   if (lane != 0) return;
   uint32_t L = e >= 4u ? min(e / 4u - 1u, 253u) << 7 : 0u, W = kWinKeys;
-  if (found && n_b >= kWinNarrowBlocks) {
+  if (p.usum) {
+    // kBinUnits: the threshold of a plan is that of all blocks or lower, so most of the window
+    // lies below the predicted bin: it ends 80 to 207 keys above its middle
+    const uint32_t top = (e * 32u + 16u + 80u + 127u) & ~127u;
+    L = min(top > kWinKeys ? top - kWinKeys : 0u, 32768u - kWinKeys);
+  } else if (found && n_b >= kWinNarrowBlocks) {
     L = (uint32_t)min(max((int32_t)(e * 32u + 16u) - (int32_t)kWinNarrow / 2, 0), 32768 - (int32_t)kWinNarrow);
     W = kWinNarrow;
   }
@@ -1137,6 +1210,85 @@ __global__ void __launch_bounds__(kSelThreads) ties_window_finish(const IndexLau
   }
 }
 
+// TIES after masking: the threshold of each (expert, group) from the sums of its units' bins (all
+// units for the catalog, the selected ones for a plan), by one warp, or a mark with the coarse bin
+// and rank for the fine pass when it lies outside the window
+__global__ void __launch_bounds__(kSelThreads) ties_units_finish(const IndexLaunch p) {
+  const uint64_t x = select_pair();
+  if (x >= (uint64_t)p.K * p.n_groups) return;
+  const unsigned long long k = p.kth[x % p.n_groups];
+  const unsigned long long* h = p.usum + x * kUnitBins;
+  const uint32_t L = p.win[x] & 0xFFFFu;
+  uint32_t tau = kTauNone, j = 0;
+  unsigned long long before = 0;
+  bool miss = false;
+  if (k > h[0]) {
+    tau = 0;  // more than there are nonzero deltas
+  } else if (k != 0) {
+    if (!warp_kth<(int)kUnitBins / 32, true>(h, k, j, before)) {
+      // in bin 0, which is key 0 (L = 0) or the keys below 128
+      tau = j = 0;
+      miss = L != 0;
+    } else if (j < L >> 7) {
+      miss = true;  // below the window: bin j is coarse bin j
+    } else if (j > (L >> 7) + kWinKeys + 1u) {
+      miss = true;
+      j -= kWinKeys;
+    } else {  // key t + L at bin t + (L + t) / 128
+      const uint32_t v = j - (L >> 7);
+      tau = L + 128u * (v / 129u) + v % 129u;
+    }
+  }
+  if ((threadIdx.x & 31u) != 0) return;
+  if (miss) {
+    p.estar[x] = j;
+    p.rank[x] = k - before;
+    p.gmiss[x] = 1u;
+    atomicOr(p.miss, 1u);
+  } else {
+    p.tau[x] = tau;
+  }
+}
+
+// the sums of a plan's selected units, for ties_units_finish.  One CTA per (expert, window of
+// kUnitWin blocks); a thread owns four bins and adds them for each group the window touches.
+constexpr uint32_t kUnitWin = 32;
+
+__global__ void __launch_bounds__(kUnitBins / 4) ties_units_sum(const IndexLaunch p, uint32_t n_win) {
+  __shared__ uint32_t s_b[kUnitWin], s_g[kUnitWin], s_n;
+  const uint32_t i = blockIdx.x / n_win, tid = threadIdx.x;
+  const uint64_t b0 = (uint64_t)(blockIdx.x % n_win) * kUnitWin;
+  if (tid < 32u) {  // the selected blocks of the window
+    const uint64_t b = b0 + tid;
+    const bool sel = b < p.n_blocks && ((p.mask[b] >> i) & 1u);
+    const uint32_t v = __ballot_sync(0xFFFFFFFFu, sel), at = __popc(v & ((1u << tid) - 1u));
+    if (sel) {
+      s_b[at] = tid;
+      s_g[at] = p.blk_group[b];
+    }
+    if (tid == 0) s_n = __popc(v);
+  }
+  __syncthreads();
+  const uint32_t n = s_n;
+  const uint4* uh = reinterpret_cast<const uint4*>(p.unit_hist + ((uint64_t)i * p.n_blocks + b0) * kUnitBins) + tid;
+  for (uint32_t a = 0; a < n;) {
+    const uint32_t g = s_g[a];
+    unsigned long long c[4] = {0, 0, 0, 0};
+#pragma unroll 4
+    for (; a < n && s_g[a] == g; ++a) {
+      const uint4 q = uh[(size_t)s_b[a] * (kUnitBins / 4)];
+      c[0] += q.x;
+      c[1] += q.y;
+      c[2] += q.z;
+      c[3] += q.w;
+    }
+    unsigned long long* us = p.usum + ((uint64_t)i * p.n_groups + g) * kUnitBins + tid * 4u;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (c[e]) atomicAdd(us + e, c[e]);
+  }
+}
+
 // the TIES threshold from the coarse bins of the whole family: select the bin, count
 // the lower key bits inside it (a second pass over the blocks that can reach it; experts
 // addressed with origin 0), select the threshold
@@ -1167,13 +1319,12 @@ template <bool BF16, int KG, int BM>
 cudaError_t launch_pass(const IndexLaunch& p, uint32_t G, uint64_t n_items, int sms, unsigned long long* work,
                         cudaStream_t st) {
   constexpr bool ties = BM != kBinNone;
-  constexpr uint32_t NB = BM == kBinNone ? 1u : (BM == kBinWindow ? kWinBins : 256u);
-  const size_t smem = sizeof(IxSmem<KG, IxGeo<ties, KG>::kSlots, IxGeo<ties, KG>::kSlotBytes, NB>);
-  static_assert(IxGeo<ties, KG>::kCtasPerSm *
-                        (sizeof(IxSmem<KG, IxGeo<ties, KG>::kSlots, IxGeo<ties, KG>::kSlotBytes, NB>) + 1024) <=
-                    228u * 1024u,
+  constexpr uint32_t NB = key_bins<BM>();
+  using Geo = IxGeo<ties, KG, BM == kBinUnits>;
+  const size_t smem = sizeof(IxSmem<KG, Geo::kSlots, Geo::kSlotBytes, NB>);
+  static_assert(Geo::kCtasPerSm * (sizeof(IxSmem<KG, Geo::kSlots, Geo::kSlotBytes, NB>) + 1024) <= 228u * 1024u,
                 "the CTAs per SM that the grid assumes fit one SM's shared memory");
-  uint64_t grid = (uint64_t)sms * IxGeo<ties, KG>::kCtasPerSm;
+  uint64_t grid = (uint64_t)sms * Geo::kCtasPerSm;
   if (grid > n_items) grid = n_items;
   cudaError_t e;
   auto k = index_tma_kernel<BF16, KG, BM>;
@@ -1218,12 +1369,19 @@ cudaError_t launch_ties_t(const IndexLaunch& p, cudaStream_t st) {
   ties_window_select<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
   count_launches(2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  IndexLaunch q = p;  // the selects of the fallback ride in its passes
+  q.select_in_pass = 1;
+  if (p.usum) {  // TIES after masking: one pass gives the units' bins and the coarse bins too
+    if ((e = launch_pass<BF16, KG, kBinUnits>(p, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
+    ties_units_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
+    count_launches(1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return ties_finish_t<BF16, KG>(q, st);
+  }
   if ((e = launch_pass<BF16, KG, kBinWindow>(p, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
   ties_window_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
   count_launches(1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  IndexLaunch q = p;  // the selects of the fallback ride in its passes
-  q.select_in_pass = 1;
   if ((e = launch_pass<BF16, KG, kBinCoarse>(q, G, n_items, sms, p.work + 1, st)) != cudaSuccess) return e;
   return ties_finish_t<BF16, KG>(q, st);
 }
@@ -1268,7 +1426,7 @@ cudaError_t by_ties_items(uint32_t K, F f) {
 
 template <bool BF16>
 cudaError_t launch_dtype(const IndexLaunch& p, cudaStream_t st) {
-  if (p.coarse) return by_ties_items(p.K, [&](auto kg) { return launch_ties_t<BF16, decltype(kg)::value>(p, st); });
+  if (p.kth) return by_ties_items(p.K, [&](auto kg) { return launch_ties_t<BF16, decltype(kg)::value>(p, st); });
   if (p.K <= 1) return launch_plain_t<BF16, 1>(p, st);
   if (p.K <= 2) return launch_plain_t<BF16, 2>(p, st);
   if (p.K <= 4) return launch_plain_t<BF16, 4>(p, st);
@@ -1308,6 +1466,17 @@ cudaError_t launch_ties_window_end(const IndexLaunch& p, cudaStream_t st) {
 
 cudaError_t launch_ties_masked(const IndexLaunch& p, cudaStream_t st) {
   if (!p.unit_hist || !p.mask || p.n_blocks == 0) return cudaErrorInvalidValue;
+  if (p.usum) {
+    const uint32_t n_win = (uint32_t)((p.n_blocks + kUnitWin - 1) / kUnitWin);
+    ties_units_sum<<<p.K * n_win, kUnitBins / 4, 0, st>>>(p, n_win);
+    ties_units_finish<<<select_grid((uint64_t)p.K * p.n_groups), kSelThreads, 0, st>>>(p);
+    count_launches(2);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    IndexLaunch q = p;
+    q.select_in_pass = 1;
+    return launch_ties_finish(q, st);
+  }
   const uint32_t n_win = (uint32_t)((p.n_blocks + kMaskWin - 1) / kMaskWin);
   ties_masked_coarse<<<p.K * n_win, 256, 0, st>>>(p, n_win);
   count_launches(1);

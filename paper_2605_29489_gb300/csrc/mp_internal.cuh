@@ -77,7 +77,11 @@ struct mp_index_s {
   uint32_t* d_blk_tensor;  // [n_blocks] tensor of each block
   uint32_t* d_t_blk0;      // [n_tensors + 1] first block of each tensor, then n_blocks
   bool has_missing;        // some entry has nnz == kNnzMissing (imported catalogs only)
-  uint32_t* d_unit_hist;   // [K][n_blocks][256] coarse key histograms (TIES_MASKED only)
+  // TIES_MASKED only: the units' key histograms, [K][n_blocks][256] (coarse bins) or, with a
+  // window, [K][n_blocks][kUnitHistBins]; the windows; k of each trim group
+  uint32_t* d_unit_hist;
+  uint32_t* d_win;                  // null: coarse bins only
+  const unsigned long long* d_kth;  // [n_groups]
   // the traversal order of the first operator planned on this index, kept for later plans
   // with the same operator (written once, then only read; guarded by order_mu on the host)
   mp::Alloc order_mem;
@@ -185,6 +189,16 @@ struct NvtxScope {
 };
 
 // ---- index (index.cu) -------------------------------------------------------------------
+constexpr uint32_t kUnitHistBins = 640;  // bins of a unit's histogram with a window: 384 keys and 256 binades
+
+// Such histograms for blocks of this many elements or more on average: 2.5 KiB per unit instead of
+// 1 KiB, in exchange for a second and a third pass over the experts.  Catalog / merge of two Llama
+// layers with 4 experts 1.71 / 1.54 -> 0.81 / 0.59 ms; 20M elements with 4 experts in blocks of 4096
+// 168 / 220 -> 136 / 73 us.  With 16 experts in blocks of 1000 (where writing the histograms moves
+// more than the experts hold) the merge took 437 instead of 701 us but the catalog 1436 instead of
+// 1224.
+constexpr uint64_t kUnitHistElems = 2048;
+
 struct IndexLaunch {
   mp_dtype dtype;
   uint32_t K;
@@ -209,8 +223,11 @@ struct IndexLaunch {
   // TIES after masking: the catalog keeps each unit's coarse key histogram (256 bins, zero
   // deltas in bin 0); the fine pass then reads only the blocks the plan selected and counts
   // the expert bytes it reads
-  uint32_t* unit_hist;         // [K][n_blocks][256] or null
-  // TIES with a predicted window (device-resident experts, not after masking; null
+  uint32_t* unit_hist;         // [K][n_blocks][256], with usum [K][n_blocks][kUnitHistBins], or null
+  // with a window for each (expert, group) (device-resident experts, large blocks): the sums
+  // of the units' histograms over all blocks (catalog) or the plan's, or null
+  unsigned long long* usum;    // [K][n_groups][kUnitHistBins]
+  // TIES with a predicted window (also after masking, with usum; null
   // otherwise): a sample of each trim group predicts the coarse bin of its threshold, the
   // catalog pass counts the keys of a window around it at full resolution, and the
   // two-level select runs only for the (expert, group) pairs whose threshold left the window
@@ -253,9 +270,10 @@ cudaError_t launch_ties_finish(const IndexLaunch& p, cudaStream_t st);
 cudaError_t launch_ties_window_begin(const IndexLaunch& p, cudaStream_t st);
 cudaError_t launch_index_pass(const IndexLaunch& p, bool window, cudaStream_t st);
 cudaError_t launch_ties_window_end(const IndexLaunch& p, cudaStream_t st);
-// the TIES_MASKED threshold of a plan: coarse bins summed from the per-unit histograms of
-// the selected blocks (zero entries for the others), then the select, fine pass and select
-// of launch_ties_finish restricted to the selected blocks (p.mask)
+// the TIES_MASKED threshold of a plan.  With windows (p.usum): the sums of the selected blocks'
+// histograms, which give it unless it leaves its window.  Without: coarse bins summed from the
+// per-unit histograms of the selected blocks (zero entries for the others), then the select, fine
+// pass and select of launch_ties_finish restricted to the selected blocks (p.mask)
 cudaError_t launch_ties_masked(const IndexLaunch& p, cudaStream_t st);
 
 // ---- plan (plan.cu) ---------------------------------------------------------------------
