@@ -17,7 +17,8 @@
 //     the candidates straight from the unit order, so equal scores stay in ascending unit
 //     order; a later digit that is the same for every key is skipped.  A pass is two barriers:
 //     every warp counts its slice's digits, and after the barrier every CTA adds up the
-//     counts before its own and scatters.
+//     counts before its own and scatters.  (Up to kRankUnits units: each candidate's position
+//     from comparisons with all of them instead, without a barrier.)
 //  D  costs in that order: every position before the first prefix sum > B is selected.
 //  E  after that first overflow only candidates with cost <= the remaining budget R0 can
 //     ever be taken (R only shrinks): every CTA compacts those of its slice while the
@@ -33,7 +34,7 @@
 // take, where the cooperative grid's in global memory takes 3 us) and whose CTAs read each
 // other's digit counts from shared memory; above, a cooperative grid of one 256-thread CTA per
 // SM, because a pass is then bound by the SMs' scattered stores.  Measured, first plan of an
-// index / later plan, us: 2,048 units 45 / 15 in the cluster, 80 / 20 in the grid; 62 K 65 / 22
+// index / later plan, us: 2,048 units 34 / 15 in the cluster (45 / 15 with the radix sort), 80 / 20 in the grid; 62 K 65 / 22
 // and 82 / 23; 384 K 184 / 40 and 114 / 32.  (Before, as 21 phases of the grid alone, with a
 // compaction, a scan phase in every pass and one atomic ballot per taken tail candidate:
 // 119 / 35 at 2,048 units, 116 / 43 at 62 K, 180 / 70 at 384 K, 1124 / 348 at 3.9 M where it now
@@ -48,6 +49,11 @@ constexpr uint32_t kClusterMax = 16;     // CTAs of the cluster launch (non-port
 constexpr int kClusterThreads = 1024;    // threads per CTA of the cluster launch
 constexpr int kGridThreads = 256;        // threads per CTA of the cooperative launch
 constexpr uint64_t kClusterUnits = 1ull << 17;  // most units planned by one cluster
+// Most units that are ordered by comparing each with every other (rank_units) instead of by four
+// passes of the radix sort, whose barriers and round trips take 5 to 6 us each however few the
+// units.  First plan, sort / compare: 400 units 38 / 31 us, 1,000 43 / 29, 2,048 45 / 34, 3,000
+// 44 / 39, 4,000 44 / 51.
+constexpr uint32_t kRankUnits = 3072;
 constexpr uint32_t kBarrierLimit = 1u << 24;
 
 // summary words (plan handle)
@@ -386,6 +392,83 @@ __device__ __forceinline__ uint32_t peer_count(const uint32_t* own, uint32_t g) 
   return v;
 }
 
+// A and C for up to kRankUnits units: every CTA of the cluster scores all of them and compacts the
+// candidates in its shared memory (mem, 32 KiB), and a candidate's position in the order is the
+// number of candidates with a smaller key, or an equal one before it.  The CTAs share the
+// candidates in runs of 32, a run's warps share the keys it is compared with.  Writes the order;
+// Q is the number of candidates.  The caller's barrier follows.
+template <int PT>
+__device__ __forceinline__ void rank_units(const PlanLaunch& p, const Scratch& s, uint32_t U, uint32_t* mem,
+                                           uint32_t& Q) {
+  constexpr uint32_t W = PT / 32, R = kRankUnits / PT;
+  static_assert(kRankUnits % PT == 0 && kRankUnits <= 65536, "runs of R units per thread, 16-bit unit numbers");
+  static_assert(kRankUnits * 6 + PT * 4 <= W * 1024, "keys, units and positions fit the digit counters' memory");
+  uint32_t* s_key = mem;                                             // [kRankUnits]
+  uint16_t* s_unit = reinterpret_cast<uint16_t*>(mem + kRankUnits);  // [kRankUnits]
+  uint32_t* s_pos = mem + kRankUnits + kRankUnits / 2;               // [PT] of this CTA's candidates
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, G = gridDim.x, c = blockIdx.x;
+  const uint32_t r = (U + PT - 1) / PT, u0 = tid * r;  // this thread's units u0 .. u0 + r - 1
+  uint32_t key[R], n = 0;
+  bool cand[R], miss = false;
+#pragma unroll
+  for (uint32_t e = 0; e < R; ++e) {
+    cand[e] = false;
+    if (e < r && u0 + e < U) {
+      const Unit x = score_unit(p, s, u0 + e);
+      miss |= x.missing;
+      key[e] = x.key;
+      cand[e] = x.cand;
+      n += x.cand ? 1u : 0u;
+    }
+  }
+  uint32_t at = block_scan<PT, uint32_t>(n, Q);
+#pragma unroll
+  for (uint32_t e = 0; e < R; ++e)
+    if (cand[e]) {
+      s_key[at] = key[e];
+      s_unit[at++] = (uint16_t)(u0 + e);
+    }
+  if (tid < 3 && Q + tid < kRankUnits) s_key[Q + tid] = 0xFFFFFFFFu;  // below no key: whole vectors of keys
+  s_pos[tid] = 0u;
+  if (c == 0 && miss) s.x[X_MISSING] = 1ull;  // cleared by this CTA before the scan
+  __syncthreads();
+  const uint32_t runs = (Q + 31u) / 32u, per = (runs + G - 1) / G, g0 = c * per;
+  const uint32_t mine = g0 < runs ? min(per, runs - g0) : 0u;  // at most W (launch_plan)
+  if (mine != 0u) {
+    const uint32_t share = W / mine, g = warp / share, part = warp % share;
+    if (g < mine) {
+      const uint32_t i0 = (g0 + g) * 32u, i = i0 + lane;
+      const uint32_t ki = i < Q ? s_key[i] : 0u;
+      const uint32_t step = ((Q + share - 1) / share + 3u) & ~3u;
+      const uint32_t j0 = min(part * step, Q), j1 = min(j0 + step, Q);
+      uint32_t k = 0;
+      const uint4* v = reinterpret_cast<const uint4*>(s_key);
+#pragma unroll 4
+      for (uint32_t j = j0; j < min(j1, i0); j += 4) {  // before the run: equal keys come first
+        const uint4 q = v[j / 4u];
+        k += (q.x <= ki) + (q.y <= ki) + (q.z <= ki) + (q.w <= ki);
+      }
+      for (uint32_t j = max(j0, i0); j < min(j1, i0 + 32u); ++j) k += s_key[j] < ki || (s_key[j] == ki && j < i);
+#pragma unroll 4
+      for (uint32_t j = max(j0, i0 + 32u); j < j1; j += 4) {
+        const uint4 q = v[j / 4u];
+        k += (q.x < ki) + (q.y < ki) + (q.z < ki) + (q.w < ki);
+      }
+      if (k) atomicAdd(&s_pos[g * 32u + lane], k);
+    }
+  }
+  __syncthreads();
+  if (tid < mine * 32u && g0 * 32u + tid < Q) {
+    const uint32_t pos = s_pos[tid], u = s_unit[g0 * 32u + tid];
+    if (kChecked && pos >= U) {  // checked build: a position past U
+      atomicOr((unsigned long long*)&p.summary[S_ERR], (unsigned long long)kErrBounds);
+      return;
+    }
+    p.order[pos] = u;
+    if (p.cache_order_out) p.cache_order_out[pos] = u;
+  }
+}
+
 template <int PT, bool CL>
 __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch s) {
   constexpr int W = PT / 32;
@@ -456,13 +539,23 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
       if (!phase_sync<CL>(s.x, gen, p.summary)) return;
     }
 
+    bool ranked = false;
+    if constexpr (CL) {
+      if (U <= kRankUnits) {
+        rank_units<PT>(p, s, U, &s_cnt[0][0], Q);
+        own_slice(Q);
+        if (p.cache_q_out && gt == 0) *p.cache_q_out = Q;
+        if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+        ranked = true;
+      }
+    }
     // ---- A and C: candidates, then a stable LSD radix sort by 8-bit digits ----
     // Pass 0 takes the candidates of this warp's slice of the units, later passes its slice of
     // the pass before; the first kHold tiles' keys stay in registers from count to scatter.
     const uint2* in = nullptr;
     uint2* out = s.kv_a;
     bool ordered = false;  // the last pass has put the units into p.order
-    for (uint32_t pass = 0; pass < 4; ++pass) {
+    for (uint32_t pass = 0; pass < 4 && !ranked; ++pass) {
       const uint32_t shift = 8u * pass;
       const uint64_t r0 = pass == 0 ? ua : a, r1 = pass == 0 ? ub : b;
       auto load = [&](uint64_t j, uint32_t& key, uint32_t& val) -> bool {  // false: no candidate
@@ -566,9 +659,9 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
     }
     // the sorted units are in p.order unless the last pass was skipped (a uniform fact: every
     // CTA made the same skip decisions)
-    if (!ordered)
+    if (!ordered && !ranked)
       for (uint64_t j = a + lane; j < b; j += 32) p.order[j] = in[j].y;
-    if (p.cache_order_out) {  // keep the order for later plans with the same operator
+    if (p.cache_order_out && !ranked) {  // keep the order for later plans with the same operator
       for (uint64_t j = a + lane; j < b; j += 32) p.cache_order_out[j] = ordered ? p.order[j] : in[j].y;
       if (gt == 0) *p.cache_q_out = Q;
     }
@@ -799,9 +892,10 @@ cudaError_t launch_plan(const PlanLaunch& p, void* scratch, cudaStream_t st) {
   carve(scratch, U, n_pairs, &s);
   cudaError_t e;
   if (U <= kClusterUnits) {
-    // half a unit per thread, then more, in one cluster
+    // half a unit per thread, then more, in one cluster; where the units are compared with one
+    // another, 2^16 comparisons per CTA, then more
     uint32_t grid = 1;
-    while (grid < kClusterMax && grid * 512ull < U) grid *= 2;
+    while (grid < kClusterMax && (grid * 512ull < U || (U <= kRankUnits && U * U > (uint64_t)grid << 16))) grid *= 2;
     auto k = plan_kernel<kClusterThreads, true>;
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

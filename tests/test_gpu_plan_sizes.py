@@ -87,3 +87,12 @@ def test_a_tail_that_fits_at_once():
         n[:, 0] = 1.0
         return n * (1 + 1e-3 * r.random(s))
     _check(numels, 1 << 20, 1, norms, (0.01, 0.05, 0.5, 1.0))
+
+
+@pytest.mark.parametrize("norms", [lognormal, lambda r, s: 2.0 ** r.integers(-3, 3, s), lambda r, s: np.zeros(s)],
+                         ids=["lognormal", "powers", "zero"])
+@pytest.mark.parametrize("n_blocks,K", [(7, 1), (257, 2), (1023, 1), (1365, 2), (3072, 1), (1024, 3), (3073, 1)])
+def test_units_ranked_by_comparison(n_blocks, K, norms):
+    # up to 3,072 units; candidates fewer than units, not a multiple of 4 or 32, tensors with missing entries
+    _check([256 * n_blocks - 7], 256, K, norms, (0.0, 0.3, 1.0), zero_frac=0.13, seed=n_blocks)
+    _check([256 * (n_blocks - 3) - 7, 300, 5], 256, K, norms, (0.3, 1.0), missing=0.01, seed=n_blocks)
