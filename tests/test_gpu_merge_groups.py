@@ -56,3 +56,13 @@ def test_a_chunk_across_the_carry_of_the_mask_counter(kind):
     del fam, base, expert
     torch.cuda.empty_cache()
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("K", [3, 6, 11])
+@pytest.mark.parametrize("n_blocks", [150, 152 * 3 * 8 + 5, 152 * 4 * 16 - 1, 152 * 4 * 24 + 9])
+def test_chunks_taken_one_two_and_three_at_a_time(n_blocks, K):
+    """the number of chunks of a grab follows the size of the merge (one chunk per block here)"""
+    fam = synth.custom([n_blocks * 512 - 3, 77], dtype=synth.BF16, block_elems=512, K=K, active_frac=0.5,
+                       name=f"grabs-{n_blocks}")
+    base, experts = fam.host_arrays()
+    run_case(fam, base, experts, ("ta", "ties", "dare", "avg_renorm", "dare_ties"), [0.4])
