@@ -360,13 +360,12 @@ __device__ __forceinline__ bool checked_item(const IndexLaunch& p, uint64_t b, u
   return false;
 }
 
-// The k-th largest of the keys counted in h[0 .. 32 N) (SKIP0: h[0] apart), by one warp: lane l sums the N bins
-// that rank l-th from the top, a warp scan finds the lane where the running count reaches k,
-// and that lane walks its own bins.  True (on every lane) when h holds at least k keys; then
-// bin is the bin of the k-th largest and before the number of keys above it; false: before is
-// the number of keys.  One thread
-// walking the bins waits for a load per bin: 256 to 384 of them took 30-46 us whatever the
-// number of pairs, this takes two.
+// The k-th largest of the keys counted in h[0 .. 32 N) (SKIP0: h[0] apart), by one warp: lane l
+// sums the N bins that rank l-th from the top, a warp scan finds the lane where the running count
+// reaches k, and that lane walks its own bins.  True (on every lane) when h holds at least k keys;
+// then bin is the bin of the k-th largest and before the number of keys above it; false: before
+// is the number of keys.  One thread walking the bins waits for a load per bin: 256 to 384 of
+// them took 30-46 us whatever the number of pairs, this takes two.
 template <int N, bool SKIP0 = false>
 __device__ __forceinline__ bool warp_kth(const unsigned long long* h, unsigned long long k, uint32_t& bin,
                                          unsigned long long& before) {
@@ -414,7 +413,8 @@ __device__ __forceinline__ void coarse_select_pair(const IndexLaunch& p, uint64_
   uint32_t e = kNoBin;
   unsigned long long before = 0, r = 0;
   if (k != 0) {
-    if (!warp_kth<8>(p.coarse + x * 256u, k, e, before)) e = 0u;  // unreachable for k <= numel
+    // bin 0 is what the others leave: after masking the omitted elements, zeros, are not counted
+    if (!warp_kth<8, true>(p.coarse + x * 256u, k, e, before)) e = 0u;
     r = k - before;
   }
   if ((threadIdx.x & 31u) == 0) {
@@ -453,11 +453,23 @@ __device__ __forceinline__ bool last_cta(unsigned long long* done, volatile int*
   return true;
 }
 
+// f(x) for every marked pair x, by one warp each of the WARPS of a CTA.  The marks are read 32 to a
+// warp: a warp that read one pair's after the other's took 84 us for 2,948 pairs.
+template <int WARPS, typename F>
+__device__ __forceinline__ void for_marked_pairs(const IndexLaunch& p, F f) {
+  const uint64_t n = (uint64_t)p.K * p.n_groups;
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint64_t x0 = (threadIdx.x >> 5) * 32u; x0 < n; x0 += WARPS * 32u) {
+    uint32_t m = __ballot_sync(0xFFFFFFFFu, x0 + lane < n && p.gmiss[x0 + lane] != 0u);
+    for (; m; m &= m - 1u) f(x0 + (uint32_t)(__ffs(m) - 1));
+  }
+}
+
 // the end of a fallback coarse pass: its last CTA makes the coarse select of the marked pairs
 // (few or none as a rule), which saves a launch that would return at once
 __device__ __forceinline__ void coarse_pass_end(const IndexLaunch& p, volatile int* s_last) {
   if (!p.select_in_pass || !last_cta<kIxThreads>(p.work + 2, s_last)) return;
-  for (uint64_t x = threadIdx.x >> 5; x < (uint64_t)p.K * p.n_groups; x += kIxThreads / 32) coarse_select_pair(p, x);
+  for_marked_pairs<kIxThreads / 32>(p, [&](uint64_t x) { coarse_select_pair(p, x); });
 }
 
 template <bool BF16, int KG, int BM>
@@ -988,39 +1000,12 @@ __global__ void __launch_bounds__(256) ties_fine_kernel(const IndexLaunch p) {
   }
   // the windowed catalog's fallback: the last CTA makes the fine select of the marked pairs
   if (!p.select_in_pass || !last_cta<256>(p.work + 3, &s_last)) return;
-  for (uint64_t x = tid >> 5; x < (uint64_t)p.K * p.n_groups; x += 8) fine_select_pair(p, x);
+  for_marked_pairs<8>(p, [&](uint64_t x) { fine_select_pair(p, x); });
 }
 
 __global__ void __launch_bounds__(kSelThreads) ties_fine_select(const IndexLaunch p) {
   const uint64_t x = select_pair();
   if (x < (uint64_t)p.K * p.n_groups) fine_select_pair(p, x);
-}
-
-// TIES after masking: the coarse bins of (expert i, group) summed over a window of blocks:
-// a selected block adds its catalog histogram, an unselected one adds its elements to bin 0
-// (omitted entries are zeros).  One CTA per (expert, window of kMaskWin blocks); thread e
-// owns bin e and adds its sum for each group the window touches.
-constexpr uint32_t kMaskWin = 256;
-
-__global__ void __launch_bounds__(256) ties_masked_coarse(const IndexLaunch p, uint32_t n_win) {
-  const uint32_t i = blockIdx.x / n_win;
-  const uint64_t b0 = (uint64_t)(blockIdx.x % n_win) * kMaskWin;
-  const uint64_t b1 = b0 + kMaskWin < p.n_blocks ? b0 + kMaskWin : p.n_blocks;
-  const uint32_t e = threadIdx.x;
-  const uint32_t* uh = p.unit_hist + ((uint64_t)i * p.n_blocks << 8);
-  uint32_t grp = p.blk_group[b0];
-  unsigned long long acc = 0;
-  for (uint64_t b = b0; b < b1; ++b) {
-    const uint32_t g = p.blk_group[b];
-    if (g != grp) {
-      if (acc) atomicAdd(&p.coarse[((uint64_t)i * p.n_groups + grp) * 256u + e], acc);
-      acc = 0;
-      grp = g;
-    }
-    if ((p.mask[b] >> i) & 1u) acc += uh[(b << 8) + e];
-    else if (e == 0) acc += p.blk_len[b];
-  }
-  if (acc) atomicAdd(&p.coarse[((uint64_t)i * p.n_groups + grp) * 256u + e], acc);
 }
 
 // ---- TIES thresholds with a predicted window ----------------------------------------------
@@ -1250,11 +1235,14 @@ __global__ void __launch_bounds__(kSelThreads) ties_units_finish(const IndexLaun
   }
 }
 
-// the sums of a plan's selected units, for ties_units_finish.  One CTA per (expert, window of
-// kUnitWin blocks); a thread owns four bins and adds them for each group the window touches.
+// The sums of a plan's selected units (NB = kUnitBins: for ties_units_finish, 256: the coarse bins).
+// One CTA per (expert, window of kUnitWin blocks); a thread owns four bins and adds them for each
+// group the window touches, several units' bins in flight.  (One thread per bin that walked 256
+// blocks one after the other, each behind its mask word, took 43 us on 1,104 blocks with 7 experts.)
 constexpr uint32_t kUnitWin = 32;
 
-__global__ void __launch_bounds__(kUnitBins / 4) ties_units_sum(const IndexLaunch p, uint32_t n_win) {
+template <uint32_t NB>
+__global__ void __launch_bounds__(NB / 4) ties_units_sum(const IndexLaunch p, uint32_t n_win) {
   __shared__ uint32_t s_b[kUnitWin], s_g[kUnitWin], s_n;
   const uint32_t i = blockIdx.x / n_win, tid = threadIdx.x;
   const uint64_t b0 = (uint64_t)(blockIdx.x % n_win) * kUnitWin;
@@ -1270,19 +1258,19 @@ __global__ void __launch_bounds__(kUnitBins / 4) ties_units_sum(const IndexLaunc
   }
   __syncthreads();
   const uint32_t n = s_n;
-  const uint4* uh = reinterpret_cast<const uint4*>(p.unit_hist + ((uint64_t)i * p.n_blocks + b0) * kUnitBins) + tid;
+  const uint4* uh = reinterpret_cast<const uint4*>(p.unit_hist + ((uint64_t)i * p.n_blocks + b0) * NB) + tid;
   for (uint32_t a = 0; a < n;) {
     const uint32_t g = s_g[a];
     unsigned long long c[4] = {0, 0, 0, 0};
 #pragma unroll 4
     for (; a < n && s_g[a] == g; ++a) {
-      const uint4 q = uh[(size_t)s_b[a] * (kUnitBins / 4)];
+      const uint4 q = uh[(size_t)s_b[a] * (NB / 4)];
       c[0] += q.x;
       c[1] += q.y;
       c[2] += q.z;
       c[3] += q.w;
     }
-    unsigned long long* us = p.usum + ((uint64_t)i * p.n_groups + g) * kUnitBins + tid * 4u;
+    unsigned long long* us = (NB == kUnitBins ? p.usum : p.coarse) + ((uint64_t)i * p.n_groups + g) * NB + tid * 4u;
 #pragma unroll
     for (int e = 0; e < 4; ++e)
       if (c[e]) atomicAdd(us + e, c[e]);
@@ -1466,23 +1454,20 @@ cudaError_t launch_ties_window_end(const IndexLaunch& p, cudaStream_t st) {
 
 cudaError_t launch_ties_masked(const IndexLaunch& p, cudaStream_t st) {
   if (!p.unit_hist || !p.mask || p.n_blocks == 0) return cudaErrorInvalidValue;
+  const uint32_t n_win = (uint32_t)((p.n_blocks + kUnitWin - 1) / kUnitWin);
+  IndexLaunch q = p;
   if (p.usum) {
-    const uint32_t n_win = (uint32_t)((p.n_blocks + kUnitWin - 1) / kUnitWin);
-    ties_units_sum<<<p.K * n_win, kUnitBins / 4, 0, st>>>(p, n_win);
+    ties_units_sum<kUnitBins><<<p.K * n_win, kUnitBins / 4, 0, st>>>(p, n_win);
     ties_units_finish<<<select_grid((uint64_t)p.K * p.n_groups), kSelThreads, 0, st>>>(p);
-    count_launches(2);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    IndexLaunch q = p;
+    count_launches(1);
     q.select_in_pass = 1;
-    return launch_ties_finish(q, st);
+  } else {
+    ties_units_sum<256><<<p.K * n_win, 64, 0, st>>>(p, n_win);
   }
-  const uint32_t n_win = (uint32_t)((p.n_blocks + kMaskWin - 1) / kMaskWin);
-  ties_masked_coarse<<<p.K * n_win, 256, 0, st>>>(p, n_win);
   count_launches(1);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_ties_finish(p, st);
+  return launch_ties_finish(q, st);
 }
 
 cudaError_t launch_ties_finish(const IndexLaunch& p, cudaStream_t st) {
