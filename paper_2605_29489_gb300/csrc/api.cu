@@ -521,6 +521,7 @@ cudaError_t walk_segments(const IndexLaunch& p, const mp_index_s* ix, cudaStream
     ps.expert_origin = g.e0;
     ps.ext.x_span = span;
     ps.defer_ties_select = 1;
+    ps.follows = false;  // the segment waits for its gather
     ps.work = p.work + s;
     for (uint32_t i = 0; i < p.K; ++i) ps.experts.p[i] = hp.buf(b, i);
     const int tk = trace_begin(MP_TRACE_SEGMENT, (uint32_t)s, 0, cs);
@@ -561,6 +562,7 @@ cudaError_t index_host_pool(IndexLaunch p, const mp_index_s* ix, cudaStream_t cs
     p.b_begin = 0;
     p.b_end = p.n_blocks;
     p.expert_origin = 0;
+    p.follows = false;
     e = launch_ties_finish(p, cs);
   }
   return e;
@@ -925,6 +927,7 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   p.b_end = g.n_blocks;
   p.expert_origin = 0;
   p.ext = Extents{g.span_elems, g.span_elems};
+  p.follows = true;  // the initial kernel
   if (family->experts_location == 0) {
     if ((e = launch_index(p, cs)) != cudaSuccess) return bail(e, "index kernels");
   } else {
@@ -1303,6 +1306,7 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
     q.ext = Extents{g.span_elems, g.span_elems};
     q.wait_limit = g_stall_rounds.load(std::memory_order_relaxed);
     q.stall = q.wait_limit ? 1u : 0u;
+    q.follows = true;  // the fill
     if ((e = launch_ties_masked(q, cs)) != cudaSuccess) return bail(e, "masked TIES threshold");
   }
 
@@ -1349,6 +1353,7 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   p.touched_only = touched_only ? 1u : 0u;
   p.wait_limit = g_stall_rounds.load(std::memory_order_relaxed);
   p.stall = p.wait_limit ? 1u : 0u;
+  p.follows = family->experts_location == 0;  // the fill, or the threshold's last kernel
   if (family->experts_location == 0) {
     if ((e = launch_merge(p, cs)) != cudaSuccess) return bail(e, "merge kernels");
   } else {

@@ -13,6 +13,7 @@
 // would wait for all of it.  A host buffer these kernels read is pinned memory, which the
 // device reaches through its host mapping.
 #include "mp_internal.cuh"
+#include "tma.cuh"
 
 namespace mp {
 namespace {
@@ -61,6 +62,7 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const GatherLaunch g) 
 // the ranges of an InitList: blockIdx.y is the range.  One launch of about 3 us takes the place
 // of up to eight (each 2-2.5 us on the device and 3-4 us of the host's time)
 __global__ void __launch_bounds__(kThreads) init_kernel(const InitList l) {
+  kernel_begin();
   const InitSeg g = l.seg[blockIdx.y];
   const size_t tid = (size_t)blockIdx.x * kThreads + threadIdx.x, nt = (size_t)gridDim.x * kThreads;
   const size_t nv = g.bytes / 16u;
@@ -72,6 +74,7 @@ __global__ void __launch_bounds__(kThreads) init_kernel(const InitList l) {
 }
 
 __global__ void __launch_bounds__(kThreads) fill_kernel(char* dst, uint32_t v, size_t bytes) {
+  kernel_begin();
   const size_t tid = (size_t)blockIdx.x * kThreads + threadIdx.x, nt = (size_t)gridDim.x * kThreads;
   const uint32_t w = (v & 0xFFu) * 0x01010101u;
   if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {

@@ -475,6 +475,7 @@ __device__ __forceinline__ void coarse_pass_end(const IndexLaunch& p, volatile i
 template <bool BF16, int KG, int BM>
 __global__ void __launch_bounds__(kIxThreads, IxGeo<BM != kBinNone, KG, BM == kBinUnits>::kCtasPerSm)
     index_tma_kernel(const IndexLaunch p, uint32_t G, uint64_t n_items, unsigned long long* work) {
+  kernel_begin();
   constexpr bool TIES = BM != kBinNone;
   constexpr uint32_t NB = key_bins<BM>();  // key bins per expert
   using Geo = IxGeo<TIES, KG, BM == kBinUnits>;
@@ -929,12 +930,14 @@ __device__ __forceinline__ uint64_t select_pair() {
 inline unsigned select_grid(uint64_t pairs) { return (unsigned)((pairs + kSelThreads / 32 - 1) / (kSelThreads / 32)); }
 
 __global__ void __launch_bounds__(kSelThreads) ties_coarse_select(const IndexLaunch p) {
+  kernel_begin();
   const uint64_t x = select_pair();
   if (x < (uint64_t)p.K * p.n_groups) coarse_select_pair(p, x);
 }
 
 template <bool BF16, int KG>
 __global__ void __launch_bounds__(256) ties_fine_kernel(const IndexLaunch p) {
+  kernel_begin();
   constexpr int V = BF16 ? 8 : 4;
   __shared__ uint32_t s_fine[KG][128];
   __shared__ int s_last;
@@ -1004,6 +1007,7 @@ __global__ void __launch_bounds__(256) ties_fine_kernel(const IndexLaunch p) {
 }
 
 __global__ void __launch_bounds__(kSelThreads) ties_fine_select(const IndexLaunch p) {
+  kernel_begin();
   const uint64_t x = select_pair();
   if (x < (uint64_t)p.K * p.n_groups) fine_select_pair(p, x);
 }
@@ -1044,6 +1048,7 @@ constexpr uint32_t kSampleBins = 1024;
 
 template <bool BF16, int KG>
 __global__ void __launch_bounds__(256, 4) ties_sample_kernel(const IndexLaunch p) {
+  kernel_begin();
   constexpr uint32_t V = BF16 ? 8u : 4u;
   __shared__ uint32_t hist[KG][kSampleBins];
   __shared__ unsigned long long s_n;  // sampled elements
@@ -1118,6 +1123,7 @@ __global__ void __launch_bounds__(256, 4) ties_sample_kernel(const IndexLaunch p
 // the window of each (expert, group) from its sample, by one warp: around the bin e of the k_s-th
 // largest sampled key, or the three binades around that bin's binade
 __global__ void __launch_bounds__(kSelThreads) ties_window_select(const IndexLaunch p) {
+  kernel_begin();
   const uint64_t x = select_pair();
   if (x >= (uint64_t)p.K * p.n_groups) return;
   const uint32_t lane = threadIdx.x & 31u, g = (uint32_t)(x % p.n_groups);
@@ -1170,6 +1176,7 @@ __global__ void __launch_bounds__(kSelThreads) ties_window_select(const IndexLau
 // the threshold of each (expert, group) from its window counts, or a mark for the
 // two-level select when it lies outside the window
 __global__ void __launch_bounds__(kSelThreads) ties_window_finish(const IndexLaunch p) {
+  kernel_begin();
   const uint64_t x = select_pair();
   if (x >= (uint64_t)p.K * p.n_groups) return;
   const unsigned long long k = p.kth[x % p.n_groups];
@@ -1199,6 +1206,7 @@ __global__ void __launch_bounds__(kSelThreads) ties_window_finish(const IndexLau
 // units for the catalog, the selected ones for a plan), by one warp, or a mark with the coarse bin
 // and rank for the fine pass when it lies outside the window
 __global__ void __launch_bounds__(kSelThreads) ties_units_finish(const IndexLaunch p) {
+  kernel_begin();
   const uint64_t x = select_pair();
   if (x >= (uint64_t)p.K * p.n_groups) return;
   const unsigned long long k = p.kth[x % p.n_groups];
@@ -1243,6 +1251,7 @@ constexpr uint32_t kUnitWin = 32;
 
 template <uint32_t NB>
 __global__ void __launch_bounds__(NB / 4) ties_units_sum(const IndexLaunch p, uint32_t n_win) {
+  kernel_begin();
   __shared__ uint32_t s_b[kUnitWin], s_g[kUnitWin], s_n;
   const uint32_t i = blockIdx.x / n_win, tid = threadIdx.x;
   const uint64_t b0 = (uint64_t)(blockIdx.x % n_win) * kUnitWin;
@@ -1281,7 +1290,7 @@ __global__ void __launch_bounds__(NB / 4) ties_units_sum(const IndexLaunch p, ui
 // the lower key bits inside it (a second pass over the blocks that can reach it; experts
 // addressed with origin 0), select the threshold
 template <bool BF16, int KG>
-cudaError_t ties_finish_t(const IndexLaunch& p, cudaStream_t st) {
+cudaError_t ties_finish_t(const IndexLaunch& p, bool follows, cudaStream_t st) {
   const uint32_t G = (p.K + KG - 1) / KG;
   const uint64_t nsel = (uint64_t)p.K * p.n_groups;
   const unsigned sgrid = select_grid(nsel);
@@ -1295,17 +1304,19 @@ cudaError_t ties_finish_t(const IndexLaunch& p, cudaStream_t st) {
   uint64_t fgrid = (uint64_t)sms * (per_sm > 0 ? per_sm : 1);
   if (fgrid > p.n_blocks * G) fgrid = p.n_blocks * G;
   if (fgrid == 0) fgrid = 1;
-  if (!p.select_in_pass) ties_coarse_select<<<sgrid, kSelThreads, 0, st>>>(p);
-  ties_fine_kernel<BF16, KG><<<(unsigned)fgrid, 256, 0, st>>>(p);
-  if (!p.select_in_pass) ties_fine_select<<<sgrid, kSelThreads, 0, st>>>(p);
-  count_launches(p.select_in_pass ? 1 : 3);
-  return cudaGetLastError();
+  if (!p.select_in_pass) {
+    if ((e = launch_kernel(follows, ties_coarse_select, sgrid, kSelThreads, 0, st, p)) != cudaSuccess) return e;
+    follows = true;
+  }
+  if ((e = launch_kernel(follows, ties_fine_kernel<BF16, KG>, (unsigned)fgrid, 256, 0, st, p)) != cudaSuccess) return e;
+  if (!p.select_in_pass) e = launch_kernel(true, ties_fine_select, sgrid, kSelThreads, 0, st, p);
+  return e;
 }
 
 // one persistent launch of the catalog kernel with binning mode BM
 template <bool BF16, int KG, int BM>
-cudaError_t launch_pass(const IndexLaunch& p, uint32_t G, uint64_t n_items, int sms, unsigned long long* work,
-                        cudaStream_t st) {
+cudaError_t launch_pass(const IndexLaunch& p, bool follows, uint32_t G, uint64_t n_items, int sms,
+                        unsigned long long* work, cudaStream_t st) {
   constexpr bool ties = BM != kBinNone;
   constexpr uint32_t NB = key_bins<BM>();
   using Geo = IxGeo<ties, KG, BM == kBinUnits>;
@@ -1317,9 +1328,7 @@ cudaError_t launch_pass(const IndexLaunch& p, uint32_t G, uint64_t n_items, int 
   cudaError_t e;
   auto k = index_tma_kernel<BF16, KG, BM>;
   if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  k<<<(unsigned)grid, kIxThreads, smem, st>>>(p, G, n_items, work);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_kernel(follows, k, (unsigned)grid, kIxThreads, smem, st, p, G, n_items, work);
 }
 
 template <bool BF16, int KG>
@@ -1332,7 +1341,17 @@ cudaError_t launch_plain_t(const IndexLaunch& p, cudaStream_t st) {
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  return launch_pass<BF16, KG, kBinNone>(p, G, n_items, sms, p.work, st);
+  return launch_pass<BF16, KG, kBinNone>(p, p.follows, G, n_items, sms, p.work, st);
+}
+
+template <bool BF16, int KG>
+cudaError_t window_begin_t(const IndexLaunch& p, cudaStream_t st) {
+  const uint32_t G = (p.K + KG - 1) / KG;
+  const uint64_t nsel = (uint64_t)p.K * p.n_groups;
+  if (p.n_samp_spans == 0 || nsel == 0) return cudaSuccess;
+  const cudaError_t e = launch_kernel(p.follows, ties_sample_kernel<BF16, KG>, dim3(p.n_samp_spans, G), 256, 0, st, p);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(true, ties_window_select, select_grid(nsel), kSelThreads, 0, st, p);
 }
 
 template <bool BF16, int KG>
@@ -1346,43 +1365,25 @@ cudaError_t launch_ties_t(const IndexLaunch& p, cudaStream_t st) {
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if (!p.win) {  // the two-level select for every pair
-    if ((e = launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
+    if ((e = launch_pass<BF16, KG, kBinCoarse>(p, p.follows, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
     if (p.defer_ties_select) return cudaSuccess;
-    return ties_finish_t<BF16, KG>(p, st);
+    return ties_finish_t<BF16, KG>(p, true, st);
   }
   // predicted windows: sample, windowed catalog pass, thresholds from the windows, then the
   // two-level select for the pairs whose threshold left its window (a no-op when none did)
-  const uint64_t nsel = (uint64_t)p.K * p.n_groups;
-  ties_sample_kernel<BF16, KG><<<dim3(p.n_samp_spans, G), 256, 0, st>>>(p);
-  ties_window_select<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
-  count_launches(2);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const unsigned sgrid = select_grid((uint64_t)p.K * p.n_groups);
+  if ((e = window_begin_t<BF16, KG>(p, st)) != cudaSuccess) return e;
   IndexLaunch q = p;  // the selects of the fallback ride in its passes
   q.select_in_pass = 1;
   if (p.usum) {  // TIES after masking: one pass gives the units' bins and the coarse bins too
-    if ((e = launch_pass<BF16, KG, kBinUnits>(p, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
-    ties_units_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
-    count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return ties_finish_t<BF16, KG>(q, st);
+    if ((e = launch_pass<BF16, KG, kBinUnits>(p, true, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
+    if ((e = launch_kernel(true, ties_units_finish, sgrid, kSelThreads, 0, st, p)) != cudaSuccess) return e;
+    return ties_finish_t<BF16, KG>(q, true, st);
   }
-  if ((e = launch_pass<BF16, KG, kBinWindow>(p, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
-  ties_window_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
-  count_launches(1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_pass<BF16, KG, kBinCoarse>(q, G, n_items, sms, p.work + 1, st)) != cudaSuccess) return e;
-  return ties_finish_t<BF16, KG>(q, st);
-}
-
-template <bool BF16, int KG>
-cudaError_t window_begin_t(const IndexLaunch& p, cudaStream_t st) {
-  const uint32_t G = (p.K + KG - 1) / KG;
-  const uint64_t nsel = (uint64_t)p.K * p.n_groups;
-  if (p.n_samp_spans == 0 || nsel == 0) return cudaSuccess;
-  ties_sample_kernel<BF16, KG><<<dim3(p.n_samp_spans, G), 256, 0, st>>>(p);
-  ties_window_select<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
-  count_launches(2);
-  return cudaGetLastError();
+  if ((e = launch_pass<BF16, KG, kBinWindow>(p, true, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
+  if ((e = launch_kernel(true, ties_window_finish, sgrid, kSelThreads, 0, st, p)) != cudaSuccess) return e;
+  if ((e = launch_pass<BF16, KG, kBinCoarse>(q, true, G, n_items, sms, p.work + 1, st)) != cudaSuccess) return e;
+  return ties_finish_t<BF16, KG>(q, true, st);
 }
 
 template <bool BF16, int KG>
@@ -1395,8 +1396,8 @@ cudaError_t pass_t(const IndexLaunch& p, bool window, cudaStream_t st) {
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  return window ? launch_pass<BF16, KG, kBinWindow>(p, G, n_items, sms, p.work, st)
-                : launch_pass<BF16, KG, kBinCoarse>(p, G, n_items, sms, p.work, st);
+  return window ? launch_pass<BF16, KG, kBinWindow>(p, false, G, n_items, sms, p.work, st)
+                : launch_pass<BF16, KG, kBinCoarse>(p, false, G, n_items, sms, p.work, st);
 }
 
 // f(KG) with the experts per item of the TIES kernels as a constant.  More than 4 experts take
@@ -1447,33 +1448,31 @@ cudaError_t launch_ties_window_end(const IndexLaunch& p, cudaStream_t st) {
   if (!p.win || !p.coarse) return cudaErrorInvalidValue;
   const uint64_t nsel = (uint64_t)p.K * p.n_groups;
   if (nsel == 0) return cudaSuccess;
-  ties_window_finish<<<select_grid(nsel), kSelThreads, 0, st>>>(p);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_kernel(false, ties_window_finish, select_grid(nsel), kSelThreads, 0, st, p);
 }
 
 cudaError_t launch_ties_masked(const IndexLaunch& p, cudaStream_t st) {
   if (!p.unit_hist || !p.mask || p.n_blocks == 0) return cudaErrorInvalidValue;
   const uint32_t n_win = (uint32_t)((p.n_blocks + kUnitWin - 1) / kUnitWin);
   IndexLaunch q = p;
+  cudaError_t e;
   if (p.usum) {
-    ties_units_sum<kUnitBins><<<p.K * n_win, kUnitBins / 4, 0, st>>>(p, n_win);
-    ties_units_finish<<<select_grid((uint64_t)p.K * p.n_groups), kSelThreads, 0, st>>>(p);
-    count_launches(1);
+    e = launch_kernel(p.follows, ties_units_sum<kUnitBins>, p.K * n_win, kUnitBins / 4, 0, st, p, n_win);
+    if (e != cudaSuccess) return e;
+    e = launch_kernel(true, ties_units_finish, select_grid((uint64_t)p.K * p.n_groups), kSelThreads, 0, st, p);
     q.select_in_pass = 1;
   } else {
-    ties_units_sum<256><<<p.K * n_win, 64, 0, st>>>(p, n_win);
+    e = launch_kernel(p.follows, ties_units_sum<256>, p.K * n_win, 64, 0, st, p, n_win);
   }
-  count_launches(1);
-  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  q.follows = true;
   return launch_ties_finish(q, st);
 }
 
 cudaError_t launch_ties_finish(const IndexLaunch& p, cudaStream_t st) {
   return by_ties_items(p.K, [&](auto kg) {
     constexpr int KG = decltype(kg)::value;
-    return p.dtype == MP_BF16 ? ties_finish_t<true, KG>(p, st) : ties_finish_t<false, KG>(p, st);
+    return p.dtype == MP_BF16 ? ties_finish_t<true, KG>(p, p.follows, st) : ties_finish_t<false, KG>(p, p.follows, st);
   });
 }
 

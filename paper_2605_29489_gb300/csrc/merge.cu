@@ -339,6 +339,7 @@ __device__ __forceinline__ void merge_end(const MergeLaunch& p, volatile int* s_
 template <bool BF16, int OPC>
 __global__ void __launch_bounds__(Geo::kThreads, Geo::kCtasPerSm)
     merge_tma_kernel(const MergeLaunch p, uint32_t cpb, uint32_t grab, uint64_t n_chunks, unsigned long long* work) {
+  kernel_begin();
   static_assert(OPC == OP_ADD || OPC == OP_RENORM, "streaming consumers: AVG/TA and the renormalised AVG");
   constexpr int kConsumers = Geo::kConsumers;
   constexpr uint32_t ES = BF16 ? 2u : 4u;
@@ -611,6 +612,7 @@ struct __align__(128) TcSmem {
 template <bool BF16, int OPC, int KC>
 __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCtasPerSm)
     merge_chunk_kernel(const MergeLaunch p, uint32_t cpb, uint32_t grab, uint64_t n_chunks, unsigned long long* work) {
+  kernel_begin();
   static_assert(OPC == OP_TIES || OPC == OP_DARE || OPC == OP_DTIES, "groups of fills: TIES, DARE, DARE-TIES");
   // the packed counts C = 2^23 + c+ + 2^CB c-: CB = 4 bits for up to 8 experts, 6 for 32
   constexpr uint32_t CB = KC <= 8 ? 4u : 6u;
@@ -1062,9 +1064,8 @@ cudaError_t launch_chunk(const MergeLaunch& p, cudaStream_t st) {
     return e;
   uint64_t grid = (uint64_t)sms * Geo::kCtasPerSm;
   if (grid > n_chunks) grid = n_chunks;
-  kern<<<(unsigned)grid, Geo::kThreads, smem, st>>>(p, cpb, grab_of<Geo::kGrab>(n_chunks, grid), n_chunks, p.work);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_kernel(p.follows, kern, (unsigned)grid, Geo::kThreads, smem, st, p, cpb,
+                       grab_of<Geo::kGrab>(n_chunks, grid), n_chunks, p.work);
 }
 
 template <bool BF16, int OPC>
@@ -1091,10 +1092,8 @@ cudaError_t launch_op(const MergeLaunch& p, cudaStream_t st) {
     return e;
   uint64_t grid = (uint64_t)sms * Geo::kCtasPerSm;
   if (grid > n_chunks) grid = n_chunks;
-  merge_tma_kernel<BF16, OPC>
-      <<<(unsigned)grid, Geo::kThreads, smem, st>>>(p, cpb, grab_of<Geo::kGrab>(n_chunks, grid), n_chunks, p.work);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_kernel(p.follows, merge_tma_kernel<BF16, OPC>, (unsigned)grid, Geo::kThreads, smem, st, p, cpb,
+                       grab_of<Geo::kGrab>(n_chunks, grid), n_chunks, p.work);
 }
 
 template <bool BF16>

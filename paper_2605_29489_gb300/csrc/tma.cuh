@@ -20,6 +20,15 @@ __device__ __forceinline__ uint32_t wait_limit_of(uint32_t launch_limit) {
   return launch_limit ? launch_limit : kWaitLimit;
 }
 
+// The first statement of every kernel that launch_kernel may start before the one ahead of it on
+// its stream has ended: lets the kernel behind it start likewise, then waits until the one ahead
+// has ended and what it wrote is visible.  Nothing is read or written before it.  Without such a
+// launch on either side it does nothing.
+__device__ __forceinline__ void kernel_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
