@@ -360,8 +360,7 @@ mp_status alloc_hashes(mp_index_s* ix, cudaStream_t cs);
 
 // ---- experts in pinned host memory: segment pipeline -------------------------------------
 //
-// The family is walked in segments of consecutive blocks (about kSegmentElems elements
-// each).  Two HBM staging buffers alternate: while the kernels of the caller's stream
+// The family is walked in segments of consecutive blocks (segment_elems elements at most).  Two HBM staging buffers alternate: while the kernels of the caller's stream
 // work on segment s, segment s+1 is brought in on a side stream by a gather kernel that
 // reads the host experts over the host mapping — every expert block for the index pass,
 // only the planned (block, expert) pairs for the merge.  The planned blocks are scattered
@@ -371,21 +370,35 @@ mp_status alloc_hashes(mp_index_s* ix, cudaStream_t cs);
 namespace {
 
 constexpr uint64_t kSegmentElems = 32ull << 20;
+constexpr uint64_t kStagingBytes = 192ull << 20;
+
+// Most elements of a segment.  Families of up to 16 segments take smaller ones where both staging
+// buffers then stay within what the pool keeps: mapping them anew in every call, and gathering a
+// segment of 32M elements before any kernel of the catalog ran, took 1.2 of 9.9 ms (index, plan and
+// merge) on 166M elements with 4 experts, 10.7 of 23.4 ms on 30M with 32.  Larger families keep
+// large segments, whose gathers of small budgets are long against the 8 us between two of them.
+uint64_t segment_elems(const Geometry& g) {
+  if (g.n_params > 16u * kSegmentElems) return kSegmentElems;
+  const uint64_t e = kStagingBytes / (2u * (uint64_t)g.K * g.elem_size);
+  return e < kSegmentElems / 8u ? kSegmentElems / 8u : (e > kSegmentElems ? kSegmentElems : e);
+}
 constexpr int kSide = 1;  // side streams of the host-pool gathers (one gather kernel saturates the link)
 
 struct Segment {
   uint64_t b0, b1, e0, e1;  // blocks [b0, b1), elements [e0, e1)
 };
 
-std::vector<Segment> make_segments(const std::vector<uint64_t>& off, const std::vector<uint32_t>& len,
-                                   uint64_t& max_span) {
+std::vector<Segment> make_segments(const mp_index_s* ix, uint64_t& max_span) {
+  const std::vector<uint64_t>& off = ix->h_blk_off;
+  const std::vector<uint32_t>& len = ix->h_blk_len;
+  const uint64_t most = segment_elems(ix->g);
   std::vector<Segment> segs;
   max_span = 0;
   const uint64_t nb = off.size();
   uint64_t b0 = 0;
   while (b0 < nb) {
     uint64_t b1 = b0, acc = 0;
-    while (b1 < nb && (b1 == b0 || acc + len[b1] <= kSegmentElems)) acc += len[b1++];
+    while (b1 < nb && (b1 == b0 || acc + len[b1] <= most)) acc += len[b1++];
     const uint64_t e0 = off[b0], e1 = off[b1 - 1] + len[b1 - 1];
     segs.push_back({b0, b1, e0, e1});
     if (e1 - e0 > max_span) max_span = e1 - e0;
@@ -479,7 +492,7 @@ template <typename Stage>
 cudaError_t walk_segments(const IndexLaunch& p, const mp_index_s* ix, cudaStream_t cs, const uint32_t* gate,
                           Stage stage) {
   uint64_t span = 0;
-  const std::vector<Segment> segs = make_segments(ix->h_blk_off, ix->h_blk_len, span);
+  const std::vector<Segment> segs = make_segments(ix, span);
   HostPipe hp;
   cudaError_t e = hp.init(cs, p.K, span, ix->g.elem_size);
   for (size_t s = 0; s < segs.size() && e == cudaSuccess; ++s) {
@@ -547,7 +560,7 @@ cudaError_t index_host_pool(IndexLaunch p, const mp_index_s* ix, cudaStream_t cs
       return e;
     if ((e = launch_ties_window_end(p, cs)) != cudaSuccess) return e;
     IndexLaunch q = p;
-    q.work = p.work + 2 * (size_t)(ix->g.n_params / kSegmentElems) + 2;  // the second walk's counters
+    q.work = p.work + 2 * (size_t)(ix->g.n_params / segment_elems(ix->g)) + 2;  // the second walk's counters
     if ((e = walk_segments(q, ix, cs, p.miss, [&](const IndexLaunch& ps) { return launch_index_pass(ps, false, cs); })) !=
         cudaSuccess)
       return e;
@@ -570,7 +583,7 @@ cudaError_t index_host_pool(IndexLaunch p, const mp_index_s* ix, cudaStream_t cs
 
 cudaError_t merge_host_pool(MergeLaunch p, const mp_index_s* ix, cudaStream_t cs) {
   uint64_t span = 0;
-  const std::vector<Segment> segs = make_segments(ix->h_blk_off, ix->h_blk_len, span);
+  const std::vector<Segment> segs = make_segments(ix, span);
   const uint32_t es = ix->g.elem_size;
   HostPipe hp;
   cudaError_t e = hp.init(cs, p.K, span, es);
@@ -813,8 +826,8 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   auto slot = [&](size_t bytes) { size_t r = o; o += align_up(bytes); return r; };
   // the index kernels' work counters: for device-resident experts the two passes' and the two
   // counts of finished CTAs; for a host pool one per segment of both walks (any two consecutive
-  // segments together exceed kSegmentElems)
-  const size_t n_work = family->experts_location == 0 ? 4 : 2 * (2 * (size_t)(g.n_params / kSegmentElems) + 2);
+  // segments together exceed segment_elems)
+  const size_t n_work = family->experts_location == 0 ? 4 : 2 * (2 * (size_t)(g.n_params / segment_elems(g)) + 2);
   const size_t o_work = slot(n_work * 8);
   size_t o_coarse = 0, o_fine = 0, o_kth = 0, o_est = 0, o_rank = 0;
   size_t o_wfine = 0, o_wabove = 0, o_win = 0, o_gmiss = 0, o_miss = 0, o_wend = 0;
@@ -1241,7 +1254,7 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   const size_t m_gmiss = mslot(KG * 4), m_miss = mslot(16), m_work = mslot(4 * 8), m_zero = mo;
   const size_t m_est = mslot(KG * 4), m_rank = mslot(KG * 8), m_tau = mslot(KG * 4);
   // the merge kernel's work counter (one per segment of a host pool) and its count of finished CTAs
-  const size_t n_work = family->experts_location == 0 ? 1 : 2 * (size_t)(g.n_params / kSegmentElems) + 2;
+  const size_t n_work = family->experts_location == 0 ? 1 : 2 * (size_t)(g.n_params / segment_elems(g)) + 2;
   const size_t scratch_off = align_up(back_bytes + (n_work + 1) * 8);
   const size_t zero_bytes = masked ? scratch_off + m_zero : back_bytes + (n_work + 1) * 8;
   if ((st = dev_alloc(mf->mem, scratch_off + (masked ? mo : 0), cs)) != MP_OK) {
