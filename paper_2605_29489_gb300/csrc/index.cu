@@ -1,18 +1,18 @@
 // Catalog pass (Sec. 3 "Catalog"; the Analyze reads of Sec. 2): per-(expert, block)
 // statistics of Delta = M_i - M_0 and, for TIES, the per-(expert, trim group) threshold.
 //
-// Mapping: one CTA of 256 threads per (block, group of up to 8 experts).  Thread l is
+// Mapping: an item is a block and up to 8 of its experts (4 for TIES).  Consumer thread l is
 // lane l of the fixed summation order: it streams 16-byte vectors l, l+256, ... of the
 // block (base once, each expert of the group), keeps a sequential fma chain of delta^2
 // per expert, then the lanes are combined by a xor butterfly inside each warp and over
 // the 8 warp sums.  That order is part of the definition of the norm (it decides the
 // plan), so it must not change with tuning.
 //
-// TIES threshold (k-th largest 15-bit key bits(bf16(|delta|)) & 0x7FFF per trim group)
-// is a two-level radix select: the index pass histograms the upper 8 key bits in shared
-// memory; a select kernel finds the bin holding the k-th key; a second pass over only the
-// blocks that can hold keys in that bin histograms the lower 7 bits; a last select kernel
-// finishes the threshold.
+// TIES threshold (k-th largest 15-bit key bits(bf16(|delta|)) & 0x7FFF per trim group): a sample
+// predicts a window of keys, the index pass counts those in shared memory and the threshold
+// comes from the counts.  Where it lies outside the window a two-level radix select finds it:
+// the upper 8 key bits' bins, the bin holding the k-th key, a second pass over only the blocks
+// that can hold keys in that bin with bins of the lower 7 bits, the key.
 #include <cuda_bf16.h>
 
 #include <type_traits>
@@ -165,7 +165,7 @@ constexpr uint32_t key_bins() {
 
 template <int KG, int NS, uint32_t SB, uint32_t NB>
 struct __align__(128) IxSmem {
-  uint32_t hist[KG][NB];  // first: its byte addresses stay below 2^16 (ties_win2k packs two)
+  uint32_t hist[KG][NB];  // first: its byte addresses stay below 2^16 (ties_win2 packs two)
   alignas(128) uint8_t slot[NS][SB];
   IxMeta meta[NS];
   uint64_t full[NS];
