@@ -604,7 +604,9 @@ struct __align__(128) TcSmem {
   uint32_t thr[TIES ? G : 1][KC];  // producer only, TIES: bits threshold of (chunk of the grab, expert)
   uint64_t full[NS];
   uint64_t empty[NS];
-  float2 ntab[kTcMaxK + 1];  // {-c, RN(1/c)} for the counts c = 0..32 (entry 0: {-1, 1})
+  // -c and RN(1/c) for the counts c = 0..32 (entry 0: -1, 1); apart, so that two elements' entries
+  // load into the register pairs that the packed operations take
+  float nneg[kTcMaxK + 1], nrcp[kTcMaxK + 1];
   uint32_t nf[NS];           // producer only: fills held by the group of each entry
   int abort, last;
 };
@@ -614,8 +616,11 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
     merge_chunk_kernel(const MergeLaunch p, uint32_t cpb, uint32_t grab, uint64_t n_chunks, unsigned long long* work) {
   kernel_begin();
   static_assert(OPC == OP_TIES || OPC == OP_DARE || OPC == OP_DTIES, "groups of fills: TIES, DARE, DARE-TIES");
-  // the packed counts C = 2^23 + c+ + 2^CB c-: CB = 4 bits for up to 8 experts, 6 for 32
-  constexpr uint32_t CB = KC <= 8 ? 4u : 6u;
+  // the packed counts C = 2^23 + c+ + 2^8 c-, a byte each, which one byte selection extracts (with
+  // CB = 4 or 6 a shift, a select and a mask; that and the split table above: four Llama layers
+  // TIES K = 4 0.924 -> 0.910 ms, Qwen2.5-1.5B (8 layers) DARE-TIES K = 16 2.181 -> 2.152, K = 4
+  // 2.142 -> 2.116, K = 8 2.159 -> 2.126)
+  constexpr uint32_t CB = 8u;
   constexpr int GF = TcGeo<OPC, KC>::kGroup;
   constexpr int NS = TcGeo<OPC, KC>::kSlots;
   constexpr int kConsumers = TcGeo<OPC, KC>::kConsumers;
@@ -644,7 +649,8 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
   }
   if (tid <= kTcMaxK) {
     const float c = tid == 0 ? 1.0f : (float)tid;
-    S.ntab[tid] = make_float2(-c, __fdiv_rn(1.0f, c));
+    S.nneg[tid] = -c;
+    S.nrcp[tid] = __fdiv_rn(1.0f, c);
   }
   __syncthreads();
 
@@ -970,7 +976,8 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
       const bool pos = Pp[u][v] > -Nn[u][v], any = Pp[u][v] != -Nn[u][v];
       num = any ? (pos ? Pp[u][v] : Nn[u][v]) : 0.0f;
       const uint32_t cb = __float_as_uint(Cc[u][v]);
-      cv = (pos ? cb : cb >> CB) & ((1u << CB) - 1u);
+      static_assert(CB == 8u && kTcMaxK < 256u, "a byte holds a count");
+      cv = __byte_perm(cb, 0u, pos ? 0x4440u : 0x4441u);  // byte 0 or 1
     };
     // q = RN(num * y), then Markstein's correction q + RN(num - q c) * y, and the output
     // fma(lambda, q, M_0), two elements per instruction.  Numerators 0 < |num| < 2^-100 need the
@@ -981,8 +988,7 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
       float a;
       uint32_t cv;
       num_c(u, v, a, cv);
-      const float2 t = S.ntab[cv];
-      return __fmaf_rn(p.lambda, div_small(a, -t.x, t.y), x0[u][v]);
+      return __fmaf_rn(p.lambda, div_small(a, -S.nneg[cv], S.nrcp[cv]), x0[u][v]);
     };
     auto finalise = [&](auto checked) {
       // 2 |bits| - 2 wraps the zeros to the top: its minimum over the vector is below
@@ -1006,10 +1012,10 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
         num_c(u, v, a0, c0);
         num_c(u, v + 1, a1, c1);
         if constexpr (decltype(checked)::value && kWhole) look(a0, a1);
-        const float2 t0 = S.ntab[c0], t1 = S.ntab[c1];
-        f2_mul(a0, a1, t0.y, t1.y, q0, q1);
-        f2_fma(q0, q1, t0.x, t1.x, a0, a1, r0, r1);
-        f2_fma(r0, r1, t0.y, t1.y, q0, q1, q0, q1);
+        const float n0 = S.nneg[c0], n1 = S.nneg[c1], i0 = S.nrcp[c0], i1 = S.nrcp[c1];
+        f2_mul(a0, a1, i0, i1, q0, q1);
+        f2_fma(q0, q1, n0, n1, a0, a1, r0, r1);
+        f2_fma(r0, r1, i0, i1, q0, q1, q0, q1);
         f2_fma(p.lambda, p.lambda, q0, q1, x0[u][v], x0[u][v + 1], y0, y1);
       };
       // a class that keeps its state over groups has no registers for the words beside it: it
