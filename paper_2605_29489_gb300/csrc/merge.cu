@@ -611,6 +611,20 @@ struct __align__(128) TcSmem {
   int abort, last;
 };
 
+// DARE-TIES: a rescaled delta d whose keep word passes goes to P and c+ or to N and c- by its sign
+// (C = 2^23 + c+ + 256 c-).  Predicated adds, which the FMA pipe takes, instead of keep factors as
+// floats from two more compares and packed multiply-adds: the ALU pipe was the busy one (67 %).
+// Qwen2.5-1.5B (8 layers) K = 16 2.152 -> 1.930 ms, K = 4 2.116 -> 1.905, K = 8 2.126 -> 1.943,
+// Qwen2.5-0.5B (8 layers) K = 32 1.598 -> 1.424, fp32 K = 8 1.175 -> 1.125.  TIES, which tests two
+// thresholds and no keep word, lost by the same (K = 16 0.939 -> 0.986).
+__device__ __forceinline__ void keep_signed(uint32_t kw, uint32_t T16, float d, float& P, float& N, float& C) {
+  asm("{\n .reg .pred q, a, b;\n setp.ge.u32 q, %3, %4;\n setp.gt.and.f32 a, %5, 0f00000000, q;\n"
+      " setp.lt.and.f32 b, %5, 0f00000000, q;\n @a add.rn.f32 %0, %0, %5;\n @b add.rn.f32 %1, %1, %5;\n"
+      " @a add.rn.f32 %2, %2, 0f3F800000;\n @b add.rn.f32 %2, %2, 0f43800000;\n}"
+      : "+f"(P), "+f"(N), "+f"(C)
+      : "r"(kw), "r"(T16), "f"(d));
+}
+
 template <bool BF16, int OPC, int KC>
 __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCtasPerSm)
     merge_chunk_kernel(const MergeLaunch p, uint32_t cpb, uint32_t grab, uint64_t n_chunks, unsigned long long* work) {
@@ -818,7 +832,7 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
   // TIES: P and N, the sums of the kept positive and negative deltas, and both counts in one
   // float C = 2^23 + c+ + 2^CB c- (exact: every value is an integer below 2^24, so the low bits
   // of C hold c+ and c-).  DARE-TIES keeps, instead, every nonzero rescaled delta s = d sigma
-  // whose keep word passes (no magnitude trim).  A delta d is kept positive when d >= thr and kept
+  // whose keep word passes (no magnitude trim; keep_signed).  A TIES delta d is kept positive when d >= thr and kept
   // negative when d <= -thr (thr > 0: |d| >= thr and the sign in one compare each); the keep
   // factors k+ and k- are 1 or 0, and P = fma(k+, d, P), N = fma(k-, d, N): a factor 1 adds d with
   // the one rounding of P + d, a factor 0 adds a zero, which leaves P and N unchanged (they start
@@ -916,24 +930,18 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
             if (kw[v + 1] >= p.dare_T16) acc[u][v + 1] = __fmaf_rn(a, d1, acc[u][v + 1]);
             return;
           }
-          float t0, t1, kp0, kp1, kn0, kn1;
           if constexpr (OPC == OP_DTIES) {
-            // keep factors as 1.0 / 0.0 straight from compares joined with the keep test
-            asm("{\n .reg .pred q;\n setp.ge.u32 q, %4, %5;\n set.gt.and.f32.f32 %0, %6, 0f00000000, q;\n"
-                " set.lt.and.f32.f32 %1, %6, 0f00000000, q;\n setp.ge.u32 q, %7, %5;\n"
-                " set.gt.and.f32.f32 %2, %8, 0f00000000, q;\n set.lt.and.f32.f32 %3, %8, 0f00000000, q;\n}"
-                : "=f"(kp0), "=f"(kn0), "=f"(kp1), "=f"(kn1)
-                : "r"(kw[v]), "r"(p.dare_T16), "f"(d0), "r"(kw[v + 1]), "f"(d1));
-          } else {
-            kp0 = d0 >= thr ? 1.0f : 0.0f;
-            kp1 = d1 >= thr ? 1.0f : 0.0f;
-            kn0 = d0 <= -thr ? 1.0f : 0.0f;
-            kn1 = d1 <= -thr ? 1.0f : 0.0f;
+            keep_signed(kw[v], p.dare_T16, d0, Pp[u][v], Nn[u][v], Cc[u][v]);
+            keep_signed(kw[v + 1], p.dare_T16, d1, Pp[u][v + 1], Nn[u][v + 1], Cc[u][v + 1]);
+            return;
           }
+          float t0, t1;
+          const float kp0 = d0 >= thr ? 1.0f : 0.0f, kp1 = d1 >= thr ? 1.0f : 0.0f;
+          const float kn0 = d0 <= -thr ? 1.0f : 0.0f, kn1 = d1 <= -thr ? 1.0f : 0.0f;
           f2_fma(kp0, kp1, d0, d1, Pp[u][v], Pp[u][v + 1], Pp[u][v], Pp[u][v + 1]);
           f2_fma(kn0, kn1, d0, d1, Nn[u][v], Nn[u][v + 1], Nn[u][v], Nn[u][v + 1]);
-          f2_fma(kn0, kn1, (float)(1u << CB), (float)(1u << CB), kp0, kp1, t0, t1);
-          f2_add(Cc[u][v], Cc[u][v + 1], t0, t1, Cc[u][v], Cc[u][v + 1]);
+          f2_fma(kn0, kn1, (float)(1u << CB), (float)(1u << CB), Cc[u][v], Cc[u][v + 1], t0, t1);
+          f2_add(kp0, kp1, t0, t1, Cc[u][v], Cc[u][v + 1]);
         };
         delta_pairs<BF16>(r, x0[u], fold_pair);
       }
