@@ -1,7 +1,8 @@
 """TIES thresholds at the edges of the sampling rule and of the warp-wide selects.
 
 The sample takes 8, 32 or up to 128 vectors of a block by the number of blocks in its trim
-group (64 or more, 16 or more, fewer); the selects give each lane a run of 4, 8 or 12 bins.
+group (256 or more, 64 or more, fewer), groups of 16 blocks or more get a narrow window; the
+selects give each lane a run of 4, 8, 12 or 20 bins.
 Group sizes on both sides of each line, one-vector tensors, and ranks from the largest key
 (k = 1) to the smallest (k = numel) must give the oracle's thresholds.
 """
@@ -21,7 +22,7 @@ E = 1024
 
 
 @pytest.mark.parametrize("dtype", [synth.BF16, synth.F32], ids=["bf16", "fp32"])
-@pytest.mark.parametrize("n_b", [1, 15, 16, 63, 64, 65])
+@pytest.mark.parametrize("n_b", [1, 15, 16, 63, 64, 65, 255, 256])
 def test_thresholds_at_the_edges_of_the_sampling_rule(n_b, dtype):
     fam = synth.custom([n_b * E - 5, 3, 8, n_b * E // 2 + 1], dtype=dtype, block_elems=E, K=5, active_frac=0.6,
                        name="sample-edges")
