@@ -821,6 +821,14 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
     for (uint32_t q = 0; q < n_groups; ++q)
       h_kth[q] = (unsigned long long)floor((double)op->density * (double)gnumel[q]);
   }
+  // TIES takes its thresholds from predicted windows, TIES after masking where the units' larger
+  // histograms (2.5 KiB) are small against what they count, and fit the device's memory
+  const bool windowed = ties && op->kind == MP_OP_TIES;
+  const bool masked = ties && !windowed;
+  bool units = masked && family->experts_location == 0 && g.n_params >= g.n_blocks * kUnitHistElems;
+  mp_index_s* ix = nullptr;
+  char* m = nullptr;
+  InitList init;
   // the index kernels' work space after the handle's own arrays
   size_t o = 0;
   auto slot = [&](size_t bytes) { size_t r = o; o += align_up(bytes); return r; };
@@ -828,56 +836,56 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
   // counts of finished CTAs; for a host pool one per segment of both walks (any two consecutive
   // segments together exceed segment_elems)
   const size_t n_work = family->experts_location == 0 ? 4 : 2 * (2 * (size_t)(g.n_params / segment_elems(g)) + 2);
-  const size_t o_work = slot(n_work * 8);
+  size_t o_work = 0, o_usum = 0, o_shist = 0, o_scnt = 0, o_spans = 0;
   size_t o_coarse = 0, o_fine = 0, o_kth = 0, o_est = 0, o_rank = 0;
   size_t o_wfine = 0, o_wabove = 0, o_win = 0, o_gmiss = 0, o_miss = 0, o_wend = 0;
-  // TIES takes its thresholds from predicted windows, TIES after masking where the units' larger
-  // histograms (2.5 KiB) are small against what they count
-  const bool windowed = ties && op->kind == MP_OP_TIES;
-  const bool masked = ties && !windowed;
-  const bool units = masked && family->experts_location == 0 && g.n_params >= g.n_blocks * kUnitHistElems;
-  size_t o_usum = 0;
-  if (ties) {
-    o_coarse = slot(units ? 0 : KG * 256 * 8);
-    o_fine = slot(KG * 128 * 8);
-    o_usum = slot(units ? KG * kUnitHistBins * 8 : 0);
-    o_kth = slot(n_groups * 8);
-    o_est = slot(KG * 4);
-    o_rank = slot(KG * 8);
-  }
   // the sampling CTAs' spans: up to span_blocks blocks of one trim group each, 64 for large
   // families and as few as 8 (one per warp) for small ones, so that about 300 CTAs (two per
   // SM) share the sample of a small family too
   std::vector<uint32_t> h_spans;
   uint64_t span_blocks = 64;
   while (span_blocks > 8 && g.n_blocks < span_blocks * 304) span_blocks /= 2;
-  size_t o_shist = 0, o_scnt = 0, o_spans = 0;
-  if (windowed || units) {
-    for (uint32_t q = 0; q < n_groups; ++q) {
-      const uint64_t b0 = scope == 0 ? g.t_first_block[q] : 0;
-      const uint64_t b1 = scope == 0 ? (q + 1 < g.n_tensors ? g.t_first_block[q + 1] : g.n_blocks) : g.n_blocks;
-      for (uint64_t b = b0; b < b1; b += span_blocks) {
-        h_spans.push_back(q);
-        h_spans.push_back((uint32_t)b);
-      }
+  for (;;) {
+    o = 0;
+    h_spans.clear();
+    o_work = slot(n_work * 8);
+    if (ties) {
+      o_coarse = slot(units ? 0 : KG * 256 * 8);
+      o_fine = slot(KG * 128 * 8);
+      o_usum = slot(units ? KG * kUnitHistBins * 8 : 0);
+      o_kth = slot(n_groups * 8);
+      o_est = slot(KG * 4);
+      o_rank = slot(KG * 8);
     }
-    // zeroed together: window counts, keys above, marks, the flag, sampled bins and counts
-    o_wfine = slot(units ? 0 : KG * 384 * 8);
-    o_wabove = slot(units ? 0 : KG * 8);
-    o_gmiss = slot(KG * 4);
-    o_miss = slot(16);
-    o_shist = slot(KG * 1024 * 4);
-    o_scnt = slot(n_groups * 8);
-    o_wend = o;
-    o_win = slot(KG * 4);
-    o_spans = slot(h_spans.size() * 4);
+    if (windowed || units) {
+      for (uint32_t q = 0; q < n_groups; ++q) {
+        const uint64_t b0 = scope == 0 ? g.t_first_block[q] : 0;
+        const uint64_t b1 = scope == 0 ? (q + 1 < g.n_tensors ? g.t_first_block[q + 1] : g.n_blocks) : g.n_blocks;
+        for (uint64_t b = b0; b < b1; b += span_blocks) {
+          h_spans.push_back(q);
+          h_spans.push_back((uint32_t)b);
+        }
+      }
+      // zeroed together: window counts, keys above, marks, the flag, sampled bins and counts
+      o_wfine = slot(units ? 0 : KG * 384 * 8);
+      o_wabove = slot(units ? 0 : KG * 8);
+      o_gmiss = slot(KG * 4);
+      o_miss = slot(16);
+      o_shist = slot(KG * 1024 * 4);
+      o_scnt = slot(n_groups * 8);
+      o_wend = o;
+      o_win = slot(KG * 4);
+      o_spans = slot(h_spans.size() * 4);
+    }
+    st = new_index(g, op, family->experts_location != 0, units ? kUnitHistBins : (masked ? 256u : 0u), o, cs, init, &ix, &m);
+    if (st == MP_OK) break;
+    // without the memory for the larger histograms: the smaller ones
+    size_t fr = 0, total = 0;
+    if (st != MP_ERR_OOM || !units || cudaMemGetInfo(&fr, &total) != cudaSuccess ||
+        fr >= o + (uint64_t)g.K * g.n_blocks * kUnitHistBins * 4)
+      return st;
+    units = false;
   }
-  mp_index_s* ix = nullptr;
-  char* m = nullptr;
-  InitList init;
-  if ((st = new_index(g, op, family->experts_location != 0, units ? kUnitHistBins : (masked ? 256u : 0u), o, cs, init,
-                      &ix, &m)) != MP_OK)
-    return st;
 
   cudaError_t e;
   auto bail = [&](cudaError_t err, const char* what) {

@@ -48,3 +48,39 @@ def test_sample_that_misleads():
         x = torch.from_numpy((base.astype(np.uint32) << 16).view(np.float32) + d)
         experts[i] = x.to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
     run_case(fam, base, experts, ("ties_masked", "ties_masked1"), [0.1, 0.5, 1.0])
+
+
+def test_little_memory_takes_the_smaller_histograms():
+    """1.28 million units: 3.3 GB with the larger histograms, 1.3 GB with the smaller ones; with 2.4 GB
+    free the catalog takes the latter, and the thresholds, the plan and the output are the same"""
+    import torch
+
+    import paper_2605_29489_gb300 as mp
+
+    n, K = 2048 * 40000, 32
+    g = torch.Generator(device="cuda").manual_seed(5)
+    base = torch.randn(n, generator=g, device="cuda").mul_(0.02).to(torch.bfloat16)
+    expert = (base.float() + 1e-3 * torch.randn(n, generator=g, device="cuda")).to(torch.bfloat16)
+    fam = mp.family([(0, n // 2), (n // 2, n // 2)], base, [expert] * K, 2048, mp.MP_BF16, 0)
+    op = mp.make_op(mp.MP_OP_TIES_MASKED, lam=1.0, density=0.2)
+
+    def run():
+        out = torch.zeros_like(base)
+        with mp.mp_index_blocks(fam, op) as idx:
+            torch.cuda.synchronize()
+            free = torch.cuda.mem_get_info()[0]
+            tau = mp.mp_index_stats(idx)[3]
+            with mp.mp_plan(idx, op, mp.mp_budget_from_fraction(fam, 0.3)) as plan:
+                with mp.mp_merge(fam, idx, plan, out) as man:
+                    digest = mp.mp_manifest_info(man, K)["digest"]
+        return tau, digest, out, free
+
+    tau, digest, out, _ = run()
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (2400 << 20), dtype=torch.uint8, device="cuda")
+    tau2, digest2, out2, free = run()
+    assert free > 512 << 20  # the larger histograms would not have fitted
+    del hold
+    assert np.array_equal(tau, tau2) and digest == digest2
+    assert torch.equal(out.view(torch.int16), out2.view(torch.int16))
