@@ -607,7 +607,6 @@ struct __align__(128) TcSmem {
   // -c and RN(1/c) for the counts c = 0..32 (entry 0: -1, 1); apart, so that two elements' entries
   // load into the register pairs that the packed operations take
   float nneg[kTcMaxK + 1], nrcp[kTcMaxK + 1];
-  uint32_t nf[NS];           // producer only: fills held by the group of each entry
   int abort, last;
 };
 
@@ -680,6 +679,12 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
     uint32_t seq = 0;   // groups published
     uint32_t head = 0;  // oldest published group not yet seen released
     uint32_t used = 0;  // slots held by groups head .. seq - 1
+    // Lane e: the fills held by the group of entry e, read by a shuffle.  (In shared memory a lane that
+    // lagged behind in reserve() could read the count that lane 0 had written for the next group of the
+    // same entry: with all entries outstanding, as in a run of chunks that select no expert, the entry
+    // just freed is the one published next.)
+    static_assert(NS <= 32, "one lane per entry");
+    uint32_t nf = 0;
     bool ok = true;
     // wait until entry seq % NS is free and nfill slots are free; groups are released in order,
     // so the oldest one is the next to free its slots
@@ -687,7 +692,7 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
       while (seq - head >= (uint32_t)NS || used + nfill > (uint32_t)NS) {
         const uint32_t he = head % NS;
         if (!warp_wait(&S.empty[he], (head / NS) & 1u, abort_flag, wl)) return false;
-        used -= S.nf[he];
+        used -= __shfl_sync(0xFFFFFFFFu, nf, (int)he);
         ++head;
       }
       return true;
@@ -776,8 +781,8 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
               ce.flags = (first ? kFirst : 0u) | (done + nexp == nsel ? kLast : 0u) | (nsel ? 0u : kNone) | fast;
               ce.s0 = fill % NS;
               ce.nexp = nexp;
-              S.nf[e] = nfill;
             }
+            if (lane == e) nf = nfill;
             __syncwarp();  // the entry is written before it is published
             // test hook: the first group is never armed, so the consumers' wait for it runs out
             const bool arm = !(seq == 0 && p.stall);
@@ -806,7 +811,6 @@ __global__ void __launch_bounds__(TcGeo<OPC, KC>::kThreads, TcGeo<OPC, KC>::kCta
       const uint32_t e = seq % NS;
       if (lane == 0) {
         S.ce[e].flags = kEndGroup;
-        S.nf[e] = 0u;
         if (!(seq == 0 && p.stall)) mbar_arrive_expect_tx(&S.full[e], 0u);
       }
       ++seq;

@@ -66,3 +66,40 @@ def test_chunks_taken_one_two_and_three_at_a_time(n_blocks, K):
                        name=f"grabs-{n_blocks}")
     base, experts = fam.host_arrays()
     run_case(fam, base, experts, ("ta", "ties", "dare", "avg_renorm", "dare_ties"), [0.4])
+
+
+@pytest.mark.parametrize("K", [3, 6, 11])
+def test_long_runs_of_chunks_that_select_no_expert(K):
+    """blocks that differ from the base 12 blocks apart, so that between two of them a CTA's ring is
+    held by one-slot groups only: every group entry is then outstanding, and the entry just released
+    is the one published next.  Repeated, because what can go wrong there depends on timing."""
+    E, nb = 65536, 733
+    n = nb * E - 1001
+    g = torch.Generator(device="cuda").manual_seed(K)
+    base = torch.randn(n, generator=g, device="cuda").mul_(0.02).to(torch.bfloat16)
+    experts = [base.clone() for _ in range(K)]
+    active = sorted({*range(5, nb, 12), nb - 1})
+    for i, x in enumerate(experts):
+        for b in active[i % 2::2] if i else active:
+            v = x[b * E:(b + 1) * E]
+            v.copy_((v.float() + 1e-3 * torch.randn(v.numel(), generator=g, device="cuda")).to(torch.bfloat16))
+    fam = mp.family([(0, n)], base, experts, E, mp.MP_BF16, 0)
+    raw = lambda t: t.view(torch.int16).cpu().numpy().view(np.uint16)  # noqa: E731
+    untouched = (base.float() + 0.0).to(torch.bfloat16)  # M_0 plus the zero that the operator adds
+    kw = dict(lam=0.8, density=0.02, drop_p=0.5, seed=3, alpha=[1.0 / K] * K)
+    for gk, ok in [(mp.MP_OP_TIES, oracle.TIES), (mp.MP_OP_DARE, oracle.DARE), (mp.MP_OP_DARE_TIES, oracle.DARE_TIES)]:
+        gop, oop = mp.make_op(gk, **kw), oracle.Op(ok, K, **kw)
+        with mp.mp_index_blocks(fam, gop) as idx, mp.mp_plan(idx, gop, mp.mp_budget_from_fraction(fam, 1.0)) as plan:
+            pi = mp.mp_plan_info(plan, idx)
+            tau = mp.mp_index_stats(idx)[3][:, 0] if gk == mp.MP_OP_TIES else None
+            want = untouched.clone()
+            for b in np.nonzero(pi["mask"])[0]:
+                s = slice(int(b) * E, min((int(b) + 1) * E, n))
+                w = oracle.merge_block(synth.BF16, s.start, raw(base[s]), [raw(x[s]) for x in experts],
+                                       int(pi["mask"][b]), oop, tau)
+                want[s].copy_(torch.from_numpy(w.view(np.int16)).view(torch.bfloat16))
+            for it in range(10):
+                out = torch.full_like(base, float("nan"))
+                with mp.mp_merge(fam, idx, plan, out) as man:
+                    assert mp.mp_manifest_info(man, K)["realized_total"] == pi["chat"], (gk, it)
+                assert torch.equal(out.view(torch.int16), want.view(torch.int16)), (gk, it)
