@@ -35,7 +35,8 @@
  *    catalog, the plans and the merges from the buffers' current contents into the
  *    handles made during the capture.  The accessors of those handles then wait for
  *    the whole device (a captured event cannot be waited for from the host).  Free
- *    such handles before the graph is destroyed.  Host-resident pools, TIES after
+ *    such handles before the graph is destroyed; a handle made before the capture that a captured
+ *    call uses is needed by every replay, and mp_free does not wait for replays.  Host-resident pools, TIES after
  *    masking and mp_index_import are not capturable.  Errors found by a kernel (a
  *    non-finite delta, a timed-out wait) are reported by the next accessor on
  *    that handle or on a handle derived from it.
@@ -312,8 +313,10 @@ mp_status mp_plan_noalloc(uint32_t K, uint64_t n_blocks, uint32_t n_groups, mp_d
                           const uint32_t* index_err, const mp_op* op, uint64_t budget_bytes,
                           uint32_t* mask, uint32_t* order, uint64_t* summary, mp_stream stream);
 
-/* Release an mp_index, mp_plan_t or mp_manifest (waits for its pending work).  NULL is a
-   no-op.  Passing anything else is undefined. */
+/* Release an mp_index, mp_plan_t or mp_manifest.  Waits for its pending work and for that of the
+   calls enqueued on it (the plans, merges, hashes and validations that read an index or a plan),
+   so a handle may be freed at any time after the calls that use it have returned.  NULL is a no-op.
+   Passing anything else is undefined. */
 void mp_free(void* handle);
 
 /* Host copies of the index statistics, expert-major [K][n_blocks]; tau is [K][n_groups]

@@ -6,8 +6,10 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -173,8 +175,11 @@ mp_status dev_alloc(Alloc& a, size_t bytes, cudaStream_t st) {
   return MP_OK;
 }
 
+// Memory of a stream-ordered pool goes back as it is: cudaFree does not wait for the work that uses
+// it, and the pool hands it to the next call on any stream.  So every caller has waited for that work
+// before (mp_free for the handle's own and for its users, the failure paths for the stream).
 void dev_free(Alloc& a) {
-  if (a.ptr) cudaFree(a.ptr);  // synchronising free: no pending work can still use it
+  if (a.ptr) cudaFree(a.ptr);
   a.ptr = nullptr;
 }
 
@@ -335,9 +340,60 @@ cudaError_t stream_wait(cudaStream_t cs, cudaEvent_t ev, bool ev_captured, bool 
   return cudaSuccess;
 }
 
-cudaError_t wait_handle(cudaEvent_t done, bool captured) {
+cudaError_t wait_handle(const Event& done, bool captured) {
   if (captured) return cudaDeviceSynchronize();
-  return done ? cudaEventSynchronize(done) : cudaSuccess;
+  return done ? done.sync() : cudaSuccess;
+}
+
+Event::Box::~Box() {
+  if (e) cudaEventDestroy(e);
+}
+
+cudaError_t Event::make(bool again) {
+  try {
+    p = std::make_shared<Box>();
+  } catch (const std::bad_alloc&) {
+    return cudaErrorMemoryAllocation;
+  }
+  p->again = again;
+  const cudaError_t r = cudaEventCreateWithFlags(&p->e, cudaEventDisableTiming);
+  if (r != cudaSuccess) p.reset();
+  return r;
+}
+
+cudaError_t Event::sync() const {
+  if (over()) return cudaSuccess;
+  const cudaError_t r = cudaEventSynchronize(p->e);
+  if (r == cudaSuccess && !p->again) p->over.store(true, std::memory_order_release);
+  return r;
+}
+
+// from so many remembered calls on, the runtime is asked which of them are done
+constexpr size_t kUsersKept = 16;
+
+void Users::add(const Event& e) {
+  std::lock_guard<std::mutex> lk(mu);
+  auto forget = [&](auto is_done) { ev.erase(std::remove_if(ev.begin(), ev.end(), is_done), ev.end()); };
+  forget([&](const Event& x) { return x == e || x.over(); });
+  if (ev.size() >= kUsersKept) {
+    // an event query is refused while another thread captures in global mode
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    forget([](const Event& x) { return cudaEventQuery(x.get()) == cudaSuccess; });
+    cudaGetLastError();  // of those that are not done
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  try {
+    ev.push_back(e);
+  } catch (const std::bad_alloc&) {
+    e.sync();  // nothing to remember then
+  }
+}
+
+void Users::wait() {
+  std::lock_guard<std::mutex> lk(mu);
+  for (const Event& x : ev) x.sync();
+  ev.clear();
 }
 
 mp_status cuda_fail(cudaError_t e, const char* what) {
@@ -677,7 +733,6 @@ mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, uint32_t
   ix->trim_scope = scope;
   ix->n_groups = n_groups;
   ix->has_missing = false;
-  ix->done = nullptr;
   ix->captured = capturing(cs);
   ix->order_captured = false;
   ix->order_ready = nullptr;
@@ -736,8 +791,8 @@ mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, uint32_t
 // the handle is complete once the stream reaches this point
 cudaError_t finish_index(mp_index_s* ix, cudaStream_t cs) {
   cudaError_t e;
-  if ((e = cudaEventCreateWithFlags(&ix->done, cudaEventDisableTiming)) != cudaSuccess) return e;
-  return cudaEventRecord(ix->done, cs);
+  if ((e = ix->done.make(true)) != cudaSuccess) return e;
+  return cudaEventRecord(ix->done.get(), cs);
 }
 
 // the catalog's hash arrays (base, then K experts), allocated once per index
@@ -759,7 +814,6 @@ void discard_index(mp_index_s* ix, cudaStream_t cs) {
   dev_free(ix->hash_mem);
   dev_free(ix->order_mem);
   dev_free(ix->mem);
-  if (ix->done) cudaEventDestroy(ix->done);
   if (ix->order_ready) cudaEventDestroy(ix->order_ready);
   delete ix->order_mu;
   delete ix;
@@ -1067,7 +1121,6 @@ mp_status mp_plan(const mp_index* index, const mp_op* op, uint64_t budget_bytes,
   pl->seed = op->seed;
   pl->budget = budget_bytes;
   pl->n_groups = index->n_groups;
-  pl->done = nullptr;
   pl->captured = capturing(cs);
   pl->h_summary = static_cast<uint64_t*>(pin_get(64));
   if (!pl->h_summary) {
@@ -1094,12 +1147,11 @@ mp_status mp_plan(const mp_index* index, const mp_op* op, uint64_t budget_bytes,
     if (scratch.ptr) cudaFree(scratch.ptr);
     dev_free(pl->mem);
     pin_put(pl->h_summary, 64);
-    if (pl->done) cudaEventDestroy(pl->done);
     delete pl;
     return r;
   };
   cudaError_t e;
-  if ((e = stream_wait(cs, index->done, index->captured, pl->captured)) != cudaSuccess) return bail(e, "stream wait");
+  if ((e = stream_wait(cs, index->done.get(), index->captured, pl->captured)) != cudaSuccess) return bail(e, "stream wait");
   const uint64_t n_pairs = index->has_missing ? (uint64_t)g.K * g.n_tensors : 0ull;
   if ((e = malloc_async(&scratch.ptr, plan_scratch_bytes(U, n_pairs), cs)) != cudaSuccess) {
     scratch.ptr = nullptr;
@@ -1181,8 +1233,9 @@ mp_status mp_plan(const mp_index* index, const mp_op* op, uint64_t budget_bytes,
   }
   if ((e = cudaFreeAsync(scratch.ptr, cs)) != cudaSuccess) return bail(e, "free scratch");
   scratch.ptr = nullptr;
-  if ((e = cudaEventCreateWithFlags(&pl->done, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "event");
-  if ((e = cudaEventRecord(pl->done, cs)) != cudaSuccess) return bail(e, "event record");
+  if ((e = pl->done.make()) != cudaSuccess) return bail(e, "event");
+  if ((e = cudaEventRecord(pl->done.get(), cs)) != cudaSuccess) return bail(e, "event record");
+  if (!pl->captured) index->users.add(pl->done);
   *out = pl;
   return MP_OK;
 }
@@ -1238,9 +1291,7 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
   mf->device = plan->device;
   mf->K = g.K;
   mf->n_blocks = g.n_blocks;
-  mf->done = nullptr;
   mf->captured = capturing(cs);
-  mf->valid_done = nullptr;
   for (uint32_t i = 0; i <= kMaxK; ++i) mf->lineage[i] = (family->lineage_ids && i <= g.K) ? family->lineage_ids[i] : 0u;
   const size_t counters_bytes = (size_t)kCounterSlots * g.K * 8;
   // the counters (64 slots x K), the plan summary, the error word and the TIES_MASKED
@@ -1277,13 +1328,12 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
     cudaStreamSynchronize(cs);
     dev_free(mf->mem);
     release_pinned();
-    if (mf->done) cudaEventDestroy(mf->done);
     delete mf;
     return r;
   };
   cudaError_t e;
-  if ((e = stream_wait(cs, index->done, index->captured, mf->captured)) != cudaSuccess) return bail(e, "stream wait");
-  if ((e = stream_wait(cs, plan->done, plan->captured, mf->captured)) != cudaSuccess) return bail(e, "stream wait");
+  if ((e = stream_wait(cs, index->done.get(), index->captured, mf->captured)) != cudaSuccess) return bail(e, "stream wait");
+  if ((e = stream_wait(cs, plan->done.get(), plan->captured, mf->captured)) != cudaSuccess) return bail(e, "stream wait");
   if ((e = launch_fill(mf->mem.ptr, 0, zero_bytes, cs)) != cudaSuccess) return bail(e, "fill");
   uint32_t* masked_tau = nullptr;
   if (masked) {
@@ -1382,8 +1432,12 @@ mp_status merge_common(const mp_family* family, const mp_index* index, const mp_
       return bail(cudaErrorInvalidValue, "an index of a host-resident pool is needed for a host-pool merge");
     if ((e = merge_host_pool(p, index, cs)) != cudaSuccess) return bail(e, "merge (host pool)");
   }
-  if ((e = cudaEventCreateWithFlags(&mf->done, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "event");
-  if ((e = cudaEventRecord(mf->done, cs)) != cudaSuccess) return bail(e, "event record");
+  if ((e = mf->done.make()) != cudaSuccess) return bail(e, "event");
+  if ((e = cudaEventRecord(mf->done.get(), cs)) != cudaSuccess) return bail(e, "event record");
+  if (!mf->captured) {
+    index->users.add(mf->done);
+    plan->users.add(mf->done);
+  }
   *man_out = mf;
   return MP_OK;
 }
@@ -1408,9 +1462,9 @@ void mp_free(void* handle) {
   if (magic == kMagicIndex) {
     mp_index_s* ix = static_cast<mp_index_s*>(handle);
     wait_handle(ix->done, ix->captured);
-    if (ix->done) cudaEventDestroy(ix->done);
+    ix->users.wait();
     if (ix->order_ready) {
-      wait_handle(ix->order_ready, ix->order_captured);
+      if (ix->order_captured) cudaDeviceSynchronize();  // else the plan that recorded it is among the users
       cudaEventDestroy(ix->order_ready);
     }
     dev_free(ix->hash_mem);
@@ -1423,7 +1477,7 @@ void mp_free(void* handle) {
   } else if (magic == kMagicPlan) {
     mp_plan_s* pl = static_cast<mp_plan_s*>(handle);
     wait_handle(pl->done, pl->captured);
-    if (pl->done) cudaEventDestroy(pl->done);
+    pl->users.wait();
     dev_free(pl->mem);
     pin_put(pl->h_summary, 64);
     pl->magic = 0;
@@ -1431,8 +1485,7 @@ void mp_free(void* handle) {
   } else if (magic == kMagicManifest) {
     mp_manifest_s* mf = static_cast<mp_manifest_s*>(handle);
     wait_handle(mf->done, mf->captured);
-    if (mf->done) cudaEventDestroy(mf->done);
-    if (mf->valid_done) cudaEventSynchronize(mf->valid_done), cudaEventDestroy(mf->valid_done);
+    if (mf->valid_done) mf->valid_done.sync();
     dev_free(mf->valid_mem);
     dev_free(mf->mem);
     pin_put(mf->h_realized, (size_t)kCounterSlots * mf->K * 8 + 64 + 16 + 16);
@@ -1536,7 +1589,8 @@ mp_status mp_index_hashes(const mp_family* family, mp_index* index, mp_stream st
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
   cudaError_t e;
   // after whatever built the index; the index's event then covers the hashes too
-  if (index->done && (e = cudaStreamWaitEvent(cs, index->done, 0)) != cudaSuccess) return cuda_fail(e, "stream wait");
+  if (index->done && (e = cudaStreamWaitEvent(cs, index->done.get(), 0)) != cudaSuccess)
+    return cuda_fail(e, "stream wait");
   if ((st = alloc_hashes(index, cs)) != MP_OK) return st;
   HashLaunch p;
   memset(&p, 0, sizeof(p));
@@ -1552,7 +1606,7 @@ mp_status mp_index_hashes(const mp_family* family, mp_index* index, mp_stream st
   p.ext = Extents{g.span_elems, g.span_elems};
   p.err = index->d_err;
   if ((e = launch_hash(p, cs)) != cudaSuccess) return cuda_fail(e, "hash kernel");
-  if ((e = cudaEventRecord(index->done, cs)) != cudaSuccess) return cuda_fail(e, "event record");
+  if ((e = cudaEventRecord(index->done.get(), cs)) != cudaSuccess) return cuda_fail(e, "event record");
   return MP_OK;
 }
 
@@ -1597,8 +1651,15 @@ mp_status mp_manifest_validate(const mp_family* family, const mp_index* index, c
     man->d_out_hash = man->d_vresult + 4;
   }
   // after the merge (its output) and the index's own work (the hashes, perhaps added later)
-  if ((e = cudaStreamWaitEvent(cs, man->done, 0)) != cudaSuccess) return cuda_fail(e, "stream wait");
-  if ((e = cudaStreamWaitEvent(cs, index->done, 0)) != cudaSuccess) return cuda_fail(e, "stream wait");
+  if ((e = cudaStreamWaitEvent(cs, man->done.get(), 0)) != cudaSuccess) return cuda_fail(e, "stream wait");
+  if ((e = cudaStreamWaitEvent(cs, index->done.get(), 0)) != cudaSuccess) return cuda_fail(e, "stream wait");
+  // and after an earlier validation, which wrote the same results (and whose end valid_done marks so far)
+  const bool now_captured = capturing(cs);
+  if (man->valid_done && !man->valid_captured && !now_captured &&
+      (e = cudaStreamWaitEvent(cs, man->valid_done.get(), 0)) != cudaSuccess)
+    return cuda_fail(e, "stream wait");
+  Event valid_done = man->valid_done;  // made before the launch, so that what is enqueued has an end to wait for
+  if (!valid_done && (e = valid_done.make(true)) != cudaSuccess) return cuda_fail(e, "event");
   if ((e = cudaMemsetAsync(man->d_vresult, 0, 16, cs)) != cudaSuccess) return cuda_fail(e, "memset");
   if ((e = cudaMemsetAsync(man->d_vresult + 2, 0xFF, 8, cs)) != cudaSuccess) return cuda_fail(e, "memset");
   HashLaunch p;
@@ -1620,9 +1681,13 @@ mp_status mp_manifest_validate(const mp_family* family, const mp_index* index, c
   p.ext = Extents{g.span_elems, g.span_elems};
   p.err = man->d_err;
   if ((e = launch_hash(p, cs)) != cudaSuccess) return cuda_fail(e, "hash kernel");
-  if (!man->valid_done && (e = cudaEventCreateWithFlags(&man->valid_done, cudaEventDisableTiming)) != cudaSuccess)
-    return cuda_fail(e, "event");
-  if ((e = cudaEventRecord(man->valid_done, cs)) != cudaSuccess) return cuda_fail(e, "event record");
+  if ((e = cudaEventRecord(valid_done.get(), cs)) != cudaSuccess) return cuda_fail(e, "event record");
+  man->valid_done = valid_done;
+  man->valid_captured = now_captured;
+  if (!now_captured) {
+    index->users.add(man->valid_done);
+    plan->users.add(man->valid_done);
+  }
   return MP_OK;
 }
 
@@ -1631,7 +1696,7 @@ mp_status mp_manifest_validation(const mp_manifest* man, uint64_t* checked, uint
   if ((st = check_handle(man, kMagicManifest, "manifest")) != MP_OK) return st;
   if (!man->valid_done) return fail(MP_ERR_INVALID_ARG, "the manifest was not validated (mp_manifest_validate)");
   cudaError_t e;
-  if ((e = cudaEventSynchronize(man->valid_done)) != cudaSuccess) return cuda_fail(e, "validation work");
+  if ((e = man->valid_done.sync()) != cudaSuccess) return cuda_fail(e, "validation work");
   unsigned long long r[3];
   if ((e = cudaMemcpy(r, man->d_vresult, sizeof(r), cudaMemcpyDeviceToHost)) != cudaSuccess) return cuda_fail(e, "copy");
   uint32_t err = 0;

@@ -5,8 +5,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <string>
+#include <atomic>
+#include <memory>
 #include <mutex>
+#include <string>
 #include <utility>
 #include <vector>
 
@@ -59,6 +61,42 @@ struct Alloc {
   cudaStream_t stream = nullptr;
 };
 
+// a timing-less event, shared between the handle whose work it ends and the handles which that
+// work uses; destroyed with the last of them
+class Event {
+ public:
+  // again: the event may be recorded more than once (what has been waited for is not remembered then)
+  cudaError_t make(bool again = false);
+  cudaError_t sync() const;  // waits on the host; no runtime call once that has succeeded
+  bool over() const { return p->over.load(std::memory_order_acquire); }
+  cudaEvent_t get() const { return p ? p->e : nullptr; }
+  explicit operator bool() const { return (bool)p; }
+  bool operator==(const Event& o) const { return p == o.p; }
+
+ private:
+  struct Box {
+    cudaEvent_t e = nullptr;
+    bool again = false;
+    std::atomic<bool> over{false};
+    ~Box();
+  };
+  std::shared_ptr<Box> p;
+};
+
+// The ends of the calls that use a handle's device memory (the plans, merges, hashes and validations
+// enqueued on it), which mp_free waits for before the memory goes back to the pool.  Calls under
+// stream capture are not among them: their events cannot be waited for from the host, and a
+// graph's replays need its handles anyway.
+class Users {
+ public:
+  void add(const Event& e);
+  void wait();
+
+ private:
+  std::mutex mu;
+  std::vector<Event> ev;
+};
+
 }  // namespace mp
 
 struct mp_index_s {
@@ -99,7 +137,8 @@ struct mp_index_s {
   uint32_t* d_nnz;         // [K][n_blocks]
   uint32_t* d_tau;         // [K][n_groups] (TIES only)
   uint32_t* d_err;         // error word
-  cudaEvent_t done;
+  mp::Event done;
+  mutable mp::Users users;
   bool captured;           // built under stream capture: waits go through the device
   std::vector<std::pair<void*, size_t>> pinned;  // pinned staging of the uploads (released by mp_free)
   std::vector<uint64_t> h_blk_off;  // host copy of the block table (segments of a host pool)
@@ -125,7 +164,8 @@ struct mp_plan_s {
   uint32_t* d_order;       // [K*n_blocks] traversal order (first n_cand valid)
   uint64_t* d_summary;     // [8] chat, n_sel, n_cand, set_hash, digest, touched, err, pad
   uint64_t* h_summary;     // pinned host copy of d_summary
-  cudaEvent_t done;
+  mp::Event done;
+  mutable mp::Users users;
   bool captured;           // built under stream capture: waits go through the device
 };
 
@@ -141,7 +181,7 @@ struct mp_manifest_s {
   uint32_t* h_err;
   uint64_t planned, touched, digest;
   uint64_t lineage[mp::kMaxK + 1];  // caller ids of M_0..M_K (zeros when none were given)
-  cudaEvent_t done;
+  mp::Event done;
   bool captured;                    // built under stream capture: waits go through the device
   // hash validation (mp_manifest_validate): checked / mismatched / first bad item, and
   // the output's block hashes
@@ -149,7 +189,8 @@ struct mp_manifest_s {
   unsigned long long* d_vresult;   // [3]
   unsigned long long* d_out_hash;  // [n_blocks]
   uint64_t n_blocks;
-  cudaEvent_t valid_done;
+  mp::Event valid_done;
+  bool valid_captured;             // the validation was enqueued under stream capture
 };
 
 namespace mp {

@@ -68,3 +68,45 @@ def test_threads_on_their_own_streams():
     for t in ts:
         t.join()
     assert not bad
+
+
+@pytest.mark.parametrize("kind", ["ties", "ties_masked", "dare"])
+def test_handles_freed_while_a_merge_runs(kind):
+    """index and plan are freed as soon as the merge is enqueued, and other calls on a second stream
+    take memory at once: the free waits for the merge, whose output and manifest are what they are
+    when the handles are kept"""
+    g = torch.Generator(device="cuda").manual_seed(11)
+    n, K, E = 40_000_000 - 123, 4, 16384
+    base = torch.randn(n, generator=g, device="cuda").mul_(0.02).to(torch.bfloat16)
+    experts = [(base.float() + 1e-3 * torch.randn(n, generator=g, device="cuda")).to(torch.bfloat16) for _ in range(K)]
+    fam = mp.family([(0, n)], base, experts, E, mp.MP_BF16, 0)
+    other = mp.family([(0, n // 8)], experts[0], experts[1:3], 4096, mp.MP_BF16, 0)
+    op = {"ties": mp.make_op(mp.MP_OP_TIES, density=0.2), "ties_masked": mp.make_op(mp.MP_OP_TIES_MASKED, density=0.2),
+          "dare": mp.make_op(mp.MP_OP_DARE, alpha=[0.25] * K, drop_p=0.5, seed=2)}[kind]
+    B = mp.mp_budget_from_fraction(fam, 0.4)
+
+    def read(out, man):
+        mi = mp.mp_manifest_info(man, K)
+        return out.view(torch.int16).clone(), mi["digest"], mi["realized"].tolist()
+
+    out = torch.empty_like(base)
+    with mp.mp_index_blocks(fam, op) as idx, mp.mp_plan(idx, op, B) as plan, mp.mp_merge(fam, idx, plan, out) as man:
+        want = read(out, man)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    out2 = torch.empty_like(experts[0])
+    for it in range(8):
+        out.fill_(float("nan"))
+        torch.cuda.synchronize()
+        idx = mp.mp_index_blocks(fam, op, stream=s1)
+        plan = mp.mp_plan(idx, op, B, stream=s1)
+        man = mp.mp_merge(fam, idx, plan, out, stream=s1)
+        for h in ((idx, plan) if it % 2 else (plan, idx)):
+            h.free()
+        assert s1.query(), it  # nothing that reads them is left
+        with mp.mp_index_blocks(other, mp.make_op(mp.MP_OP_TIES, density=0.1), stream=s2) as i2:
+            p2 = mp.mp_plan(i2, mp.make_op(mp.MP_OP_TIES, density=0.1), 1 << 24, stream=s2)
+            m2 = mp.mp_merge(other, i2, p2, out2, stream=s2)
+            got = read(out, man)
+            assert torch.equal(got[0], want[0]) and got[1:] == want[1:], it
+            for h in (m2, p2, man):
+                h.free()

@@ -1,0 +1,124 @@
+"""The library's host code on a CUDA runtime without a device (CPU).
+
+The library's own sources are linked against `probes/fake_cudart.cpp`, where kernels do nothing, work on a
+stream is done only when something waits for it, and device memory is host memory against a limit.
+What the host code waits for, which allocations it makes and which launches it chooses can then be
+seen without a GPU, also for what must not be tried on one: memory handed back while a kernel
+may still read it, a device that is nearly full, a planner that gives up.
+"""
+import concurrent.futures as cf
+import ctypes
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_2605_29489_gb300 as mp
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+OOM, TIMEOUT = -3, -6
+DEVICE_GB = 280
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    from paper_2605_29489_gb300 import build
+
+    d = str(tmp_path_factory.mktemp("fake_runtime"))
+    srcs = sorted(glob.glob(os.path.join(build.CSRC, "*.cu"))) + [os.path.join(HERE, "probes", "fake_cudart.cpp")]
+    objs = [os.path.join(d, os.path.basename(s) + ".o") for s in srcs]
+    # PTX only: nothing here is run on a device
+    flags = ["-gencode", "arch=compute_103a,code=compute_103a", "-std=c++17", "-O1", "-Xcompiler", "-fPIC",
+             "--expt-relaxed-constexpr", "-I", build.INCLUDE, "-I", build.CSRC]
+    with cf.ThreadPoolExecutor(max_workers=os.cpu_count() or 4) as ex:
+        list(ex.map(lambda so: subprocess.check_call([build.nvcc(), *flags, "-c", so[0], "-o", so[1]]), zip(srcs, objs)))
+    path = os.path.join(d, "libmergepipe_fake.so")
+    subprocess.check_call(["g++", "-shared", "-Wl,-Bsymbolic", "-o", path, *objs])
+    return path
+
+
+@pytest.fixture
+def rt(fake_lib, monkeypatch):
+    """the package's binding over the library on the fake runtime; the runtime's own controls"""
+    monkeypatch.setattr(mp, "library_path", lambda: fake_lib)
+    monkeypatch.setattr(mp, "_lib", None)
+    L = mp.lib()
+    for n in ("fake_used", "fake_pending", "fake_most_pending_at_free"):
+        getattr(L, n).restype = ctypes.c_uint64
+    L.fake_memory.argtypes = [ctypes.c_size_t, ctypes.c_size_t]
+    L.fake_launched.argtypes = [ctypes.c_char_p]
+    L.cudaDeviceSynchronize()
+    L.fake_reset()
+    yield L
+    mp.mp_debug_inject_fault(mp.MP_FAULT_ALLOC, 0)
+
+
+def family(n_blocks=64, K=3, block=4096, tail=0):
+    """no data is read: the kernels do nothing"""
+    buf = np.zeros(64, np.uint8)
+    p = (buf.ctypes.data + 15) & ~15
+    n = n_blocks * block - tail
+    far = [p + 16 * n * (i + 1) for i in range(K + 1)]  # the buffers do not overlap the output
+    fam = mp.family([(0, n)], p, far[:K], block, mp.MP_BF16, 0)
+    fam.keep = buf
+    return fam, far[K]
+
+
+S1, S2 = 0x1000, 0x2000
+TA = lambda K: mp.make_op(mp.MP_OP_TA, alpha=[0.5] * K)  # noqa: E731
+
+
+# ---- a handle's memory goes back only when nothing reads it any more --------------------------
+
+def test_freeing_waits_for_the_calls_that_use_the_handle(rt):
+    """index and plan freed right after a merge was enqueued, on the merge's stream and on another: what
+    they hold is read by kernels that have not run"""
+    for plan_stream, merge_stream in ((S1, S1), (S1, S2), (S2, S1)):
+        for first in ("index", "plan"):
+            fam, out = family()
+            idx = mp.mp_index_blocks(fam, TA(3), stream=S1)
+            plan = mp.mp_plan(idx, TA(3), 1 << 20, stream=plan_stream)
+            man = mp.mp_merge(fam, idx, plan, out, stream=merge_stream)
+            assert rt.fake_pending() > 0
+            for h in ((idx, plan) if first == "index" else (plan, idx)):
+                h.free()
+            assert rt.fake_most_pending_at_free() == 0, (plan_stream, merge_stream, first)
+            man.free()
+
+
+def test_freeing_an_index_waits_for_plans_hashes_and_validation(rt):
+    fam, out = family()
+    idx = mp.mp_index_blocks(fam, TA(3), stream=S1)
+    plan = mp.mp_plan(idx, TA(3), 1 << 20, stream=S2)
+    idx.free()
+    assert rt.fake_most_pending_at_free() == 0
+    plan.free()
+
+    idx = mp.mp_index_blocks(fam, TA(3), stream=S1)
+    mp.mp_index_hashes(fam, idx, stream=S2)
+    plan = mp.mp_plan(idx, TA(3), 1 << 20, stream=S1)
+    man = mp.mp_merge(fam, idx, plan, out, stream=S1)
+    mp.mp_manifest_info(man, 3, check=False)
+    mp.mp_manifest_validate(fam, idx, plan, out, man, stream=S1)
+    mp.mp_manifest_validate(fam, idx, plan, out, man, stream=S2)
+    plan.free()
+    assert rt.fake_most_pending_at_free() == 0
+    idx.free()
+    man.free()
+    assert rt.fake_most_pending_at_free() == 0
+
+
+def test_one_index_used_by_many_merges_keeps_few_events(rt):
+    """a long-lived index: the calls that are done are forgotten"""
+    fam, out = family()
+    idx = mp.mp_index_blocks(fam, TA(3), stream=S1)
+    for _ in range(300):
+        plan = mp.mp_plan(idx, TA(3), 1 << 20, stream=S1)
+        man = mp.mp_merge(fam, idx, plan, out, stream=S2)
+        for h in (man, plan):
+            h.free()
+    used = rt.fake_used()
+    idx.free()
+    assert rt.fake_used() < used and rt.fake_most_pending_at_free() == 0
