@@ -341,7 +341,7 @@ mp_status mp_plan_info(const mp_plan_t* plan, uint64_t* planned_bytes, uint64_t*
 /* Manifest (waits for the merge): realized expert-read bytes per expert (K words),
    their total, touched blocks (#{b : mask_b != 0}) and the plan digest.  Errors:
    MP_ERR_INVALID_ARG (not a manifest), MP_ERR_TIMEOUT (a bounded device wait in the merge
-   gave up), MP_ERR_CUDA (the merge kernels reported another error), MP_ERR_BUDGET (realized
+   gave up, or in the index or planner kernels of its plan), MP_ERR_CUDA (the merge kernels reported another error), MP_ERR_BUDGET (realized
    reads above the planned bytes: never expected). */
 mp_status mp_manifest_info(const mp_manifest* man, uint64_t* realized_bytes_per_expert,
                            uint64_t* realized_total, uint64_t* touched_blocks, uint64_t* digest);
@@ -447,7 +447,9 @@ mp_status mp_trace_read(mp_trace_range* out, uint64_t n);
  * mp_debug_stall_pipeline(rounds): the index and merge kernels launched from now on never arm
  * the first slot of each CTA's shared-memory ring (its bulk copy is not issued), so the
  * consumers' wait for it cannot complete, and every pipeline wait (producer or consumer
- * mbarrier) gives up after `rounds` polling rounds instead of the default 2^21.  The wait
+ * mbarrier) gives up after `rounds` polling rounds instead of the default 2^21; in mp_plan calls of
+ * more than 2^17 units one CTA of the planner's grid never comes to its barrier, where the
+ * others give up after `rounds` polls.  The wait
  * that runs out sets the handle's error word; the accessors of that handle and of the
  * handles built from it return MP_ERR_TIMEOUT.  The waits that drain a CTA's own bulk
  * copies before it exits keep the full limit, so no copy is in flight when a kernel

@@ -383,7 +383,8 @@ def mp_debug_inject_fault(kind: int, n: int) -> None:
 
 def mp_debug_stall_pipeline(rounds: int) -> None:
     """Test hook: index and merge kernels launched from now on never arm their first ring
-    slot and give up a pipeline wait after `rounds` polling rounds (0 = off)."""
+    slot and give up a pipeline wait after `rounds` polling rounds; one CTA of a planner's grid (more
+    than 2^17 units) never comes to its barrier (0 = off)."""
     lib().mp_debug_stall_pipeline(int(rounds))
 
 

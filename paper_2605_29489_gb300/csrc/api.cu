@@ -1198,7 +1198,11 @@ mp_status mp_plan(const mp_index* index, const mp_op* op, uint64_t budget_bytes,
   const std::vector<uint8_t> order_key = hdr;  // everything the traversal order depends on
   put_u64(hdr, budget_bytes);
   p.digest_state = plan_digest_state(hdr.data(), hdr.size());
+  // until the kernel has come to its end the plan counts as one whose waits gave up
+  for (int k = 0; k < 8; ++k) pl->h_summary[k] = k == 6 ? (uint64_t)kErrTimeout : 0ull;
   p.host_summary = pl->h_summary;
+  p.wait_limit = g_stall_rounds.load(std::memory_order_relaxed);
+  p.stall = p.wait_limit ? 1u : 0u;
 
   // the first operator planned on this index leaves its traversal order behind; later
   // plans with the same operator start from it (the order is written once, by a launch
@@ -1544,7 +1548,7 @@ mp_status mp_plan_info(const mp_plan_t* plan, uint64_t* planned_bytes, uint64_t*
     return cuda_fail(e, "copy");
   if (s[6] & kErrNonfinite) return fail(MP_ERR_NONFINITE, "the index saw a NaN or infinite delta");
   if (s[6] & kErrMissing) return fail(MP_ERR_UNSUPPORTED, "a catalog entry without statistics and no tensor map");
-  if (s[6] & kErrTimeout) return fail(MP_ERR_TIMEOUT, "a bounded device wait in the index gave up");
+  if (s[6] & kErrTimeout) return fail(MP_ERR_TIMEOUT, "a bounded device wait in the index or the planner gave up");
   if (s[6] & kErrBounds) return fail(MP_ERR_CUDA, "a bounds check of the checked build failed in the index kernels");
   if (s[6]) return fail(MP_ERR_CUDA, "an internal check of the index or plan kernels failed");
   if (s[0] > plan->budget) return fail(MP_ERR_BUDGET, "planned bytes exceed the budget");
@@ -1573,6 +1577,8 @@ mp_status mp_manifest_info(const mp_manifest* man, uint64_t* realized_per_expert
   if (err & kErrTimeout) return fail(MP_ERR_TIMEOUT, "a bounded device wait in the merge gave up");
   if (err & kErrBounds) return fail(MP_ERR_CUDA, "a bounds check of the checked build failed in the merge kernels");
   if (err) return fail(MP_ERR_CUDA, "merge kernels reported an error");
+  // a plan that gave up has left a part of its mask
+  if (s[6] & kErrTimeout) return fail(MP_ERR_TIMEOUT, "a bounded device wait in the index or the planner gave up");
   if (tot > s[0]) return fail(MP_ERR_BUDGET, "realized expert reads exceed the planned bytes");
   return MP_OK;
 }

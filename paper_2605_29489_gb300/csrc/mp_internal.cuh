@@ -375,7 +375,11 @@ struct PlanLaunch {
   uint32_t* mask;
   uint32_t* order;
   uint64_t* summary;
-  uint64_t* host_summary;  // pinned host copy of the summary, or null
+  // pinned host copy of the summary, or null: written at the end of the kernel, but the error word also
+  // by a CTA that gives up a barrier
+  uint64_t* host_summary;
+  uint32_t wait_limit;     // polls of the grid barrier (0: the default)
+  uint32_t stall;          // test hook: one CTA of a cooperative launch never comes to a barrier
   uint64_t digest_state;   // FNV-1a state after the digest header (plan_digest_state)
 };
 // FNV-1a 64 over the digest header (op, theta, B): the part of the digest known to the host

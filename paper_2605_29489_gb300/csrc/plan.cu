@@ -121,8 +121,10 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned long long* p) {
 }
 
 // barrier of the cooperative grid: the last CTA to arrive bumps the generation; the others wait for it with
-// a bounded number of polls.  Returns false (uniformly inside the CTA) if the wait expired.
-__device__ __forceinline__ bool grid_sync(unsigned long long* x, unsigned& gen, uint64_t* summary) {
+// a bounded number of polls.  Returns false (uniformly inside the CTA) if the wait expired: the CTA then
+// returns, and as the host's copy of the summary is otherwise written at the very end only, the error
+// word goes there too.
+__device__ __forceinline__ bool grid_sync(const PlanLaunch& p, unsigned long long* x, unsigned& gen) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -134,11 +136,13 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* x, unsigned& gen, 
       __threadfence();
       atomicExch(&x[X_BAR_GEN], (unsigned long long)target);
     } else {
+      const uint32_t limit = p.wait_limit ? p.wait_limit : kBarrierLimit;
       uint32_t k = 0;
       while (ld_acquire(&x[X_BAR_GEN]) != target) {
-        if (++k > kBarrierLimit) {
+        if (++k > limit) {
           ok = 0;
-          atomicOr((unsigned long long*)&summary[S_ERR], (unsigned long long)kErrTimeout);
+          atomicOr((unsigned long long*)&p.summary[S_ERR], (unsigned long long)kErrTimeout);
+          if (p.host_summary) *(volatile uint64_t*)&p.host_summary[S_ERR] = (uint64_t)kErrTimeout;
           break;
         }
         __nanosleep(32);
@@ -153,7 +157,8 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* x, unsigned& gen, 
 }
 
 // barrier of the cluster: every thread arrives, and what any of them wrote before is visible
-// to all of them after
+// to all of them after.  No limit is needed: the CTAs of a cluster run at the same time, and the hardware
+// waits for the threads that have not exited, all of which come here or exit.
 __device__ __forceinline__ void cluster_sync() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -161,12 +166,12 @@ __device__ __forceinline__ void cluster_sync() {
 
 // the barrier between phases; false (uniformly inside the CTA) when the wait expired
 template <bool CL>
-__device__ __forceinline__ bool phase_sync(unsigned long long* x, unsigned& gen, uint64_t* summary) {
+__device__ __forceinline__ bool phase_sync(const PlanLaunch& p, unsigned long long* x, unsigned& gen) {
   if constexpr (CL) {
     cluster_sync();
     return true;
   } else {
-    return grid_sync(x, gen, summary);
+    return grid_sync(p, x, gen);
   }
 }
 
@@ -498,6 +503,9 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
     s.x[X_MISSING] = 0;
     if (p.cache_q_out) *p.cache_q_out = ~0ull;  // an invalid count until the sort is complete
   }
+  // test hook: this CTA never comes to a barrier.  Its share of the mask is zero by now, as that of a CTA
+  // which gives up is: a mask that was not finished selects some units or none, never an expert past K
+  if (!CL && p.stall && c == 1) return;
   bool bad_order = false, miss = false;
   uint32_t Q = 0, len = 0, a = 0, b = 0;  // candidates; this warp's slice [a, b) of them
   auto own_slice = [&](uint32_t q) {
@@ -520,7 +528,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
       const uint32_t n_pairs = p.K * p.n_tensors;
       for (uint32_t k = gt; k < n_pairs; k += gn) s.pair_flag[k] = 0u;
       for (uint32_t k = gt; k < p.n_tensors; k += gn) s.sel_bits[k] = 0u;
-      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+      if (!phase_sync<CL>(p, s.x, gen)) return;
       // 0a: flag the pairs holding an entry without statistics (one atomic per pair and warp)
       for (uint64_t t0 = ua; t0 < ub; t0 += 32) {
         const uint64_t u = t0 + lane;
@@ -532,11 +540,11 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
         const uint32_t peers = __match_any_sync(0xFFFFFFFFu, pr);
         if (pr != 0xFFFFFFFFu && lane == (uint32_t)(__ffs(peers) - 1)) atomicOr(&s.pair_flag[pr], 1u);
       }
-      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+      if (!phase_sync<CL>(p, s.x, gen)) return;
       // 0b: the flagged pairs' units, one warp each
       for (uint32_t pr = gw; pr < n_pairs; pr += G * W)
         if (s.pair_flag[pr]) fallback_pair(p, s, pr, lane);
-      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+      if (!phase_sync<CL>(p, s.x, gen)) return;
     }
 
     bool ranked = false;
@@ -545,7 +553,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
         rank_units<PT>(p, s, U, &s_cnt[0][0], Q);
         own_slice(Q);
         if (p.cache_q_out && gt == 0) *p.cache_q_out = Q;
-        if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+        if (!phase_sync<CL>(p, s.x, gen)) return;
         ranked = true;
       }
     }
@@ -596,7 +604,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
         if constexpr (CL) s_hist[tid] = n;
         else s.hist[(uint64_t)c * 256u + tid] = n;
       }
-      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+      if (!phase_sync<CL>(p, s.x, gen)) return;
       // digit starts, the counts of the CTAs before this one, then each warp's start
       uint32_t before = 0, tot = 0;
       if (tid < 256u) {
@@ -615,7 +623,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
       }
       // one digit holds every key: nothing moves (uniform over the grid: the same totals)
       if (pass > 0 && (__syncthreads_or(tid < 256u && tot == Q) != 0 || Q == 0)) {
-        if (!phase_sync<CL>(s.x, gen, p.summary)) return;  // every CTA has read the counts
+        if (!phase_sync<CL>(p, s.x, gen)) return;  // every CTA has read the counts
         continue;
       }
       if (tid < 256u) {
@@ -652,7 +660,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
         const bool valid = load(t0 + lane, key, val);
         scatter(valid, key, val);
       }
-      if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+      if (!phase_sync<CL>(p, s.x, gen)) return;
       ordered = pass == 3;
       in = out;
       out = in == s.kv_a ? s.kv_b : s.kv_a;
@@ -682,7 +690,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
       if (lane == 0) s.cta_b[c] = t;
     }
   }
-  if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+  if (!phase_sync<CL>(p, s.x, gen)) return;
   unsigned long long total_cost;
   {
     unsigned long long own;
@@ -705,7 +713,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
       }
     }
   }
-  if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+  if (!phase_sync<CL>(p, s.x, gen)) return;
   const unsigned long long P = s.x[X_P];
   const unsigned long long pbp = P == kNoP ? 0ull : s.x[X_PBP];
   const unsigned long long R0 = P == kNoP ? 0ull : p.budget - pbp;
@@ -750,7 +758,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
       if (tid == 0) s.cta_a[c] = n_cta;
     }
   }
-  if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+  if (!phase_sync<CL>(p, s.x, gen)) return;
   unsigned long long tail_sum = 0;
   if (c == 0 && P != kNoP) {
     // greedy with skip over the compacted tail, in order, from shared memory; once R is
@@ -832,7 +840,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
   }
   if (p.fallback) {
     // a taken fallback unit's expert bit goes into every block of its tensor
-    if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+    if (!phase_sync<CL>(p, s.x, gen)) return;
     unsigned long long t = 0;
     for (uint64_t k = gt; k < p.n_blocks; k += gn) {
       uint32_t m = p.mask[k];
@@ -845,7 +853,7 @@ __global__ void __launch_bounds__(PT, 1) plan_kernel(const PlanLaunch p, Scratch
     }
     t = block_sum<PT, unsigned long long>(t);
     if (tid == 0 && t) atomicAdd((unsigned long long*)&p.summary[S_TOUCHED], t);
-    if (!phase_sync<CL>(s.x, gen, p.summary)) return;
+    if (!phase_sync<CL>(p, s.x, gen)) return;
   }
   if (gt != 0) return;
   // ---- F: the digest: FNV-1a 64 over the header (hashed by the host) and C_hat, n_sel, set_hash ----

@@ -5,7 +5,8 @@
   pipeline wait after a few thousand polling rounds, so their consumers' wait for that slot
   runs out.  The kernels record the timeout and return (the waits that drain their own
   copies keep the full limit); the accessors report MP_ERR_TIMEOUT for the index, for a
-  plan built on it and for the manifest of a merge.
+  plan built on it and for the manifest of a merge.  The planner's grid barrier likewise, for the
+  plan and for the manifest of a merge with it.
 * Failures made on the host (mp_debug_inject_fault): the n-th device allocation or the
   n-th host-pool gather launch fails; the call returns its error and produces no handle
   (Alg. 2: a run either publishes or leaves no visible state), and the next calls work.
@@ -189,3 +190,45 @@ def test_injected_gather_failure_in_host_pool(restore_hooks):
     assert np.array_equal(host(fam, out)[cov], want[cov])
     for x in (man, plan, idx):
         x.free()
+
+
+def test_planner_barrier_that_runs_out_is_reported_as_timeout(restore_hooks):
+    """above 2^17 units the planner is a cooperative grid whose barrier gives up after a number of polls;
+    with the hook one CTA never comes to it.  The plan and the manifest of a merge with it report the
+    timeout, and the same call without the hook gives the oracle's plan."""
+    fam = synth.custom([4300 * 256 - 40], dtype=synth.BF16, block_elems=256, K=32, active_frac=0.5, name="plan-timeout")
+    base, experts = fam.host_arrays()
+    mf, b, ex = upload(fam, base, experts)
+    K = fam.K
+    gop, oop = mp.make_op(mp.MP_OP_TA, alpha=[0.3] * K), oracle.Op(oracle.TA, K, alpha=[0.3] * K)
+    B = mp.mp_budget_from_fraction(mf, 0.5)
+    out = torch.empty_like(b)
+    idx = mp.mp_index_blocks(mf, gop)
+    assert mp.mp_index_shape(idx)[1] > 1 << 17
+    good = mp.mp_plan(idx, gop, B)  # its pinned slot is used again below
+    assert mp.mp_plan_info(good, idx)["n_sel"] > 0
+    good.free()
+    for _ in range(2):
+        mp.mp_debug_stall_pipeline(STALL_ROUNDS)
+        bad = mp.mp_plan(idx, gop, B)
+        mp.mp_debug_stall_pipeline(0)
+        with pytest.raises(mp.MergePipeError) as e:
+            mp.mp_plan_info(bad, idx)
+        assert e.value.status == TIMEOUT
+        man = mp.mp_merge(mf, idx, bad, out)
+        with pytest.raises(mp.MergePipeError) as e:
+            mp.mp_manifest_info(man, K)
+        assert e.value.status == TIMEOUT
+        man.free()
+        bad.free()
+    idx.free()
+    idx = mp.mp_index_blocks(mf, gop)  # (the plan above was to leave its order with the other index)
+    plan = mp.mp_plan(idx, gop, B)
+    pi = mp.mp_plan_info(plan, idx)
+    of = oracle_family(fam, base, experts)
+    norm, maxabs, nnz = oracle.index(of)
+    _, bl, bt = fam.block_table()
+    opl = oracle.plan(K, bl, bt, 1, fam.elem_size, oop, norm, maxabs, nnz, None, B)
+    assert pi["digest"] == opl["digest"] and np.array_equal(pi["mask"], opl["mask"])
+    plan.free()
+    idx.free()

@@ -122,3 +122,19 @@ def test_one_index_used_by_many_merges_keeps_few_events(rt):
     used = rt.fake_used()
     idx.free()
     assert rt.fake_used() < used and rt.fake_most_pending_at_free() == 0
+
+
+# ---- a planner that gives up ------------------------------------------------------------------
+
+def test_a_plan_that_did_not_finish_is_reported(rt):
+    """the planner writes its summary to the host at its very end; one that gave up before (here: that
+    did not run) is a timeout, not the plan of whatever handle had the pinned slot before"""
+    fam, out = family()
+    idx = mp.mp_index_blocks(fam, TA(3), stream=S1)
+    for _ in range(3):  # the slot is used again and again
+        plan = mp.mp_plan(idx, TA(3), 1 << 20, stream=S1)
+        with pytest.raises(mp.MergePipeError) as e:
+            mp.mp_plan_info(plan)
+        assert e.value.status == TIMEOUT
+        plan.free()
+    idx.free()
