@@ -26,6 +26,7 @@ thread_local const char* g_static_error = nullptr;  // set instead of g_last_err
 // to the event that fails; 0 = disarmed.
 std::atomic<int64_t> g_fault_left[MP_FAULT_GATHER + 1];
 thread_local bool g_injected = false;  // the error being reported was injected
+thread_local bool g_was_injected = false;  // the error last reported was
 std::atomic<uint32_t> g_stall_rounds{0};  // mp_debug_stall_pipeline: wait rounds of stalled launches (0: off)
 
 // true when this event of the given kind is the one armed to fail (it then disarms)
@@ -399,6 +400,7 @@ void Users::wait() {
 mp_status cuda_fail(cudaError_t e, const char* what) {
   cudaGetLastError();
   g_static_error = nullptr;
+  g_was_injected = g_injected;
   if (g_injected) {
     g_injected = false;
     g_last_error = std::string(what) + ": injected fault (test hook)";
@@ -931,13 +933,12 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
       o_win = slot(KG * 4);
       o_spans = slot(h_spans.size() * 4);
     }
+    g_was_injected = false;
     st = new_index(g, op, family->experts_location != 0, units ? kUnitHistBins : (masked ? 256u : 0u), o, cs, init, &ix, &m);
     if (st == MP_OK) break;
-    // without the memory for the larger histograms: the smaller ones
-    size_t fr = 0, total = 0;
-    if (st != MP_ERR_OOM || !units || cudaMemGetInfo(&fr, &total) != cudaSuccess ||
-        fr >= o + (uint64_t)g.K * g.n_blocks * kUnitHistBins * 4)
-      return st;
+    // without the memory for the larger histograms: the smaller ones (whatever the device says is free: an
+    // allocation can fail with more than its size free)
+    if (st != MP_ERR_OOM || !units || g_was_injected) return st;
     units = false;
   }
 

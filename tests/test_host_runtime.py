@@ -138,3 +138,41 @@ def test_a_plan_that_did_not_finish_is_reported(rt):
         assert e.value.status == TIMEOUT
         plan.free()
     idx.free()
+
+
+# ---- TIES after masking on a device that is nearly full ---------------------------------------
+
+UNITS = 640_000  # 20,000 blocks of 2,048 elements, 32 experts: the line of the larger histograms
+LARGE, SMALL = UNITS * 640 * 4, UNITS * 256 * 4
+MASKED = mp.make_op(mp.MP_OP_TIES_MASKED, density=0.2)
+
+
+def _masked_catalog(rt):
+    """bytes held by a catalog of TIES after masking"""
+    fam, _ = family(n_blocks=20_000, K=32, block=2048)
+    before = rt.fake_used()
+    with mp.mp_index_blocks(fam, MASKED, stream=S1):
+        return rt.fake_used() - before
+
+
+def test_smaller_histograms_whenever_the_larger_ones_do_not_fit(rt):
+    assert _masked_catalog(rt) > LARGE
+    tables = UNITS * 12 + 20_000 * 20
+    for free, largest in ((LARGE - 1, 1 << 40),             # not even the histograms
+                          (LARGE + tables // 2, 1 << 40),   # those, but not the tables and statistics beside them
+                          (64 << 30, LARGE - 1)):           # enough in all, but not in one piece
+        rt.fake_memory(free, largest)
+        held = _masked_catalog(rt)
+        assert SMALL < held < LARGE, (free, largest)
+    rt.fake_memory(SMALL, 1 << 40)  # too little for those either
+    with pytest.raises(mp.MergePipeError) as e:
+        _masked_catalog(rt)
+    assert e.value.status == OOM
+
+
+def test_an_injected_failure_is_not_taken_for_a_full_device(rt):
+    mp.mp_debug_inject_fault(mp.MP_FAULT_ALLOC, 1)
+    with pytest.raises(mp.MergePipeError) as e:
+        _masked_catalog(rt)
+    assert e.value.status == OOM and "injected" in str(e.value)
+    assert _masked_catalog(rt) > LARGE
