@@ -160,7 +160,8 @@ typedef struct mp_manifest_s mp_manifest;
  * and also keeps every (expert, block)'s key histogram, from which each merge finds its
  * plan's threshold: 256 bins of the upper 8 key bits (1 KB per unit), or, for experts in
  * device memory and blocks of 2,048 elements or more on average, 640 bins that also hold the
- * single keys around tau (2.5 KB per unit; 256 bins where the memory for them is lacking).
+ * single keys around tau (2.5 KB per unit; 256 bins where the difference is more than 64 MiB and
+ * more than 1/32 of the device's free memory, or where the larger ones cannot be allocated).
  * op may be NULL for non-TIES use.
  * The family's buffers must stay valid and unchanged until the stream reaches this work.
  * Errors: MP_ERR_INVALID_ARG (bad family or op), MP_ERR_OOM, MP_ERR_CUDA; a non-finite

@@ -808,6 +808,19 @@ mp_status alloc_hashes(mp_index_s* ix, cudaStream_t cs) {
   return MP_OK;
 }
 
+// whether the larger histograms of TIES after masking leave the caller's memory alone
+bool unit_hist_affordable(const Geometry& g) {
+  const uint64_t more = (uint64_t)g.K * g.n_blocks * (kUnitHistBins - 256) * 4;
+  if (more <= kUnitHistSmall) return true;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // no part of a capture
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  size_t fr = 0, total = 0;
+  const cudaError_t e = cudaMemGetInfo(&fr, &total);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess && more <= fr / kUnitHistShare;
+}
+
 // frees a handle whose construction failed (after the stream's work on it is done)
 void discard_index(mp_index_s* ix, cudaStream_t cs) {
   cudaStreamSynchronize(cs);
@@ -878,10 +891,11 @@ mp_status mp_index_blocks(const mp_family* family, const mp_op* op, mp_stream st
       h_kth[q] = (unsigned long long)floor((double)op->density * (double)gnumel[q]);
   }
   // TIES takes its thresholds from predicted windows, TIES after masking where the units' larger
-  // histograms (2.5 KiB) are small against what they count, and fit the device's memory
+  // histograms (2.5 KiB) are small against what they count and against the device's free memory
   const bool windowed = ties && op->kind == MP_OP_TIES;
   const bool masked = ties && !windowed;
-  bool units = masked && family->experts_location == 0 && g.n_params >= g.n_blocks * kUnitHistElems;
+  bool units = masked && family->experts_location == 0 && g.n_params >= g.n_blocks * kUnitHistElems &&
+               unit_hist_affordable(g);
   mp_index_s* ix = nullptr;
   char* m = nullptr;
   InitList init;

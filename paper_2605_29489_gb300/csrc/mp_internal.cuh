@@ -263,6 +263,12 @@ constexpr uint32_t kUnitHistBins = 640;  // bins of a unit's histogram with a wi
 // merge took 437 instead of 701 us but the catalog 1436 instead of 1224.
 constexpr uint64_t kUnitHistElems = 2048;
 
+// And only where the 1.5 KiB per unit that they take more are little against the memory which the
+// device has left for the caller's next allocations, an output for instance: at blocks of 2,048 bf16
+// elements the larger histograms come to 0.6 of the experts.  Up to kUnitHistSmall bytes nothing is asked.
+constexpr uint64_t kUnitHistSmall = 64ull << 20;
+constexpr uint64_t kUnitHistShare = 32;  // of the free memory, the part that they may take more
+
 struct IndexLaunch {
   mp_dtype dtype;
   uint32_t K;

@@ -158,12 +158,11 @@ def _masked_catalog(rt):
 def test_smaller_histograms_whenever_the_larger_ones_do_not_fit(rt):
     assert _masked_catalog(rt) > LARGE
     tables = UNITS * 12 + 20_000 * 20
-    for free, largest in ((LARGE - 1, 1 << 40),             # not even the histograms
-                          (LARGE + tables // 2, 1 << 40),   # those, but not the tables and statistics beside them
-                          (64 << 30, LARGE - 1)):           # enough in all, but not in one piece
-        rt.fake_memory(free, largest)
+    for largest in (LARGE - 1,             # not even the histograms
+                    LARGE + tables // 2):  # those, but not the tables and statistics beside them
+        rt.fake_memory(64 << 30, largest)
         held = _masked_catalog(rt)
-        assert SMALL < held < LARGE, (free, largest)
+        assert SMALL < held < LARGE, largest
     rt.fake_memory(SMALL, 1 << 40)  # too little for those either
     with pytest.raises(mp.MergePipeError) as e:
         _masked_catalog(rt)
@@ -176,3 +175,16 @@ def test_an_injected_failure_is_not_taken_for_a_full_device(rt):
         _masked_catalog(rt)
     assert e.value.status == OOM and "injected" in str(e.value)
     assert _masked_catalog(rt) > LARGE
+
+
+def test_larger_histograms_only_where_the_caller_keeps_nearly_all_of_the_free_memory(rt):
+    """983 MB more than the smaller ones: more than a 32nd of 20 GB, less than that of 40 GB"""
+    rt.fake_memory(20 << 30, 1 << 40)
+    assert SMALL < _masked_catalog(rt) < LARGE
+    rt.fake_memory(40 << 30, 1 << 40)
+    assert _masked_catalog(rt) > LARGE
+    rt.fake_memory(1 << 30, 1 << 40)  # 40,000 units: 61 MB more, as before
+    fam, _ = family(n_blocks=40_000, K=1, block=2048)
+    before = rt.fake_used()
+    with mp.mp_index_blocks(fam, MASKED, stream=S1):
+        assert rt.fake_used() - before > 40_000 * 640 * 4
