@@ -50,6 +50,12 @@
  *    return MP_ERR_CUDA with "a bounds check of the checked build failed".  mp_version()
  *    names the build.  Meant for debugging; its checks cost little (within 1 % of the
  *    default build on a Qwen2.5-0.5B-shaped task-arithmetic step).
+ *  - Device memory for handles and scratch comes, in stream order, from a pool of the
+ *    library's own on each device, which keeps at most 256 MiB of unused memory between
+ *    calls (mp_trim gives it back, and an allocation of the same process that would fail for want
+ *    of memory is served from it).  A caller that has set a memory pool of its own
+ *    on the device (cudaDeviceSetMemPool) has the library use that one instead; under stream
+ *    capture the memory belongs to the graph.
  *  - On an error return no handle is produced and *out is set to NULL; the
  *    contents of a merge output buffer are then unspecified.
  *  - mp_last_error() returns a thread-local message for the last failure.
@@ -319,6 +325,10 @@ mp_status mp_plan_noalloc(uint32_t K, uint64_t n_blocks, uint32_t n_groups, mp_d
    so a handle may be freed at any time after the calls that use it have returned.  NULL is a no-op.
    Passing anything else is undefined. */
 void mp_free(void* handle);
+
+/* Gives the unused device memory that the library keeps on the current device back to the system
+   (memory freed by work that is still running stays until the next call).  Errors: MP_ERR_CUDA. */
+mp_status mp_trim(void);
 
 /* Host copies of the index statistics, expert-major [K][n_blocks]; tau is [K][n_groups]
    (n_groups = n_tensors for trim_scope 0, 1 for trim_scope 1).  Any pointer may be NULL.

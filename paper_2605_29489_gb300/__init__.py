@@ -23,7 +23,8 @@ import numpy as np
 __all__ = [
     "MP_OK", "MP_BF16", "MP_F32", "MP_OP_AVG", "MP_OP_TA", "MP_OP_TIES", "MP_OP_DARE", "MP_OP_AVG_RENORM", "MP_OP_DARE_TIES",
     "MP_OP_TIES_MASKED", "mp_manifest_threshold_reads", "MergePipeError",
-    "family", "make_op", "mp_index_blocks", "mp_plan", "mp_merge", "mp_merge_touched", "mp_free", "mp_index_stats",
+    "family", "make_op", "mp_index_blocks", "mp_plan", "mp_merge", "mp_merge_touched", "mp_free", "mp_trim",
+    "mp_index_stats",
     "mp_index_shape", "mp_plan_info", "mp_manifest_info", "mp_manifest_lineage", "mp_budget_from_fraction", "mp_last_error",
     "mp_version", "mp_kernel_launch_count", "mp_plan_noalloc", "mp_index_import", "MP_NNZ_MISSING", "mp_index_hashes",
     "mp_index_hash_values", "mp_manifest_validate", "mp_manifest_validation", "lib",
@@ -108,6 +109,7 @@ def lib():
             f = getattr(L, name)
             f.restype, f.argtypes = st, args
         L.mp_free.restype, L.mp_free.argtypes = None, [vp]
+        L.mp_trim.restype, L.mp_trim.argtypes = st, []
         L.mp_budget_from_fraction.restype, L.mp_budget_from_fraction.argtypes = u64, [vp, ctypes.c_double]
         L.mp_last_error.restype, L.mp_last_error.argtypes = ctypes.c_char_p, []
         L.mp_version.restype, L.mp_version.argtypes = ctypes.c_char_p, []
@@ -301,6 +303,11 @@ def mp_merge_touched(fam: Family, index: Handle, plan: Handle, out, stream=None)
 def mp_free(h: Handle | None):
     if h is not None:
         h.free()
+
+
+def mp_trim():
+    """give the unused device memory that the library keeps (at most 256 MiB) back to the system"""
+    _check(lib().mp_trim())
 
 
 def mp_index_shape(index: Handle):

@@ -42,21 +42,33 @@ bool inject_fault(int kind) {
 // device, so that a program which frees its handles after every merge had each call map its
 // memory anew (mp_index_blocks spent 140-270 us on the host, 40 us more to free it; host-pool
 // staging about 1.4 ms).  This pool keeps at most kPoolKeep bytes of unused memory between
-// calls; what is above goes back at the next wait, and all of it when an allocation fails.
-// cudaMallocFromPoolAsync orders every block's reuse by stream, from any thread.
+// calls; what is above goes back at the next wait, and all of it when an allocation of the library
+// fails, on mp_trim, and when another allocation of the process needs it (the driver's own retry:
+// cudaMalloc got 64 of 96 MiB kept here and not reported as free).  A caller that has made
+// a pool of its own the device's current one has its memory used instead, as before there was this
+// one.  cudaMallocFromPoolAsync orders every block's reuse by stream, from any thread.
 constexpr uint64_t kPoolKeep = 256ull << 20;
 constexpr int kPoolDevices = 64;
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[kPoolDevices];
+cudaMemPool_t g_pool[kPoolDevices];          // the library's
+cudaMemPool_t g_default_pool[kPoolDevices];  // the device's, which never changes
 
-// the current device's pool, created on first use; null where there is none
+// the current device's pool, created on first use; null where there is none, or where the caller
+// has set a memory pool of its own
 cudaMemPool_t device_pool() {
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices) {
+  cudaMemPool_t cur = nullptr;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices ||
+      cudaDeviceGetMemPool(&cur, dev) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
   std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (!g_default_pool[dev] && cudaDeviceGetDefaultMemPool(&g_default_pool[dev], dev) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (cur != g_default_pool[dev]) return nullptr;
   if (!g_pool[dev]) {
     cudaMemPoolProps props;
     memset(&props, 0, sizeof(props));
@@ -1473,6 +1485,19 @@ mp_status mp_merge(const mp_family* family, const mp_index* index, const mp_plan
 mp_status mp_merge_touched(const mp_family* family, const mp_index* index, const mp_plan_t* plan, void* out_buf,
                            mp_stream stream, mp_manifest** man_out) {
   return merge_common(family, index, plan, out_buf, stream, man_out, true);
+}
+
+mp_status mp_trim(void) {
+  int dev = -1;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return cuda_fail(e, "device");
+  cudaMemPool_t pool = nullptr;
+  if (dev >= 0 && dev < kPoolDevices) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    pool = g_pool[dev];
+  }
+  if (pool && (e = cudaMemPoolTrimTo(pool, 0)) != cudaSuccess) return cuda_fail(e, "pool trim");
+  return MP_OK;
 }
 
 void mp_free(void* handle) {

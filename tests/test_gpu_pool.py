@@ -110,3 +110,27 @@ def test_handles_freed_while_a_merge_runs(kind):
             assert torch.equal(got[0], want[0]) and got[1:] == want[1:], it
             for h in (m2, p2, man):
                 h.free()
+
+
+def test_kept_memory_is_within_the_callers_reach():
+    """what the pool keeps unused goes to an allocation of the process that would fail without it, and
+    back to the system on mp_trim"""
+    b = torch.zeros(3000 * 256, dtype=torch.bfloat16, device="cuda")
+    mf = mp.family([(0, 3000 * 256)], b, [b] * 32, 256, mp.MP_BF16, 0)
+    op = mp.make_op(mp.MP_OP_TIES_MASKED, density=0.2)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    mp.mp_trim()
+    free = torch.cuda.mem_get_info()[0]
+    mp.mp_index_blocks(mf, op).free()
+    torch.cuda.synchronize()
+    kept = free - torch.cuda.mem_get_info()[0]
+    assert 64 << 20 < kept <= 256 << 20
+    hold = torch.empty(free - kept + (16 << 20), dtype=torch.uint8, device="cuda")  # more than is reported free
+    del hold
+    torch.cuda.empty_cache()
+    mp.mp_index_blocks(mf, op).free()
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] > 64 << 20
+    mp.mp_trim()
+    assert free - torch.cuda.mem_get_info()[0] <= 4 << 20
