@@ -451,7 +451,9 @@ mp_status mp_trace_read(mp_trace_range* out, uint64_t n);
  *                    returns MP_ERR_OOM and no handle;
  *   MP_FAULT_GATHER  a host-pool gather launch (mp_index_blocks / mp_merge with experts in
  *                    pinned host memory) is not made: the call returns MP_ERR_CUDA and no
- *                    handle, after the work already enqueued has been joined.
+ *                    handle, after the work already enqueued has been joined;
+ *   MP_FAULT_CLUSTER a planner launch (mp_plan, mp_plan_noalloc) finds no room on the device for its
+ *                    thread-block cluster: the call takes the cooperative grid instead and succeeds.
  * mp_last_error() then names the injected fault.  Returns MP_ERR_INVALID_ARG for an unknown
  * kind.
  *
@@ -468,6 +470,7 @@ mp_status mp_trace_read(mp_trace_range* out, uint64_t n);
  */
 #define MP_FAULT_ALLOC 1
 #define MP_FAULT_GATHER 2
+#define MP_FAULT_CLUSTER 3
 mp_status mp_debug_inject_fault(int32_t kind, uint64_t n);
 void mp_debug_stall_pipeline(uint32_t rounds);
 

@@ -28,7 +28,7 @@ __all__ = [
     "mp_index_shape", "mp_plan_info", "mp_manifest_info", "mp_manifest_lineage", "mp_budget_from_fraction", "mp_last_error",
     "mp_version", "mp_kernel_launch_count", "mp_plan_noalloc", "mp_index_import", "MP_NNZ_MISSING", "mp_index_hashes",
     "mp_index_hash_values", "mp_manifest_validate", "mp_manifest_validation", "lib",
-    "MP_FAULT_ALLOC", "MP_FAULT_GATHER", "mp_debug_inject_fault", "mp_debug_stall_pipeline",
+    "MP_FAULT_ALLOC", "MP_FAULT_GATHER", "MP_FAULT_CLUSTER", "mp_debug_inject_fault", "mp_debug_stall_pipeline",
     "MP_TRACE_INDEX", "MP_TRACE_PLAN", "MP_TRACE_MERGE", "MP_TRACE_GATHER", "MP_TRACE_SEGMENT",
     "mp_trace_start", "mp_trace_stop", "library_path",
 ]
@@ -39,7 +39,7 @@ MP_ERR = {-1: "MP_ERR_INVALID_ARG", -2: "MP_ERR_CUDA", -3: "MP_ERR_OOM", -4: "MP
 MP_BF16, MP_F32 = 0, 1
 MP_OP_AVG, MP_OP_TA, MP_OP_TIES, MP_OP_DARE, MP_OP_AVG_RENORM, MP_OP_DARE_TIES, MP_OP_TIES_MASKED = 0, 1, 2, 3, 4, 5, 6
 MP_NNZ_MISSING = 0xFFFFFFFF   # catalog entry without block statistics (tensor-level fallback)
-MP_FAULT_ALLOC, MP_FAULT_GATHER = 1, 2  # test hooks: kinds of injected host-side failures
+MP_FAULT_ALLOC, MP_FAULT_GATHER, MP_FAULT_CLUSTER = 1, 2, 3  # test hooks: kinds of injected host-side failures
 # kinds of traced device-time ranges (mp_trace_start)
 MP_TRACE_INDEX, MP_TRACE_PLAN, MP_TRACE_MERGE, MP_TRACE_GATHER, MP_TRACE_SEGMENT = 1, 2, 3, 4, 5
 
@@ -384,7 +384,8 @@ def mp_kernel_launch_count() -> int:
 
 def mp_debug_inject_fault(kind: int, n: int) -> None:
     """Test hook: the n-th device allocation (MP_FAULT_ALLOC) or host-pool gather launch
-    (MP_FAULT_GATHER) from now on fails once, on the host; n = 0 disarms."""
+    (MP_FAULT_GATHER) from now on fails once, on the host, or the n-th planner launch finds no room
+    for its cluster (MP_FAULT_CLUSTER); n = 0 disarms."""
     _check(lib().mp_debug_inject_fault(int(kind), int(n)))
 
 

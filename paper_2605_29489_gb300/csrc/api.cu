@@ -24,7 +24,7 @@ thread_local const char* g_static_error = nullptr;  // set instead of g_last_err
 // test hooks: failures injected on the host (mp_debug_inject_fault) and device waits made to
 // run out (mp_debug_stall_pipeline); nothing faults the GPU.  g_fault_left[kind] counts down
 // to the event that fails; 0 = disarmed.
-std::atomic<int64_t> g_fault_left[MP_FAULT_GATHER + 1];
+std::atomic<int64_t> g_fault_left[MP_FAULT_CLUSTER + 1];
 thread_local bool g_injected = false;  // the error being reported was injected
 thread_local bool g_was_injected = false;  // the error last reported was
 std::atomic<uint32_t> g_stall_rounds{0};  // mp_debug_stall_pipeline: wait rounds of stalled launches (0: off)
@@ -33,7 +33,7 @@ std::atomic<uint32_t> g_stall_rounds{0};  // mp_debug_stall_pipeline: wait round
 bool inject_fault(int kind) {
   if (g_fault_left[kind].load(std::memory_order_relaxed) <= 0) return false;
   if (g_fault_left[kind].fetch_sub(1) != 1) return false;
-  g_injected = true;
+  g_injected = kind != MP_FAULT_CLUSTER;  // no call fails for that one
   return true;
 }
 
@@ -331,6 +331,8 @@ void set_error(const std::string& msg) {
 }
 
 void set_static_error(const char* msg) { g_static_error = msg; }
+
+bool cluster_refused() { return inject_fault(MP_FAULT_CLUSTER); }
 
 void count_launches(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
@@ -861,7 +863,7 @@ const char* mp_version(void) {
 uint64_t mp_kernel_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 mp_status mp_debug_inject_fault(int32_t kind, uint64_t n) {
-  if (kind != MP_FAULT_ALLOC && kind != MP_FAULT_GATHER) return fail(MP_ERR_INVALID_ARG, "unknown fault kind");
+  if (kind < MP_FAULT_ALLOC || kind > MP_FAULT_CLUSTER) return fail(MP_ERR_INVALID_ARG, "unknown fault kind");
   g_fault_left[kind].store(n > (uint64_t)INT64_MAX ? INT64_MAX : (int64_t)n, std::memory_order_relaxed);
   return MP_OK;
 }

@@ -225,6 +225,8 @@ inline cudaError_t launch_kernel(bool follows, void (*k)(P...), dim3 grid, unsig
 void set_error(const std::string& msg);
 // records a string literal as the last error without allocating
 void set_static_error(const char* msg);
+// test hook: this launch of the planner is to find no room for its cluster
+bool cluster_refused();
 mp_status cuda_fail(cudaError_t e, const char* what);
 
 // CUDA graphs: a call made while its stream is being captured records its work (and its

@@ -899,7 +899,8 @@ cudaError_t launch_plan(const PlanLaunch& p, void* scratch, cudaStream_t st) {
   Scratch s;
   carve(scratch, U, n_pairs, &s);
   cudaError_t e;
-  if (U <= kClusterUnits) {
+  bool cluster = U <= kClusterUnits;
+  if (cluster) {
     // half a unit per thread, then more, in one cluster; where the units are compared with one
     // another, 2^16 comparisons per CTA, then more
     uint32_t grid = 1;
@@ -917,9 +918,19 @@ cudaError_t launch_plan(const PlanLaunch& p, void* scratch, cudaStream_t st) {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if ((e = cudaLaunchKernelEx(&cfg, k, p, s)) != cudaSuccess) return e;
-    count_launches(1);
-    return cudaGetLastError();
+    // Up to 16 whole SMs of one GPC, more than a partition of the device or a limit on its SMs may leave
+    // this process: without room for the cluster the cooperative grid below plans any number of units.
+    int room = 0;
+    if ((e = cudaOccupancyMaxActiveClusters(&room, k, &cfg)) != cudaSuccess) {
+      cudaGetLastError();
+      room = 0;
+    }
+    cluster = room > 0 && !cluster_refused();
+    if (cluster) {
+      if ((e = cudaLaunchKernelEx(&cfg, k, p, s)) != cudaSuccess) return e;
+      count_launches(1);
+      return cudaGetLastError();
+    }
   }
   int dev = 0, sms = 0, per_sm = 0;
   auto kern = plan_kernel<kGridThreads, false>;

@@ -96,3 +96,23 @@ def test_units_ranked_by_comparison(n_blocks, K, norms):
     # up to 3,072 units; candidates fewer than units, not a multiple of 4 or 32, tensors with missing entries
     _check([256 * n_blocks - 7], 256, K, norms, (0.0, 0.3, 1.0), zero_frac=0.13, seed=n_blocks)
     _check([256 * (n_blocks - 3) - 7, 300, 5], 256, K, norms, (0.3, 1.0), missing=0.01, seed=n_blocks)
+
+
+@pytest.mark.parametrize("n_blocks,K", [(1, 1), (33, 1), (700, 3), (3073, 1), (16385, 2)])
+def test_plan_without_room_for_a_cluster(n_blocks, K):
+    """what one cluster plans otherwise, by the cooperative grid: single units, fewer than its warps, and
+    sizes of both ways of ordering; the first plan and one from the kept order"""
+    class Refused:
+        def __enter__(self):
+            self.plan = mp.mp_plan
+            def plan(*a, **k):
+                mp.mp_debug_inject_fault(mp.MP_FAULT_CLUSTER, 1)
+                return self.plan(*a, **k)
+            mp.mp_plan = plan
+        def __exit__(self, *a):
+            mp.mp_plan = self.plan
+            mp.mp_debug_inject_fault(mp.MP_FAULT_CLUSTER, 0)
+
+    with Refused():
+        _check([256 * n_blocks - 7], 256, K, lognormal, (0.0, 0.3, 1.0), zero_frac=0.13)
+        _check([256 * n_blocks - 7, 300, 5], 256, K, lognormal, (0.3, 1.0), missing=0.01)

@@ -211,3 +211,16 @@ def test_trim_gives_the_kept_memory_back(rt):
     n = rt.fake_trims()
     mp.mp_trim()
     assert rt.fake_trims() == n + 1
+
+
+# ---- a device without room for the planner's cluster ------------------------------------------
+
+def test_planner_takes_the_grid_where_no_cluster_fits(rt):
+    fam, out = family()
+    idx = mp.mp_index_blocks(fam, TA(3), stream=S1)
+    mp.mp_plan(idx, TA(3), 1 << 20, stream=S1).free()
+    assert rt.fake_launched(b"cluster:") == 1 and rt.fake_launched(b"cooperative:") == 0
+    rt.fake_cluster_room(0)
+    mp.mp_plan(idx, TA(3), 1 << 20, stream=S1).free()
+    assert rt.fake_launched(b"cluster:") == 1 and rt.fake_launched(b"cooperative:") == 1
+    idx.free()
