@@ -461,9 +461,9 @@ def native(args, rank, world, local_rank):
         for h in hs:
             h.free()
     graph = None
-    # device-resident families whose calls enqueue only kernels (TIES after masking and
-    # imported catalogs copy host arrays in, which a capture cannot hold)
-    if not host_pool and catalog is None and gop.kind != mp.MP_OP_TIES_MASKED:
+    # device-resident families whose calls enqueue only kernels (an imported catalog copies host
+    # arrays in, which a capture cannot hold)
+    if not host_pool and catalog is None:
         graph = graph_replay(mp, step, mf)
 
     if not touched_mode:   # touched-only outputs hold only the touched blocks

@@ -27,8 +27,8 @@
  *    mp_merge_touched enqueue kernels only (their small tables and results move
  *    through pinned memory that kernels read and write), so bulk transfers the
  *    caller runs on other streams do not hold them up; the exceptions use
- *    cudaMemcpyAsync: a block table above 8 MiB, the thresholds of TIES after
- *    masking, and the arrays that mp_index_import copies in.
+ *    cudaMemcpyAsync: a block table above 8 MiB and the arrays that mp_index_import
+ *    copies in.
  *  - CUDA graphs: for a family whose experts are in device memory, a step made of
  *    mp_index_blocks, mp_plan and mp_merge / mp_merge_touched calls can be captured
  *    on a stream (stream capture) and the graph replayed; each replay recomputes the
@@ -36,8 +36,8 @@
  *    handles made during the capture.  The accessors of those handles then wait for
  *    the whole device (a captured event cannot be waited for from the host).  Free
  *    such handles before the graph is destroyed; a handle made before the capture that a captured
- *    call uses is needed by every replay, and mp_free does not wait for replays.  Host-resident pools, TIES after
- *    masking and mp_index_import are not capturable.  Errors found by a kernel (a
+ *    call uses is needed by every replay, and mp_free does not wait for replays.  Host-resident pools and
+ *    mp_index_import are not capturable.  Errors found by a kernel (a
  *    non-finite delta, a timed-out wait) are reported by the next accessor on
  *    that handle or on a handle derived from it.
  *  - Checked build: libmergepipe_checked.so exports the same entry points from the same

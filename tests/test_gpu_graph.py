@@ -24,8 +24,8 @@ def _same(fam, a, b):
                for o, n in zip(offs.tolist(), nums.tolist()))
 
 
-def _family():
-    fam = synth.custom([3 * 4096 + 77, 5 * 4096, 999], dtype=synth.BF16, block_elems=4096, K=3, active_frac=0.5,
+def _family(E):
+    fam = synth.custom([3 * 4096 + 77, 5 * 4096, 999], dtype=synth.BF16, block_elems=E, K=3, active_frac=0.5,
                        name="graph")
     base, experts = fam.device_arrays()
     offs, nums, _ = fam.layout()
@@ -33,10 +33,15 @@ def _family():
     return fam, base, experts, mf
 
 
-@pytest.mark.parametrize("kind", ["ties", "ta", "dare"])
-def test_captured_step_replays_the_eager_step(kind):
-    fam, base, experts, mf = _family()
+@pytest.mark.parametrize("kind,E", [("ties", 4096), ("ta", 4096), ("dare", 4096), ("dare_ties", 4096),
+                                    ("avg_renorm", 4096), ("ties_masked", 4096), ("ties_masked", 512)],
+                         ids=["ties", "ta", "dare", "dare_ties", "avg_renorm", "ties_masked", "ties_masked-small"])
+def test_captured_step_replays_the_eager_step(kind, E):
+    fam, base, experts, mf = _family(E)  # (after masking: both sides of the line of the larger histograms)
     gop = {"ties": mp.make_op(mp.MP_OP_TIES, density=0.2),
+           "dare_ties": mp.make_op(mp.MP_OP_DARE_TIES, drop_p=0.5, seed=7),
+           "avg_renorm": mp.make_op(mp.MP_OP_AVG_RENORM, alpha=[0.2, 0.3, 0.5]),
+           "ties_masked": mp.make_op(mp.MP_OP_TIES_MASKED, density=0.2),
            "ta": mp.make_op(mp.MP_OP_TA, alpha=[0.3] * 3),
            "dare": mp.make_op(mp.MP_OP_DARE, alpha=[1 / 3] * 3, drop_p=0.9, seed=5)}[kind]
     Bs = [mp.mp_budget_from_fraction(mf, f) for f in (1.0, 0.25)]
