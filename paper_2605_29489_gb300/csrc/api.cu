@@ -144,9 +144,25 @@ void* pin_get(size_t bytes) {
   return p;
 }
 
+// pinned memory of its own for data above the largest slot; pin_put gives it back
+void* pin_get_large(size_t bytes) {
+  void* p = nullptr;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t e = cudaHostAlloc(&p, bytes, cudaHostAllocDefault);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e == cudaSuccess) return p;
+  cudaGetLastError();
+  return nullptr;
+}
+
 void pin_put(void* p, size_t bytes) {
   int c = pin_class(bytes);
-  if (!p || c < 0) return;
+  if (!p) return;
+  if (c < 0) {
+    cudaFreeHost(p);
+    return;
+  }
   std::lock_guard<std::mutex> lk(g_pin_mu);
   g_pin_free[c].push_back(p);
 }
@@ -155,10 +171,12 @@ size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // Host data into the index's device memory: staged in a pinned slot that the handle keeps until
 // mp_free, and copied by the init kernel over the host mapping.  Data larger than the largest
-// slot goes by cudaMemcpyAsync.
+// slot goes by cudaMemcpyAsync, but under stream capture: a replay reads the source again, which
+// therefore has to stay with the handle too.
 cudaError_t upload(mp_index_s* ix, InitList& init, void* dst, const void* src, size_t bytes, cudaStream_t cs) {
   if (bytes == 0) return cudaSuccess;
   void* h = pin_get(bytes);
+  if (!h && ix->captured && !(h = pin_get_large(bytes))) return cudaErrorMemoryAllocation;
   if (!h) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, cs);
   memcpy(h, src, bytes);
   ix->pinned.push_back({h, bytes});

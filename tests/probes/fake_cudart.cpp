@@ -34,7 +34,8 @@ std::map<void*, size_t> g_mem;
 std::vector<std::string> g_launched;
 size_t g_limit = (size_t)280 << 30, g_used = 0, g_largest = ~(size_t)0, g_pool_kept = 0;
 unsigned long long g_most_pending_at_free = 0;
-unsigned g_from_pool = 0, g_from_current = 0, g_trims = 0;
+unsigned g_from_pool = 0, g_from_current = 0, g_trims = 0, g_copies = 0;
+int g_host_blocks = 0, g_capturing = 0;
 int g_own_pool = 0, g_cluster_room = 1;
 int g_pool_obj[3];  // the default pool, the caller's, the library's
 cudaError_t g_last = cudaSuccess;
@@ -99,7 +100,8 @@ void fake_reset() {
   g_limit = (size_t)280 << 30;
   g_largest = ~(size_t)0;
   g_most_pending_at_free = 0;
-  g_from_pool = g_from_current = g_trims = 0;
+  g_from_pool = g_from_current = g_trims = g_copies = 0;
+  g_capturing = 0;
   g_own_pool = 0;
   g_cluster_room = 1;
   g_launched.clear();
@@ -111,6 +113,9 @@ unsigned long long fake_most_pending_at_free() { return g_most_pending_at_free; 
 unsigned fake_from_pool() { return g_from_pool; }
 unsigned fake_from_current() { return g_from_current; }
 unsigned fake_trims() { return g_trims; }
+unsigned fake_copies() { return g_copies; }
+int fake_host_blocks() { return g_host_blocks; }
+void fake_capturing(int on) { g_capturing = on; }
 void fake_callers_pool(int on) { g_own_pool = on; }
 void fake_cluster_room(int clusters) { g_cluster_room = clusters; }
 int fake_launched(const char* what) {
@@ -241,7 +246,13 @@ cudaError_t cudaFreeAsync(void* p, cudaStream_t s) {
 }
 cudaError_t cudaHostAlloc(void** p, size_t bytes, unsigned) {
   *p = calloc(1, bytes);
+  g_host_blocks += *p != nullptr;
   return *p ? cudaSuccess : fail(cudaErrorMemoryAllocation);
+}
+cudaError_t cudaFreeHost(void* p) {
+  g_host_blocks -= p != nullptr;
+  free(p);
+  return cudaSuccess;
 }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, enum cudaMemcpyKind) {
   memcpy(d, s, n);
@@ -249,6 +260,7 @@ cudaError_t cudaMemcpy(void* d, const void* s, size_t n, enum cudaMemcpyKind) {
 }
 cudaError_t cudaMemcpyAsync(void* d, const void* src, size_t n, enum cudaMemcpyKind, cudaStream_t s) {
   memcpy(d, src, n);
+  ++g_copies;
   op(s);
   return cudaSuccess;
 }
@@ -274,7 +286,7 @@ cudaError_t cudaStreamSynchronize(cudaStream_t s) {
   return cudaSuccess;
 }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, enum cudaStreamCaptureStatus* c) {
-  *c = cudaStreamCaptureStatusNone;
+  *c = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
 cudaError_t cudaThreadExchangeStreamCaptureMode(enum cudaStreamCaptureMode*) { return cudaSuccess; }

@@ -133,3 +133,40 @@ def test_capture_while_the_pinned_staging_is_in_use():
     for h in (man, pl, idx, idx_e, held):
         h.free()
     del g
+
+
+def test_capture_of_a_catalog_with_a_large_block_table():
+    """450,000 blocks: 9 MB of table, above the largest pinned slot; the replay copies it in again"""
+    n = 450_000 * 256 - 5
+    g0 = torch.Generator(device="cuda").manual_seed(1)
+    base = torch.randn(n, generator=g0, device="cuda").mul_(0.02).to(torch.bfloat16)
+    expert = (base.float() + 1e-3 * torch.randn(n, generator=g0, device="cuda")).to(torch.bfloat16)
+    mf = mp.family([(0, n)], base, [expert], 256, mp.MP_BF16, 0)
+    gop = mp.make_op(mp.MP_OP_TA, alpha=[0.5])
+    B = mp.mp_budget_from_fraction(mf, 0.25)
+    s = torch.cuda.Stream()
+
+    def step(out):
+        idx = mp.mp_index_blocks(mf, gop, s)
+        pl = mp.mp_plan(idx, gop, B, s)
+        return [mp.mp_merge(mf, idx, pl, out, s), pl, idx]
+
+    want, out = torch.empty_like(base), torch.zeros_like(base)
+    with torch.cuda.stream(s):
+        hs = step(want)
+    s.synchronize()
+    for h in hs:
+        h.free()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        hs = step(out)
+    junk = [np.full(450_000 * 20 // 8, 0x7F7F7F7F, np.int64) for _ in range(8)]  # takes what the call freed on the host
+    for _ in range(2):
+        out.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int16), want.view(torch.int16))
+    assert mp.mp_manifest_info(hs[0], 1)["realized_total"] <= B and len(junk) == 8
+    for h in hs:
+        h.free()
+    del g

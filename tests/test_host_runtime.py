@@ -224,3 +224,22 @@ def test_planner_takes_the_grid_where_no_cluster_fits(rt):
     mp.mp_plan(idx, TA(3), 1 << 20, stream=S1).free()
     assert rt.fake_launched(b"cluster:") == 1 and rt.fake_launched(b"cooperative:") == 1
     idx.free()
+
+
+# ---- capture of a catalog whose block table is above the largest pinned slot ------------------
+
+def test_a_captured_upload_keeps_its_source(rt):
+    """500,000 blocks, 10 MB of table: a replay copies it in again, so the copy's source has to live as
+    long as the handle; outside a capture it is done when the call returns"""
+    fam, out = family(n_blocks=500_000, K=1, block=256)
+    idx = mp.mp_index_blocks(fam, TA(1), stream=S1)
+    assert rt.fake_copies() == 1
+    idx.free()
+    blocks = rt.fake_host_blocks()
+    rt.fake_reset()
+    rt.fake_capturing(1)
+    idx = mp.mp_index_blocks(fam, TA(1), stream=S1)
+    rt.fake_capturing(0)
+    assert rt.fake_copies() == 0 and rt.fake_host_blocks() == blocks + 1
+    idx.free()
+    assert rt.fake_host_blocks() == blocks
