@@ -442,20 +442,16 @@ mp_status cuda_fail(cudaError_t e, const char* what) {
   return e == cudaErrorMemoryAllocation ? MP_ERR_OOM : MP_ERR_CUDA;
 }
 
-mp_status new_index(const Geometry& g, const mp_op* op, bool host_pool, size_t work_bytes, cudaStream_t cs,
-                    InitList& init, mp_index_s** out, char** work);
-cudaError_t finish_index(mp_index_s* ix, cudaStream_t cs);
 void discard_index(mp_index_s* ix, cudaStream_t cs);
-mp_status alloc_hashes(mp_index_s* ix, cudaStream_t cs);
 
 // ---- experts in pinned host memory: segment pipeline -------------------------------------
 //
-// The family is walked in segments of consecutive blocks (segment_elems elements at most).  Two HBM staging buffers alternate: while the kernels of the caller's stream
-// work on segment s, segment s+1 is brought in on a side stream by a gather kernel that
-// reads the host experts over the host mapping — every expert block for the index pass,
-// only the planned (block, expert) pairs for the merge.  The planned blocks are scattered
-// (one copy call per run of consecutive blocks would mean ~10^5 calls per merge), and the
-// kernel reads them at the host link's rate.
+// The family is walked in segments of consecutive blocks (segment_elems elements at most).  Two HBM
+// staging buffers alternate: while the kernels of the caller's stream work on segment s, segment
+// s+1 is brought in on a side stream by a gather kernel that reads the host experts over the host
+// mapping — every expert block for the index pass, only the planned (block, expert) pairs for
+// the merge.  The planned blocks are scattered (one copy call per run of consecutive blocks would
+// mean ~10^5 calls per merge), and the kernel reads them at the host link's rate.
 
 namespace {
 
@@ -640,8 +636,8 @@ cudaError_t walk_segments(const IndexLaunch& p, const mp_index_s* ix, cudaStream
 cudaError_t index_host_pool(IndexLaunch p, const mp_index_s* ix, cudaStream_t cs) {
   cudaError_t e;
   if (p.win) {
-    // the windowed TIES catalog: the sample reads the host experts in place (32 vectors per
-    // block), one walk counts every pair's window, the finish marks the pairs whose threshold
+    // the windowed TIES catalog: the sample reads the host experts in place (8 to 128 vectors per
+    // block, by the size of its group), one walk counts every pair's window, the finish marks the pairs whose threshold
     // left it; a second walk, whose gathers and kernels do nothing unless some pair was
     // marked, bins the marked groups coarsely for the two-level select
     if ((e = launch_ties_window_begin(p, cs)) != cudaSuccess) return e;

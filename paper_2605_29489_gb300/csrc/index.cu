@@ -141,6 +141,7 @@ constexpr uint32_t kWinBins = kWinKeys + 2;  // + below + above
 // Qwen2.5-0.5B with 8 experts (items of 4 instead of 8 besides) 2.65 -> 1.88.  128 keys gave 1.59,
 // 0.92 and, with missed windows, 2.49 ms (items of 8), 192 keys 1.59, 0.93 and 2.44.
 constexpr uint32_t kWinNarrow = 160, kWinNarrowBlocks = 16;
+static_assert(kWinNarrow >= 1 && kWinNarrow <= kWinKeys, "the counts of a window fit its bins, and key - L + 1 16 bits");
 
 // the window in 16-bit lanes: 1 - L (added to the keys) and W + 1 (the clamp, the bin above)
 __device__ __forceinline__ void win_words(uint32_t win, uint32_t& neg, uint32_t& top) {
@@ -258,12 +259,13 @@ __device__ __forceinline__ void deltas(const uint4 r, const float* x0, float* d)
 // one address share a wavefront, and a predicate on the increment cost more than it saved (it
 // becomes a branch: 537 instead of 425 million warp instructions on a Llama layer).  Both keys
 // at once in 16-bit lanes:
-// one add and one clamp at zero and W + 1 (k - L + 1 lies in [-32383, 32768]; it wraps only for
-// the NaN key 0x7FFF at L = 0, whose bin the clamp still keeps in range and whose NaN the
-// statistics report), and one multiply-add for both byte addresses (h2 = h in both lanes, which
-// the caller keeps below 2^16 - 4 * 385).  An exact zero has key 0: below the window, or, with
-// L = 0, in key 0's bin, where it can only decide a threshold of key 0, the one that an
-// uncounted zero gives too.  Returns the two keys.
+// one add and one clamp at zero and W + 1 (L is at most 32768 - W, so k - L + 1 lies in
+// [W - 32767, 32768], from -32607 up in a narrow window; it wraps only for the NaN key 0x7FFF at
+// L = 0, whose bin the clamp still keeps in range and whose NaN the statistics report), and one
+// multiply-add for both byte addresses (h2 = h in both lanes, which the caller keeps below
+// 2^16 - 4 * 385).  An exact zero has key 0: below the window, or, with L = 0, in key 0's bin, where it
+// can only decide a threshold of key 0, the one that an uncounted zero gives too.  Returns the two
+// keys.
 __device__ __forceinline__ uint32_t ties_win2(float d0, float d1, uint32_t neg, uint32_t top, uint32_t h2) {
   const __nv_bfloat162 hb = __floats2bfloat162_rn(d0, d1);
   const uint32_t w = *reinterpret_cast<const uint32_t*>(&hb) & 0x7FFF7FFFu;
