@@ -132,15 +132,21 @@ constexpr uint32_t kWinKeys = 384;           // most keys of a window (three bin
 constexpr uint32_t kWinBins = kWinKeys + 2;  // + below + above
 
 // The window of one (expert, trim group), as ties_window_select leaves it: L | W << 16.
-// Groups of kWinNarrowBlocks blocks or more get a window of kWinNarrow keys (64 keys, a factor of
-// 1.4 or more, either side of the predicted bin of 32), smaller ones, whose sample is small, three
+// Groups of kWinNarrowBlocks blocks or more get a window of kWinNarrow keys (80 keys, a factor of
+// 1.45 or more, either side of the predicted bin of 32), smaller ones, whose sample is small, three
 // whole binades.  The increments are what bounds the pass: with three binades for every group
 // they took 5.5 wavefronts each and the LSU data pipe was 88 % busy (every block active); in a
-// narrow window most lanes share the bins below and above it (1.5 wavefronts).  Index of four
-// Llama layers with 4 experts 1.82 -> 1.61 ms, of two with every block active 1.26 -> 0.94, of
-// Qwen2.5-0.5B with 8 experts (items of 4 instead of 8 besides) 2.65 -> 1.88.  128 keys gave 1.59,
-// 0.92 and, with missed windows, 2.49 ms (items of 8), 192 keys 1.59, 0.93 and 2.44.
-constexpr uint32_t kWinNarrow = 160, kWinNarrowBlocks = 16;
+// narrow window most lanes share the bins below and above it (1.5 wavefronts).  A pair that misses
+// its window costs a pass over its group's blocks.  TIES index in ms by the keys of a narrow window
+// (four Llama layers with 4 experts, three seeds / two layers, every block active / Qwen2.5-0.5B with 8
+// experts, two seeds / with 16 / Qwen2.5-1.5B, 8 layers, with 16 / Llama-3-8B with 4):
+//    96: 1.61 1.56 1.42 / 0.91 / 1.59 1.83 / 3.30 / 3.98 / 12.95   (misses)
+//   128: 1.42 1.56 1.42 / 0.91 / 1.59 1.78 / 3.25 / 3.97 / 12.44   (a miss)
+//   160: 1.43 1.44 1.44 / 0.93 / 1.62 1.81 / 3.30 / 3.91 / 12.58
+//   192: 1.43 1.43 1.43 / 0.93 / 1.61 1.80 / 3.27 / 3.86 / 12.47
+//   256: 1.45 1.45 1.45 / 1.01 / 1.66 1.84 / 3.35 / 3.89 / 12.73
+//   384: 1.59 1.59 1.59 / 1.14 / 1.78 1.95 / 3.61 / 3.91 / 13.94
+constexpr uint32_t kWinNarrow = 192, kWinNarrowBlocks = 16;
 static_assert(kWinNarrow >= 1 && kWinNarrow <= kWinKeys, "the counts of a window fit its bins, and key - L + 1 16 bits");
 
 // the window in 16-bit lanes: 1 - L (added to the keys) and W + 1 (the clamp, the bin above)
