@@ -473,8 +473,18 @@ __device__ __forceinline__ void for_marked_pairs(const IndexLaunch& p, F f) {
   }
 }
 
-// the end of a fallback coarse pass: its last CTA makes the coarse select of the marked pairs
-// (few or none as a rule), which saves a launch that would return at once
+// The selects of the fallback ride in its passes, whose last CTA makes those of the marked pairs, up to
+// so many (expert, group) pairs; above they are launches of their own, with a warp for each pair.  A
+// launch that finds no pair marked costs 1 us; one CTA that selects them all costs more the more there
+// are, as with density 1 on deltas without zeros, where every pair misses its window.  Index of fp32
+// families in blocks of 4096, us, in the pass / own launches: 256 pairs, none marked 53 / 55, all 132 /
+// 86; 512 63 / 65, 185 / 104; 1,024 69 / 71, 279 / 110; 2,948 123 / 126, 818 / 234; 9,600 337 / 342,
+// 2551 / 686.
+constexpr uint64_t kPassSelectPairs = 512;
+inline uint32_t selects_in_pass(uint64_t pairs) { return pairs <= kPassSelectPairs ? 1u : 0u; }
+
+// the end of a fallback coarse pass: with few pairs its last CTA makes the coarse select of the marked
+// ones, which saves a launch that as a rule would return at once
 __device__ __forceinline__ void coarse_pass_end(const IndexLaunch& p, volatile int* s_last) {
   if (!p.select_in_pass || !last_cta<kIxThreads>(p.work + 2, s_last)) return;
   for_marked_pairs<kIxThreads / 32>(p, [&](uint64_t x) { coarse_select_pair(p, x); });
@@ -939,6 +949,7 @@ inline unsigned select_grid(uint64_t pairs) { return (unsigned)((pairs + kSelThr
 
 __global__ void __launch_bounds__(kSelThreads) ties_coarse_select(const IndexLaunch p) {
   kernel_begin();
+  if (p.miss && *p.miss == 0u) return;  // windowed thresholds: no pair needs it
   const uint64_t x = select_pair();
   if (x < (uint64_t)p.K * p.n_groups) coarse_select_pair(p, x);
 }
@@ -1009,13 +1020,14 @@ __global__ void __launch_bounds__(256) ties_fine_kernel(const IndexLaunch p) {
     }
     __syncthreads();  // the next item clears s_fine
   }
-  // the windowed catalog's fallback: the last CTA makes the fine select of the marked pairs
+  // the windowed catalog's fallback, with few pairs: the last CTA makes the fine select of the marked ones
   if (!p.select_in_pass || !last_cta<256>(p.work + 3, &s_last)) return;
   for_marked_pairs<8>(p, [&](uint64_t x) { fine_select_pair(p, x); });
 }
 
 __global__ void __launch_bounds__(kSelThreads) ties_fine_select(const IndexLaunch p) {
   kernel_begin();
+  if (p.miss && *p.miss == 0u) return;
   const uint64_t x = select_pair();
   if (x < (uint64_t)p.K * p.n_groups) fine_select_pair(p, x);
 }
@@ -1312,7 +1324,7 @@ cudaError_t ties_finish_t(const IndexLaunch& p, bool follows, cudaStream_t st) {
   uint64_t fgrid = (uint64_t)sms * (per_sm > 0 ? per_sm : 1);
   if (fgrid > p.n_blocks * G) fgrid = p.n_blocks * G;
   if (fgrid == 0) fgrid = 1;
-  if (!p.select_in_pass) {
+  if (!p.select_in_pass && !p.usum) {  // after masking the units' bins have given the coarse bin
     if ((e = launch_kernel(follows, ties_coarse_select, sgrid, kSelThreads, 0, st, p)) != cudaSuccess) return e;
     follows = true;
   }
@@ -1381,8 +1393,8 @@ cudaError_t launch_ties_t(const IndexLaunch& p, cudaStream_t st) {
   // two-level select for the pairs whose threshold left its window (a no-op when none did)
   const unsigned sgrid = select_grid((uint64_t)p.K * p.n_groups);
   if ((e = window_begin_t<BF16, KG>(p, st)) != cudaSuccess) return e;
-  IndexLaunch q = p;  // the selects of the fallback ride in its passes
-  q.select_in_pass = 1;
+  IndexLaunch q = p;
+  q.select_in_pass = selects_in_pass((uint64_t)p.K * p.n_groups);
   if (p.usum) {  // TIES after masking: one pass gives the units' bins and the coarse bins too
     if ((e = launch_pass<BF16, KG, kBinUnits>(p, true, G, n_items, sms, p.work, st)) != cudaSuccess) return e;
     if ((e = launch_kernel(true, ties_units_finish, sgrid, kSelThreads, 0, st, p)) != cudaSuccess) return e;
@@ -1468,7 +1480,7 @@ cudaError_t launch_ties_masked(const IndexLaunch& p, cudaStream_t st) {
     e = launch_kernel(p.follows, ties_units_sum<kUnitBins>, p.K * n_win, kUnitBins / 4, 0, st, p, n_win);
     if (e != cudaSuccess) return e;
     e = launch_kernel(true, ties_units_finish, select_grid((uint64_t)p.K * p.n_groups), kSelThreads, 0, st, p);
-    q.select_in_pass = 1;
+    q.select_in_pass = selects_in_pass((uint64_t)p.K * p.n_groups);
   } else {
     e = launch_kernel(p.follows, ties_units_sum<256>, p.K * n_win, 64, 0, st, p, n_win);
   }

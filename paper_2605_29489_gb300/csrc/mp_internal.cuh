@@ -320,7 +320,7 @@ struct IndexLaunch {
   unsigned long long* thr_reads;  // expert bytes read by the fine pass, or null
   // item counters of the dynamic scheduler, zeroed with the handle: work[0] of the catalog
   // pass, work[1] of the fallback pass; work[2] and work[3] count the CTAs of the fallback pass
-  // and of the fine pass that are done (the last one selects, when select_in_pass is set)
+  // and of the fine pass that are done (the last one selects, when select_in_pass is set: few pairs)
   unsigned long long* work;
   uint32_t select_in_pass;
   // the launch covers blocks [b_begin, b_end); expert pointers address element

@@ -1,12 +1,11 @@
 """TIES thresholds taken from predicted windows: both exact paths against the oracle.
 
 For device-resident experts the catalog predicts, from a sample of every block of each
-trim group, the coarse key bin that holds the threshold, and counts a window of 384 keys
-around it at full resolution.  A pair whose threshold lies
-outside its window takes the two-level select instead.  The families here are built so
-that the sample mispredicts (the blocks it weighs most carry deltas far larger than the
-others'), or so that the threshold is the key of an exact zero; thresholds,
-plans and merges must still be the oracle's, bit for bit.
+trim group, the bin of keys that holds the threshold, and counts a window of keys around it at
+full resolution.  A pair whose threshold lies outside its window takes the two-level select
+instead.  The families here are built so that the sample mispredicts (outliers exactly where it
+reads), so that every pair misses (density 1 on deltas without zeros), or so that the threshold is the
+key of an exact zero; thresholds, plans and merges must still be the oracle's, bit for bit.
 """
 import numpy as np
 import pytest
@@ -15,6 +14,7 @@ import torch
 import oracle
 from conftest import oracle_family
 from test_gpu_parity import run_case, upload
+from test_gpu_ties_sample import _sampled_vectors
 
 pytestmark = pytest.mark.gpu
 
@@ -51,35 +51,32 @@ def _with_deltas(fam, scale_of_block, seed):
 
 @pytest.mark.parametrize("host_experts", [False, True], ids=["device", "host_pool"])
 def test_sample_that_misses_the_threshold_falls_back_to_the_two_level_select(host_experts):
-    """The sample reads 32 vectors of every block longer than 4096 elements and every vector
-    of a shorter one, so short blocks weigh far more in it.  Here the short blocks (a
-    tensor's tail, small tensors) carry deltas about 10^4 times larger than the full
-    blocks: the sample predicts a window among the large keys while the threshold lies
-    among the small ones — for tensor 0 with per-tensor trim groups, and for the single
-    group of trim scope 1.  The two-level select must give the oracle's thresholds — also
-    with the experts in pinned host memory, where the sample reads them in place and the
-    fallback walk's gathers run only because a pair was marked."""
+    """Deltas of 0.5 in the vectors that the sample reads of tensors 0 and 1, deltas of 1e-3 everywhere
+    else: the sample predicts a window among the large keys while the threshold lies among the small
+    ones — for both tensors with per-tensor trim groups, and for the single group of trim
+    scope 1 (the positions are the same: the group's size class and its whole blocks' length
+    are).  The two-level select must give the oracle's thresholds — also with the experts in
+    pinned host memory, where the sample reads them in place and the fallback walk's gathers run
+    only because a pair was marked."""
     E = 65536
-    shapes = [2 * E + 4000, 16 * E] + [4096] * 20 + [70001]
+    shapes = [18 * E + 4000, 16 * E] + [4096] * 8 + [70001]
     fam = synth.custom(shapes, dtype=synth.BF16, block_elems=E, K=3, active_frac=0.5, name="window-miss")
-    _, bl, bt = fam.block_table()
-
-    def scale(i, b):
-        t = int(bt[b])
-        if t <= 1:
-            return 0.5 if bl[b] <= 4096 else 1e-4
-        if t < len(shapes) - 1:
-            return 0.5
-        return 1e-3 * (1 + i)
-
-    base, experts = _with_deltas(fam, scale, seed=11)
+    base, experts = _with_deltas(fam, lambda i, b: 1e-3 * (1 + i), seed=11)
+    bo, bl, bt = fam.block_table()
+    assert fam.n_blocks < 64  # one size class of the sample for tensors and the whole family
+    for i in range(fam.K):
+        x = _f32(base).copy()
+        for b in np.nonzero(bt <= 1)[0]:
+            for v in _sampled_vectors(int(b), int((bt == bt[b]).sum()), (int(bl[b]) + 7) // 8, E // 8):
+                s = slice(int(bo[b]) + 8 * v, min(int(bo[b]) + 8 * v + 8, int(bo[b] + bl[b])))
+                experts[i][s] = _bf16_bits(x[s] + 0.5)
     run_case(fam, base, experts, ("ties", "ties1"), [1.0, 0.5, 0.25], host_experts=host_experts)
-    # the threshold of tensor 0 lies among its small deltas, far below the sampled ones
+    # the thresholds of tensors 0 and 1 lie among their small deltas, far below the sampled ones
     mf, _, _ = upload(fam, base, experts, host_experts)
     idx = mp.mp_index_blocks(mf, mp.make_op(mp.MP_OP_TIES, lam=1.0, density=0.2))
     tau = mp.mp_index_stats(idx)[3]
     key_mid = int(_bf16_bits(np.float32([1e-2]))[0]) & 0x7FFF
-    assert np.all(tau[:, 0] < key_mid)
+    assert np.all(tau[:, :2] < key_mid)
     idx.free()
 
 
@@ -99,3 +96,23 @@ def test_threshold_at_the_key_of_an_exact_zero(density, host_experts):
     assert np.array_equal(tau, want)
     assert np.all(want == 0)
     idx.free()
+
+
+@pytest.mark.parametrize("n_tensors", [128, 129])
+def test_every_pair_misses_on_both_sides_of_the_selects_line(n_tensors):
+    """512 and 516 (expert, tensor) pairs: the selects of the marked pairs are made by the last CTA of
+    the fallback's passes, or by launches of their own.  With density 1 the threshold is the smallest key,
+    which no sample of a large tensor holds; after masking, a small budget leaves most thresholds
+    far below the window of the full deltas."""
+    fam = synth.custom([12000 + 7 * t for t in range(n_tensors)], dtype=synth.F32, block_elems=E, K=4, active_frac=1.0,
+                       name=f"all-miss-{n_tensors}")
+    base, experts = fam.host_arrays()
+    mf, _, _ = upload(fam, base, experts)
+    of = oracle_family(fam, base, experts)
+    for kind in (mp.MP_OP_TIES, mp.MP_OP_TIES_MASKED):
+        for density in (1.0, 0.9999, 0.2):
+            idx = mp.mp_index_blocks(mf, mp.make_op(kind, lam=1.0, density=density))
+            tau = mp.mp_index_stats(idx)[3]
+            idx.free()
+            assert np.array_equal(tau, oracle.ties_thresholds(of, float(np.float32(density)))), (kind, density)
+    run_case(fam, base, experts, ("ties", "ties_masked"), [0.03, 0.3])
