@@ -28,7 +28,7 @@ def test_hostpool_parity_small_families(make):
 
 
 def test_hostpool_multi_segment_matches_oracle_and_device_path(pool):  # noqa: F811
-    """Qwen2.5-0.5B shapes (494M params, 16 segments), K=8: TA and TIES against the oracle's
+    """Qwen2.5-0.5B shapes (494M params, some 80 segments), K=8: TA and TIES against the oracle's
     catalog, thresholds and plans, sampled merged blocks, and the device-resident run"""
     fam = synth.qwen25_05b()
     K = fam.K

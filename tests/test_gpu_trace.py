@@ -1,7 +1,7 @@
 """Device-time trace of the calls (mp_trace_start / mp_trace_stop).
 
 On device-resident inputs a traced index, plan and merge give one range each, in stream
-order.  On a host-resident pool (Qwen2.5-0.5B shapes, 16 segments) every segment adds a
+order.  On a host-resident pool (Qwen2.5-0.5B shapes, some 80 segments with 8 experts) every segment adds a
 gather range on the side stream and a kernel range on the caller's stream; the trace then
 shows the pipeline's two dependencies: a segment's kernels start after its gather ends
 (the staging buffer is full), and the gather of segment s + 2 starts after the kernels of
