@@ -53,9 +53,9 @@
  *  - Device memory for handles and scratch comes, in stream order, from a pool of the
  *    library's own on each device, which keeps at most 256 MiB of unused memory between
  *    calls (mp_trim gives it back, and an allocation of the same process that would fail for want
- *    of memory is served from it).  A caller that has set a memory pool of its own
- *    on the device (cudaDeviceSetMemPool) has the library use that one instead; under stream
- *    capture the memory belongs to the graph.
+ *    of memory is served from it).  A memory pool that the caller has set on the device
+ *    (cudaDeviceSetMemPool) is not used, except under stream capture, where the memory belongs
+ *    to the graph.
  *  - On an error return no handle is produced and *out is set to NULL; the
  *    contents of a merge output buffer are then unspecified.
  *  - mp_last_error() returns a thread-local message for the last failure.

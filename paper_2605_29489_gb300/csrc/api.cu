@@ -44,31 +44,23 @@ bool inject_fault(int kind) {
 // staging about 1.4 ms).  This pool keeps at most kPoolKeep bytes of unused memory between
 // calls; what is above goes back at the next wait, and all of it when an allocation of the library
 // fails, on mp_trim, and when another allocation of the process needs it (the driver's own retry:
-// cudaMalloc got 64 of 96 MiB kept here and not reported as free).  A caller that has made
-// a pool of its own the device's current one has its memory used instead, as before there was this
-// one.  cudaMallocFromPoolAsync orders every block's reuse by stream, from any thread.
+// cudaMalloc got 64 of 96 MiB kept here and not reported as free).  A pool that the caller has set on
+// the device is not looked for: with that query made, a profiler's replay of a kernel that uses memory of
+// this pool ended in a failed launch.  cudaMallocFromPoolAsync orders every block's reuse by stream,
+// from any thread.
 constexpr uint64_t kPoolKeep = 256ull << 20;
 constexpr int kPoolDevices = 64;
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[kPoolDevices];          // the library's
-cudaMemPool_t g_default_pool[kPoolDevices];  // the device's, which never changes
+cudaMemPool_t g_pool[kPoolDevices];
 
-// the current device's pool, created on first use; null where there is none, or where the caller
-// has set a memory pool of its own
+// the current device's pool, created on first use; null where there is none
 cudaMemPool_t device_pool() {
   int dev = -1;
-  cudaMemPool_t cur = nullptr;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices ||
-      cudaDeviceGetMemPool(&cur, dev) != cudaSuccess) {
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices) {
     cudaGetLastError();
     return nullptr;
   }
   std::lock_guard<std::mutex> lk(g_pool_mu);
-  if (!g_default_pool[dev] && cudaDeviceGetDefaultMemPool(&g_default_pool[dev], dev) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  if (cur != g_default_pool[dev]) return nullptr;
   if (!g_pool[dev]) {
     cudaMemPoolProps props;
     memset(&props, 0, sizeof(props));

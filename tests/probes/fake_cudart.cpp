@@ -34,10 +34,10 @@ std::map<void*, size_t> g_mem;
 std::vector<std::string> g_launched;
 size_t g_limit = (size_t)280 << 30, g_used = 0, g_largest = ~(size_t)0, g_pool_kept = 0;
 unsigned long long g_most_pending_at_free = 0;
-unsigned g_from_pool = 0, g_from_current = 0, g_trims = 0, g_copies = 0;
+unsigned g_trims = 0, g_copies = 0;
 int g_host_blocks = 0, g_capturing = 0;
-int g_own_pool = 0, g_cluster_room = 1;
-int g_pool_obj[3];  // the default pool, the caller's, the library's
+int g_cluster_room = 1;
+int g_pool_obj;  // the library's pool
 cudaError_t g_last = cudaSuccess;
 
 // kernels register before this file's own objects are made
@@ -100,9 +100,8 @@ void fake_reset() {
   g_limit = (size_t)280 << 30;
   g_largest = ~(size_t)0;
   g_most_pending_at_free = 0;
-  g_from_pool = g_from_current = g_trims = g_copies = 0;
+  g_trims = g_copies = 0;
   g_capturing = 0;
-  g_own_pool = 0;
   g_cluster_room = 1;
   g_launched.clear();
 }
@@ -110,13 +109,10 @@ void fake_memory(size_t limit, size_t largest) { g_limit = g_used + limit, g_lar
 unsigned long long fake_used() { return g_used; }
 unsigned long long fake_pending() { return pending(); }
 unsigned long long fake_most_pending_at_free() { return g_most_pending_at_free; }
-unsigned fake_from_pool() { return g_from_pool; }
-unsigned fake_from_current() { return g_from_current; }
 unsigned fake_trims() { return g_trims; }
 unsigned fake_copies() { return g_copies; }
 int fake_host_blocks() { return g_host_blocks; }
 void fake_capturing(int on) { g_capturing = on; }
-void fake_callers_pool(int on) { g_own_pool = on; }
 void fake_cluster_room(int clusters) { g_cluster_room = clusters; }
 int fake_launched(const char* what) {
   int n = 0;
@@ -209,29 +205,19 @@ cudaError_t cudaMemGetInfo(size_t* fr, size_t* total) {
   *total = g_limit;
   return cudaSuccess;
 }
-cudaError_t cudaDeviceGetDefaultMemPool(cudaMemPool_t* p, int) {
-  *p = (cudaMemPool_t)&g_pool_obj[0];
-  return cudaSuccess;
-}
-cudaError_t cudaDeviceGetMemPool(cudaMemPool_t* p, int) {
-  *p = (cudaMemPool_t)&g_pool_obj[g_own_pool ? 1 : 0];
-  return cudaSuccess;
-}
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const struct cudaMemPoolProps*) {
-  *p = (cudaMemPool_t)&g_pool_obj[2];
+  *p = (cudaMemPool_t)&g_pool_obj;
   return cudaSuccess;
 }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, enum cudaMemPoolAttr, void*) { return cudaSuccess; }
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t p, size_t) {
-  if (p == (cudaMemPool_t)&g_pool_obj[2]) ++g_trims;
+  if (p == (cudaMemPool_t)&g_pool_obj) ++g_trims;
   return cudaSuccess;
 }
 cudaError_t cudaMallocAsync(void** p, size_t bytes, cudaStream_t) {
-  ++g_from_current;
   return take(p, bytes);
 }
 cudaError_t cudaMallocFromPoolAsync(void** p, size_t bytes, cudaMemPool_t, cudaStream_t) {
-  ++g_from_pool;
   return take(p, bytes);
 }
 cudaError_t cudaFree(void* p) { return give(p); }

@@ -190,20 +190,7 @@ def test_larger_histograms_only_where_the_caller_keeps_nearly_all_of_the_free_me
         assert rt.fake_used() - before > 40_000 * 640 * 4
 
 
-# ---- whose memory the library takes -----------------------------------------------------------
-
-def test_a_pool_that_the_caller_has_set_is_used(rt):
-    fam, out = family()
-    mp.mp_index_blocks(fam, TA(3), stream=S1).free()
-    assert rt.fake_from_pool() > 0 and rt.fake_from_current() == 0  # the library's own
-    rt.fake_reset()
-    rt.fake_callers_pool(1)
-    mp.mp_index_blocks(fam, TA(3), stream=S1).free()
-    assert rt.fake_from_pool() == 0 and rt.fake_from_current() > 0
-    rt.fake_callers_pool(0)
-    mp.mp_index_blocks(fam, TA(3), stream=S1).free()
-    assert rt.fake_from_pool() > 0
-
+# ---- the memory that the library keeps --------------------------------------------------------
 
 def test_trim_gives_the_kept_memory_back(rt):
     fam, out = family()
