@@ -125,12 +125,13 @@ def test_kept_memory_is_within_the_callers_reach():
     mp.mp_index_blocks(mf, op).free()
     torch.cuda.synchronize()
     kept = free - torch.cuda.mem_get_info()[0]
-    assert 64 << 20 < kept <= 256 << 20
+    # a catalog of 98 MB, mapped in pieces of 32 MiB of which one or two may have been there before
+    assert 32 << 20 <= kept <= 256 << 20
     hold = torch.empty(free - kept + (16 << 20), dtype=torch.uint8, device="cuda")  # more than is reported free
     del hold
     torch.cuda.empty_cache()
     mp.mp_index_blocks(mf, op).free()
     torch.cuda.synchronize()
-    assert free - torch.cuda.mem_get_info()[0] > 64 << 20
+    assert free - torch.cuda.mem_get_info()[0] >= 32 << 20
     mp.mp_trim()
     assert free - torch.cuda.mem_get_info()[0] <= 4 << 20
