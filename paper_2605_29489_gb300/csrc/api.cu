@@ -393,20 +393,19 @@ cudaError_t Event::sync() const {
   return r;
 }
 
-// from so many remembered calls on, the runtime is asked which of them are done
-constexpr size_t kUsersKept = 16;
 
 void Users::add(const Event& e) {
   std::lock_guard<std::mutex> lk(mu);
   auto forget = [&](auto is_done) { ev.erase(std::remove_if(ev.begin(), ev.end(), is_done), ev.end()); };
   forget([&](const Event& x) { return x == e || x.over(); });
-  if (ev.size() >= kUsersKept) {
+  if (ev.size() >= ask) {
     // an event query is refused while another thread captures in global mode
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
     forget([](const Event& x) { return cudaEventQuery(x.get()) == cudaSuccess; });
     cudaGetLastError();  // of those that are not done
     cudaThreadExchangeStreamCaptureMode(&mode);
+    ask = std::max(kUsersAsk, 2 * ev.size());  // with many in flight not for every call again
   }
   try {
     ev.push_back(e);
@@ -1537,7 +1536,7 @@ void mp_free(void* handle) {
   } else if (magic == kMagicManifest) {
     mp_manifest_s* mf = static_cast<mp_manifest_s*>(handle);
     wait_handle(mf->done, mf->captured);
-    if (mf->valid_done) mf->valid_done.sync();
+    if (mf->valid_done) wait_handle(mf->valid_done, mf->valid_captured);
     dev_free(mf->valid_mem);
     dev_free(mf->mem);
     pin_put(mf->h_realized, (size_t)kCounterSlots * mf->K * 8 + 64 + 16 + 16);

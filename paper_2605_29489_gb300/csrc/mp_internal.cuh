@@ -93,8 +93,10 @@ class Users {
   void wait();
 
  private:
+  static constexpr size_t kUsersAsk = 16;
   std::mutex mu;
   std::vector<Event> ev;
+  size_t ask = kUsersAsk;  // from so many remembered calls on, the runtime is asked which of them are done
 };
 
 }  // namespace mp

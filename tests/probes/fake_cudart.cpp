@@ -35,7 +35,7 @@ std::vector<std::string> g_launched;
 size_t g_limit = (size_t)280 << 30, g_used = 0, g_largest = ~(size_t)0, g_pool_kept = 0;
 unsigned long long g_most_pending_at_free = 0;
 unsigned g_trims = 0, g_copies = 0;
-int g_host_blocks = 0, g_capturing = 0;
+int g_host_blocks = 0, g_capturing = 0, g_events = 0, g_queries = 0;
 int g_cluster_room = 1;
 int g_pool_obj;  // the library's pool
 cudaError_t g_last = cudaSuccess;
@@ -112,6 +112,8 @@ unsigned long long fake_most_pending_at_free() { return g_most_pending_at_free; 
 unsigned fake_trims() { return g_trims; }
 unsigned fake_copies() { return g_copies; }
 int fake_host_blocks() { return g_host_blocks; }
+int fake_events() { return g_events; }
+int fake_queries() { return g_queries; }
 void fake_capturing(int on) { g_capturing = on; }
 void fake_cluster_room(int clusters) { g_cluster_room = clusters; }
 int fake_launched(const char* what) {
@@ -278,11 +280,13 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, enum cudaStreamCaptureStatus* c)
 cudaError_t cudaThreadExchangeStreamCaptureMode(enum cudaStreamCaptureMode*) { return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
   *e = (cudaEvent_t) new Event();
+  ++g_events;
   return cudaSuccess;
 }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { return cudaEventCreateWithFlags(e, 0); }
 cudaError_t cudaEventDestroy(cudaEvent_t e) {
   delete (Event*)e;
+  --g_events;
   return cudaSuccess;
 }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
@@ -296,6 +300,7 @@ cudaError_t cudaEventSynchronize(cudaEvent_t e) {
 }
 cudaError_t cudaEventQuery(cudaEvent_t e) {
   Event* v = (Event*)e;
+  ++g_queries;
   return !v->s || v->s->done >= v->upto ? cudaSuccess : cudaErrorNotReady;
 }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) {

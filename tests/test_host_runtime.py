@@ -111,7 +111,8 @@ def test_freeing_an_index_waits_for_plans_hashes_and_validation(rt):
 
 
 def test_one_index_used_by_many_merges_keeps_few_events(rt):
-    """a long-lived index: the calls that are done are forgotten"""
+    """a long-lived index: calls that are done are forgotten, and with many in flight the runtime is not
+    asked about all of them again for every call"""
     fam, out = family()
     idx = mp.mp_index_blocks(fam, TA(3), stream=S1)
     for _ in range(300):
@@ -119,9 +120,18 @@ def test_one_index_used_by_many_merges_keeps_few_events(rt):
         man = mp.mp_merge(fam, idx, plan, out, stream=S2)
         for h in (man, plan):
             h.free()
+    n = rt.fake_events()
+    assert n <= 64
+    plan = mp.mp_plan(idx, TA(3), 1 << 20, stream=S1)
+    asked = rt.fake_queries()
+    mans = [mp.mp_merge(fam, idx, plan, out, stream=S2) for _ in range(1000)]  # none of them runs
+    assert rt.fake_queries() - asked <= 2 * 2 * 2000  # two handles, each asked at 16, 32, 64, ...
     used = rt.fake_used()
     idx.free()
+    plan.free()
     assert rt.fake_used() < used and rt.fake_most_pending_at_free() == 0
+    for m in mans:
+        m.free()
 
 
 # ---- a planner that gives up ------------------------------------------------------------------
